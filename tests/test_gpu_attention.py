@@ -103,3 +103,33 @@ def test_attention_ignores_memory_it_never_wrote():
     _run_case(32, 32, [412], [100], 700, seed=3, poison=True)
     _run_case(28, 4, [300, 17], [40, 9], 500, seed=4, poison=True)
     _run_case(8, 2, [129, 5, 250], [3, 0, 60], 320, attn_impl=1, seed=5, poison=True)
+
+
+@pytest.mark.parametrize("hq,hkv,F,rows", [
+    (32, 32, [525 + 3 * b for b in range(7)], [50] * 7),      # five and more key tiles per CTA, the last cached one ragged
+    (32, 32, [490, 493], [43, 38]),                            # the same on clusters of 2
+])
+def test_attention_repeats_bit_for_bit_with_ragged_tiles(hq, hkv, F, rows):
+    """The rows of a ragged V tile past the last key are cleared in shared memory; done while the stage still waited for an
+    earlier tile, the clear took rows of that tile's V (one launch in four on the first case).  Repeated launches over several
+    layers (more K/V than the L2 cache holds) must give the first launch's bits."""
+    from paper_2603_05454_b200 import LSPDecoder, SchedCfg
+    dh, B, L = 128, len(rows), 8
+    sh = S.ModelShape(L, 128 * hq, hq, hkv, dh, 64, 256, dtype="bf16")
+    z = lambda *s: torch.zeros(*s, dtype=torch.bfloat16, device=DEV)
+    d = sh.d_model
+    layer = dict(attn_norm=z(d), w_qkv=z((hq + 2 * hkv) * dh, d), w_o=z(d, hq * dh), ffn_norm=z(d), w_gate=z(64, d), w_up=z(64, d),
+                 w_down=z(d, 64))
+    dec = LSPDecoder(sh, dict(embed=z(256, d), w_head=z(256, d), final_norm=z(d), layers=[layer] * L), SchedCfg(), B, max(F) + max(rows),
+                     device=DEV)
+    M, bf = int(sum(rows)), torch.bfloat16
+    q, kn, vn = (S.normal((M, h * dh), 0, i, 1.0, bf, DEV) for i, h in ((1, hq), (2, hkv), (3, hkv)))
+    dec.kv_view().normal_(generator=torch.Generator(device=DEV).manual_seed(0))
+    out = torch.empty(M, hq * dh, dtype=bf, device=DEV)
+    first = [dec.op_attention(l, q, kn, vn, out, F, rows).clone() for l in range(L)]
+    wrong = 0
+    for _ in range(100):
+        for l in range(L):
+            wrong += not torch.equal(dec.op_attention(l, q, kn, vn, out, F, rows), first[l])
+    dec.close()
+    assert wrong == 0, f"{wrong} of {100 * L} launches differ"
