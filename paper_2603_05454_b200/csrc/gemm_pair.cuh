@@ -1,0 +1,442 @@
+// bf16 GEMM on pairs of SMs (tcgen05.mma.cta_group::2), for passes of more than 256 activation rows.
+//
+//   acc[m, c] = sum_k A[m, k] * Wt[c, k]        operands and fused epilogues as k_gemm_stream (gemm_umma.cuh)
+//
+// With several row groups a layer GEMM is bound by the tensor pipe.  One SM working alone on a 128 x 256 tile takes in
+// 48 KB per 64-element K atom; a cluster of two CTAs computing one 256 x BN tile takes in 32 KB per SM at BN = 256: each
+// loads its own 128 activation rows and one half of the weight tile's BN rows (the MMA reads the other half from its peer)
+// and keeps its own 128 accumulator rows in tensor memory.
+//   * What bounds it otherwise is the producer and the issuer, one thread each: a turn of the stage ring (wait, arm, copies,
+//     MMAs, commit) costs 300 ns whatever its size.  So a stage holds two K atoms and each operand of it is ONE copy (a 4-D
+//     tensor map, see umma_map4), the MMAs of a stage share one commit, and whole warps run the loops with one elected
+//     thread issuing (a lane branch around tcgen05.mma costs about 130 cycles per instruction, elect.sync 48 to 88).  With
+//     one atom per stage and a copy per box the same kernel ran 4096 x 4096 outputs (K 4096) in 104 us, so 98, and
+//     512 x 4096 in 25.3, so 17.8.
+//   * Persistent: pair p takes tiles p, p + P, ...; the accumulators are double-buffered (2 x BN of 512 columns), so the
+//     epilogue of a tile overlaps the next tile's MMAs.
+//   * BN is a run-time multiple of 32 (64 for the rotary epilogue), chosen so that the last wave of tiles is full (see
+//     pair_width).
+// Measured (B200, back to back, weights from a ring larger than L2; row-major k_gemm_stream before -> now, us):
+//   rows    12288 x 4096   4096 x 4096   2 x 12288 x 4096 SwiGLU   4096 x 12288
+//    512      58 -> 42      31 -> 17            111 -> 76          56 -> 45
+//   1000     104 -> 74      41 -> 28            153 -> 139          86 -> 75
+//   4096     313 -> 271     129 -> 99            559 -> 512         311 -> 297
+//   8240     646 -> 551     260 -> 202           1205 -> 1050        657 -> 596
+//   * The weight tile's two halves come from the two tensors / row ranges whose columns a fused epilogue pairs (gate and
+//     up, rotate-half partners), so CTA 0 always loads the first and CTA 1 the second of the pair.
+//   * Eight epilogue warps: two per quarter of the accumulator rows, each taking half of the 16-column chunks.  The
+//     residual epilogue fetches its rows of x while it waits for the accumulators.
+// Warp roles (320 threads): warp 0 = TMA producer, warp 1 = TMEM allocator and, in the pair's first CTA, MMA issuer,
+// warps 2..9 = epilogue.  Every wait is bounded; on expiry the kernel records (code, site) in the status word, drains and
+// returns.
+#pragma once
+#include "gemm_stream.cuh"
+
+namespace lsp {
+
+constexpr int PR_THREADS = 320;
+constexpr int PR_MAX_STAGES = 8;
+constexpr int PR_ROWS = 256;               // activation rows per tile
+
+struct PairArgs {
+  int M;            // activation rows
+  int n_pairs;      // dual: pair indices; plain: output columns
+  int n_tiles;      // column tiles
+  int row_groups;   // groups of 256 activation rows
+  int band;         // row groups per band: tiles are ordered band by band, within a band column tile by column tile
+  int kc;           // chunks of 128 K elements (two atoms; the last one may be half empty: zero-filled)
+  int bn;           // tile width
+  int unit;         // rotary epilogue: weight rows per copy when a half tile is not made of whole head halves (else 0)
+  int stages;
+  unsigned* status;
+};
+
+// One box of a 4-D map (umma_map4) into this CTA's shared memory; the bytes are counted on the barrier `bar` (a
+// shared::cluster address: the barrier of the pair's first CTA).
+__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* map, int r0, int blk, int a0, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+      ::"r"(dst), "l"(map), "r"(0), "r"(r0), "r"(blk), "r"(a0), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void tc_mma_f16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                                uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// arrives at the barrier at this offset in both CTAs of the pair once the issued MMAs have completed
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+               "h"((uint16_t)3)
+               : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+template <typename Epi>
+__global__ void __launch_bounds__(PR_THREADS, 1)
+k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b0,
+            const __grid_constant__ CUtensorMap map_b1, PairArgs args, Epi epi) {
+  extern __shared__ uint8_t smem_raw[];
+  pdl_release();
+  constexpr int A_ATOM = UM_BM * 128;                     // this CTA's 128 activation rows of one K atom
+  constexpr uint32_t TMEM_COLS = 512;
+  constexpr bool kRope = std::is_same<Epi, EpiQKVRope<bf16>>::value;
+  const int BN = args.bn, HALF = BN / 2;
+  const int B_ATOM = HALF * 128;
+  const int STAGE_BYTES = 2 * (A_ATOM + B_ATOM);          // two K atoms
+  const int S = args.stages;
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)S * STAGE_BYTES);
+  // bars[0..S) full (used in the first CTA), [S..2S) empty, [2S..2S+2) accumulators full, [2S+2..2S+4) accumulators empty
+  // (used in the first CTA)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 4);
+  volatile uint32_t* abort_flag = tmem_slot + 1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t bar_base = smem_u32(bars);
+  auto full_bar = [&](int s) { return bar_base + 8u * s; };
+  auto empty_bar = [&](int s) { return bar_base + 8u * (S + s); };
+  auto accf_bar = [&](int b) { return bar_base + 8u * (2 * S + b); };
+  auto acce_bar = [&](int b) { return bar_base + 8u * (2 * S + 2 + b); };
+
+  const int rank = (int)cluster_ctarank();
+  const int P = gridDim.x >> 1, pair = blockIdx.x >> 1;
+  const int T = args.n_tiles * args.row_groups;
+  const int my_tiles = (T - pair + P - 1) / P;            // the host launches at most T pairs
+  const int kc = args.kc;
+  const int n_units = my_tiles * kc;
+  // i-th tile of this pair -> column tile and row group
+  auto tile_of = [&](int i, int& tile, int& rg) {
+    const int t = pair + i * P;
+    const int per_band = args.band * args.n_tiles;
+    const int b = t / per_band, r = t - b * per_band;
+    const int rows = min(args.band, args.row_groups - b * args.band);
+    tile = r / rows;
+    rg = b * args.band + r % rows;
+  };
+  const uint32_t full0 = cluster_map(bar_base, 0);        // the first CTA's full barriers, in the cluster's window
+  const CUtensorMap* map_b = rank ? &map_b1 : &map_b0;    // this CTA's half of the weight tile
+  auto load_weights = [&](int tile, int c, int s) {
+    const uint32_t sb = smem_u32(smem + (size_t)s * STAGE_BYTES) + 2 * A_ATOM;
+    if constexpr (kRope) {
+      // blocks of the map are head halves; a half tile is HALF consecutive pair indices
+      const int j = tile * HALF;
+      if (args.unit == 0) {
+        tma_load_4d_pair(sb, map_b, 0, j / epi.half, 2 * c, full0 + 8u * s);
+      } else {
+        for (int b = 0; b < HALF; b += args.unit)
+          for (int a = 0; a < 2; ++a)
+            tma_load_4d_pair(sb + a * B_ATOM + b * 128, map_b, (j + b) % epi.half, (j + b) / epi.half, 2 * c + a, full0 + 8u * s);
+      }
+    } else {
+      tma_load_4d_pair(sb, map_b, Epi::kDual ? tile * HALF : tile * BN + rank * HALF, 0, 2 * c, full0 + 8u * s);
+    }
+  };
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(full_bar(s), 1);
+      mbar_init(empty_bar(s), 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(accf_bar(b), 1);
+      mbar_init(acce_bar(b), 16);           // eight epilogue warps of each CTA
+    }
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();                            // both CTAs' barriers and tensor memory are set up
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  if (warp == 0) {
+    // ---------------- TMA producer ----------------
+    const int n_pre = n_units < S ? n_units : S;
+    int tile = 0, rg = 0, c = 0, i = 0;
+    tile_of(0, tile, rg);
+    // weights are never written by any kernel: the first stages' are requested while the preceding kernel still runs
+    {
+      int t2 = tile, rg2 = rg, c2 = 0, i2 = 0;
+      for (int it = 0; it < n_pre; ++it) {
+        if (elect_one()) {
+          if (rank == 0) mbar_expect_tx(full_bar(it), 2 * STAGE_BYTES);
+          load_weights(t2, c2, it);
+        }
+        __syncwarp();
+        if (++c2 == kc) { c2 = 0; if (++i2 < my_tiles) tile_of(i2, t2, rg2); }
+      }
+    }
+    pdl_wait();
+    int s = 0, issued = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int it = 0; it < n_units; ++it) {
+      if (it >= n_pre) {
+        ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, abort_flag));
+        if (!ok) {
+          if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 41u; }
+          break;
+        }
+      }
+      if (elect_one()) {
+        if (it >= n_pre) {
+          if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE_BYTES);
+          load_weights(tile, c, s);
+        }
+        tma_load_4d_pair(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_a, rg * PR_ROWS + rank * UM_BM, 0, 2 * c, full0 + 8u * s);
+      }
+      __syncwarp();
+      ++issued;
+      if (++s == S) { s = 0; ph ^= 1u; }
+      if (++c == kc) { c = 0; if (++i < my_tiles) tile_of(i, tile, rg); }
+    }
+    // do not leave while copies may still be landing: the first CTA's barriers count both CTAs' copies, and the cluster
+    // barrier at the end holds the second CTA until the first has seen them
+    volatile uint32_t no_abort = 0;
+    if (rank == 0) {
+      for (int it = issued > S ? issued - S : 0; it < issued; ++it) mbar_wait(full_bar(it % S), (uint32_t)(it / S) & 1u, &no_abort);
+    }
+    if (!ok) {                             // after a failure the peer may not have counted these copies: let them land
+      const uint64_t t0 = globaltimer_ns();
+      while (globaltimer_ns() - t0 < 1000000ull) {}
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer (first CTA; the whole warp waits, one elected thread issues) ----------------
+    if (rank == 0) {
+      const uint32_t idesc = (make_idesc(BN) & ~(31u << 24)) | ((uint32_t)(PR_ROWS >> 4) << 24);
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int i = 0; i < my_tiles && ok; ++i) {
+        const int buf = i & 1, use = i >> 1;
+        if (use >= 1) ok = mbar_wait(acce_bar(buf), (uint32_t)(use - 1) & 1u, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) {
+          if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 42u; }
+          break;
+        }
+        tc_fence_after();
+        const uint32_t d = tmem_base + (uint32_t)(buf * 256);
+        for (int c = 0; c < kc; ++c) {
+          ok = mbar_wait(full_bar(s), ph, abort_flag);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) {
+            if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 43u; }
+            break;
+          }
+          tc_fence_after();
+          const uint32_t sa = smem_u32(smem + (size_t)s * STAGE_BYTES);
+          if (elect_one()) {
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+              const uint64_t da = make_smem_desc(sa + a * A_ATOM), db = make_smem_desc(sa + 2 * A_ATOM + a * B_ATOM);
+#pragma unroll
+              for (int k = 0; k < 4; ++k)
+                tc_mma_f16_pair(d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (c | a | k) != 0 ? 1u : 0u);
+            }
+            tc_commit_pair(empty_bar(s));
+            if (c == kc - 1) tc_commit_pair(accf_bar(buf));
+          }
+          __syncwarp();
+          if (++s == S) { s = 0; ph ^= 1u; }
+        }
+      }
+    }
+  } else {
+    // ---------------- epilogue ----------------
+    pdl_wait();
+    const int q = warp & 3;                                       // the quarter of tensor-memory lanes this warp may read
+    const int h = (warp - 2) >> 2;                                // column half
+    const int r_in = q * 32 + lane;
+    const int CH = Epi::kDual ? HALF : BN;                        // pair indices (dual) or columns (plain) per tile
+    const int nch = CH >> 4, mid = (nch + 1) >> 1;
+    const int ch_lo = h ? mid : 0, ch_hi = h ? nch : mid;
+    const uint32_t acce0 = cluster_map(acce_bar(0), 0);
+    for (int i = 0; i < my_tiles; ++i) {
+      const int buf = i & 1, use = i >> 1;
+      int tile, rg;
+      tile_of(i, tile, rg);
+      const int m = rg * PR_ROWS + rank * UM_BM + r_in;
+      const int j0 = tile * CH;
+      const bool live = m < args.M;
+      uint4 xr[16];
+      if constexpr (std::is_same<Epi, EpiResidual<bf16>>::value) {
+        // this thread's part of the residual rows, fetched while the MMAs run
+        const uint4* xp = reinterpret_cast<const uint4*>(epi.x + (size_t)m * epi.ld + j0 + ch_lo * 16);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if (live && ch_lo + k < ch_hi && j0 + (ch_lo + k) * 16 < args.n_pairs) {
+            xr[2 * k] = xp[2 * k];
+            xr[2 * k + 1] = xp[2 * k + 1];
+          }
+        }
+      }
+      if (!mbar_wait(accf_bar(buf), (uint32_t)use & 1u, abort_flag)) {
+        if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 44u; }
+        break;
+      }
+      tc_fence_after();
+      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256);
+      if constexpr (std::is_same<Epi, EpiResidual<bf16>>::value) {
+        uint4* xp = reinterpret_cast<uint4*>(epi.x + (size_t)m * epi.ld + j0 + ch_lo * 16);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if (ch_lo + k < ch_hi) {                                // uniform per warp
+            float a[16];
+            tc_ld16(t_row + (uint32_t)((ch_lo + k) * 16), a);
+            if (live && j0 + (ch_lo + k) * 16 < args.n_pairs) {
+#pragma unroll
+              for (int hh = 0; hh < 2; ++hh) {
+                float x[8];
+                unpack8(xr[2 * k + hh], x);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) x[e] += a[8 * hh + e];
+                xp[2 * k + hh] = pack8(x);
+              }
+            }
+          }
+        }
+      } else {
+        Top2 red = top2_empty();
+        auto consume = [&](int ch, float (&a0)[16], float (&a1)[16]) {
+          const int j = j0 + ch * 16;
+          if constexpr (Epi::kReduce) top2_push16(red, a0, j, epi);
+          else if (live && j < args.n_pairs) epi16(epi, m, j, a0, a1);
+        };
+        auto request = [&](int ch, float (&a0)[16], float (&a1)[16]) {
+          tc_ld16_nowait(t_row + (uint32_t)(ch * 16), a0);
+          if (Epi::kDual) tc_ld16_nowait(t_row + (uint32_t)(HALF + ch * 16), a1);
+        };
+        // the next chunk's tensor-memory loads are in flight while this one is converted and stored
+        float p0[16], p1[16], q0[16], q1[16];
+        if (ch_lo < ch_hi) request(ch_lo, p0, p1);
+#pragma unroll 1
+        for (int ch = ch_lo; ch < ch_hi; ch += 2) {
+          tc_wait_ld();
+          tc_pin16(p0);
+          if (Epi::kDual) tc_pin16(p1);
+          if (ch + 1 < ch_hi) request(ch + 1, q0, q1);
+          consume(ch, p0, p1);
+          if (ch + 1 < ch_hi) {
+            tc_wait_ld();
+            tc_pin16(q0);
+            if (Epi::kDual) tc_pin16(q1);
+            if (ch + 2 < ch_hi) request(ch + 2, p0, p1);
+            consume(ch + 1, q0, q1);
+          }
+        }
+        if constexpr (Epi::kReduce) {
+          if (live) epi.part[(size_t)m * epi.n_tiles + 2 * tile + h] = red;      // one partial per column half
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(acce0 + 8u * buf);
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();          // nobody leaves while its peer may still read its shared memory or signal its barriers
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+  }
+}
+
+// ---- host side ------------------------------------------------------------------------------------------------
+// Tile width.  A tile costs about bn + 44 in units of one column's MMA time (the constant: what a tile costs whatever its
+// width; per round of 4096 K elements 11.4 / 13.5 / 16.1 / 18.9 / 21.8 / 24.6 us at 96 / 128 / 160 / 192 / 224 / 256), and the launch takes as many rounds as its fullest pair, so the width that gives the least rounds x (bn + 44)
+// wins.  step: widths are multiples of 32, or 64 for the rotary epilogue (a half tile is then made of whole 32-row boxes
+// inside one head half).
+inline int pair_width(int M, int cols, int n_pairs_of_sms, int step) {
+  const long rg = (M + PR_ROWS - 1) / PR_ROWS;
+  int best = 256;
+  double best_cost = 1e30;
+  for (int bn = 256; bn >= 96; bn -= step) {
+    const long t = (long)((cols + bn - 1) / bn) * rg;
+    const double cost = (double)((t + n_pairs_of_sms - 1) / n_pairs_of_sms) * (bn + 44);
+    if (cost < best_cost - 1e-9) { best_cost = cost; best = bn; }
+  }
+  return best;
+}
+
+template <typename Epi>
+int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
+                int n_rows_w, const Epi& epi, unsigned* status) {
+  constexpr bool kRope = std::is_same<Epi, EpiQKVRope<bf16>>::value;
+  const int cols = Epi::kDual ? 2 * NP : NP;
+  const int pairs = st.max_clusters[2];
+  int bn = Epi::kReduce ? UM_HEAD_BN : pair_width(M, cols, pairs, kRope ? 64 : 32);
+  if (st.pair_bn > 0 && !Epi::kReduce) bn = st.pair_bn;
+  int unit = 0;
+  if constexpr (kRope) {
+    if ((bn / 2) % epi.half) unit = 32;
+    if (epi.half % 32) { st.err = "unsupported head_dim for the paired GEMM"; return -6; }
+  }
+  const int stage = 2 * (UM_BM * 128 + bn / 2 * 128);
+  const int aux = 1024 + 8 * (2 * PR_MAX_STAGES + 4) + 16;
+  int stages = (st.max_smem - aux) / stage;
+  if (stages > PR_MAX_STAGES) stages = PR_MAX_STAGES;
+  if (stages < 2) { st.err = "not enough shared memory for the paired GEMM"; return -2; }
+  const size_t smem = (size_t)stages * stage + aux;
+  static bool attr_set = false;   // per instantiation
+  if (!attr_set) {
+    cudaError_t e = cudaFuncSetAttribute(k_gemm_pair<Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, st.max_smem);
+    if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -3; }
+    attr_set = true;
+  }
+  CUtensorMap ma, mb0, mb1;
+  {
+    const CUtensorMap* p = umma_map4(st, A, M, M, 1, K, UM_BM, 1, 2);
+    if (!p) return -4;
+    ma = *p;
+    if constexpr (kRope) {
+      const int blocks = n_rows_w / (2 * epi.half), br = unit ? unit : epi.half, bb = unit ? 1 : bn / 2 / epi.half;
+      p = umma_map4(st, W0, epi.half, 2 * epi.half, blocks, K, br, bb, unit ? 1 : 2);
+      if (!p) return -4;
+      mb0 = *p;
+      p = umma_map4(st, W1 + (size_t)epi.half * K, epi.half, 2 * epi.half, blocks, K, br, bb, unit ? 1 : 2);
+    } else {
+      p = umma_map4(st, W0, n_rows_w, n_rows_w, 1, K, bn / 2, 1, 2);
+      if (!p) return -4;
+      mb0 = *p;
+      p = umma_map4(st, W1, n_rows_w, n_rows_w, 1, K, bn / 2, 1, 2);
+    }
+    if (!p) return -4;
+    mb1 = *p;
+  }
+  const int per_tile = Epi::kDual ? bn / 2 : bn;
+  const int n_tiles = (NP + per_tile - 1) / per_tile;
+  const int rg = (M + PR_ROWS - 1) / PR_ROWS;
+  const long T = (long)n_tiles * rg;
+  if (T > (1l << 24)) { st.err = "too many tiles for the paired GEMM"; return -9; }
+  // Bands of row groups whose activation rows (at most about 40 MB) stay in L2 while the weights stream past them once per
+  // band: 8240 x 12288 x 2 (K 4096) 1146 us in one band, 1067 in bands of 16; 8240 x 4096 (K 12288) 648 in one, 589 in bands
+  // of 4, 751 in bands of 2 (then the weights, streamed too often, are the larger part).
+  int band_max = (int)(40e6 / ((double)PR_ROWS * K * 2));
+  if (band_max < 4) band_max = 4;
+  if (st.pair_band > 0) band_max = st.pair_band;
+  const int n_bands = (rg + band_max - 1) / band_max, band = (rg + n_bands - 1) / n_bands;
+  const int grid = 2 * (int)(T < pairs ? T : pairs);
+  PairArgs args{M, NP, n_tiles, rg, band, (K + 2 * UM_BK - 1) / (2 * UM_BK), bn, unit, stages, status};
+  cudaError_t e = launch_k(st.pdl, k_gemm_pair<Epi>, dim3(grid), dim3(PR_THREADS), smem, stream, 2, ma, mb0, mb1, args, epi);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -5; }
+  return 0;
+}
+
+}  // namespace lsp

@@ -88,6 +88,23 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar)
       : "memory");
 }
+// True in one thread of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+// One box of a 4-D map (umma_map4): rows r0.. of block blk.., 64-element K atoms a0..
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int r0, int blk, int a0, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+      ::"r"(dst), "l"(map), "r"(0), "r"(r0), "r"(blk), "r"(a0), "r"(bar)
+      : "memory");
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
@@ -245,6 +262,7 @@ typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_
 struct UmmaState {
   PFN_encodeTiled encode = nullptr;
   std::map<std::tuple<const void*, int, int, int>, CUtensorMap> cache;
+  std::map<std::tuple<const void*, int, int, int, int, int>, CUtensorMap> cache4;
   int max_smem = 0;
   int n_sm = 148;
   float* scratch = nullptr;        // split-K partial tiles (device), scratch_bytes long
@@ -271,6 +289,9 @@ struct UmmaState {
   int swap_min_rows = 129;         // row counts [min, max] that take the operand-swapped kernel (gemm_swap.cuh); max 0 = never
   int swap_max_rows = 256;
   int swap_force = 0;              // 1: take it whenever it can run (tests), not only where it was measured to pay
+  int pair_min_rows = 257;         // fewest rows that take the kernel on pairs of SMs (gemm_pair.cuh)
+  int pair_bn = 0;                 // its tile width (0 = automatic)
+  int pair_band = 0;               // its row groups per band (0 = automatic)
   int stream_grid_mode = 2;        // its grid: 0 = by row count, 1 = one CTA per SM (even shares), 2 = multiple of the tile count
   int stream_even_max_rows = 0;    // mode 0: even shares up to this many activation rows
   std::string err;
@@ -291,6 +312,32 @@ inline int umma_init(UmmaState& st) {
   cudaDeviceGetAttribute(&st.n_sm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&st.sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   return 0;
+}
+
+// bf16 tensor [rows, K] row-major seen as [K / 64 atoms][blocks of block_rows rows, block_stride rows apart][rows][64], so
+// that one copy brings `atoms` K atoms of box_blocks x box_rows rows, each atom a [rows x 128 bytes] swizzled tile of its own
+// behind the previous one (K atoms past the end are zero-filled).  Copies are issued by one thread at a cost that hardly
+// depends on their size, so fewer and larger ones keep the producer ahead.  base: the first row (a rotary map starts at the
+// head's first or second half).
+inline const CUtensorMap* umma_map4(UmmaState& st, const void* base, int block_rows, int block_stride, int blocks, int K, int box_rows,
+                                    int box_blocks, int atoms) {
+  auto key = std::make_tuple(base, block_rows, block_stride, blocks, K, box_rows * 4096 + box_blocks * 16 + atoms);
+  auto it = st.cache4.find(key);
+  if (it != st.cache4.end()) return &it->second;
+  if (st.cache4.size() > 4096) st.cache4.clear();
+  CUtensorMap m;
+  cuuint64_t dims[4] = {(cuuint64_t)UM_BK, (cuuint64_t)block_rows, (cuuint64_t)blocks, (cuuint64_t)(K / UM_BK)};
+  cuuint64_t strides[3] = {(cuuint64_t)K * 2, (cuuint64_t)block_stride * K * 2, (cuuint64_t)UM_BK * 2};
+  cuuint32_t box[4] = {(cuuint32_t)UM_BK, (cuuint32_t)box_rows, (cuuint32_t)box_blocks, (cuuint32_t)atoms};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = st.encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    st.err = "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
+    return nullptr;
+  }
+  return &st.cache4.emplace(key, m).first->second;
 }
 
 // 2-D bf16 tensor [rows, K] row-major, box = [64 (K), box_rows], 128-byte swizzle, zero fill out of bounds.
@@ -314,12 +361,20 @@ inline const CUtensorMap* umma_map(UmmaState& st, const void* base, int rows, in
 }
 
 constexpr int UM_HEAD_BN = 256;
-inline int umma_head_tiles(int vocab) { return (vocab + UM_HEAD_BN - 1) / UM_HEAD_BN; }
+// several row groups: pairs of SMs (gemm_pair.cuh)
+inline bool umma_takes_pairs(const UmmaState& st, int M) { return M >= st.pair_min_rows; }
+// Partials per row the head GEMM of M rows leaves: one per vocabulary tile, or (k_gemm_pair) one per half tile.
+inline int umma_head_tiles(const UmmaState& st, int M, int vocab) {
+  return (vocab + UM_HEAD_BN - 1) / UM_HEAD_BN * (umma_takes_pairs(st, M) ? 2 : 1);
+}
 
 template <typename Epi> int stream_row_tiles(const UmmaState& st, int M, int NP, int K, int bn);
 template <int NACC, typename Epi>
 int swap_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
                 int n_rows_w, const Epi& epi, unsigned* status, int box_rows);
+template <typename Epi>
+int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
+                int n_rows_w, const Epi& epi, unsigned* status);
 template <int BN, int MT, int NI, typename Epi>
 int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
                   int n_rows_w, const Epi& epi, unsigned* status, int box_rows);
@@ -359,6 +414,7 @@ template <typename Epi>
 int umma_gemm(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
               int n_rows_w, const Epi& epi, unsigned* status) {
   if (K % UM_BK) { st.err = "K must be a multiple of 64"; return -6; }
+  if (umma_takes_pairs(st, M)) return pair_launch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
   if constexpr (Epi::kReduce) {
     {
       const int smt = stream_row_tiles<Epi>(st, M, NP, K, UM_HEAD_BN);

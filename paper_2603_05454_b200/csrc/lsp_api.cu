@@ -21,6 +21,7 @@
 #ifndef LSP_NO_UMMA
 #include "gemm_stream.cuh"
 #include "gemm_swap.cuh"
+#include "gemm_pair.cuh"
 #include "attention_umma.cuh"
 #endif
 
@@ -175,7 +176,7 @@ struct Layout {
 constexpr size_t kGemmScratchBytes = 80u << 20;   // split-K partial tiles (the streaming GEMM needs 74 MiB at its widest)
 constexpr int kGemmCounters = 4096;               // split-K arrival counters
 
-int head_tiles_max(const lsp_model_cfg* m) { return (m->vocab + 63) / 64; }
+int head_tiles_max(const lsp_model_cfg* m) { return std::max(2, (m->vocab + 63) / 64); }
 
 Layout make_layout(const lsp_model_cfg* m, int max_batch, int max_len) {
   const size_t esz = m->dtype == 0 ? 4 : 2;
@@ -256,7 +257,7 @@ int run_head(lsp_ctx* c, const T* hidden, int rows, int* n_tiles_out) {
   epi.exclude_id = c->s.exclude_mask_logit ? m.mask_id : -1;
   int n_tiles = (m.vocab + SG_BN - 1) / SG_BN;
 #ifndef LSP_NO_UMMA
-  if (std::is_same<T, bf16>::value && c->gemm_impl == 1) n_tiles = umma_head_tiles(m.vocab);
+  if (std::is_same<T, bf16>::value && c->gemm_impl == 1) n_tiles = umma_head_tiles(c->umma, rows, m.vocab);
 #endif
   epi.n_tiles = n_tiles;
   *n_tiles_out = n_tiles;
@@ -798,6 +799,9 @@ int lsp_debug_set(lsp_ctx* c, int key, int value) {
   else if (key == 24) c->umma.stream_big_mt = (value == 1 || value == 2) ? value : 3;
   else if (key == 20) c->umma.stream_bn2 = (value == 256 || value == 128) ? value : 0;
   else if (key == 23) c->umma.stream_bn = (value == 256 || value == 128) ? value : 0;
+  else if (key == 40) c->umma.pair_min_rows = value;
+  else if (key == 41) c->umma.pair_bn = (value >= 96 && value <= 256 && value % 32 == 0) ? value : 0;
+  else if (key == 42) c->umma.pair_band = value < 0 ? 0 : value;
   else if (key == 21) c->umma.stream_atoms = value;
   else if (key == 22) c->umma.stream_min_stages2 = value < 2 ? 2 : value;
 #endif

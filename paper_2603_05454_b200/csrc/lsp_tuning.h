@@ -35,6 +35,9 @@ extern "C" {
  *      default), or through global scratch by the last CTA to arrive (0)
  *   32 tile width of the dual (SwiGLU) GEMM: 0 = automatic (default), 192 or 256
  *   33 a cluster of 2 exchanges half tiles (1, default) or publishes whole partial tiles like larger clusters (0)
+ * GEMM on pairs of SMs:
+ *   40 fewest rows that take it (default 257)   41 its tile width (0 = automatic, 96 ... 256 in steps of 32)
+ *   42 most row groups of 256 per band (0 = automatic)
  * tcgen05 attention:
  *   28 fewest (query row x group head) rows of a (sequence, KV head) for which the tcgen05 kernel is used (default 0)
  *   30 it splits a row tile's keys over a thread block cluster when there are few CTAs (1, default)

@@ -300,3 +300,60 @@ def test_linear_bf16_second_row_tile_of_64_rows(case):
     ref = x0 + a @ w.T
     np.testing.assert_allclose(f64(xr), dlm.round_bf16(ref), rtol=rtol, atol=rtol * np.abs(ref).max() * 0.05)
     dec.close()
+
+
+@pytest.mark.parametrize("case", [
+    # (M, N, K, tile width 0 = automatic): row groups of 256 (one row of a second group, a group less one row), a ragged last
+    # column tile, a half-empty last K chunk (odd multiples of 64), more tiles than pairs of SMs, several bands
+    (257, 64, 64, 0), (511, 1152, 192, 0), (513, 4112, 320, 160), (300, 2048, 1024, 256), (700, 9600, 448, 96),
+    (1030, 4096, 512, 224), (4610, 576, 4096, 0), (2600, 1040, 2048, 128),
+])
+def test_linear_bf16_on_pairs_of_sms(case):
+    """More than 256 rows: the GEMM on pairs of SMs, at the edges of its tiles, against fp64 products of the same operands.
+    One bf16 ulp of the result (1/128 relative), plus a twentieth of that of the largest, as in the tests above; the SwiGLU
+    product has two factors."""
+    M, N, K, bn = case
+    dec = _dec("bf16")
+    dec.debug_set(41, bn)
+    A = S.normal((M, K), 11, 1, 1.0, torch.bfloat16, DEV)
+    W = S.normal((N, K), 11, 2, 0.05, torch.bfloat16, DEV)
+    W2 = S.normal((N, K), 11, 3, 0.05, torch.bfloat16, DEV)
+    X0 = S.normal((M, N), 11, 4, 1.0, torch.bfloat16, DEV)
+    ref, up = A.double() @ W.double().t(), A.double() @ W2.double().t()
+    near = lambda got, want, ulps=1: bool(((got.double() - want).abs() <= ulps / 128 * want.abs() + want.abs().max() / 2560).all())
+    out = torch.full((M + 1, N), 7.0, dtype=torch.bfloat16, device=DEV)
+    dec.op_linear(0, A, W, None, out[:M])
+    assert near(out[:M], ref) and bool((out[M] == 7.0).all())
+    x = torch.cat([X0, out[M:]])
+    dec.op_linear(1, A, W, None, x[:M])
+    assert near(x[:M], X0.double() + ref) and bool((x[M] == 7.0).all())
+    dec.op_linear(2, A, W, W2, out[:M])
+    assert near(out[:M], torch.nn.functional.silu(ref) * up, 2) and bool((out[M] == 7.0).all())
+    dec.close()
+
+
+@pytest.mark.parametrize("dh,hq,hkv,bn", [(128, 4, 2, 128), (128, 4, 2, 192), (128, 5, 5, 256), (64, 6, 2, 192), (64, 6, 2, 128)])
+def test_rotary_projection_on_pairs_of_sms(dh, hq, hkv, bn):
+    """The rotary QKV projection of more than 256 rows (half tiles of whole head halves, or of 32-row pieces of them): the
+    first layer's cached keys and values against the CUDA-core GEMM's.  Both round the same fp32 value up to the order of its
+    sum, so they differ by at most one bf16 ulp (1/128 relative), with a floor of a ulp of the typical value for sums that
+    cancel."""
+    from paper_2603_05454_b200 import LSPDecoder, SchedCfg
+    d, B, P, G = hq * dh, 2, 170, 9
+    sh = S.ModelShape(1, d, hq, hkv, dh, 128, 256, dtype="bf16")
+    w = S.make_weights(sh, 5, device=DEV)
+    kv = []
+    for impl in (1, 0):
+        dec = LSPDecoder(sh, w, SchedCfg(), B, P + G, device=DEV)
+        dec.set_option(0, impl)
+        dec.debug_set(41, bn)
+        tokens = torch.zeros(B, P + G, dtype=torch.int32, device=DEV)
+        tokens[:, :P] = S.make_prompt(B, P, sh, 6).to(DEV)
+        dec.begin(tokens, [P] * B, [G] * B)
+        dec.denoise_step()
+        dec.commit()
+        torch.cuda.synchronize()
+        kv.append(dec.kv_view()[0, :, :, :P].double())
+        dec.close()
+    typical = kv[1].square().mean().sqrt()
+    assert bool(((kv[0] - kv[1]).abs() <= (kv[1].abs() + typical) / 128).all())
