@@ -47,6 +47,7 @@ struct EpiSwiGLU {
   static constexpr bool kReduce = false;
   T* out;
   int ld;
+  int flip = 0;      // the kernel's first accumulator is the up projection's (vectorised row-major epilogue only)
   __device__ __forceinline__ int row0(int j) const { return j; }
   __device__ __forceinline__ int row1(int j) const { return j; }
   __device__ __forceinline__ void elem(int m, int j, float g, float u) const {

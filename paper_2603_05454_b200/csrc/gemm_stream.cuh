@@ -21,6 +21,10 @@
 //     order whoever finishes, so results are deterministic) before running the fused epilogue.
 // Tile width: measured per shape and row count (see umma_gemm): 128 columns for plain epilogues in the streaming
 // regime (no K split needed with 96 tiles), 256 for dual epilogues and for every problem with several row groups.
+// Producer and issuers are whole warps with one elected thread issuing, and each operand of a stage is one copy (4-D and 5-D
+// tensor maps, gemm_umma.cuh): against a lane branch and a copy per half tile and K atom 2 x 12288 x 4096 SwiGLU at 101 rows
+// 38.7 -> 35.5 us, 12288 x 4096 25.7 -> 24.7, 3584 x 18944 at 9 rows 28.8 -> 26.4; a LLaDA-shaped pass of 9 rows
+// 4.20 -> 3.95 ms, of 101 rows 4.82 -> 4.51.
 // Warp roles: warp 0 = TMA producer, warp 1 = TMEM allocator + MMA issuer, warps 2..5 = epilogue, warp 6 = second MMA
 // issuer (see the note on issue rate in the kernel).
 // Every wait is bounded; on expiry the kernel records (code, site) in the status word, drains and returns.
@@ -46,7 +50,8 @@ struct StreamArgs {
   int kc;           // K chunks (one per stage) per tile
   int a_rows;       // activation box rows (M rounded up to a multiple of 8)
   int atoms;        // 64-element K atoms per stage (1 or 2)
-  int box_rows;     // weight rows per TMA box: BN/2, or fewer when the rows of a half tile are not contiguous (rotary pairs)
+  int one_copy;     // 1: one copy brings both halves and all atoms of a stage's weight tile (map_b0); 0: one per half and atom
+  int half;         // rotary epilogue: pair indices per head (half its width), else 0
   int stages;
   int half_tile1;   // two row tiles, every CTA one whole tile, at most 192 rows: the second row tile's MMAs span 64
                     // accumulator rows instead of 128 (its rows sit in the lower half of every warp's tensor-memory lanes)
@@ -155,23 +160,22 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
   auto pos_next = [&](Pos& p) {
     if (++p.c == args.kc) pos_set(p, p.vt + 1, 0);
   };
-  // weight boxes of one stage: the atoms of a row group back to back (AT x 128 contiguous bytes per weight row)
+  // the weight tile of one stage: both halves of every K atom (see umma_map5)
   auto load_weights = [&](const Pos& p, int s) {
     const uint32_t sb = smem_u32(smem + (size_t)s * STAGE_BYTES) + AT * A_ATOM;
-    const int k0 = p.c * AT * UM_BK;
-    for (int b = 0; b < HALF; b += args.box_rows) {
-      int row_b0, row_b1;
-      if (Epi::kDual) { row_b0 = epi.row0(p.tile * HALF + b); row_b1 = epi.row1(p.tile * HALF + b); }
-      else { row_b0 = p.tile * BN + b; row_b1 = p.tile * BN + HALF + b; }
-      for (int j = 0; j < AT; ++j) tma_load_2d(sb + j * B_ATOM + b * 128, &map_b0, k0 + 64 * j, row_b0, full_bar(s));
-      for (int j = 0; j < AT; ++j)
-        tma_load_2d(sb + j * B_ATOM + B_HALF_ATOM + b * 128, &map_b1, k0 + 64 * j, row_b1, full_bar(s));
+    const int j = p.tile * (Epi::kDual ? HALF : BN);
+    const int r0 = args.half ? 0 : j, blk = args.half ? j / args.half : 0;
+    if (args.one_copy) {
+      tma_load_5d(sb, &map_b0, r0, blk, 0, p.c * AT, full_bar(s));
+    } else {
+      for (int a = 0; a < AT; ++a) {
+        tma_load_5d(sb + a * B_ATOM, &map_b0, r0, blk, 0, p.c * AT + a, full_bar(s));
+        tma_load_5d(sb + a * B_ATOM + B_HALF_ATOM, &map_b1, r0, blk, 0, p.c * AT + a, full_bar(s));
+      }
     }
   };
   auto load_acts = [&](const Pos& p, int s) {
-    const uint32_t sa = smem_u32(smem + (size_t)s * STAGE_BYTES);
-    const int k0 = p.c * AT * UM_BK;
-    for (int j = 0; j < AT; ++j) tma_load_2d(sa + j * A_ATOM, &map_a, k0 + 64 * j, p.rg * ROWS, full_bar(s));
+    tma_load_4d(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_a, p.rg * ROWS, 0, p.c * AT, full_bar(s));
   };
 
   const int n_pre = n_units < S ? n_units : S;      // stages whose weights are requested before the predecessor is done
@@ -188,14 +192,20 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     *epi_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 0) {
     // The weights are never written by any kernel, so the first stages' weight tiles can be requested at once, while a
     // preceding kernel (launched with programmatic serialisation) is still running; the activations follow after
-    // pdl_wait().  This thread is also the producer below.
+    // pdl_wait().  This warp is also the producer below.
+    __syncwarp();
     Pos p;
     pos_set(p, (int)(u0 / args.kc), (int)(u0 % args.kc));
     for (int it = 0; it < n_pre; ++it) {
-      mbar_expect_tx(full_bar(it), STAGE_BYTES);
-      load_weights(p, it);
+      if (elect_one()) {
+        mbar_expect_tx(full_bar(it), STAGE_BYTES);
+        load_weights(p, it);
+      }
+      __syncwarp();
       pos_next(p);
     }
   }
@@ -213,39 +223,40 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
 
   if (warp == 0) {
     // ---------------- TMA producer: one uninterrupted stream over this CTA's units ----------------
-    if (lane == 0) {
-      int issued = 0;
-      Pos p;
-      pos_set(p, (int)(u0 / args.kc), (int)(u0 % args.kc));
-      int s = 0;
-      uint32_t ph = 0;
-      for (int it = 0; it < n_units; ++it) {
-        if (it < n_pre) {
-          load_acts(p, s);                   // the stage is armed and its weights are on their way
-        } else {
-          if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) {
-            if (!*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 11u; }
-            break;
-          }
+    int issued = 0;
+    Pos p;
+    pos_set(p, (int)(u0 / args.kc), (int)(u0 % args.kc));
+    int s = 0;
+    uint32_t ph = 0;
+    for (int it = 0; it < n_units; ++it) {
+      if (it >= n_pre) {
+        if (!__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, abort_flag))) {
+          if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 11u; }
+          break;
+        }
+      }
+      if (elect_one()) {
+        if (it >= n_pre) {                   // else the stage is armed and its weights are on their way
           mbar_expect_tx(full_bar(s), STAGE_BYTES);
           load_weights(p, s);
-          load_acts(p, s);
         }
-        ++issued;
-        if (++s == S) { s = 0; ph ^= 1u; }
-        pos_next(p);
+        load_acts(p, s);
       }
-      // do not leave while copies may still be landing in this CTA's shared memory
-      const int first = issued > S ? issued - S : 0;
-      for (int it = first; it < issued; ++it) {
-        volatile uint32_t no_abort = 0;
-        mbar_wait(full_bar((int)(it % S)), (uint32_t)(it / S) & 1u, &no_abort);
-      }
+      __syncwarp();
+      ++issued;
+      if (++s == S) { s = 0; ph ^= 1u; }
+      pos_next(p);
+    }
+    // do not leave while copies may still be landing in this CTA's shared memory
+    const int first = issued > S ? issued - S : 0;
+    for (int it = first; it < issued; ++it) {
+      volatile uint32_t no_abort = 0;
+      mbar_wait(full_bar((int)(it % S)), (uint32_t)(it / S) & 1u, &no_abort);
     }
   } else if (warp == 1 || warp == 6) {
-    // ---------------- MMA issuers ----------------
+    // ---------------- MMA issuers (the whole warp waits, one elected thread issues) ----------------
     const int is = warp == 1 ? 0 : 1;                   // issuer index
-    if (lane == 0 && is < NI) {
+    if (is < NI) {
       const uint32_t idesc = (MT == 2 && is == 1 && args.half_tile1) ? make_idesc_m64(BN) : make_idesc(BN);
       int seg = 0;
       bool ok = true;
@@ -256,39 +267,43 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         const int seg_end = min(u1, (vt + 1) * args.kc);
         const int buf = seg % NBUF, use = seg / NBUF;
         // wait until the epilogue has drained this accumulator set (its previous use was segment seg - NBUF)
-        if (use >= 1 && !mbar_wait(acce_bar(buf), (uint32_t)(use - 1) & 1u, abort_flag)) {
-          if (!*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 12u; }
-          ok = false;
+        if (use >= 1) ok = __all_sync(0xffffffffu, mbar_wait(acce_bar(buf), (uint32_t)(use - 1) & 1u, abort_flag));
+        if (!ok) {
+          if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 12u; }
           break;
         }
         tc_fence_after();
         // this issuer's accumulator: row tile `is` (two row tiles) or K-parity accumulator `is` (one row tile)
         const uint32_t d_tmem = tmem_base + (uint32_t)(buf * SET_COLS + (NI == 2 ? is * BN : 0));
-        bool first = true;
+        uint32_t acc = 0;                               // 0: the segment's first MMA overwrites the accumulator
         for (; u < seg_end; ++u) {
-          if (!mbar_wait(full_bar(s), ph, abort_flag)) {
-            if (!*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 13u; }
-            ok = false;
+          ok = __all_sync(0xffffffffu, mbar_wait(full_bar(s), ph, abort_flag));
+          if (!ok) {
+            if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 13u; }
             break;
           }
           tc_fence_after();
           const uint32_t sa = smem_u32(smem + (size_t)s * STAGE_BYTES);
           const uint32_t sb = sa + AT * A_ATOM;
-          for (int j = 0; j < AT; ++j) {
-            // row tile 1 starts 128 rows = 16 KB (1024 descriptor units) further into the activation atom
-            const uint64_t da = make_smem_desc(sa + j * A_ATOM) + (uint64_t)((MT == 2 && is == 1) ? 1024 : 0);
-            const uint64_t db = make_smem_desc(sb + j * B_ATOM);
+          if (elect_one()) {
+            for (int j = 0; j < AT; ++j) {
+              // row tile 1 starts 128 rows = 16 KB (1024 descriptor units) further into the activation atom
+              const uint64_t da = make_smem_desc(sa + j * A_ATOM) + (uint64_t)((MT == 2 && is == 1) ? 1024 : 0);
+              const uint64_t db = make_smem_desc(sb + j * B_ATOM);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              if (MT == 1 && NI == 2 && (k & 1) != is) continue;       // alternate K steps
-              tc_mma_f16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, first ? 0u : 1u);
-              first = false;
+              for (int k = 0; k < 4; ++k) {
+                if (MT == 1 && NI == 2 && (k & 1) != is) continue;       // alternate K steps
+                const int step = (MT == 1 && NI == 2) ? k >> 1 : k;
+                tc_mma_f16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, acc | (uint32_t)(j | step));
+              }
             }
+            tc_commit(empty_bar(s));
+            if (u == seg_end - 1) tc_commit(accf_bar(buf));
           }
-          tc_commit(empty_bar(s));
+          __syncwarp();
+          acc = 1;
           if (++s == S) { s = 0; ph ^= 1u; }
         }
-        if (ok) tc_commit(accf_bar(buf));
         ++seg;
       }
     }
@@ -740,7 +755,7 @@ inline void stream_query_clusters(UmmaState& st) {
 
 template <int BN, int MT, int NI, typename Epi>
 int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
-                  int n_rows_w, const Epi& epi, unsigned* status, int box_rows) {
+                  int n_rows_w, const Epi& epi, unsigned* status) {
   const StreamShape sh = stream_shape(st, stream_a_rows(M, MT), BN, MT, K);
   if (sh.stages < 2) { st.err = "not enough shared memory for the streaming GEMM"; return -2; }
   const size_t smem = (size_t)sh.stages * sh.stage_bytes + sh.aux;
@@ -750,12 +765,32 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
     if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -3; }
     attr_set = true;
   }
-  if (st.cache.size() > 4096) st.cache.clear();
-  if (box_rows <= 0 || box_rows > BN / 2 || (BN / 2) % box_rows || box_rows % 8) box_rows = BN / 2;
-  const CUtensorMap* ma = umma_map(st, A, M, K, sh.a_rows);
-  const CUtensorMap* mb0 = umma_map(st, W0, n_rows_w, K, box_rows);
-  const CUtensorMap* mb1 = umma_map(st, W1, n_rows_w, K, box_rows);
-  if (!ma || !mb0 || !mb1) return -4;
+  const CUtensorMap* ma = umma_map4(st, A, M, M, 1, K, sh.a_rows, 1, sh.atoms);
+  if (!ma) return -4;
+  WeightView v{W0, n_rows_w, 1, n_rows_w, 1, 0, BN, 1};
+  int one_copy = 1, rot_half = 0;
+  Epi e2 = epi;
+  if constexpr (std::is_same<Epi, EpiQKVRope<bf16>>::value) {
+    rot_half = epi.half;
+    v = WeightView{W0, rot_half, n_rows_w / (2 * rot_half), 2 * rot_half, 2, (size_t)rot_half * K * 2, rot_half, BN / 2 / rot_half};
+  } else if constexpr (Epi::kDual) {
+    // gate and up are two tensors: the halves' distance is that of the tensors (either may come first)
+    const bool flip = (uintptr_t)W1 < (uintptr_t)W0;
+    const size_t dist = flip ? (const char*)W0 - (const char*)W1 : (const char*)W1 - (const char*)W0;
+    v = WeightView{flip ? W1 : W0, n_rows_w, 1, n_rows_w, 2, dist, BN / 2, 1};
+    if (dist == 0 || dist >= ((size_t)1 << 40) || (dist & 15) || st.stream_split_copies) { one_copy = 0; v.base = W0; v.halves = 1; }
+    else if (flip) e2.flip = 1;
+  }
+  const CUtensorMap* mb0 = umma_map5(st, v, K, one_copy ? sh.atoms : 1);
+  if (!mb0) return -4;
+  const CUtensorMap mb0v = *mb0;
+  CUtensorMap mb1v = mb0v;
+  if (!one_copy) {
+    v.base = W1;
+    const CUtensorMap* mb1 = umma_map5(st, v, K, 1);
+    if (!mb1) return -4;
+    mb1v = *mb1;
+  }
   const int per_tile = Epi::kDual ? BN / 2 : BN;
   const int n_tiles = (NP + per_tile - 1) / per_tile;
   const int kc = K / (sh.atoms * UM_BK);
@@ -780,10 +815,10 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
   // at most 192 rows on two row tiles, every CTA one unsplit tile: 64-row MMAs for the second row tile
   const int half_tile1 = (MT == 2 && !Epi::kReduce && st.stream_half_tile1 && row_groups == 1 && M <= UM_BM + 64 && grid == (int)T &&
                           cluster == 0) ? 1 : 0;
-  StreamArgs args{M, NP, n_tiles, row_groups, whole, cluster, cl_rounds, kc, sh.a_rows, sh.atoms, box_rows, sh.stages, half_tile1,
+  StreamArgs args{M, NP, n_tiles, row_groups, whole, cluster, cl_rounds, kc, sh.a_rows, sh.atoms, one_copy, rot_half, sh.stages, half_tile1,
                   st.scratch, st.counters, status};
-  cudaError_t e = launch_k(st.pdl, k_gemm_stream<BN, MT, NI, Epi>, dim3(grid), dim3(ST_THREADS), smem, stream, cluster, *ma, *mb0,
-                           *mb1, args, epi);
+  cudaError_t e = launch_k(st.pdl, k_gemm_stream<BN, MT, NI, Epi>, dim3(grid), dim3(ST_THREADS), smem, stream, cluster, *ma, mb0v,
+                           mb1v, args, e2);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -5; }
   return 0;

@@ -88,7 +88,16 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar)
       : "memory");
 }
-// True in one thread of a converged warp.
+// One box of a 5-D map (umma_map5): rows r0.. of blocks blk.., both halves, 64-element K atoms a0..
+__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, int r0, int blk, int half, int a0, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+      ::"r"(dst), "l"(map), "r"(0), "r"(r0), "r"(blk), "r"(half), "r"(a0), "r"(bar)
+      : "memory");
+}
+// True in one thread of a converged warp.  A tcgen05.mma behind a lane test (if (lane == 0)) costs its issuer about 130 cycles
+// whatever its width when a commit follows every fourth, behind elect.sync 88; a turn of a stage ring costs a producer or
+// issuer about 300 ns in all, so stages are large and each operand of a stage is one copy.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile(
@@ -218,7 +227,10 @@ __device__ __forceinline__ void epi16(const EpiSwiGLU<bf16>& e, int m, int j, co
 #pragma unroll
   // __fdividef (reciprocal + multiply, 2 ulp): the IEEE division's slow path is a subroutine call inside the epilogue,
   // and its mere presence cost the whole kernel 5-7 us at every row count (39.4 -> 34.4 us at 2 rows, 61.7 -> 54.6 at 256)
-  for (int i = 0; i < 16; ++i) r[i] = __fdividef(g[i], 1.f + __expf(-g[i])) * u[i];
+  for (int i = 0; i < 16; ++i) {
+    const float gi = e.flip ? u[i] : g[i], ui = e.flip ? g[i] : u[i];
+    r[i] = __fdividef(gi, 1.f + __expf(-gi)) * ui;
+  }
   uint4* p = reinterpret_cast<uint4*>(e.out + (size_t)m * e.ld + j);
   p[0] = pack8(r);
   p[1] = pack8(r + 8);
@@ -263,6 +275,7 @@ struct UmmaState {
   PFN_encodeTiled encode = nullptr;
   std::map<std::tuple<const void*, int, int, int>, CUtensorMap> cache;
   std::map<std::tuple<const void*, int, int, int, int, int>, CUtensorMap> cache4;
+  std::map<std::tuple<const void*, size_t, int, int, int, int>, CUtensorMap> cache5;
   int max_smem = 0;
   int n_sm = 148;
   float* scratch = nullptr;        // split-K partial tiles (device), scratch_bytes long
@@ -285,6 +298,7 @@ struct UmmaState {
   int stream_exchange = 1;         // clusters of 2 exchange half tiles instead of publishing whole partial tiles
   int stream_atoms = 0;            // K atoms per stage: 0 = two when stream_min_stages2 such stages fit, else 1 or 2 as given
   int stream_min_stages2 = 3;
+  int stream_split_copies = 0;     // a dual tile's weights by one copy per half and atom even where one copy can bring them all
   int stream_half_tile1 = 1;       // 129..192 rows on two row tiles, unsplit: 64-row MMAs for the second row tile
   int swap_min_rows = 129;         // row counts [min, max] that take the operand-swapped kernel (gemm_swap.cuh); max 0 = never
   int swap_max_rows = 256;
@@ -319,6 +333,16 @@ inline int umma_init(UmmaState& st) {
 // behind the previous one (K atoms past the end are zero-filled).  Copies are issued by one thread at a cost that hardly
 // depends on their size, so fewer and larger ones keep the producer ahead.  base: the first row (a rotary map starts at the
 // head's first or second half).
+inline CUresult umma_encode4(PFN_encodeTiled encode, CUtensorMap* m, const void* base, int block_rows, int block_stride, int blocks, int K,
+                             int box_rows, int box_blocks, int atoms) {
+  cuuint64_t dims[4] = {(cuuint64_t)UM_BK, (cuuint64_t)block_rows, (cuuint64_t)blocks, (cuuint64_t)(K / UM_BK)};
+  cuuint64_t strides[3] = {(cuuint64_t)K * 2, (cuuint64_t)block_stride * K * 2, (cuuint64_t)UM_BK * 2};
+  cuuint32_t box[4] = {(cuuint32_t)UM_BK, (cuuint32_t)box_rows, (cuuint32_t)box_blocks, (cuuint32_t)atoms};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
 inline const CUtensorMap* umma_map4(UmmaState& st, const void* base, int block_rows, int block_stride, int blocks, int K, int box_rows,
                                     int box_blocks, int atoms) {
   auto key = std::make_tuple(base, block_rows, block_stride, blocks, K, box_rows * 4096 + box_blocks * 16 + atoms);
@@ -326,18 +350,45 @@ inline const CUtensorMap* umma_map4(UmmaState& st, const void* base, int block_r
   if (it != st.cache4.end()) return &it->second;
   if (st.cache4.size() > 4096) st.cache4.clear();
   CUtensorMap m;
-  cuuint64_t dims[4] = {(cuuint64_t)UM_BK, (cuuint64_t)block_rows, (cuuint64_t)blocks, (cuuint64_t)(K / UM_BK)};
-  cuuint64_t strides[3] = {(cuuint64_t)K * 2, (cuuint64_t)block_stride * K * 2, (cuuint64_t)UM_BK * 2};
-  cuuint32_t box[4] = {(cuuint32_t)UM_BK, (cuuint32_t)box_rows, (cuuint32_t)box_blocks, (cuuint32_t)atoms};
-  cuuint32_t estr[4] = {1, 1, 1, 1};
-  CUresult r = st.encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  const CUresult r = umma_encode4(st.encode, &m, base, block_rows, block_stride, blocks, K, box_rows, box_blocks, atoms);
   if (r != CUDA_SUCCESS) {
     st.err = "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
     return nullptr;
   }
   return &st.cache4.emplace(key, m).first->second;
+}
+
+// Weight tiles of the row-major kernels: [K / 64 atoms][halves][blocks][rows][64], so that ONE copy brings both halves of a
+// tile (gate / up rows, rotate-half partners) for `atoms` K atoms, laid out as the MMA wants them: per atom, the rows of the
+// first half and then those of the second.
+struct WeightView {
+  const void* base;
+  int rows, blocks, block_stride, halves;      // block_stride in rows
+  size_t half_stride;                          // bytes between the halves
+  int box_rows, box_blocks;                    // rows x blocks of a half tile
+};
+inline CUresult umma_encode5(PFN_encodeTiled encode, CUtensorMap* m, const WeightView& v, int K, int box_halves, int atoms) {
+  cuuint64_t dims[5] = {(cuuint64_t)UM_BK, (cuuint64_t)v.rows, (cuuint64_t)v.blocks, (cuuint64_t)v.halves, (cuuint64_t)(K / UM_BK)};
+  cuuint64_t strides[4] = {(cuuint64_t)K * 2, (cuuint64_t)v.block_stride * K * 2, (cuuint64_t)(v.halves > 1 ? v.half_stride : 16),
+                           (cuuint64_t)UM_BK * 2};
+  cuuint32_t box[5] = {(cuuint32_t)UM_BK, (cuuint32_t)v.box_rows, (cuuint32_t)v.box_blocks, (cuuint32_t)box_halves, (cuuint32_t)atoms};
+  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  return encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(v.base), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
+inline const CUtensorMap* umma_map5(UmmaState& st, const WeightView& v, int K, int atoms) {
+  auto key = std::make_tuple(v.base, v.half_stride, v.rows, v.blocks, K, ((v.box_rows * 16 + v.box_blocks) * 4 + v.halves) * 16 + atoms);
+  auto it = st.cache5.find(key);
+  if (it != st.cache5.end()) return &it->second;
+  if (st.cache5.size() > 4096) st.cache5.clear();
+  CUtensorMap m;
+  const CUresult r = umma_encode5(st.encode, &m, v, K, v.halves, atoms);
+  if (r != CUDA_SUCCESS) {
+    st.err = "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
+    return nullptr;
+  }
+  return &st.cache5.emplace(key, m).first->second;
 }
 
 // 2-D bf16 tensor [rows, K] row-major, box = [64 (K), box_rows], 128-byte swizzle, zero fill out of bounds.
@@ -377,16 +428,16 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
                 int n_rows_w, const Epi& epi, unsigned* status);
 template <int BN, int MT, int NI, typename Epi>
 int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
-                  int n_rows_w, const Epi& epi, unsigned* status, int box_rows);
+                  int n_rows_w, const Epi& epi, unsigned* status);
 
 // Instantiation choice for the streaming kernel: tile width 128 or 256, one or two row tiles, one or two MMA issuers
 // (two row tiles always have two).
 template <typename Epi>
 int stream_dispatch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
-                    int n_rows_w, const Epi& epi, unsigned* status, int box_rows, int bn, int mt, int ni) {
+                    int n_rows_w, const Epi& epi, unsigned* status, int bn, int mt, int ni) {
 #define LSP_STREAM_CASE(BN_, MT_, NI_) \
   if (bn == BN_ && mt == MT_ && ni == NI_) \
-    return stream_launch<BN_, MT_, NI_, Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status, box_rows)
+    return stream_launch<BN_, MT_, NI_, Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status)
   if (mt == 2) ni = 2;
   LSP_STREAM_CASE(256, 1, 1);
   LSP_STREAM_CASE(256, 1, 2);
@@ -419,7 +470,7 @@ int umma_gemm(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0,
     {
       const int smt = stream_row_tiles<Epi>(st, M, NP, K, UM_HEAD_BN);
       if (smt > 0)
-        return stream_dispatch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status, 0, UM_HEAD_BN, smt,
+        return stream_dispatch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status, UM_HEAD_BN, smt,
                                     st.stream_issuers);
     }
     st.err = "the tcgen05 head GEMM cannot take this shape";
@@ -470,7 +521,7 @@ int umma_gemm(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0,
       }
       const int smt = stream_row_tiles<Epi>(st, M, NP, K, sbn);
       if (smt > 0 && (sbn == 128 || sbn == 256 || sbn == 192))
-        return stream_dispatch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status, box_rows, sbn, smt,
+        return stream_dispatch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status, sbn, smt,
                                     st.stream_issuers);
     }
     st.err = "the tcgen05 GEMM cannot take this shape";

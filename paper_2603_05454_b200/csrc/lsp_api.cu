@@ -802,6 +802,7 @@ int lsp_debug_set(lsp_ctx* c, int key, int value) {
   else if (key == 40) c->umma.pair_min_rows = value;
   else if (key == 41) c->umma.pair_bn = (value >= 96 && value <= 256 && value % 32 == 0) ? value : 0;
   else if (key == 42) c->umma.pair_band = value < 0 ? 0 : value;
+  else if (key == 43) c->umma.stream_split_copies = value ? 1 : 0;
   else if (key == 21) c->umma.stream_atoms = value;
   else if (key == 22) c->umma.stream_min_stages2 = value < 2 ? 2 : value;
 #endif
@@ -1285,16 +1286,6 @@ void static_msg(char* err, size_t err_len, const char* fmt, ...) {
   va_end(ap);
 }
 
-bool static_map(PFN_encodeTiled encode, CUtensorMap* m, const void* base, int rows, int K, int box_rows) {
-  cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-  cuuint32_t box[2] = {(cuuint32_t)UM_BK, (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  return encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 }  // namespace
 
 int lsp_linear_static(const void* A, const void* W, void* out, int M, int N, int K, void* cuda_stream, char* err,
@@ -1351,7 +1342,8 @@ int lsp_linear_static(const void* A, const void* W, void* out, int M, int N, int
   if (stages > ST_MAX_STAGES) stages = ST_MAX_STAGES;
   const size_t smem = (size_t)stages * atoms * atom + aux;
   CUtensorMap ma, mb;
-  if (stages < 2 || !static_map(sd.encode, &ma, A, M, K, a_rows) || !static_map(sd.encode, &mb, W, N, K, kStaticBN / 2)) {
+  if (stages < 2 || umma_encode4(sd.encode, &ma, A, M, M, 1, K, a_rows, 1, atoms) != CUDA_SUCCESS ||
+      umma_encode5(sd.encode, &mb, WeightView{W, N, 1, N, 1, 0, kStaticBN, 1}, K, 1, atoms) != CUDA_SUCCESS) {
     static_msg(err, err_len, "lsp_linear_static: could not describe the operands to the copy engine");
     return LSP_ERR_CUDA;
   }
@@ -1370,7 +1362,7 @@ int lsp_linear_static(const void* A, const void* W, void* out, int M, int N, int
     static_msg(err, err_len, "lsp_linear_static: clearing the counters failed (%s)", cudaGetErrorString(e));
     return LSP_ERR_CUDA;
   }
-  StreamArgs args{M, N, n_tiles, 1, 0, 0, 1, kc, a_rows, atoms, kStaticBN / 2, stages, 0, partials, counters, status};
+  StreamArgs args{M, N, n_tiles, 1, 0, 0, 1, kc, a_rows, atoms, 1, 0, stages, 0, partials, counters, status};
   EpiStore<bf16> epi{(bf16*)out, N};
   k_gemm_stream<kStaticBN, 1, 2, EpiStore<bf16>><<<grid, ST_THREADS, smem, stream>>>(ma, mb, mb, args, epi);
   e = cudaGetLastError();

@@ -34,6 +34,7 @@ extern "C" {
  *   29 the K slices of a split tile run as one thread block cluster, reduced through distributed shared memory (1,
  *      default), or through global scratch by the last CTA to arrive (0)
  *   32 tile width of the dual (SwiGLU) GEMM: 0 = automatic (default), 192 or 256
+ *   43 a SwiGLU tile's weights come by one copy per half and K atom even where one copy can bring them all (0, default)
  *   33 a cluster of 2 exchanges half tiles (1, default) or publishes whole partial tiles like larger clusters (0)
  * GEMM on pairs of SMs:
  *   40 fewest rows that take it (default 257)   41 its tile width (0 = automatic, 96 ... 256 in steps of 32)

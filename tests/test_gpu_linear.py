@@ -357,3 +357,22 @@ def test_rotary_projection_on_pairs_of_sms(dh, hq, hkv, bn):
         dec.close()
     typical = kv[1].square().mean().sqrt()
     assert bool(((kv[0] - kv[1]).abs() <= (kv[1].abs() + typical) / 128).all())
+
+
+@pytest.mark.parametrize("M,N,K,opts", [(5, 12288, 256, {}), (100, 384, 192, {}), (200, 12288, 320, {}), (128, 1152, 576, {43: 1}),
+                                        (200, 12288, 320, {43: 1}), (64, 9600, 1024, {29: 0})])
+@pytest.mark.parametrize("up_first", [False, True])
+def test_swiglu_weights_by_one_copy_in_either_order(M, N, K, opts, up_first):
+    """At most 256 rows: one copy brings a SwiGLU tile's gate and up rows whichever of the two tensors lies first in memory
+    (the accumulators then come in that order), and by one copy per half and atom.  Two bf16 ulps: the product has two factors."""
+    dec = _dec("bf16")
+    for k, v in opts.items():
+        dec.debug_set(k, v)
+    W = S.normal((2, N, K), 12, 2, 0.05, torch.bfloat16, DEV)
+    A = S.normal((M, K), 12, 1, 1.0, torch.bfloat16, DEV)
+    gate, up = (W[1], W[0]) if up_first else (W[0], W[1])
+    out = torch.empty(M, N, dtype=torch.bfloat16, device=DEV)
+    dec.op_linear(2, A, gate, up, out)
+    want = torch.nn.functional.silu(A.double() @ gate.double().t()) * (A.double() @ up.double().t())
+    assert bool(((out.double() - want).abs() <= want.abs() / 64 + want.abs().max() / 2560).all())
+    dec.close()
