@@ -100,6 +100,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
               const __grid_constant__ CUtensorMap map_b1, StreamArgs args, Epi epi) {
   extern __shared__ uint8_t smem_raw[];
   pdl_release();
+  constexpr bool kRope = std::is_same<Epi, EpiQKVRope<bf16>>::value;
   constexpr int HALF = BN / 2;
   constexpr int B_HALF_ATOM = HALF * 128;               // bytes of one half-tile atom (64 K elements)
   constexpr int B_ATOM = BN * 128;
@@ -209,6 +210,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       pos_next(p);
     }
   }
+  if (threadIdx.x == 64) tma_prefetch_map(&map_a);      // its first use comes right after pdl_wait()
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(TMEM_COLS)
@@ -322,6 +324,12 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       const int seg_end = min(u1, tile_u0 + args.kc);
       const bool whole = (u == tile_u0) && (seg_end == tile_u0 + args.kc);
       const int buf = seg % NBUF, use = seg / NBUF;
+      const int j0 = tile * CH;
+      // what the first chunk's epilogue reads is fetched while the MMAs run (see EpiPre)
+      EpiPre<Epi> preA, preB;
+      if constexpr (!Epi::kReduce) {
+        if (whole && row0 + r_in < args.M && j0 < args.n_pairs) preA.load(epi, row0 + r_in, j0);
+      }
       if (!mbar_wait(accf_bar(buf), (uint32_t)use & 1u, abort_flag)) {
         if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 14u; }
         ok = false;
@@ -329,7 +337,6 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       }
       tc_fence_after();
       const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * SET_COLS);
-      const int j0 = tile * CH;
       if (whole) {
         // the accumulator is complete in tensor memory: each thread owns one row of every row tile
 #pragma unroll 1
@@ -339,7 +346,12 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
           Top2 red = top2_empty();
           // one chunk of 16 columns (or pairs) at a time; the next chunk's tensor-memory loads are in flight while this
           // one is converted and stored (with K-parity accumulators the extra loads are not pipelined)
-          auto consume = [&](int c, float (&a0)[16], float (&a1)[16]) {
+          auto fetch = [&](int c, EpiPre<Epi>& pre) {
+            if constexpr (!Epi::kReduce) {
+              if (m < args.M && c < CH && j0 + c < args.n_pairs) pre.load(epi, m, j0 + c);
+            }
+          };
+          auto consume = [&](int c, float (&a0)[16], float (&a1)[16], const EpiPre<Epi>& pre) {
             if constexpr (ACC == 2) {               // add the second K-parity accumulator
               float b0[16];
               tc_ld16(t_row + BN + c, b0);
@@ -354,13 +366,28 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             if constexpr (Epi::kReduce) {
               top2_push16(red, a0, j0 + c, epi);
             } else {
-              if (m < args.M && j0 + c < args.n_pairs) epi16(epi, m, j0 + c, a0, a1);
+              if (m < args.M && j0 + c < args.n_pairs) epi16(epi, m, j0 + c, a0, a1, pre);
             }
           };
           auto request = [&](int c, float (&a0)[16], float (&a1)[16]) {
             tc_ld16_nowait(t_row + mt * ACC * BN + c, a0);
             if (Epi::kDual) tc_ld16_nowait(t_row + mt * ACC * BN + HALF + c, a1);
           };
+          if (mt > 0) fetch(0, preA);
+          if constexpr (kRope) {
+            // (the table entries of two chunks take the registers a second set of accumulator values would)
+            float p0[16], p1[16];
+#pragma unroll 1
+            for (int c = 0; c < CH; c += 16) {
+              request(c, p0, p1);
+              fetch(c + 16, preB);
+              tc_wait_ld();
+              tc_pin16(p0);
+              tc_pin16(p1);
+              consume(c, p0, p1, preA);
+              preA = preB;
+            }
+          } else {
           float p0[16], p1[16], q0[16], q1[16];
           request(0, p0, p1);
 #pragma unroll 1
@@ -369,14 +396,17 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             tc_pin16(p0);
             if (Epi::kDual) tc_pin16(p1);
             if (c + 16 < CH) request(c + 16, q0, q1);
-            consume(c, p0, p1);
+            fetch(c + 16, preB);
+            consume(c, p0, p1, preA);
             if (c + 16 < CH) {                     // CH is a multiple of 16, not always of 32 (48 pairs per tile)
               tc_wait_ld();
               tc_pin16(q0);
               if (Epi::kDual) tc_pin16(q1);
               if (c + 32 < CH) request(c + 32, p0, p1);
-              consume(c + 16, q0, q1);
+              fetch(c + 32, preA);
+              consume(c + 16, q0, q1, preB);
             }
+          }
           }
           if constexpr (Epi::kReduce) {
             if (m < args.M) epi.part[(size_t)m * epi.n_tiles + tile] = red;
@@ -402,6 +432,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
 #pragma unroll 1
             for (int mt = 0; mt < MT; ++mt) {
               const int m = mt * UM_BM + r_in;
+              if (row0 + mt * UM_BM + q * 32 >= args.M) break;  // none of this warp's rows exists
 #pragma unroll 1
               for (int ch = p_lo; ch < p_hi; ++ch) {
 #pragma unroll
@@ -431,6 +462,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
 #pragma unroll 1
         for (int mt = 0; mt < (by_tile ? 1 : MT); ++mt) {
           const int m = mt * UM_BM + r_in;              // row within the row group
+          if (row0 + mt * UM_BM + q * 32 >= args.M) break;      // none of this warp's rows exists
 #pragma unroll 1
           for (int c = 0; c < BN; c += 16) {
             float v[16];
@@ -473,7 +505,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
           const int g_lo = st_owner(U, G, tile_u0), g_hi = st_owner(U, G, tile_u0 + args.kc - 1);
           // The tile is the sum of the contributors' partial tiles.  Work items are (row, 16-column chunk), dealt over
           // the 128 epilogue threads so that a tile with few rows still uses all of them, and every item issues the
-          // loads of up to four contributors before it adds them (in CTA order: deterministic).
+          // loads of several contributors before it adds them (in CTA order: deterministic).
           constexpr int NCH = CH / 16;                 // chunks per row
           constexpr int RPP = 128 / NCH;               // rows per pass
           const int et = threadIdx.x - 64;
@@ -488,10 +520,11 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
 #pragma unroll
             for (int i = 0; i < 16; ++i) { a0[i] = 0.f; a1[i] = 0.f; }
             if (valid) {
-              for (int gb = g_lo; gb <= g_hi; gb += 4) {
-                float4 t0[4][4], t1[4][4];
+              constexpr int GB = Epi::kDual ? 2 : 4;
+              for (int gb = g_lo; gb <= g_hi; gb += GB) {
+                float4 t0[GB][4], t1[GB][4];
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
+                for (int x = 0; x < GB; ++x) {
                   const int gg = gb + x;
                   if (gg <= g_hi) {
                     // contributor gg's segment of this tile is its first one iff its share starts inside the tile
@@ -508,7 +541,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                   }
                 }
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
+                for (int x = 0; x < GB; ++x) {
                   if (gb + x <= g_hi) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
@@ -538,48 +571,81 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
   }
   if (args.cluster == 2 && args.cl_rounds == 0) {
     // Pair exchange: after the barrier each CTA adds, for its own half of the chunks, its accumulator (still in tensor
-    // memory) and the peer's published piece, and runs the fused epilogue.  One row per thread, as in the plain epilogue.
-    cluster_sync();
+    // memory) and the peer's published piece, and runs the fused epilogue.  One row per thread, as in the plain epilogue;
+    // the next chunk's piece and what its epilogue reads are requested before the current one is finished.
     if constexpr (!Epi::kReduce && ACC == 1) {
-      if (warp >= 2 && warp <= 5 && n_units > 0) {
-        constexpr int CH = Epi::kDual ? HALF : BN;
-        constexpr int P = Epi::kDual ? 2 : 1;
-        const int rank = (int)cluster_ctarank();
-        const int o_lo = (CH / 16) * rank / 2, o_hi = (CH / 16) * (rank + 1) / 2;               // this CTA's chunks
-        const int q = warp & 3, r_in = q * 32 + lane;
-        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
-        const uint32_t peer = cluster_map(smem_u32(smem), (unsigned)(rank ^ 1));
-        const int j0 = cl_tile * CH;
-        tc_fence_after();
-#pragma unroll 1
-        for (int mt = 0; mt < MT; ++mt) {
-          const int m = mt * UM_BM + r_in;
-          const bool live = cl_row0 + m < args.M;
-#pragma unroll 1
-          for (int ch = o_lo; ch < o_hi; ++ch) {
-            float a0[16], a1[16];
-            tc_ld16(t_row + mt * BN + ch * 16, a0);
-            if (Epi::kDual) tc_ld16(t_row + mt * BN + HALF + ch * 16, a1);
-            if (live) {
-              float4 t0[4], t1[4];
+      constexpr int CH = Epi::kDual ? HALF : BN;
+      constexpr int P = Epi::kDual ? 2 : 1;
+      const int rank = (int)cluster_ctarank();
+      const int o_lo = (CH / 16) * rank / 2, n_ch = (CH / 16) * (rank + 1) / 2 - o_lo;        // this CTA's chunks
+      const int q = warp & 3, r_in = q * 32 + lane;
+      const bool mine = warp >= 2 && warp <= 5 && n_units > 0;
+      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
+      const uint32_t peer = cluster_map(smem_u32(smem), (unsigned)(rank ^ 1));
+      const int j0 = cl_tile * CH;
+      auto live = [&](int it) { return it < MT * n_ch && cl_row0 + (it / n_ch) * UM_BM + r_in < args.M && j0 + (o_lo + it % n_ch) * 16 < args.n_pairs; };
+      auto fetch = [&](int it, EpiPre<Epi>& pre) {
+        if (live(it)) pre.load(epi, cl_row0 + (it / n_ch) * UM_BM + r_in, j0 + (o_lo + it % n_ch) * 16);
+      };
+      auto request = [&](int it, float4 (&t0)[4], float4 (&t1)[4]) {
+        if (live(it)) {
+          const int m = (it / n_ch) * UM_BM + r_in, k = it % n_ch;
 #pragma unroll
-              for (int i = 0; i < 4; ++i) t0[i] = ld_cluster_f4(peer + (uint32_t)(((((ch - o_lo) * P) * 4 + i) * ROWS + m) * 16));
-              if (Epi::kDual) {
+          for (int i = 0; i < 4; ++i) t0[i] = ld_cluster_f4(peer + (uint32_t)(((k * P * 4 + i) * ROWS + m) * 16));
+          if (Epi::kDual) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) t1[i] = ld_cluster_f4(peer + (uint32_t)(((((ch - o_lo) * P + 1) * 4 + i) * ROWS + m) * 16));
-              }
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                a0[4 * i] += t0[i].x; a0[4 * i + 1] += t0[i].y; a0[4 * i + 2] += t0[i].z; a0[4 * i + 3] += t0[i].w;
-                if (Epi::kDual) {
-                  a1[4 * i] += t1[i].x; a1[4 * i + 1] += t1[i].y; a1[4 * i + 2] += t1[i].z; a1[4 * i + 3] += t1[i].w;
-                }
-              }
-              if (j0 + ch * 16 < args.n_pairs) epi16(epi, cl_row0 + m, j0 + ch * 16, a0, a1);
-            }
+            for (int i = 0; i < 4; ++i) t1[i] = ld_cluster_f4(peer + (uint32_t)((((k * P + 1) * 4 + i) * ROWS + m) * 16));
           }
         }
+      };
+      auto finish = [&](int it, const float4 (&t0)[4], const float4 (&t1)[4], const EpiPre<Epi>& pre) {
+        const int mt = it / n_ch, ch = o_lo + it % n_ch;
+        float a0[16], a1[16];
+        tc_ld16(t_row + mt * BN + ch * 16, a0);
+        if (Epi::kDual) tc_ld16(t_row + mt * BN + HALF + ch * 16, a1);
+        if (live(it)) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            a0[4 * i] += t0[i].x; a0[4 * i + 1] += t0[i].y; a0[4 * i + 2] += t0[i].z; a0[4 * i + 3] += t0[i].w;
+            if (Epi::kDual) {
+              a1[4 * i] += t1[i].x; a1[4 * i + 1] += t1[i].y; a1[4 * i + 2] += t1[i].z; a1[4 * i + 3] += t1[i].w;
+            }
+          }
+          epi16(epi, cl_row0 + mt * UM_BM + r_in, j0 + ch * 16, a0, a1, pre);
+        }
+      };
+      EpiPre<Epi> preA, preB;
+      if (mine) fetch(0, preA);
+      cluster_sync();
+      // a warp whose rows do not exist has nothing to finish
+      const int n_it = (mine && cl_row0 + q * 32 < args.M) ? MT * n_ch : 0;
+      if (n_it > 0) {
+        tc_fence_after();
+        float4 a0[4], a1[4], b0[4], b1[4];
+        request(0, a0, a1);
+        if constexpr (kRope) {              // (registers: one piece at a time)
+#pragma unroll 1
+          for (int it = 0; it < n_it; ++it) {
+            finish(it, a0, a1, preA);
+            request(it + 1, a0, a1);
+            fetch(it + 1, preA);
+          }
+        } else {
+#pragma unroll 1
+        for (int it = 0; it < n_it; it += 2) {
+          request(it + 1, b0, b1);
+          fetch(it + 1, preB);
+          finish(it, a0, a1, preA);
+          if (it + 1 < n_it) {
+            request(it + 2, a0, a1);
+            fetch(it + 2, preA);
+            finish(it + 1, b0, b1, preB);
+          }
+        }
+        }
       }
+    } else {
+      cluster_sync();
     }
     cluster_sync();      // nobody leaves while its peer may still read its shared memory
   } else if (args.cluster > 1) {
@@ -609,30 +675,44 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
           }
         }
       }
-      cluster_sync();
-      if constexpr (!Epi::kReduce) {
-        if (warp >= 2 && warp <= 5 && n_units > 0) {
-          constexpr int CH = Epi::kDual ? HALF : BN;
-          constexpr int NCH = CH / 16;
-          const unsigned rank = cluster_ctarank();
-          const int ch_lo = NCH * (int)rank / C, ch_hi = NCH * ((int)rank + 1) / C;
-          const int r_first = cl_row0 + rd * PR;                       // first activation row of this round
-          const int rows_here = max(0, min(PR, args.M - r_first));
-          const int n_items = rows_here * (ch_hi - ch_lo);
+      if constexpr (Epi::kReduce) {
+        cluster_sync();
+      } else {
+        constexpr int CH = Epi::kDual ? HALF : BN;
+        constexpr int NCH = CH / 16;
+        const unsigned rank = cluster_ctarank();
+        const int ch_lo = NCH * (int)rank / C, ch_hi = NCH * ((int)rank + 1) / C;
+        const int r_first = cl_row0 + rd * PR;                       // first activation row of this round
+        const int rows_here = max(0, min(PR, args.M - r_first));
+        const int n_items = (warp >= 2 && warp <= 5 && n_units > 0) ? rows_here * (ch_hi - ch_lo) : 0;
+        const int j0 = cl_tile * CH;
+        // what an item's epilogue reads is fetched before the barrier, then one item ahead
+        EpiPre<Epi> pre, next;
+        auto fetch = [&](int idx, EpiPre<Epi>& p) {
+          if (idx >= 0 && idx < n_items) {               // (threads of the first two warps pass negative indices)
+            const int c = (ch_lo + idx / rows_here) * 16;
+            if (j0 + c < args.n_pairs) p.load(epi, r_first + idx % rows_here, j0 + c);
+          }
+        };
+        fetch((int)threadIdx.x - 64, pre);
+        cluster_sync();
+        if (n_items > 0) {
           const uint32_t base = smem_u32(smem);
           for (int idx = threadIdx.x - 64; idx < n_items; idx += 128) {
             const int mm = idx % rows_here, ch = ch_lo + idx / rows_here, c = ch * 16;
+            if (!kRope) fetch(idx + 128, next);          // (registers: a rotary item's table entries follow the item)
             float a0[16], a1[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) { a0[i] = 0.f; a1[i] = 0.f; }
             const uint32_t off0 = (uint32_t)(((c >> 4) * 4 * PR + mm) * 16);
             const uint32_t off1 = (uint32_t)((((HALF + c) >> 4) * 4 * PR + mm) * 16);
-            // up to four ranks' pieces are requested before any is added (the loads are independent; the sum stays in
-            // rank order)
-            for (int pb = 0; pb < C; pb += 4) {
-              float4 t0[4][4], t1[4][4];
+            // several ranks' pieces are requested before any is added (the loads are independent; the sum stays in rank
+            // order): four, or two where an item is a pair of chunks
+            constexpr int PB = Epi::kDual ? 2 : 4;
+            for (int pb = 0; pb < C; pb += PB) {
+              float4 t0[PB][4], t1[PB][4];
 #pragma unroll
-              for (int x = 0; x < 4; ++x) {
+              for (int x = 0; x < PB; ++x) {
                 if (pb + x < C) {
                   const uint32_t peer = cluster_map(base, (unsigned)(pb + x));
 #pragma unroll
@@ -644,7 +724,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                 }
               }
 #pragma unroll
-              for (int x = 0; x < 4; ++x) {
+              for (int x = 0; x < PB; ++x) {
                 if (pb + x < C) {
 #pragma unroll
                   for (int i = 0; i < 4; ++i) {
@@ -656,8 +736,9 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                 }
               }
             }
-            const int j0 = cl_tile * CH;
-            if (j0 + c < args.n_pairs) epi16(epi, r_first + mm, j0 + c, a0, a1);
+            if (j0 + c < args.n_pairs) epi16(epi, r_first + mm, j0 + c, a0, a1, pre);
+            if (kRope) fetch(idx + 128, pre);
+            else pre = next;
           }
         }
       }
@@ -809,7 +890,8 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
     if (splits >= 2 && splits <= 8 && kc >= splits && area >= tile_bytes) {
       cluster = splits;
       if (area < MT * tile_bytes) cl_rounds = MT;      // the partial tile is published one row tile at a time
-      if (splits == 2 && st.stream_exchange && !(MT == 1 && NI == 2) && 2 * area >= MT * tile_bytes) cl_rounds = 0;
+      // (a few rows: their items are better dealt over all epilogue threads than kept by the warp that owns the rows)
+      if (splits == 2 && st.stream_exchange && !(MT == 1 && NI == 2) && 2 * area >= MT * tile_bytes && (M >= st.stream_exchange_rows || area < MT * tile_bytes)) cl_rounds = 0;
     }
   }
   // at most 192 rows on two row tiles, every CTA one unsplit tile: 64-row MMAs for the second row tile

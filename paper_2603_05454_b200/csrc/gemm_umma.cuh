@@ -82,6 +82,10 @@ __global__ void k_wait_selftest(unsigned* status, unsigned long long limit_ns) {
     }
   }
 }
+// Fetches a tensor map ahead of the first copy that uses it (about a microsecond of its latency).
+__device__ __forceinline__ void tma_prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
@@ -211,16 +215,54 @@ __device__ __forceinline__ void epi16(const EpiStore<bf16>& e, int m, int j, con
   p[0] = pack8(a0);
   p[1] = pack8(a0 + 8);
 }
-__device__ __forceinline__ void epi16(const EpiResidual<bf16>& e, int m, int j, const float* a0, const float*) {
+// What an epilogue reads from memory for 16 columns (or pairs), fetched ahead of the accumulators: EpiPre::load early, then
+// epi16 with it.  Left to the epilogue itself, one L2 round trip (two for the rotary table, which is indexed by a loaded row
+// position) per chunk of 16 columns lies behind the last MMA: 5 us of a QKV projection, 2 to 3 of an O or down projection.
+template <typename Epi>
+struct EpiPre {
+  __device__ __forceinline__ void load(const Epi&, int, int) {}
+};
+template <>
+struct EpiPre<EpiResidual<bf16>> {
+  uint4 x[2];
+  __device__ __forceinline__ void load(const EpiResidual<bf16>& e, int m, int j) {
+    const uint4* p = reinterpret_cast<const uint4*>(e.x + (size_t)m * e.ld + j);
+    x[0] = p[0];
+    x[1] = p[1];
+  }
+};
+template <>
+struct EpiPre<EpiQKVRope<bf16>> {
+  float4 c[8];        // (cos, sin) of 16 frequencies
+  __device__ __forceinline__ void load(const EpiQKVRope<bf16>& e, int m, int j) {
+    const int h = j / e.half, i = j % e.half;
+    if (h < e.n_heads + e.n_kv_heads) {
+      const float4* c4 = reinterpret_cast<const float4*>(e.cs + (size_t)__ldg(e.row_pos + m) * e.half + i);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) c[q] = __ldg(c4 + q);
+    }
+  }
+};
+template <typename Epi>
+__device__ __forceinline__ void epi16(const Epi& e, int m, int j, const float* a0, const float* a1, const EpiPre<Epi>&) {
+  epi16(e, m, j, a0, a1);
+}
+__device__ __forceinline__ void epi16(const EpiResidual<bf16>& e, int m, int j, const float* a0, const float*,
+                                      const EpiPre<EpiResidual<bf16>>& pre) {
   uint4* p = reinterpret_cast<uint4*>(e.x + (size_t)m * e.ld + j);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     float x[8];
-    unpack8(p[h], x);
+    unpack8(pre.x[h], x);
 #pragma unroll
     for (int i = 0; i < 8; ++i) x[i] += a0[8 * h + i];
     p[h] = pack8(x);
   }
+}
+__device__ __forceinline__ void epi16(const EpiResidual<bf16>& e, int m, int j, const float* a0, const float* a1) {
+  EpiPre<EpiResidual<bf16>> pre;
+  pre.load(e, m, j);
+  epi16(e, m, j, a0, a1, pre);
 }
 __device__ __forceinline__ void epi16(const EpiSwiGLU<bf16>& e, int m, int j, const float* g, const float* u) {
   float r[16];
@@ -235,17 +277,17 @@ __device__ __forceinline__ void epi16(const EpiSwiGLU<bf16>& e, int m, int j, co
   p[0] = pack8(r);
   p[1] = pack8(r + 8);
 }
-__device__ __forceinline__ void epi16(const EpiQKVRope<bf16>& e, int m, int j, const float* a0, const float* a1) {
+__device__ __forceinline__ void epi16(const EpiQKVRope<bf16>& e, int m, int j, const float* a0, const float* a1,
+                                      const EpiPre<EpiQKVRope<bf16>>& pre) {
   const int h = j / e.half, i = j % e.half;       // 16 indices stay inside one head (half is a multiple of 16)
   const int dh = 2 * e.half;
   float r0[16], r1[16];
   bf16* dst;
   if (h >= e.n_heads && e.seq_stride > 0 && e.row_seq[m] < 0) return;      // in-place layout: a row of no sequence has no cache slot
   if (h < e.n_heads + e.n_kv_heads) {
-    const float4* c4 = reinterpret_cast<const float4*>(e.cs + (size_t)e.row_pos[m] * e.half + i);
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const float4 c = __ldg(c4 + q);             // (cos, sin) of two consecutive frequencies
+      const float4 c = pre.c[q];                  // (cos, sin) of two consecutive frequencies
       r0[2 * q] = a0[2 * q] * c.x - a1[2 * q] * c.y;
       r1[2 * q] = a1[2 * q] * c.x + a0[2 * q] * c.y;
       r0[2 * q + 1] = a0[2 * q + 1] * c.z - a1[2 * q + 1] * c.w;
@@ -264,6 +306,11 @@ __device__ __forceinline__ void epi16(const EpiQKVRope<bf16>& e, int m, int j, c
   p0[1] = pack8(r0 + 8);
   p1[0] = pack8(r1);
   p1[1] = pack8(r1 + 8);
+}
+__device__ __forceinline__ void epi16(const EpiQKVRope<bf16>& e, int m, int j, const float* a0, const float* a1) {
+  EpiPre<EpiQKVRope<bf16>> pre;
+  pre.load(e, m, j);
+  epi16(e, m, j, a0, a1, pre);
 }
 
 // ---- host side ------------------------------------------------------------------------------------------------
@@ -296,6 +343,7 @@ struct UmmaState {
   int stream_bn2 = 0;              // ... and with two row tiles
   int stream_bn_dual = 0;          // tile width of dual epilogues: 0 = automatic, 192 or 256
   int stream_exchange = 1;         // clusters of 2 exchange half tiles instead of publishing whole partial tiles
+  int stream_exchange_rows = 64;   // ... from this many rows on
   int stream_atoms = 0;            // K atoms per stage: 0 = two when stream_min_stages2 such stages fit, else 1 or 2 as given
   int stream_min_stages2 = 3;
   int stream_split_copies = 0;     // a dual tile's weights by one copy per half and atom even where one copy can bring them all

@@ -803,6 +803,7 @@ int lsp_debug_set(lsp_ctx* c, int key, int value) {
   else if (key == 41) c->umma.pair_bn = (value >= 96 && value <= 256 && value % 32 == 0) ? value : 0;
   else if (key == 42) c->umma.pair_band = value < 0 ? 0 : value;
   else if (key == 43) c->umma.stream_split_copies = value ? 1 : 0;
+  else if (key == 44) c->umma.stream_exchange_rows = value;
   else if (key == 21) c->umma.stream_atoms = value;
   else if (key == 22) c->umma.stream_min_stages2 = value < 2 ? 2 : value;
 #endif
