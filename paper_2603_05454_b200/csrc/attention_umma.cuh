@@ -58,8 +58,15 @@ __device__ __forceinline__ float ex2_approx(float x) {
 }
 __device__ __forceinline__ float ld_cluster_f1(uint32_t addr) {
   float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr));
   return v;
+}
+// One 64-element atom of the Q tile of a KV head: positions x G heads (attn_q_map).
+__device__ __forceinline__ void tma_load_5d_q(uint32_t dst, const CUtensorMap* map, int kvh, int pos, int atom, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %2, %3, %4, %5}], [%6];"
+      ::"r"(dst), "l"(map), "r"(0), "r"(kvh), "r"(pos), "r"(atom), "r"(bar)
+      : "memory");
 }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
@@ -82,10 +89,16 @@ __device__ __forceinline__ uint32_t au_swz(int r, int c) {
 }
 
 // grid = (ceil(max rows per sequence * group / 128) * cluster, n_kv_heads, batch)
+// kRolled: the softmax reads its scores from tensor memory twice, 32 at a time in rolled loops, instead of holding all 128 of
+// a row in registers.  In small passes a CTA has one or two key tiles and its instructions come anew from L2 behind a stream
+// of weights: fetching the unrolled code takes longer than the arithmetic (one tile 5.1 -> 2.8 us; a LLaDA-shaped pass of 9 /
+// 101 rows 3.92 -> 3.77, 4.43 -> 4.29 ms together with the other changes to this kernel's latency).  With many tiles per CTA the
+// second read costs more than the code (16 x 515 rows over 2000 keys: 560 us a launch unrolled, 630 rolled).
+template <bool kRolled>
 __global__ void __launch_bounds__(AU_THREADS, 1)
-k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ CUtensorMap map_cv,
-            const __grid_constant__ CUtensorMap map_sk, const __grid_constant__ CUtensorMap map_sv,
-            const bf16* __restrict__ q, bf16* __restrict__ out, StepDesc sd, int n_heads, int n_kv_heads, int max_len,
+k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_ck,
+            const __grid_constant__ CUtensorMap map_cv, const __grid_constant__ CUtensorMap map_sk,
+            const __grid_constant__ CUtensorMap map_sv, bf16* __restrict__ out, StepDesc sd, int n_heads, int n_kv_heads, int max_len,
             float scale_log2, int cluster, int inplace, unsigned* status) {
   constexpr int DH = 128;
   extern __shared__ uint8_t smem_raw[];
@@ -98,8 +111,7 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
   // bars (each + stage s = softmax group w = tile parity): 0 k_full; 2 k_empty; 4 v_full; 6 v_empty; 8 s_full; 10 s_empty;
   // 12 p_ready; 14 pv_done.  K and V stages are released separately (K by the tile's Q K^T, V by its P V), so that the
   // next tile's K is on its way while this tile's softmax runs.
-  // 16 q_ready: the eight softmax warps have put the Q tile in place (only the Q K^T issuer waits for it, so the K/V
-  // copies are already under way while Q is being loaded)
+  // 16 q_ready: the Q tile has arrived
   constexpr int B_KF = 0, B_KE = 2, B_VF = 4, B_VE = 6, B_SF = 8, B_SE = 10, B_PR = 12, B_PD = 14, B_Q = 16;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 18);
   volatile uint32_t* abort_flag = tmem_slot + 1;
@@ -112,10 +124,26 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
   const int G = n_heads / n_kv_heads;
   if (threadIdx.x == 0) {
     for (int i = 0; i < 16; ++i) mbar_init(bar(i), (i >= B_SE && i < B_PD) ? 4 : 1);     // s_empty, p_ready: four warps arrive
-    mbar_init(bar(B_Q), 8);
+    mbar_init(bar(B_Q), 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  // tile rows that stand for no position (G does not divide 128): zeros, so that every accumulator row is finite
+  for (int i = (AU_BM / G) * G * 8 + (int)threadIdx.x; i < AU_BM * 8; i += AU_THREADS) {
+    const uint32_t off = (uint32_t)((i >> 6) * 1024 + ((i >> 3) & 7) * 128 + (i & 7) * 16);
+    *reinterpret_cast<uint4*>(Qs + off) = make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(Qs + AU_ATOM + off) = make_uint4(0u, 0u, 0u, 0u);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  if (warp == AU_W_TMA && lane == 0) {
+    tma_prefetch_map(&map_q);
+    tma_prefetch_map(&map_ck);
+    tma_prefetch_map(&map_sk);
+  }
+  if (warp == AU_W_TMAV && lane == 0) {
+    tma_prefetch_map(&map_cv);
+    tma_prefetch_map(&map_sv);
   }
   if (warp == AU_W_QK) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u)
@@ -131,37 +159,19 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
 
   const int r0 = sd.row_off[b];
   const int Qn = sd.row_off[b + 1] - r0;
-  const int rows_total = Qn * G;
   // With clusters (size C along x) the C CTAs of a cluster share one row tile and deal its key tiles round-robin:
   // rank r takes tiles r, r + C, ...; their partial (m, l, O) are merged through distributed shared memory at the end.
   const int C = cluster > 1 ? cluster : 1;
   const int rank = (int)(blockIdx.x % C);
-  const int row_base = (int)(blockIdx.x / C) * AU_BM;
+  // a row tile: 128 / G whole query positions of G heads each (row r = position r / G, head r % G)
+  const int pos_tile = AU_BM / G;
+  const int pos0 = (int)(blockIdx.x / C) * pos_tile;
   // in-place layout: this pass's K/V rows already sit behind the prefix in the cache, so every key tile is a cache tile
   const int F = sd.F[b] + (inplace ? Qn : 0);
   const int n_c = (F + AU_BN - 1) / AU_BN, n_s = inplace ? 0 : (Qn + AU_BN - 1) / AU_BN;
-  const int n_all = (row_base < rows_total) ? n_c + n_s : 0;       // a CTA past the last row does nothing
+  const int n_all = (pos0 < Qn) ? n_c + n_s : 0;       // a CTA past the last row does nothing
   const int n_tiles = n_all > rank ? (n_all - rank + C - 1) / C : 0;   // this CTA's tiles; t below counts them
   const int ldq = n_heads * DH;
-
-  if (warp < 8) {
-    // ---- Q tile -> swizzled shared memory (zeros for rows past the end): row r by two threads, eight chunks each
-    const int r = threadIdx.x & 127, c0 = (threadIdx.x >> 7) * 8;
-    const int row = row_base + r;
-    const bool valid = row < rows_total;
-    if (n_tiles > 0) {
-      const int qi = valid ? row / G : 0, hg = valid ? row % G : 0;
-      const uint4* src = reinterpret_cast<const uint4*>(q + (size_t)(r0 + qi) * ldq + (kvh * G + hg) * DH);
-#pragma unroll
-      for (int c = c0; c < c0 + 8; ++c) {
-        const uint4 v = valid ? __ldg(src + c) : make_uint4(0u, 0u, 0u, 0u);
-        *reinterpret_cast<uint4*>(Qs + au_swz(r, c)) = v;
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(bar(B_Q));
-  }
 
   if (warp == AU_W_TMA || warp == AU_W_TMAV) {
     // ---------------- TMA producers: one thread streams the K tiles, another the V tiles ----------------
@@ -169,6 +179,13 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
       const bool is_v = warp == AU_W_TMAV;
       const int full = is_v ? B_VF : B_KF, empty = is_v ? B_VE : B_KE;
       int issued = 0;
+      if (!is_v && n_tiles > 0) {
+        // the Q tile (positions past the sequence's end bring other rows or zeros; rows are independent and those are never
+        // stored)
+        mbar_expect_tx(bar(B_Q), (uint32_t)(pos_tile * G * 256));
+        tma_load_5d_q(smem_u32(Qs), &map_q, kvh, r0 + pos0, 0, bar(B_Q));
+        tma_load_5d_q(smem_u32(Qs) + AU_ATOM, &map_q, kvh, r0 + pos0, 1, bar(B_Q));
+      }
       for (int t = 0; t < n_tiles; ++t) {
         const int s = t & 1;
         if (!mbar_wait(bar(empty + s), ((uint32_t)(t >> 1) & 1u) ^ 1u, abort_flag)) {
@@ -186,6 +203,10 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
         ++issued;
       }
       // do not leave while copies may still be landing in this CTA's shared memory
+      if (!is_v && n_tiles > 0) {
+        volatile uint32_t no_abort = 0;
+        mbar_wait(bar(B_Q), 0u, &no_abort);
+      }
       for (int t = issued > 2 ? issued - 2 : 0; t < issued; ++t) {
         volatile uint32_t no_abort = 0;
         mbar_wait(bar(full + (t & 1)), (uint32_t)(t >> 1) & 1u, &no_abort);
@@ -255,7 +276,7 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
     int mine = 0;                                       // tiles this group has processed
     for (int t = w; t < n_tiles; t += 2, ++mine) {
       const uint32_t par = (uint32_t)mine & 1u;
-      if (!mbar_wait(bar(B_SF + w), par, abort_flag)) {
+      if (!__all_sync(0xffffffffu, mbar_wait(bar(B_SF + w), par, abort_flag))) {
         if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 24u; }
         ok = false;
         break;
@@ -263,24 +284,46 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
       tc_fence_after();
       const int gt = rank + t * C;
       const int valid_keys = (gt < n_c) ? min(AU_BN, F - gt * AU_BN) : min(AU_BN, Qn - (gt - n_c) * AU_BN);
-      float sv[AU_BN];
-#pragma unroll
-      for (int c = 0; c < AU_BN; c += 16) tc_ld16_nowait(lane_base + 256u + (uint32_t)(w * AU_BN + c), sv + c);
-      tc_wait_ld();
-#pragma unroll
-      for (int c = 0; c < AU_BN; c += 16) tc_pin16p(sv + c);      // no use of the scores may be scheduled ahead of the wait
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(B_SE + w));       // S buffer read
+      const uint32_t s_col = lane_base + 256u + (uint32_t)(w * AU_BN);
+      __syncwarp();                                     // the loads below are collective
       // raw scores; the scale (positive) is folded into the exponent's FMA, masking only touches a ragged last tile
-      if (valid_keys < AU_BN) {
-#pragma unroll
-        for (int i = 0; i < AU_BN; ++i)
-          if (i >= valid_keys) sv[i] = -INFINITY;
-      }
+      float sv[kRolled ? 1 : AU_BN];
       float mx = -INFINITY;
+      if constexpr (!kRolled) {
 #pragma unroll
-      for (int i = 0; i < AU_BN; ++i) mx = fmaxf(mx, sv[i]);
+        for (int c = 0; c < AU_BN; c += 16) tc_ld16_nowait(s_col + (uint32_t)c, sv + c);
+        tc_wait_ld();
+#pragma unroll
+        for (int c = 0; c < AU_BN; c += 16) tc_pin16p(sv + c);      // no use of the scores may be scheduled ahead of the wait
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(B_SE + w));       // S buffer read
+        if (valid_keys < AU_BN) {
+#pragma unroll
+          for (int i = 0; i < AU_BN; ++i)
+            if (i >= valid_keys) sv[i] = -INFINITY;
+        }
+#pragma unroll
+        for (int i = 0; i < AU_BN; ++i) mx = fmaxf(mx, sv[i]);
+      }
+#pragma unroll 1
+      for (int c = kRolled ? 0 : AU_BN; c < AU_BN; c += 32) {
+        float v[32];
+        tc_ld16_nowait(s_col + (uint32_t)c, v);
+        tc_ld16_nowait(s_col + (uint32_t)(c + 16), v + 16);
+        tc_wait_ld();
+        tc_pin16p(v);
+        tc_pin16p(v + 16);
+        if (valid_keys < c + 32) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (c + i >= valid_keys) v[i] = -INFINITY;
+        }
+        float m4[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+        for (int i = 4; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], v[i]);
+        mx = fmaxf(mx, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
+      }
       mx *= scale_log2;
       float corr = 1.f;
       bool raise = false;
@@ -291,7 +334,7 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
       }
       if (mine > 0) {
         // P_w and O_w are free once the group's previous tile's P V has completed
-        if (!mbar_wait(bar(B_PD + w), (uint32_t)(mine - 1) & 1u, abort_flag)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(bar(B_PD + w), (uint32_t)(mine - 1) & 1u, abort_flag))) {
           if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 25u; }
           ok = false;
           break;
@@ -323,21 +366,59 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
           *reinterpret_cast<uint4*>(vrow + AU_ATOM + 16 * c) = make_uint4(0u, 0u, 0u, 0u);
         }
       }
-      // exponentials, sixteen keys at a time, straight into the swizzled P tile
+      __syncwarp();                                     // the loads below are collective
+      // exponentials straight into the swizzled P tile
       float sum = 0.f;
       const float neg_m = -m_used;
+      if constexpr (!kRolled) {
 #pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        uint32_t pk[4];
+        for (int c = 0; c < 16; ++c) {
+          uint32_t pk[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float p0 = ex2_approx(fmaf(sv[8 * c + 2 * j], scale_log2, neg_m));
-          const float p1 = ex2_approx(fmaf(sv[8 * c + 2 * j + 1], scale_log2, neg_m));
-          sum += p0 + p1;
-          const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
-          pk[j] = *reinterpret_cast<const uint32_t*>(&pb);
+          for (int j = 0; j < 4; ++j) {
+            const float p0 = ex2_approx(fmaf(sv[8 * c + 2 * j], scale_log2, neg_m));
+            const float p1 = ex2_approx(fmaf(sv[8 * c + 2 * j + 1], scale_log2, neg_m));
+            sum += p0 + p1;
+            const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
+            pk[j] = *reinterpret_cast<const uint32_t*>(&pb);
+          }
+          *reinterpret_cast<uint4*>(Pw + au_swz(r, c)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         }
-        *reinterpret_cast<uint4*>(Pw + au_swz(r, c)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      }
+#pragma unroll 1
+      for (int c = kRolled ? 0 : AU_BN; c < AU_BN; c += 32) {
+        float v[32];
+        tc_ld16_nowait(s_col + (uint32_t)c, v);
+        tc_ld16_nowait(s_col + (uint32_t)(c + 16), v + 16);
+        tc_wait_ld();
+        tc_pin16p(v);
+        tc_pin16p(v + 16);
+        if (valid_keys < c + 32) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (c + i >= valid_keys) v[i] = -INFINITY;
+        }
+        float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          uint32_t pk[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float p0 = ex2_approx(fmaf(v[8 * k + 2 * j], scale_log2, neg_m));
+            const float p1 = ex2_approx(fmaf(v[8 * k + 2 * j + 1], scale_log2, neg_m));
+            s0 += p0;
+            s1 += p1;
+            const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
+            pk[j] = *reinterpret_cast<const uint32_t*>(&pb);
+          }
+          *reinterpret_cast<uint4*>(Pw + au_swz(r, (c >> 3) + k)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        }
+        sum += s0 + s1;
+      }
+      if constexpr (kRolled) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(B_SE + w));       // S buffer read
       }
       l = l * corr + sum;
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -346,6 +427,7 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
       if (lane == 0) mbar_arrive(bar(B_PR + w));        // P_w ready
     }
     bool have = ok && mine > 0 && mbar_wait(bar(B_PD + w), (uint32_t)(mine - 1) & 1u, abort_flag);
+    have = __all_sync(0xffffffffu, have);
     if (have) tc_fence_after();
     // ---- the two groups' partial results of row r: weights exp2(m_w - max) as in the merge across a cluster
     if (w == 1) {
@@ -355,7 +437,8 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
     asm volatile("bar.sync 2, 256;" ::: "memory");       // the eight softmax warps
     if (w == 0) {
       const float m1 = ml1[r], l1 = ml1[AU_BM + r];
-      const bool have1 = m1 != -INFINITY;
+      // (uniform per warp: the accumulator loads below are collective, and a row of NaN scores leaves its maximum at -inf)
+      const bool have1 = __any_sync(0xffffffffu, m1 != -INFINITY);
       const float m0 = have ? m_used : -INFINITY;
       const float mm = fmaxf(m0, m1);
       const float w0 = have ? ex2_approx(m0 - mm) : 0.f, w1 = have1 ? ex2_approx(m1 - mm) : 0.f;
@@ -364,11 +447,10 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
       if (have1) tc_fence_after();
       if (C == 1) {
         if (any) {
-          const int row = row_base + r;
           const float inv = __fdividef(1.f, lsum);
           const float f0 = w0 * inv, f1 = w1 * inv;
-          const bool valid = row < rows_total;
-          const int qi = valid ? row / G : 0, hg = valid ? row % G : 0;
+          const int qi = pos0 + r / G, hg = r % G;
+          const bool valid = r < pos_tile * G && qi < Qn;
           uint4* dst = reinterpret_cast<uint4*>(out + (size_t)(r0 + qi) * ldq + (kvh * G + hg) * DH);
 #pragma unroll 1
           for (int c = 0; c < DH; c += 16) {
@@ -409,35 +491,58 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_ck, const __grid_constant__ 
     cluster_sync();
     if (warp < 4 && n_all > 0) {
       const int r = threadIdx.x;
-      const int row = row_base + r;
-      const bool valid = row < rows_total;
+      const int qi = pos0 + r / G, hg = r % G;
+      const bool valid = r < pos_tile * G && qi < Qn;
       const uint32_t base_o = smem_u32(KVs), base_m = base_o + AU_BM * DH * 4;
-      float wgt[8];
-      float mmax = -INFINITY;
-      for (int p = 0; p < C; ++p) {
-        wgt[p] = ld_cluster_f1(cluster_map(base_m + 4u * r, (unsigned)p));
-        mmax = fmaxf(mmax, wgt[p]);
+      // the ranks' (m, l) of this row, all requested before the first is used
+      float wgt[8], lp[8];
+#pragma unroll
+      for (int p = 0; p < 8; ++p) {
+        wgt[p] = -INFINITY;
+        lp[p] = 0.f;
+        if (p < C) {
+          wgt[p] = ld_cluster_f1(cluster_map(base_m + 4u * r, (unsigned)p));
+          lp[p] = ld_cluster_f1(cluster_map(base_m + 4u * (AU_BM + r), (unsigned)p));
+        }
       }
+      float mmax = -INFINITY;
+#pragma unroll
+      for (int p = 0; p < 8; ++p) mmax = fmaxf(mmax, wgt[p]);
       float L = 0.f;
-      for (int p = 0; p < C; ++p) {
+#pragma unroll
+      for (int p = 0; p < 8; ++p) {
         wgt[p] = (wgt[p] == -INFINITY) ? 0.f : ex2_approx(wgt[p] - mmax);
-        L += wgt[p] * ld_cluster_f1(cluster_map(base_m + 4u * (AU_BM + r), (unsigned)p));
+        L += wgt[p] * lp[p];
       }
       const float inv = __fdividef(1.f, L);
-      const int qi = valid ? row / G : 0, hg = valid ? row % G : 0;
       uint4* dst = reinterpret_cast<uint4*>(out + (size_t)(r0 + qi) * ldq + (kvh * G + hg) * DH);
       const int ch_lo = (DH / 16) * rank / C, ch_hi = (DH / 16) * (rank + 1) / C;
+#pragma unroll 1
       for (int ch = ch_lo; ch < ch_hi; ++ch) {
         float v[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = 0.f;
-        for (int p = 0; p < C; ++p) {
-          const uint32_t peer = cluster_map(base_o + (uint32_t)((ch * 4 * AU_BM + r) * 16), (unsigned)p);
+        const uint32_t off = (uint32_t)((ch * 4 * AU_BM + r) * 16);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float4 t4 = ld_cluster_f4(peer + (uint32_t)(i * AU_BM * 16));
-            v[4 * i] += wgt[p] * t4.x; v[4 * i + 1] += wgt[p] * t4.y; v[4 * i + 2] += wgt[p] * t4.z; v[4 * i + 3] += wgt[p] * t4.w;
-          }
+        for (int pb = 0; pb < 8; pb += 4) {            // four ranks' pieces in flight; the sum stays in rank order
+          if (pb >= C || !valid) break;
+          float4 t4[4][4];
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+            if (pb + x < C) {
+              const uint32_t peer = cluster_map(base_o + off, (unsigned)(pb + x));
+#pragma unroll
+              for (int i = 0; i < 4; ++i) t4[x][i] = ld_cluster_f4(peer + (uint32_t)(i * AU_BM * 16));
+            }
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+            if (pb + x < C) {
+              const float wp = wgt[pb + x];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                v[4 * i] += wp * t4[x][i].x; v[4 * i + 1] += wp * t4[x][i].y; v[4 * i + 2] += wp * t4[x][i].z; v[4 * i + 3] += wp * t4[x][i].w;
+              }
+            }
         }
         if (valid) {
 #pragma unroll
@@ -464,6 +569,18 @@ inline bool attn_umma_map(UmmaState& st, CUtensorMap* m, const void* base, size_
   cuuint32_t box[2] = {64, (cuuint32_t)AU_BN};
   cuuint32_t estr[2] = {1, 1};
   return st.encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// 5-D bf16 tensor map of the packed queries [rows, n_heads * 128]: [atom of 64][position][KV head][head of its group][64].
+inline bool attn_q_map(UmmaState& st, CUtensorMap* m, const void* q, size_t rows, int n_heads, int n_kv_heads) {
+  const int G = n_heads / n_kv_heads;
+  cuuint64_t dims[5] = {64, (cuuint64_t)G, (cuuint64_t)n_kv_heads, (cuuint64_t)rows, 2};
+  cuuint64_t strides[4] = {256, (cuuint64_t)G * 256, (cuuint64_t)n_heads * 256, 128};
+  cuuint32_t box[5] = {64, (cuuint32_t)G, 1, (cuuint32_t)(AU_BM / G), 1};
+  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  return st.encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(q), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }

@@ -322,9 +322,9 @@ int check_status(lsp_ctx* c) {
 
 // Suffix-over-prefix attention of layer l (Sec. 3.2: every query row of the pass sees the cached prefix [0, F_b) and all
 // of the pass's own rows).  Reads the uploaded descriptor (F, row_off), Q from q, K/V from the cache and the staging
-// planes of layer l; writes out.  max_q: most query rows of one sequence; max_keys: most keys of one sequence.
+// planes of layer l; writes out.  q_rows: rows of Qb.  max_q: most query rows of one sequence; max_keys: most keys of one sequence.
 template <typename T>
-int run_attention(lsp_ctx* c, int l, const T* Qb, T* Att, const StepDesc& sd, int B, int maxQ, int max_keys, int inplace) {
+int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const StepDesc& sd, int B, int maxQ, int max_keys, int inplace) {
   const lsp_model_cfg& m = c->m;
   const int dh = m.head_dim, kvd = m.n_kv_heads * dh;
   const size_t plane = (size_t)c->max_rows * kvd;
@@ -343,9 +343,11 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, T* Att, const StepDesc& sd, in
   if constexpr (std::is_same<T, bf16>::value) {
     // the tcgen05 kernel (128-row tiles; with few CTAs the keys of a row tile are split over a cluster); a row-count
     // threshold can send small passes to the 64-row mma.sync kernel instead
-    if (c->attn_impl == 2 && dh == 128 && !c->attn_maps.empty() && maxQ * (m.n_heads / m.n_kv_heads) >= c->attn_umma_min_rows) {
-      const int G = m.n_heads / m.n_kv_heads;
-      const int row_tiles = (maxQ * G + AU_BM - 1) / AU_BM;
+    const int G = m.n_heads / m.n_kv_heads;
+    if (c->attn_impl == 2 && dh == 128 && G <= AU_BM && !c->attn_maps.empty() && maxQ * G >= c->attn_umma_min_rows) {
+      const int row_tiles = (maxQ + AU_BM / G - 1) / (AU_BM / G);       // 128 / G whole query positions per tile
+      CUtensorMap map_q;
+      if (!attn_q_map(c->umma, &map_q, Qb, q_rows, m.n_heads, m.n_kv_heads)) return fail(c, LSP_ERR_CUDA, "attention: no tensor map of the queries");
       // few CTAs: split every row tile's keys over a cluster of 2, 4 or 8 CTAs (merged through DSMEM)
       int cl = 1;
       if (c->attn_cluster) {
@@ -357,8 +359,10 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, T* Att, const StepDesc& sd, in
       dim3 g3(row_tiles * cl, m.n_kv_heads, B);
       const float sl2 = scale * 1.4426950408889634f;
       const CUtensorMap* mp = &c->attn_maps[4 * l];
-      launch_k(c->pdl, k_attn_umma, g3, dim3(AU_THREADS), (size_t)AU_SMEM, c->stream, cl, mp[0], mp[1], mp[2], mp[3],
-               (const bf16*)Qb, Att, sd, m.n_heads, m.n_kv_heads, c->max_len, sl2, cl, inplace, c->d_status);
+      // at most two key tiles per CTA: the kernel with rolled softmax loops
+      auto kern = (max_keys + AU_BN - 1) / AU_BN <= 2 * cl ? k_attn_umma<true> : k_attn_umma<false>;
+      launch_k(c->pdl, kern, g3, dim3(AU_THREADS), (size_t)AU_SMEM, c->stream, cl, map_q, mp[0], mp[1], mp[2], mp[3],
+               Att, sd, m.n_heads, m.n_kv_heads, c->max_len, sl2, cl, inplace, c->d_status);
       c->last_attn_kernel = 2;
       c->last_attn_cluster = cl;
       done = true;
@@ -444,7 +448,7 @@ int enqueue_pass(lsp_ctx* c, const StepDesc& sd, int B, const PassDims& pd, int*
     {
       c->counters[CNT_ATTN_BYTES] += pd.attn_bytes;
       c->counters[CNT_ATTN_FLOPS] += pd.attn_flops;
-      const int rc = run_attention<T>(c, l, Qb, Att, sd, B, pd.maxQ, pd.max_keys, c->kv_inplace);
+      const int rc = run_attention<T>(c, l, Qb, M, Att, sd, B, pd.maxQ, pd.max_keys, c->kv_inplace);
       if (rc) return rc;
     }
     {
@@ -722,7 +726,8 @@ int lsp_init(lsp_ctx** out, const lsp_model_cfg* model, const lsp_sched_cfg* sch
       const int kvd = model->n_kv_heads * model->head_dim;
       const size_t plane = (size_t)max_batch * max_len * kvd * 2;      // bytes of one (layer, K|V) plane, cache and staging alike
       c->attn_maps.resize((size_t)4 * model->n_layers);
-      bool ok = cudaFuncSetAttribute(k_attn_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, AU_SMEM) == cudaSuccess;
+      bool ok = cudaFuncSetAttribute(k_attn_umma<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AU_SMEM) == cudaSuccess &&
+                cudaFuncSetAttribute(k_attn_umma<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AU_SMEM) == cudaSuccess;
       for (int l = 0; l < model->n_layers && ok; ++l) {
         const char* ck = c->kv_cache + (size_t)(2 * l) * plane;
         const char* sk = c->stage + (size_t)(2 * l) * plane;
@@ -1209,8 +1214,8 @@ int lsp_op_attention(lsp_ctx* c, int layer, const void* q, const void* k_new, co
   char* stK = c->stage + (size_t)(2 * layer) * plane;
   CU(cudaMemcpyAsync(stK, k_new, (size_t)M * kvd * c->esz, cudaMemcpyDeviceToDevice, c->stream));
   CU(cudaMemcpyAsync(stK + plane, v_new, (size_t)M * kvd * c->esz, cudaMemcpyDeviceToDevice, c->stream));
-  const int rc = c->m.dtype == 0 ? run_attention<float>(c, layer, (const float*)q, (float*)out, desc_of(c), batch, maxQ, max_keys, 0)
-                                 : run_attention<bf16>(c, layer, (const bf16*)q, (bf16*)out, desc_of(c), batch, maxQ, max_keys, 0);
+  const int rc = c->m.dtype == 0 ? run_attention<float>(c, layer, (const float*)q, M, (float*)out, desc_of(c), batch, maxQ, max_keys, 0)
+                                 : run_attention<bf16>(c, layer, (const bf16*)q, M, (bf16*)out, desc_of(c), batch, maxQ, max_keys, 0);
   if (rc) return rc;
   CU(cudaMemcpyAsync(c->h_status, c->d_status, 16, cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));

@@ -133,3 +133,16 @@ def test_attention_repeats_bit_for_bit_with_ragged_tiles(hq, hkv, F, rows):
             wrong += not torch.equal(dec.op_attention(l, q, kn, vn, out, F, rows), first[l])
     dec.close()
     assert wrong == 0, f"{wrong} of {100 * L} launches differ"
+
+
+@pytest.mark.parametrize("case", [
+    (28, 4, [0, 0], [600, 333], 640),            # 18 positions of 7 heads per row tile, no split of the keys, several tiles each
+    (28, 4, [535, 130, 7, 300], [258, 200, 190, 129], 900),
+    (5, 1, [400], [130], 640),                   # 25 positions of 5 heads; fewer CTAs, a cluster
+])
+def test_attention_row_tiles_that_a_group_does_not_fill(case):
+    """A group of G heads that does not divide 128 leaves the last rows of every tile without a query; they hold whatever
+    shared memory held unless cleared, and must neither stop the kernel nor reach the output.  Also over NaN-filled memory."""
+    hq, hkv, F, rows, max_len = case
+    _run_case(hq, hkv, F, rows, max_len)
+    _run_case(hq, hkv, F, rows, max_len, seed=1, poison=True)
