@@ -6,18 +6,20 @@
 
 namespace lsp {
 
-constexpr int AS_BQ = 16;   // queries per block (4 per warp)
+// Queries per block: 4 per warp where that still gives a block per SM, else 1 per warp (the K/V tile is then used by fewer
+// queries, but a small pass is bound by one block's serial walk over the keys: tiny model, 26 -> 19 us a launch).
 constexpr int AS_BK = 32;   // keys per tile (one per lane)
 
-// grid = (ceil(max_rows_per_seq / 16), n_heads, batch), block = 128.
+// grid = (ceil(max_rows_per_seq / (4 QW)), n_heads, batch), block = 128; QW queries per warp.
 // q: [M, n_heads*DH]; cache_k/v: this layer's planes [batch_max][max_len][n_kv*DH]; stage_k/v: this layer's
 // staged planes [M][n_kv*DH]; out: [M, n_heads*DH].
-template <typename T, int DH>
+template <typename T, int DH, int QW>
 __global__ void __launch_bounds__(128) k_attn_simt(const T* __restrict__ q, const T* __restrict__ cache_k,
                                                    const T* __restrict__ cache_v, const T* __restrict__ stage_k,
                                                    const T* __restrict__ stage_v, T* __restrict__ out, StepDesc sd,
                                                    int n_heads, int n_kv_heads, size_t cache_seq_elems,
                                                    float scale, int inplace) {
+  constexpr int AS_BQ = 4 * QW;
   __shared__ float Qs[AS_BQ][DH];
   __shared__ float Ks[AS_BK][DH + 1];
   __shared__ float Vs[AS_BK][DH];
@@ -37,10 +39,10 @@ __global__ void __launch_bounds__(128) k_attn_simt(const T* __restrict__ q, cons
     Qs[qi][d] = (q0 + qi < Qn) ? to_f(q[(size_t)(r0 + q0 + qi) * ldq + h * DH + d]) : 0.f;
   }
   constexpr int NC = DH / 32;
-  float acc[4][NC];
-  float m_run[4], l_run[4];
+  float acc[QW][NC];
+  float m_run[QW], l_run[QW];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < QW; ++i) {
     m_run[i] = -INFINITY;
     l_run[i] = 0.f;
 #pragma unroll
@@ -68,8 +70,8 @@ __global__ void __launch_bounds__(128) k_attn_simt(const T* __restrict__ q, cons
     __syncthreads();
     const bool kvalid = (s0 + lane) < S;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int qi = w * 4 + i;
+    for (int i = 0; i < QW; ++i) {
+      const int qi = w * QW + i;
       float dot = 0.f;
 #pragma unroll 8
       for (int d = 0; d < DH; ++d) dot = fmaf(Qs[qi][d], Ks[lane][d], dot);
@@ -89,8 +91,8 @@ __global__ void __launch_bounds__(128) k_attn_simt(const T* __restrict__ q, cons
     }
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int qq = q0 + w * 4 + i;
+  for (int i = 0; i < QW; ++i) {
+    const int qq = q0 + w * QW + i;
     if (qq >= Qn) continue;
     const float inv = 1.f / l_run[i];
 #pragma unroll

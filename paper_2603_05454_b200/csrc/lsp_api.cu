@@ -109,6 +109,14 @@ void count_launch(lsp_ctx* c, int cls, int n = 1) {
   c->counters[CNT_CLS_LAUNCHES + cls] += n;
 }
 
+int sm_count(const lsp_ctx* c) {
+#ifndef LSP_NO_UMMA
+  return c->umma.n_sm;
+#else
+  return 148;
+#endif
+}
+
 // Opens a timed segment of kernel class cls (only when per-class timing is on).
 void seg_begin(lsp_ctx* c, int cls) {
   if (!c->timing) return;
@@ -244,7 +252,13 @@ int run_gemm(lsp_ctx* c, const T* A, const T* W0, const T* W1, int M, int NP, in
   }
 #endif
   dim3 grid((NP + SG_BN - 1) / SG_BN, (M + SG_BM - 1) / SG_BM);
-  CU(launch_k(c->pdl, k_gemm_simt<T, Epi>, grid, dim3(256), 0, c->stream, A, W0, W1, M, NP, K, epi));
+  auto kern = k_gemm_simt<T, Epi>;
+  if ((long)grid.x * grid.y < 2l * sm_count(c)) {          // (the line: see gemm_simt.cuh)
+    using Tile = SimtTile<Epi>;
+    grid = dim3((NP + Tile::PER_TILE - 1) / Tile::PER_TILE, (M + Tile::BM - 1) / Tile::BM);
+    kern = k_gemm_simt_split<T, Epi>;
+  }
+  CU(launch_k(c->pdl, kern, grid, dim3(256), 0, c->stream, A, W0, W1, M, NP, K, epi));
   return LSP_OK;
 }
 
@@ -255,7 +269,7 @@ int run_head(lsp_ctx* c, const T* hidden, int rows, int* n_tiles_out) {
   epi.part = c->part;
   epi.vocab = m.vocab;
   epi.exclude_id = c->s.exclude_mask_logit ? m.mask_id : -1;
-  int n_tiles = (m.vocab + SG_BN - 1) / SG_BN;
+  int n_tiles = (m.vocab + SG_HEAD_BN - 1) / SG_HEAD_BN;
 #ifndef LSP_NO_UMMA
   if (std::is_same<T, bf16>::value && c->gemm_impl == 1) n_tiles = umma_head_tiles(c->umma, rows, m.vocab);
 #endif
@@ -382,14 +396,14 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const Step
       done = true;
     }
   }
-  dim3 grid((maxQ + AS_BQ - 1) / AS_BQ, m.n_heads, B);
-  if (done) {
-  } else if (dh == 128)
-    launch_k(c->pdl, k_attn_simt<T, 128>, dim3(grid), dim3(128), 0, c->stream, Qb, cK, cV, stK, stV, Att, sd, m.n_heads, m.n_kv_heads,
-                                                     (size_t)c->max_len * kvd, scale, inplace);
-  else
-    launch_k(c->pdl, k_attn_simt<T, 64>, dim3(grid), dim3(128), 0, c->stream, Qb, cK, cV, stK, stV, Att, sd, m.n_heads, m.n_kv_heads,
-                                                    (size_t)c->max_len * kvd, scale, inplace);
+  if (!done) {
+    const int qw = (long)((maxQ + 15) / 16) * m.n_heads * B >= sm_count(c) ? 4 : 1;
+    dim3 grid((maxQ + 4 * qw - 1) / (4 * qw), m.n_heads, B);
+    auto kern = dh == 128 ? (qw == 4 ? k_attn_simt<T, 128, 4> : k_attn_simt<T, 128, 1>)
+                          : (qw == 4 ? k_attn_simt<T, 64, 4> : k_attn_simt<T, 64, 1>);
+    launch_k(c->pdl, kern, dim3(grid), dim3(128), 0, c->stream, Qb, cK, cV, stK, stV, Att, sd, m.n_heads, m.n_kv_heads,
+             (size_t)c->max_len * kvd, scale, inplace);
+  }
   seg_end(c);
   CU(cudaGetLastError());
   return LSP_OK;

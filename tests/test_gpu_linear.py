@@ -376,3 +376,12 @@ def test_swiglu_weights_by_one_copy_in_either_order(M, N, K, opts, up_first):
     want = torch.nn.functional.silu(A.double() @ gate.double().t()) * (A.double() @ up.double().t())
     assert bool(((out.double() - want).abs() <= want.abs() / 64 + want.abs().max() / 2560).all())
     dec.close()
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("M,N,K", [(1, 16, 64), (31, 48, 64), (33, 1040, 192), (128, 256, 1024), (129, 384, 256),
+                                   (1200, 1024, 128), (1217, 1040, 64)])
+def test_linear_cuda_core_kernels(dtype, M, N, K):
+    """Both CUDA-core kernels (K split over a CTA's warps below two 64 x 64 tiles per SM, one tile per CTA above: the last two)
+    at the edges of their tiles, fewer K steps than warps included."""
+    _check(dtype, 0, M, N, K, seed=13)
