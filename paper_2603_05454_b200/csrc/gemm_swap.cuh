@@ -34,7 +34,8 @@ struct SwapArgs {
   int n_pairs;    // dual: pair indices; plain: output columns
   int kc;         // K chunks of 64 elements per CTA (its K slice)
   int nr;         // activation rows rounded up to 16: the MMA's N and the activation box's rows
-  int box_rows;   // weight rows per TMA box (a divisor of 64 NACC)
+  int half;       // rotary epilogue: pair indices per head (half its width), else 0
+  int one_copy;   // 1: one copy brings a stage's whole weight tile (map_b0); 0: one per accumulator's tensor (map_b0, map_b1)
   int stages;
   int cluster;    // CTAs per tile (K slices): 1, 2 or 4
   unsigned* status;
@@ -138,14 +139,10 @@ k_gemm_swap(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 
   auto load_weights = [&](int c, int s) {
     const uint32_t sb = smem_u32(smem + (size_t)s * STAGE_BYTES) + A_BYTES;
-    const int k0 = (k_first + c) * UM_BK;
-    for (int b = 0; b < HALF; b += args.box_rows) {
-      int row_b0, row_b1;
-      if (Epi::kDual) { row_b0 = epi.row0(tile * HALF + b); row_b1 = epi.row1(tile * HALF + b); }
-      else { row_b0 = tile * BN + b; row_b1 = tile * BN + HALF + b; }
-      tma_load_2d(sb + b * 128, &map_b0, k0, row_b0, full_bar(s));
-      tma_load_2d(sb + HALF * 128 + b * 128, &map_b1, k0, row_b1, full_bar(s));
-    }
+    const int j = tile * (Epi::kDual ? HALF : BN);
+    const int r0 = args.half ? 0 : j, blk = args.half ? j / args.half : 0;
+    tma_load_5d(sb, &map_b0, r0, blk, 0, k_first + c, full_bar(s));
+    if (!args.one_copy) tma_load_5d(sb + HALF * 128, &map_b1, r0, blk, 0, k_first + c, full_bar(s));
   };
   const int n_pre = kc < S ? kc : S;
   if (threadIdx.x == 0) {
@@ -158,13 +155,20 @@ k_gemm_swap(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     *epi_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 0) {
     // weights are never written by any kernel: the first stages' weight tiles are requested while the preceding kernel
-    // (launched with programmatic serialisation) is still running; this thread is also the producer below
+    // (launched with programmatic serialisation) is still running; this warp is also the producer below
+    __syncwarp();
     for (int c = 0; c < n_pre; ++c) {
-      mbar_expect_tx(full_bar(c), STAGE_BYTES);
-      load_weights(c, c);
+      if (elect_one()) {
+        mbar_expect_tx(full_bar(c), STAGE_BYTES);
+        load_weights(c, c);
+      }
+      __syncwarp();
     }
   }
+  if (threadIdx.x == 64) tma_prefetch_map(&map_a);
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(TMEM_COLS)
@@ -179,45 +183,46 @@ k_gemm_swap(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      int issued = 0, s = 0;
-      uint32_t ph = 0;
-      for (int c = 0; c < kc; ++c) {
+    int issued = 0, s = 0;
+    uint32_t ph = 0;
+    for (int c = 0; c < kc; ++c) {
+      if (c >= n_pre && !__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, abort_flag))) {
+        if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 31u; }
+        break;
+      }
+      if (elect_one()) {
         if (c >= n_pre) {
-          if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) {
-            if (!*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 31u; }
-            break;
-          }
           mbar_expect_tx(full_bar(s), STAGE_BYTES);
           load_weights(c, s);
         }
-        tma_load_2d(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_a, (k_first + c) * UM_BK, 0, full_bar(s));
-        ++issued;
-        if (++s == S) { s = 0; ph ^= 1u; }
+        tma_load_4d(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_a, 0, 0, k_first + c, full_bar(s));
       }
-      // do not leave while copies may still be landing in this CTA's shared memory
-      for (int c = issued > S ? issued - S : 0; c < issued; ++c) {
-        volatile uint32_t no_abort = 0;
-        mbar_wait(full_bar(c % S), (uint32_t)(c / S) & 1u, &no_abort);
-      }
+      __syncwarp();
+      ++issued;
+      if (++s == S) { s = 0; ph ^= 1u; }
+    }
+    // do not leave while copies may still be landing in this CTA's shared memory
+    for (int c = issued > S ? issued - S : 0; c < issued; ++c) {
+      volatile uint32_t no_abort = 0;
+      mbar_wait(full_bar(c % S), (uint32_t)(c / S) & 1u, &no_abort);
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      const uint32_t idesc = make_idesc(NR);
-      bool ok = true;
-      int s = 0;
-      uint32_t ph = 0;
-      for (int c = 0; c < kc; ++c) {
-        if (!mbar_wait(full_bar(s), ph, abort_flag)) {
-          if (!*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 32u; }
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t sa = smem_u32(smem + (size_t)s * STAGE_BYTES);
-        const uint64_t dact = make_smem_desc(sa);                     // N-side operand: the activation rows
-        const uint64_t dw = make_smem_desc(sa + A_BYTES);             // M-side operand: 128 weight rows per accumulator
+    // ---------------- MMA issuer (the whole warp waits, one elected thread issues) ----------------
+    const uint32_t idesc = make_idesc(NR);
+    bool ok = true;
+    int s = 0;
+    uint32_t ph = 0;
+    for (int c = 0; c < kc; ++c) {
+      ok = __all_sync(0xffffffffu, mbar_wait(full_bar(s), ph, abort_flag));
+      if (!ok) {
+        if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 32u; }
+        break;
+      }
+      tc_fence_after();
+      const uint32_t sa = smem_u32(smem + (size_t)s * STAGE_BYTES);
+      const uint64_t dact = make_smem_desc(sa);                     // N-side operand: the activation rows
+      const uint64_t dw = make_smem_desc(sa + A_BYTES);             // M-side operand: 128 weight rows per accumulator
+      if (elect_one()) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
 #pragma unroll
@@ -226,9 +231,10 @@ k_gemm_swap(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                        (c | k) != 0 ? 1u : 0u);
         }
         tc_commit(empty_bar(s));
-        if (++s == S) { s = 0; ph ^= 1u; }
+        if (c == kc - 1) tc_commit(acc_bar);
       }
-      if (ok) tc_commit(acc_bar);
+      __syncwarp();
+      if (++s == S) { s = 0; ph ^= 1u; }
     }
   }
   // ---------------- epilogue (warps 2..5) ----------------
@@ -316,7 +322,7 @@ k_gemm_swap(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 // Launches the swapped kernel, or returns 1 when this problem is not one it takes (the caller then uses k_gemm_stream).
 template <int NACC, typename Epi>
 int swap_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
-                int n_rows_w, const Epi& epi, unsigned* status, int box_rows) {
+                int n_rows_w, const Epi& epi, unsigned* status) {
   constexpr int BN = 128 * NACC;
   const int per_tile = Epi::kDual ? BN / 2 : BN;
   const int n_tiles = (NP + per_tile - 1) / per_tile;
@@ -354,14 +360,30 @@ int swap_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
     if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -3; }
     attr_set = true;
   }
-  if (st.cache.size() > 4096) st.cache.clear();
-  if (box_rows <= 0 || box_rows > BN / 2 || (BN / 2) % box_rows || box_rows % 8) box_rows = BN / 2;
-  const CUtensorMap* ma = umma_map(st, A, M, K, nr);
-  const CUtensorMap* mb0 = umma_map(st, W0, n_rows_w, K, box_rows);
-  const CUtensorMap* mb1 = umma_map(st, W1, n_rows_w, K, box_rows);
-  if (!ma || !mb0 || !mb1) return -4;
-  SwapArgs args{M, NP, kc, nr, box_rows, stages, C, status};
-  cudaError_t e = launch_k(st.pdl, k_gemm_swap<NACC, Epi>, dim3(n_tiles * C), dim3(SW_THREADS), smem, stream, C, *ma, *mb0, *mb1,
+  const CUtensorMap* ma = umma_map4(st, A, M, M, 1, K, nr, 1, 1);
+  if (!ma) return -4;
+  // the weight tile as it lies in a stage: 128 rows per accumulator
+  WeightView v{W0, n_rows_w, 1, n_rows_w, 1, 0, BN, 1};
+  int one_copy = 1, rot_half = 0;
+  if constexpr (std::is_same<Epi, EpiQKVRope<bf16>>::value) {
+    rot_half = epi.half;
+    v = WeightView{W0, rot_half, n_rows_w / (2 * rot_half), 2 * rot_half, 2, (size_t)rot_half * K * 2, rot_half, BN / 2 / rot_half};
+  } else if constexpr (Epi::kDual) {
+    one_copy = 0;
+    v.box_rows = BN / 2;
+  }
+  const CUtensorMap* mb0 = umma_map5(st, v, K, 1);
+  if (!mb0) return -4;
+  const CUtensorMap mb0v = *mb0;
+  CUtensorMap mb1v = mb0v;
+  if (!one_copy) {
+    v.base = W1;
+    const CUtensorMap* mb1 = umma_map5(st, v, K, 1);
+    if (!mb1) return -4;
+    mb1v = *mb1;
+  }
+  SwapArgs args{M, NP, kc, nr, rot_half, one_copy, stages, C, status};
+  cudaError_t e = launch_k(st.pdl, k_gemm_swap<NACC, Epi>, dim3(n_tiles * C), dim3(SW_THREADS), smem, stream, C, *ma, mb0v, mb1v,
                            args, epi);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -5; }

@@ -38,7 +38,7 @@ extern "C" {
  *   33 a cluster of 2 exchanges half tiles (1, default) or publishes whole partial tiles like larger clusters (0)
  * GEMM on pairs of SMs:
  *   40 fewest rows that take it (default 257)   41 its tile width (0 = automatic, 96 ... 256 in steps of 32)
- *   42 most row groups of 256 per band (0 = automatic)
+ *   42 most row groups of 256 per band (0 = automatic)   45 with 129..256 rows where it pays (1, default) or not
  * tcgen05 attention:
  *   28 fewest (query row x group head) rows of a (sequence, KV head) for which the tcgen05 kernel is used (default 0)
  *   30 it splits a row tile's keys over a thread block cluster when there are few CTAs (1, default)

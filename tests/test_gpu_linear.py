@@ -385,3 +385,25 @@ def test_linear_cuda_core_kernels(dtype, M, N, K):
     """Both CUDA-core kernels (K split over a CTA's warps below two 64 x 64 tiles per SM, one tile per CTA above: the last two)
     at the edges of their tiles, fewer K steps than warps included."""
     _check(dtype, 0, M, N, K, seed=13)
+
+
+@pytest.mark.parametrize("M", [129, 187, 256])
+@pytest.mark.parametrize("N,K", [(4096, 4096), (1152, 512), (4608, 3584), (7168, 5120), (4096, 12288), (16, 64)])
+def test_linear_bf16_one_row_group_on_pairs(M, N, K):
+    """129 to 256 rows on both sides of the rule that sends them to the pairs of SMs or to the kernels that split K."""
+    for one_group in (1, 0):
+        dec = _dec("bf16")
+        dec.debug_set(45, one_group)
+        A = S.normal((M, K), 14, 1, 1.0, torch.bfloat16, DEV)
+        W = S.normal((N, K), 14, 2, 0.05, torch.bfloat16, DEV)
+        W2 = S.normal((N, K), 14, 3, 0.05, torch.bfloat16, DEV)
+        X0 = S.normal((M, N), 14, 4, 1.0, torch.bfloat16, DEV)
+        ref, up = A.double() @ W.double().t(), A.double() @ W2.double().t()
+        near = lambda got, want, ulps=1: bool(((got.double() - want).abs() <= ulps / 128 * want.abs() + want.abs().max() / 2560).all())
+        x = X0.clone()
+        dec.op_linear(1, A, W, None, x)
+        assert near(x, X0.double() + ref)
+        out = torch.empty(M, N, dtype=torch.bfloat16, device=DEV)
+        dec.op_linear(2, A, W, W2, out)
+        assert near(out, torch.nn.functional.silu(ref) * up, 2)
+        dec.close()
