@@ -30,6 +30,9 @@ namespace lsp {
 constexpr int AU_BM = 128;        // rows per CTA
 constexpr int AU_BN = 128;        // keys per tile
 constexpr int AU_THREADS = 384;   // warps 0..3 and 4..7: the two softmax groups; 8, 11: TMA producers (K, V); 9, 10: MMA issuers
+#ifndef AU_POLY
+#define AU_POLY 0
+#endif
 constexpr int AU_W_TMA = 8, AU_W_QK = 9, AU_W_PV = 10, AU_W_TMAV = 11;
 constexpr int AU_ATOM = 128 * 128;            // bytes of one [128 rows x 64 bf16] swizzle atom
 constexpr int AU_TILE = 2 * AU_ATOM;          // one 128 x 128 bf16 operand tile
@@ -55,6 +58,45 @@ __device__ __forceinline__ float ex2_approx(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+// Two fp32 operations per instruction.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 f2_pack(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// 2^x of two values by arithmetic instead of the special-function unit: x = n + f with n the nearest integer (adding and
+// subtracting 1.5 * 2^23 rounds to it and leaves it in the low bits), 2^f by a degree-5 polynomial fitted for the least relative
+// error on [-1/2, 1/2] (7.5e-8 exact, 2.1e-7 in fp32: what ex2.approx keeps), n added to the exponent.  x below -126 counts as -126.
+__device__ __forceinline__ void exp2_poly2(f32x2 x2, float& p0, float& p1) {
+  float x0, x1;
+  f2_unpack(x2, x0, x1);
+  x2 = f2_pack(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
+  const f32x2 t = f2_add(x2, f2_pack(12582912.f, 12582912.f));
+  const f32x2 n = f2_add(t, f2_pack(-12582912.f, -12582912.f));
+  const f32x2 f = f2_fma(n, f2_pack(-1.f, -1.f), x2);
+  f32x2 r = f2_fma(f2_pack(1.327647129073739e-3f, 1.327647129073739e-3f), f, f2_pack(9.675541892647743e-3f, 9.675541892647743e-3f));
+  r = f2_fma(r, f, f2_pack(5.550713092088699e-2f, 5.550713092088699e-2f));
+  r = f2_fma(r, f, f2_pack(0.24022120237350464f, 0.24022120237350464f));
+  r = f2_fma(r, f, f2_pack(0.6931469440460205f, 0.6931469440460205f));
+  r = f2_fma(r, f, f2_pack(1.0000001192092896f, 1.0000001192092896f));
+  float t0, t1, r0, r1;
+  f2_unpack(t, t0, t1);
+  f2_unpack(r, r0, r1);
+  p0 = __int_as_float(__float_as_int(r0) + (__float_as_int(t0) << 23));
+  p1 = __int_as_float(__float_as_int(r1) + (__float_as_int(t1) << 23));
 }
 __device__ __forceinline__ float ld_cluster_f1(uint32_t addr) {
   float v;
@@ -174,24 +216,25 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   const int ldq = n_heads * DH;
 
   if (warp == AU_W_TMA || warp == AU_W_TMAV) {
-    // ---------------- TMA producers: one thread streams the K tiles, another the V tiles ----------------
-    if (lane == 0) {
-      const bool is_v = warp == AU_W_TMAV;
-      const int full = is_v ? B_VF : B_KF, empty = is_v ? B_VE : B_KE;
-      int issued = 0;
-      if (!is_v && n_tiles > 0) {
-        // the Q tile (positions past the sequence's end bring other rows or zeros; rows are independent and those are never
-        // stored)
-        mbar_expect_tx(bar(B_Q), (uint32_t)(pos_tile * G * 256));
-        tma_load_5d_q(smem_u32(Qs), &map_q, kvh, r0 + pos0, 0, bar(B_Q));
-        tma_load_5d_q(smem_u32(Qs) + AU_ATOM, &map_q, kvh, r0 + pos0, 1, bar(B_Q));
+    // ---------------- TMA producers: one warp streams the K tiles, another the V tiles (one elected thread issues) ----------------
+    const bool is_v = warp == AU_W_TMAV;
+    const int full = is_v ? B_VF : B_KF, empty = is_v ? B_VE : B_KE;
+    int issued = 0;
+    if (!is_v && n_tiles > 0 && elect_one()) {
+      // the Q tile (positions past the sequence's end bring other rows or zeros; rows are independent and those are never
+      // stored)
+      mbar_expect_tx(bar(B_Q), (uint32_t)(pos_tile * G * 256));
+      tma_load_5d_q(smem_u32(Qs), &map_q, kvh, r0 + pos0, 0, bar(B_Q));
+      tma_load_5d_q(smem_u32(Qs) + AU_ATOM, &map_q, kvh, r0 + pos0, 1, bar(B_Q));
+    }
+    __syncwarp();
+    for (int t = 0; t < n_tiles; ++t) {
+      const int s = t & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(bar(empty + s), ((uint32_t)(t >> 1) & 1u) ^ 1u, abort_flag))) {
+        if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 21u; }
+        break;
       }
-      for (int t = 0; t < n_tiles; ++t) {
-        const int s = t & 1;
-        if (!mbar_wait(bar(empty + s), ((uint32_t)(t >> 1) & 1u) ^ 1u, abort_flag)) {
-          if (!*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 21u; }
-          break;
-        }
+      if (elect_one()) {
         mbar_expect_tx(bar(full + s), AU_TILE);
         const uint32_t dst = smem_u32(KVs + (size_t)s * 2 * AU_TILE) + (is_v ? AU_TILE : 0);
         const int gt = rank + t * C;                    // tile index in the sequence's key range
@@ -200,33 +243,30 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         const CUtensorMap* mp = cache ? (is_v ? &map_cv : &map_ck) : (is_v ? &map_sv : &map_sk);
         tma_load_2d(dst, mp, kvh * DH, row, bar(full + s));
         tma_load_2d(dst + AU_ATOM, mp, kvh * DH + 64, row, bar(full + s));
-        ++issued;
       }
-      // do not leave while copies may still be landing in this CTA's shared memory
-      if (!is_v && n_tiles > 0) {
-        volatile uint32_t no_abort = 0;
-        mbar_wait(bar(B_Q), 0u, &no_abort);
-      }
-      for (int t = issued > 2 ? issued - 2 : 0; t < issued; ++t) {
-        volatile uint32_t no_abort = 0;
-        mbar_wait(bar(full + (t & 1)), (uint32_t)(t >> 1) & 1u, &no_abort);
-      }
+      __syncwarp();
+      ++issued;
     }
+    // do not leave while copies may still be landing in this CTA's shared memory
+    volatile uint32_t no_abort = 0;
+    if (!is_v && n_tiles > 0) mbar_wait(bar(B_Q), 0u, &no_abort);
+    for (int t = issued > 2 ? issued - 2 : 0; t < issued; ++t) mbar_wait(bar(full + (t & 1)), (uint32_t)(t >> 1) & 1u, &no_abort);
   } else if (warp == AU_W_QK) {
-    // ---------------- MMA issuer 1: S = Q K^T of every tile ----------------
-    if (lane == 0) {
-      constexpr uint32_t idesc_qk = make_idesc(AU_BN);
-      if (n_tiles > 0 && !mbar_wait(bar(B_Q), 0u, abort_flag)) {
-        if (!*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 26u; }
+    // ---------------- MMA issuer 1: S = Q K^T of every tile (the whole warp waits, one elected thread issues: a lane branch
+    // around the MMAs would cost more than they take, see elect_one) ----------------
+    constexpr uint32_t idesc_qk = make_idesc(AU_BN);
+    bool ok = n_tiles == 0 || __all_sync(0xffffffffu, mbar_wait(bar(B_Q), 0u, abort_flag));
+    if (!ok && lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 26u; }
+    for (int t = 0; t < n_tiles && ok; ++t) {
+      const int s = t & 1;
+      ok = __all_sync(0xffffffffu, mbar_wait(bar(B_KF + s), (uint32_t)(t >> 1) & 1u, abort_flag) &&
+                                       mbar_wait(bar(B_SE + s), ((uint32_t)(t >> 1) & 1u) ^ 1u, abort_flag));
+      if (!ok) {
+        if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 22u; }
+        break;
       }
-      for (int t = 0; t < n_tiles && !*abort_flag; ++t) {
-        const int s = t & 1;
-        if (!mbar_wait(bar(B_KF + s), (uint32_t)(t >> 1) & 1u, abort_flag) ||
-            !mbar_wait(bar(B_SE + s), ((uint32_t)(t >> 1) & 1u) ^ 1u, abort_flag)) {
-          if (!*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 22u; }
-          break;
-        }
-        tc_fence_after();
+      tc_fence_after();
+      if (elect_one()) {
         const uint32_t kd = smem_u32(KVs + (size_t)s * 2 * AU_TILE);
         const uint32_t d = tmem_base + 256u + (uint32_t)(s * AU_BN);
 #pragma unroll
@@ -238,19 +278,20 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         tc_commit(bar(B_SF + s));     // scores ready
         tc_commit(bar(B_KE + s));     // K stage free
       }
+      __syncwarp();
     }
   } else if (warp == AU_W_PV) {
     // ---------------- MMA issuer 2: O_w += P_w V of every tile (w = tile parity) ----------------
-    if (lane == 0) {
-      constexpr uint32_t idesc_pv = make_idesc(DH) | (1u << 16);          // B operand (V) is MN-major
-      for (int t = 0; t < n_tiles; ++t) {
-        const int s = t & 1;                  // K/V stage, S buffer and softmax group of this tile
-        const uint32_t par = (uint32_t)(t >> 1) & 1u;
-        if (!mbar_wait(bar(B_VF + s), par, abort_flag) || !mbar_wait(bar(B_PR + s), par, abort_flag)) {
-          if (!*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 23u; }
-          break;
-        }
-        tc_fence_after();
+    constexpr uint32_t idesc_pv = make_idesc(DH) | (1u << 16);          // B operand (V) is MN-major
+    for (int t = 0; t < n_tiles; ++t) {
+      const int s = t & 1;                  // K/V stage, S buffer and softmax group of this tile
+      const uint32_t par = (uint32_t)(t >> 1) & 1u;
+      if (!__all_sync(0xffffffffu, mbar_wait(bar(B_VF + s), par, abort_flag) && mbar_wait(bar(B_PR + s), par, abort_flag))) {
+        if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 23u; }
+        break;
+      }
+      tc_fence_after();
+      if (elect_one()) {
         const uint32_t vd = smem_u32(KVs + (size_t)s * 2 * AU_TILE) + AU_TILE;
         const uint32_t pa = smem_u32(Ps + (size_t)s * AU_TILE);
 #pragma unroll
@@ -262,6 +303,7 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         tc_commit(bar(B_VE + s));     // V stage free
         tc_commit(bar(B_PD + s));     // P_w free, O_w updated
       }
+      __syncwarp();
     }
   } else {
     // ---------------- softmax (two groups of four warps, one row per thread; group w takes the tiles of parity w, with
@@ -303,8 +345,13 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
           for (int i = 0; i < AU_BN; ++i)
             if (i >= valid_keys) sv[i] = -INFINITY;
         }
+        float m4[4] = {sv[0], sv[1], sv[2], sv[3]};      // (four chains: a single one would be 128 dependent steps)
 #pragma unroll
-        for (int i = 0; i < AU_BN; ++i) mx = fmaxf(mx, sv[i]);
+        for (int i = 4; i < AU_BN; i += 8) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) m4[k] = fmaxf(fmaxf(m4[k], sv[i + k]), i + 4 + k < AU_BN ? sv[i + 4 + k] : sv[i + k]);
+        }
+        mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
       }
 #pragma unroll 1
       for (int c = kRolled ? 0 : AU_BN; c < AU_BN; c += 32) {
@@ -371,19 +418,31 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
       float sum = 0.f;
       const float neg_m = -m_used;
       if constexpr (!kRolled) {
+        const f32x2 sc2 = f2_pack(scale_log2, scale_log2), nm2 = f2_pack(neg_m, neg_m);
+        f32x2 sum2[2] = {0ull, 0ull};
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
           uint32_t pk[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const float p0 = ex2_approx(fmaf(sv[8 * c + 2 * j], scale_log2, neg_m));
-            const float p1 = ex2_approx(fmaf(sv[8 * c + 2 * j + 1], scale_log2, neg_m));
-            sum += p0 + p1;
+            const f32x2 x2 = f2_fma(f2_pack(sv[8 * c + 2 * j], sv[8 * c + 2 * j + 1]), sc2, nm2);
+            float p0, p1;
+            if (j >= 4 - AU_POLY) {
+              exp2_poly2(x2, p0, p1);
+            } else {
+              f2_unpack(x2, p0, p1);
+              p0 = ex2_approx(p0);
+              p1 = ex2_approx(p1);
+            }
+            sum2[j & 1] = f2_add(sum2[j & 1], f2_pack(p0, p1));
             const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
             pk[j] = *reinterpret_cast<const uint32_t*>(&pb);
           }
           *reinterpret_cast<uint4*>(Pw + au_swz(r, c)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         }
+        float sa, sb;
+        f2_unpack(f2_add(sum2[0], sum2[1]), sa, sb);
+        sum = sa + sb;
       }
 #pragma unroll 1
       for (int c = kRolled ? 0 : AU_BN; c < AU_BN; c += 32) {
