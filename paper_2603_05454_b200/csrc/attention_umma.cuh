@@ -30,9 +30,6 @@ namespace lsp {
 constexpr int AU_BM = 128;        // rows per CTA
 constexpr int AU_BN = 128;        // keys per tile
 constexpr int AU_THREADS = 384;   // warps 0..3 and 4..7: the two softmax groups; 8, 11: TMA producers (K, V); 9, 10: MMA issuers
-#ifndef AU_POLY
-#define AU_POLY 0
-#endif
 constexpr int AU_W_TMA = 8, AU_W_QK = 9, AU_W_PV = 10, AU_W_TMAV = 11;
 constexpr int AU_ATOM = 128 * 128;            // bytes of one [128 rows x 64 bf16] swizzle atom
 constexpr int AU_TILE = 2 * AU_ATOM;          // one 128 x 128 bf16 operand tile
@@ -76,27 +73,6 @@ __device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
   f32x2 r;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
-}
-// 2^x of two values by arithmetic instead of the special-function unit: x = n + f with n the nearest integer (adding and
-// subtracting 1.5 * 2^23 rounds to it and leaves it in the low bits), 2^f by a degree-5 polynomial fitted for the least relative
-// error on [-1/2, 1/2] (7.5e-8 exact, 2.1e-7 in fp32: what ex2.approx keeps), n added to the exponent.  x below -126 counts as -126.
-__device__ __forceinline__ void exp2_poly2(f32x2 x2, float& p0, float& p1) {
-  float x0, x1;
-  f2_unpack(x2, x0, x1);
-  x2 = f2_pack(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
-  const f32x2 t = f2_add(x2, f2_pack(12582912.f, 12582912.f));
-  const f32x2 n = f2_add(t, f2_pack(-12582912.f, -12582912.f));
-  const f32x2 f = f2_fma(n, f2_pack(-1.f, -1.f), x2);
-  f32x2 r = f2_fma(f2_pack(1.327647129073739e-3f, 1.327647129073739e-3f), f, f2_pack(9.675541892647743e-3f, 9.675541892647743e-3f));
-  r = f2_fma(r, f, f2_pack(5.550713092088699e-2f, 5.550713092088699e-2f));
-  r = f2_fma(r, f, f2_pack(0.24022120237350464f, 0.24022120237350464f));
-  r = f2_fma(r, f, f2_pack(0.6931469440460205f, 0.6931469440460205f));
-  r = f2_fma(r, f, f2_pack(1.0000001192092896f, 1.0000001192092896f));
-  float t0, t1, r0, r1;
-  f2_unpack(t, t0, t1);
-  f2_unpack(r, r0, r1);
-  p0 = __int_as_float(__float_as_int(r0) + (__float_as_int(t0) << 23));
-  p1 = __int_as_float(__float_as_int(r1) + (__float_as_int(t1) << 23));
 }
 __device__ __forceinline__ float ld_cluster_f1(uint32_t addr) {
   float v;
@@ -427,13 +403,9 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
           for (int j = 0; j < 4; ++j) {
             const f32x2 x2 = f2_fma(f2_pack(sv[8 * c + 2 * j], sv[8 * c + 2 * j + 1]), sc2, nm2);
             float p0, p1;
-            if (j >= 4 - AU_POLY) {
-              exp2_poly2(x2, p0, p1);
-            } else {
-              f2_unpack(x2, p0, p1);
-              p0 = ex2_approx(p0);
-              p1 = ex2_approx(p1);
-            }
+            f2_unpack(x2, p0, p1);
+            p0 = ex2_approx(p0);
+            p1 = ex2_approx(p1);
             sum2[j & 1] = f2_add(sum2[j & 1], f2_pack(p0, p1));
             const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
             pk[j] = *reinterpret_cast<const uint32_t*>(&pb);

@@ -409,6 +409,12 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const Step
   return LSP_OK;
 }
 
+template <typename T>
+void run_rmsnorm(lsp_ctx* c, const T* x, const void* gains, T* out, const int* src_rows, int rows) {
+  auto kern = rows <= 1024 ? k_rmsnorm<T, true> : k_rmsnorm<T, false>;
+  launch_k(c->pdl, kern, dim3(rows), dim3(RN_THREADS), 0, c->stream, x, (const T*)gains, out, src_rows, c->m.d_model, c->m.rms_eps);
+}
+
 // Launch shape of one denoiser pass.  The row counts may be upper bounds of what the device-side descriptor says (the
 // lagged loop sizes a pass before it has read the previous block lengths): rows past the real ones are inert.
 struct PassDims {
@@ -448,7 +454,7 @@ int enqueue_pass(lsp_ctx* c, const StepDesc& sd, int B, const PassDims& pd, int*
     T* stK = c->kv_inplace ? (T*)c->kv_cache + (size_t)(2 * l) * cplane : (T*)c->stage + (size_t)(2 * l) * plane;
     T* stV = stK + (c->kv_inplace ? cplane : plane);
     seg_begin(c, CLS_MISC);
-    launch_k(c->pdl, k_rmsnorm<T>, dim3(M), dim3(256), 0, c->stream, X, (const T*)c->attn_norm[l], Nrm, nullptr, d, m.rms_eps);
+    run_rmsnorm<T>(c, X, c->attn_norm[l], Nrm, nullptr, M);
     seg_end(c);
     count_launch(c, CLS_MISC);
     CU(cudaGetLastError());
@@ -471,7 +477,7 @@ int enqueue_pass(lsp_ctx* c, const StepDesc& sd, int B, const PassDims& pd, int*
       if (rc) return rc;
     }
     seg_begin(c, CLS_MISC);
-    launch_k(c->pdl, k_rmsnorm<T>, dim3(M), dim3(256), 0, c->stream, X, (const T*)c->ffn_norm[l], Nrm, nullptr, d, m.rms_eps);
+    run_rmsnorm<T>(c, X, c->ffn_norm[l], Nrm, nullptr, M);
     seg_end(c);
     count_launch(c, CLS_MISC);
     CU(cudaGetLastError());
@@ -488,7 +494,7 @@ int enqueue_pass(lsp_ctx* c, const StepDesc& sd, int B, const PassDims& pd, int*
   }
   // masked rows only: final norm (gathered), fused head, merge, scan
   seg_begin(c, CLS_MISC);
-  launch_k(c->pdl, k_rmsnorm<T>, dim3(Mh), dim3(256), 0, c->stream, X, (const T*)c->final_norm, Nrm, c->head_src, d, m.rms_eps);
+  run_rmsnorm<T>(c, X, c->final_norm, Nrm, c->head_src, Mh);
   seg_end(c);
   count_launch(c, CLS_MISC);
   CU(cudaGetLastError());

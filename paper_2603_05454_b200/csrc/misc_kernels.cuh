@@ -77,7 +77,11 @@ __device__ __forceinline__ uint4 f_to_vec(const float (&v)[8]) {
   return r;
 }
 
-template <typename T>
+// kEarly: the gains are fetched before the wait for the preceding kernel (they are weights, written by no kernel).  In a small
+// pass they come from HBM, behind its weight stream, and would be a second round trip after the reduction: 3.6 -> 2.4 us from
+// the wait to the last store of a 101-row launch.  With many rows they stay in L2 and the registers they hold (57 a thread
+// instead of 36) cost more: 8240 rows 34 -> 41 us.
+template <typename T, bool kEarly>
 __global__ void __launch_bounds__(RN_THREADS) k_rmsnorm(const T* __restrict__ x, const T* __restrict__ g, T* __restrict__ out,
                                                        const int* __restrict__ src_rows, int d, float eps) {
   constexpr int E = Vec16<T>::N;                 // elements per 16-byte vector
@@ -88,15 +92,15 @@ __global__ void __launch_bounds__(RN_THREADS) k_rmsnorm(const T* __restrict__ x,
   uint4* o = reinterpret_cast<uint4*>(out + (size_t)r * d);
   const int nv = d / E;                          // d is a multiple of 64
   const bool in_regs = nv <= RN_VPT * RN_THREADS;
-  uint4 keep[RN_VPT], gain[RN_VPT];
+  uint4 keep[RN_VPT], gain[kEarly ? RN_VPT : 1];
   float ss = 0.f;
-  if (in_regs) {
-    // the gains are weights, written by no kernel: they come (behind a pass's weight stream: from HBM) while the preceding
-    // kernel still runs.  3.6 -> 2.4 us from the wait to the last store of a 101-row launch.
+  if constexpr (kEarly) {
+    if (in_regs) {
 #pragma unroll
-    for (int j = 0; j < RN_VPT; ++j) {
-      const int i = threadIdx.x + j * RN_THREADS;
-      gain[j] = (i < nv) ? __ldg(gr + i) : make_uint4(0u, 0u, 0u, 0u);
+      for (int j = 0; j < RN_VPT; ++j) {
+        const int i = threadIdx.x + j * RN_THREADS;
+        gain[j] = (i < nv) ? __ldg(gr + i) : make_uint4(0u, 0u, 0u, 0u);
+      }
     }
   }
   pdl_wait();
@@ -136,7 +140,7 @@ __global__ void __launch_bounds__(RN_THREADS) k_rmsnorm(const T* __restrict__ x,
       if (i < nv) {
         float v[E], gv[E];
         vec_to_f(keep[j], v);
-        vec_to_f(gain[j], gv);
+        vec_to_f(kEarly ? gain[kEarly ? j : 0] : __ldg(gr + i), gv);
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = v[e] * inv * gv[e];
         o[i] = f_to_vec(v);
