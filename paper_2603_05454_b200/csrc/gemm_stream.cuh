@@ -766,8 +766,14 @@ inline size_t stream_scratch_bytes(int n_ctas, int bn, int mt) { return (size_t)
 // to 8 CTAs, and a launch never asks for more clusters than can be resident at once: the GPC layout fits 74 / 45 / 33 /
 // 26 / 22 / 15 / 15 clusters of 2 ... 8 one-per-SM CTAs, so e.g. 48 clusters of 3 or 16 of 8 would run as two waves
 // (measured: 40 % and 100 % slower than the next smaller split).
-inline int stream_splits(const UmmaState& st, long n_tiles) {
+// With a short K (at most 512) a slice would be a stage or two, and the reduction costs more than it saves, except where the
+// epilogue reads its output's old value (see no_split): 64 x 2 x 1024 SwiGLU 9.7 -> 7.2 us, 100 x 1024 6.8 -> 5.2, 64 x 4096
+// 6.2 -> 4.9 unsplit, but a residual update of 100 x 512 7.5 -> 8.0; from K = 1024 on the split wins (64 x 512 6.8, 8.9 without).
+template <typename Epi>
+bool stream_no_split(int K) { return K <= 512 && !std::is_same<Epi, EpiResidual<bf16>>::value; }
+inline int stream_splits(const UmmaState& st, long n_tiles, bool no_split) {
   int splits = n_tiles <= st.n_sm ? (int)(st.n_sm / n_tiles) : 0;
+  if (no_split && splits > 1) return 1;
   if (st.stream_cluster && splits > 1) {
     int c = splits < 8 ? splits : 8;
     while (c > 1 && n_tiles > st.max_clusters[c]) --c;
@@ -776,9 +782,9 @@ inline int stream_splits(const UmmaState& st, long n_tiles) {
   return splits;
 }
 
-inline int stream_grid(const UmmaState& st, int n_tiles, int M) {
+inline int stream_grid(const UmmaState& st, int n_tiles, int M, bool no_split) {
   if (st.target_ctas > 0) return st.target_ctas;
-  const int splits = stream_splits(st, n_tiles);
+  const int splits = stream_splits(st, n_tiles, no_split);
   const int aligned = splits > 0 ? n_tiles * splits : st.n_sm;
   if (st.stream_grid_mode == 1) return st.n_sm;
   if (st.stream_grid_mode == 2) return aligned;
@@ -879,7 +885,7 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
   // several row groups and at least as many tiles as SMs: whole tiles per CTA; else K slices as stream_grid says
   const long T = (long)n_tiles * row_groups;
   const int whole = (row_groups > 1 && T >= st.n_sm) ? 1 : 0;
-  int grid = whole ? st.n_sm : stream_grid(st, (int)T, M);
+  int grid = whole ? st.n_sm : stream_grid(st, (int)T, M, stream_no_split<Epi>(K));
   if (grid > T * kc) grid = (int)(T * kc);
   if ((double)T * kc * (grid + 1) >= 4.0e9) { st.err = "too many work units for the streaming GEMM"; return -9; }   // 32-bit unit arithmetic
   // K slices of one tile on the CTAs of one cluster: the reduction then stays on chip
@@ -930,7 +936,7 @@ int stream_row_tiles(const UmmaState& st, int M, int NP, int K, int bn) {
       const long groups = (M + UM_BM * m - 1) / (UM_BM * m);
       const long t = n_tiles * groups;
       long ctas = t;
-      if (t < st.n_sm && st.stream_cluster && !Epi::kReduce) ctas = t * stream_splits(st, t);
+      if (t < st.n_sm && st.stream_cluster && !Epi::kReduce) ctas = t * stream_splits(st, t, stream_no_split<Epi>(K));
       const double waves = (double)((ctas + st.n_sm - 1) / st.n_sm * st.n_sm);
       return (double)ctas / waves * (double)M / (double)(groups * UM_BM * m);
     };
@@ -941,7 +947,7 @@ int stream_row_tiles(const UmmaState& st, int M, int NP, int K, int bn) {
   const long T = n_tiles * row_groups;
   if (!(row_groups > 1 && T >= st.n_sm)) {         // tiles may be split between CTAs: scratch and counters
     if (st.scratch == nullptr || T > st.n_counters ||
-        stream_scratch_bytes(stream_grid(st, (int)T, M), bn, mt) > st.scratch_bytes)
+        stream_scratch_bytes(stream_grid(st, (int)T, M, stream_no_split<Epi>(K)), bn, mt) > st.scratch_bytes)
       return 0;
   }
   return stream_shape(st, stream_a_rows(M, mt), bn, mt, K).stages >= 2 ? mt : 0;
