@@ -147,4 +147,17 @@ struct StepDesc {
   const int* Lc;       // lengths to commit (commit kernel only)
 };
 
+// The same arrays by value, for batches small enough for a kernel's parameters: the step's first kernel takes the descriptor
+// from here and leaves it in memory for the others, which saves the copy in front of it (a copy between kernels costs a
+// small pass about 3 us: the copy itself, and the kernel behind it starts only after it).
+constexpr int kDescInline = 32;
+struct DescInline {
+  int use = 0;                     // 0: the descriptor is in memory already
+  int v[6][kDescInline + 1];       // F, pend, N, row_off, head_off, Fp
+};
+struct LenInline {
+  int use = 0;
+  int v[kDescInline];
+};
+
 }  // namespace lsp

@@ -294,30 +294,32 @@ ScanParams scan_params(const lsp_ctx* c) {
   return p;
 }
 
-// merge partials -> scores, scan, copy the scan outputs to the pinned mirror (async)
+// Where the scan leaves its results: on the device and in pinned host memory -- the context's mirror, or a slot of the lagged
+// loop's ring (scan outputs, then the status word).
+ScanOut scan_out(const lsp_ctx* c, int* h_dst, bool count_flips) {
+  const int mb = c->max_batch;
+  ScanOut o;
+  o.dev = c->d_scan;
+  o.host = h_dst ? h_dst : c->h_scan;
+  o.host_status = h_dst ? (unsigned*)(h_dst + 6 * mb) : c->h_status;
+  o.status = c->d_status;
+  o.stride = mb;
+  o.head_pos = count_flips ? c->head_pos : nullptr;
+  o.prev = c->prev_yhat;
+  o.prev_stride = c->max_len;
+  return o;
+}
+
+// merge partials -> scores, scan; the scan's results reach the pinned mirror with the kernel
 int run_merge_scan(lsp_ctx* c, int rows, int n_tiles, const int* d_seq_off, int batch, bool count_flips, int* h_dst = nullptr) {
   if (rows > 0) {
     CU(launch_k(c->pdl, k_merge_partials, dim3((rows + 3) / 4), dim3(128), 0, c->stream, (const Top2*)c->part, n_tiles, rows, c->yhat,
                 c->pmax, c->margin));
   }
   const float* score = c->s.score == 1 ? c->margin : c->pmax;
-  int* o = c->d_scan;
-  const int mb = c->max_batch;
-  if (count_flips) {
-    launch_k(c->pdl, k_flip_count, dim3(batch), dim3(256), 0, c->stream, d_seq_off, (const int*)c->head_pos,
-             (const int32_t*)c->yhat, c->prev_yhat, c->max_len, o + 4 * mb, o + 5 * mb);
-    CU(cudaGetLastError());
-  }
-  launch_k(c->pdl, k_lsp_scan, dim3(batch), dim3(32), 0, c->stream, score, c->yhat, c->margin, d_seq_off, scan_params(c), o, o + mb,
-                                          (uint32_t*)(o + 2 * mb), (float*)(o + 3 * mb));
+  launch_k(c->pdl, k_lsp_scan, dim3(batch), dim3(256), 0, c->stream, score, (const int32_t*)c->yhat, (const float*)c->margin, d_seq_off, scan_params(c),
+           scan_out(c, h_dst, count_flips));
   CU(cudaGetLastError());
-  if (h_dst) {        // a slot of the lagged loop's ring: scan outputs, then the status word
-    CU(cudaMemcpyAsync(h_dst, c->d_scan, 6 * (size_t)mb * 4, cudaMemcpyDeviceToHost, c->stream));
-    CU(cudaMemcpyAsync(h_dst + 6 * mb, c->d_status, 16, cudaMemcpyDeviceToHost, c->stream));
-    return LSP_OK;
-  }
-  CU(cudaMemcpyAsync(c->h_scan, c->d_scan, 6 * (size_t)mb * 4, cudaMemcpyDeviceToHost, c->stream));
-  CU(cudaMemcpyAsync(c->h_status, c->d_status, 16, cudaMemcpyDeviceToHost, c->stream));
   return LSP_OK;
 }
 
@@ -425,7 +427,7 @@ struct PassDims {
 
 // Enqueues one pass (Algorithm 1: forward pass, scores, scan) that reads descriptor sd on the device.
 template <typename T>
-int enqueue_pass(lsp_ctx* c, const StepDesc& sd, int B, const PassDims& pd, int* h_dst) {
+int enqueue_pass(lsp_ctx* c, const StepDesc& sd, const DescInline& din, int B, const PassDims& pd, int* h_dst) {
   const lsp_model_cfg& m = c->m;
   const bool scattered = c->s.topology == 1;
   const int M = pd.M, Mh = pd.Mh;
@@ -436,7 +438,7 @@ int enqueue_pass(lsp_ctx* c, const StepDesc& sd, int B, const PassDims& pd, int*
   T* Att = (T*)c->Att;
   T* Hf = (T*)c->Hf;
   seg_begin(c, CLS_MISC);
-  launch_k(c->pdl, k_assemble_embed<T>, dim3(M), dim3(128), 0, c->stream, sd, B, c->tokens, c->tok_stride, m.mask_id, (const T*)c->embed, d, X,
+  launch_k(c->pdl, k_assemble_embed<T>, dim3(M), dim3(128), 0, c->stream, sd, din, B, c->tokens, c->tok_stride, m.mask_id, (const T*)c->embed, d, X,
                                                c->row_seq, c->row_pos, c->head_src, c->head_pos, scattered ? 1 : 0);
   CU(cudaGetLastError());
   if (scattered) {
@@ -543,19 +545,34 @@ PassDims host_descriptor(lsp_ctx* c) {
   return pd;
 }
 
+// Hands the descriptor in the pinned mirror to the next pass: by value where the batch allows it, else copied to the device.
+int send_descriptor(lsp_ctx* c, DescInline* din) {
+  const int B = c->batch, s = c->max_batch + 1;
+  din->use = B <= kDescInline ? 1 : 0;
+  if (din->use) {
+    for (int a = 0; a < 6; ++a)
+      for (int b = 0; b <= B; ++b) din->v[a][b] = (b < B || a == 3 || a == 4) ? c->h_desc[a * s + b] : 0;
+  } else {
+    // the step owns the first six arrays; the seventh (commit lengths) belongs to lsp_commit, whose upload from the same
+    // pinned mirror may still be in flight
+    CU(cudaMemcpyAsync(c->d_desc, c->h_desc, 6 * (size_t)s * 4, cudaMemcpyHostToDevice, c->stream));
+  }
+  return LSP_OK;
+}
+
 template <typename T>
 int step_impl(lsp_ctx* c, lsp_step_rec* rec) {
-  const int B = c->batch, s = c->max_batch + 1;
+  const int B = c->batch;
   const bool scattered = c->s.topology == 1;
   const PassDims pd = host_descriptor(c);
   const int M = pd.M, Mh = pd.Mh;
   if (M == 0) return fail(c, LSP_ERR_STATE, "lsp_denoise_step: every sequence is already fully committed");
   const auto host_t0 = std::chrono::steady_clock::now();
   CU(cudaEventRecord(c->ev0, c->stream));
-  // the step owns the first six arrays; the seventh (commit lengths) belongs to lsp_commit, whose upload from the same
-  // pinned mirror may still be in flight
-  CU(cudaMemcpyAsync(c->d_desc, c->h_desc, 6 * (size_t)s * 4, cudaMemcpyHostToDevice, c->stream));
-  int rc = enqueue_pass<T>(c, desc_of(c), B, pd, nullptr);
+  DescInline din;
+  int rc = send_descriptor(c, &din);
+  if (rc) return rc;
+  rc = enqueue_pass<T>(c, desc_of(c), din, B, pd, nullptr);
   if (rc) return rc;
   CU(cudaEventRecord(c->ev1, c->stream));
   // host time spent queueing the pass (everything between the two event records)
@@ -878,9 +895,9 @@ int lsp_denoise_step(lsp_ctx* c, lsp_step_rec* rec) {
 
 namespace {
 
-// Enqueues the commit kernel(s) of a step that read descriptor sd (whose Lc array holds the block lengths).
+// Enqueues the commit kernel(s) of a step that read descriptor sd; the block lengths are in len or in sd's Lc array.
 // max_pend: the longest pending block (an upper bound is enough: it only sizes the copy's grid).
-int enqueue_commit(lsp_ctx* c, const StepDesc& sd, int B, int max_pend, int max_n) {
+int enqueue_commit(lsp_ctx* c, const StepDesc& sd, const LenInline& len, int B, int max_pend, int max_n) {
   const lsp_model_cfg& m = c->m;
   const size_t kvd = (size_t)m.n_kv_heads * m.head_dim;
   const int row_v4 = (int)(kvd * c->esz / 16);
@@ -899,14 +916,14 @@ int enqueue_commit(lsp_ctx* c, const StepDesc& sd, int B, int max_pend, int max_
   if ((!scattered || max_pend > 0) && (copy || !scattered)) {
     launch_k(c->pdl, k_commit_append, dim3(grid), dim3(256), 0, c->stream, sd, (const uint4*)c->stage, (uint4*)c->kv_cache,
                                                  stage_plane_v4, cache_plane_v4, cache_seq_v4, row_v4, c->yhat,
-                                                 c->tokens, c->tok_stride, scattered ? 0 : 1, copy ? 1 : 0);
+                                                 c->tokens, c->tok_stride, scattered ? 0 : 1, copy ? 1 : 0, len);
     count_launch(c, CLS_COMMIT);
   }
   if (scattered) {
     // accept the L most confident masked positions wherever they are
     const float* score = c->s.score == 1 ? c->margin : c->pmax;
     launch_k(c->pdl, k_scatter_commit, dim3(B), dim3(256), (size_t)max_n * sizeof(float), c->stream, sd, score,
-             (const int32_t*)c->yhat, (const int*)c->head_pos, c->tokens, c->tok_stride);
+             (const int32_t*)c->yhat, (const int*)c->head_pos, c->tokens, c->tok_stride, len);
     count_launch(c, CLS_COMMIT);
   }
   seg_end(c);
@@ -989,13 +1006,14 @@ int generate_lagged(lsp_ctx* c, lsp_step_rec* recs, int max_recs, int* n_steps) 
     remaining = 0;
     for (int b = 0; b < B; ++b) remaining += c->N[b];
     if (remaining == 0) break;
+    DescInline din;
     const bool exact = (read == launched);           // the host state is that of the step about to be launched
     PassDims pd;
     if (exact) {
       pd = host_descriptor(c);
       // the device descriptor of this step: the first one is uploaded; later ones were derived on the device (k_advance)
       // from the same block lengths and are equal to the host's
-      if (launched == 0) CU(cudaMemcpyAsync(c->d_desc, c->h_desc, 6 * (size_t)s * 4, cudaMemcpyHostToDevice, c->stream));
+      if (launched == 0) { rc = send_descriptor(c, &din); if (rc) return rc; }
     } else {
       // host state is that before step launched - 1: this step's rows of sequence b are N there (if it goes on at all)
       for (int b = 0; b < B; ++b) {
@@ -1017,7 +1035,7 @@ int generate_lagged(lsp_ctx* c, lsp_step_rec* recs, int max_recs, int* n_steps) 
     const int par = launched & 1, slot = launched % R;
     const StepDesc sd = desc_of(c, par);
     CU(cudaEventRecord(c->ring_t0[slot], c->stream));
-    rc = enqueue_pass<T>(c, sd, B, pd, c->h_ring + (size_t)slot * slot_ints);
+    rc = enqueue_pass<T>(c, sd, din, B, pd, c->h_ring + (size_t)slot * slot_ints);
     if (rc) return rc;
     CU(cudaEventRecord(c->ring_t1[slot], c->stream));
     CU(cudaEventRecord(c->ring_done[slot], c->stream));
@@ -1027,7 +1045,7 @@ int generate_lagged(lsp_ctx* c, lsp_step_rec* recs, int max_recs, int* n_steps) 
     int max_pend = 0;
     if (exact) { for (int b = 0; b < B; ++b) if (c->N[b] > 0) max_pend = std::max(max_pend, c->pend[b]); }
     else max_pend = std::min(pd.maxQ, std::max(8, 2 * last_L));
-    rc = enqueue_commit(c, sc, B, max_pend, 0);
+    rc = enqueue_commit(c, sc, LenInline(), B, max_pend, 0);
     if (rc) return rc;
     launch_k(c->pdl, k_advance, dim3(1), dim3(32), 0, c->stream, sd, c->d_desc + (size_t)(par ^ 1) * 7 * s, s,
              (const int32_t*)(c->d_scan + mb), B);
@@ -1061,15 +1079,21 @@ int lsp_commit(lsp_ctx* c, const int32_t* L_override) {
       return fail(c, LSP_ERR_STATE, "lsp_commit: L[%d] = %d outside [1, %d]", b, L[b], c->N[b]);
     if (c->pend[b] > max_pend) max_pend = c->pend[b];
   }
-  int* hl = c->h_desc + 6 * s;
-  for (int b = 0; b < B; ++b) hl[b] = L[b];
-  CU(cudaMemcpyAsync(c->d_desc + 6 * s, hl, (size_t)B * 4, cudaMemcpyHostToDevice, c->stream));
+  LenInline len;
+  len.use = B <= kDescInline ? 1 : 0;
+  if (len.use) {
+    for (int b = 0; b < B; ++b) len.v[b] = L[b];
+  } else {
+    int* hl = c->h_desc + 6 * s;
+    for (int b = 0; b < B; ++b) hl[b] = L[b];
+    CU(cudaMemcpyAsync(c->d_desc + 6 * s, hl, (size_t)B * 4, cudaMemcpyHostToDevice, c->stream));
+  }
   const lsp_model_cfg& m = c->m;
   const size_t kvd = (size_t)m.n_kv_heads * m.head_dim;
   const bool scattered = c->s.topology == 1;
   int max_n = 0;
   for (int b = 0; b < B; ++b) if (c->N[b] > max_n) max_n = c->N[b];
-  const int rc = enqueue_commit(c, desc_of(c), B, max_pend, max_n);
+  const int rc = enqueue_commit(c, desc_of(c), len, B, max_pend, max_n);
   if (rc) return rc;
   for (int b = 0; b < B; ++b)
     if (c->N[b] > 0 && !c->kv_inplace) c->counters[CNT_APPEND_BYTES] += 2.0 * c->pend[b] * kvd * c->esz * 2.0 * m.n_layers;
@@ -1178,13 +1202,9 @@ int lsp_scan(lsp_ctx* c, const float* score, const int32_t* yhat, const float* m
   int rc = upload_offsets(c, seq_offsets, batch, &rows);
   if (rc) return rc;
   c->proposed = false;
-  int* o = c->d_scan;
-  const int mb = c->max_batch;
-  launch_k(c->pdl, k_lsp_scan, dim3(batch), dim3(32), 0, c->stream, score, yhat, margin, c->d_desc + 4 * (c->max_batch + 1), scan_params(c), o,
-                                          o + mb, (uint32_t*)(o + 2 * mb), (float*)(o + 3 * mb));
+  launch_k(c->pdl, k_lsp_scan, dim3(batch), dim3(256), 0, c->stream, score, yhat, margin, (const int*)(c->d_desc + 4 * (c->max_batch + 1)),
+           scan_params(c), scan_out(c, nullptr, false));
   CU(cudaGetLastError());
-  CU(cudaMemcpyAsync(c->h_scan, c->d_scan, 4 * (size_t)mb * 4, cudaMemcpyDeviceToHost, c->stream));
-  CU(cudaMemcpyAsync(c->h_status, c->d_status, 16, cudaMemcpyDeviceToHost, c->stream));
   return scan_outputs(c, batch, l_run, l_commit, flags, tau_used);
 }
 

@@ -10,25 +10,36 @@ namespace lsp {
 // One block per row.  Also fills row_seq / row_pos and the list of rows that go through the LM head.
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void k_assemble_embed(StepDesc sd, int batch, const int32_t* __restrict__ tokens, int tok_stride,
+__global__ void k_assemble_embed(StepDesc sd, const __grid_constant__ DescInline in, int batch, const int32_t* __restrict__ tokens, int tok_stride,
                                  int mask_id, const T* __restrict__ embed, int d, T* __restrict__ X,
                                  int* __restrict__ row_seq, int* __restrict__ row_pos,
                                  int* __restrict__ head_src, int* __restrict__ head_pos, int scattered) {
   pdl_begin();
   const int r = blockIdx.x;
+  if (in.use && r == 0) {              // leave the descriptor for the step's other kernels
+    for (int i = threadIdx.x; i <= batch; i += blockDim.x) {
+      const_cast<int*>(sd.F)[i] = in.v[0][i];
+      const_cast<int*>(sd.pend)[i] = in.v[1][i];
+      const_cast<int*>(sd.N)[i] = in.v[2][i];
+      const_cast<int*>(sd.row_off)[i] = in.v[3][i];
+      const_cast<int*>(sd.head_off)[i] = in.v[4][i];
+      const_cast<int*>(sd.Fp)[i] = in.v[5][i];
+    }
+  }
+  auto at = [&](int a, const int* p, int i) { return in.use ? in.v[a][i] : p[i]; };
   // The grid may be larger than the pass (a host that sizes launches from an upper bound of the row counts): rows past
   // the last real one are zero vectors that belong to no sequence, and the spare head slots point at row 0.
-  if (r >= sd.head_off[batch] && threadIdx.x == 0) head_src[r] = 0;
-  if (r >= sd.row_off[batch]) {
+  if (r >= at(4, sd.head_off, batch) && threadIdx.x == 0) head_src[r] = 0;
+  if (r >= at(3, sd.row_off, batch)) {
     if (threadIdx.x == 0) { row_seq[r] = -1; row_pos[r] = 0; }
     uint4* z = reinterpret_cast<uint4*>(X + (size_t)r * d);
     for (int i = threadIdx.x; i < d * (int)sizeof(T) / 16; i += blockDim.x) z[i] = make_uint4(0u, 0u, 0u, 0u);
     return;
   }
   int b = 0;
-  while (b + 1 < batch && r >= sd.row_off[b + 1]) ++b;
-  const int j = r - sd.row_off[b];
-  const int F = sd.F[b], pend = sd.pend[b];
+  while (b + 1 < batch && r >= at(3, sd.row_off, b + 1)) ++b;
+  const int j = r - at(3, sd.row_off, b);
+  const int F = at(0, sd.F, b), pend = at(1, sd.pend, b), head0 = at(4, sd.head_off, b);
   const int pos = F + j;
   // prefix topology: rows past the pending block are the masked suffix; scattered topology: every row reads the token
   // buffer (committed positions hold their token, the others the mask id) and k_compact_masked lists the masked rows
@@ -37,8 +48,8 @@ __global__ void k_assemble_embed(StepDesc sd, int batch, const int32_t* __restri
     row_seq[r] = b;
     row_pos[r] = pos;
     if (!scattered && j >= pend) {
-      head_src[sd.head_off[b] + (j - pend)] = r;
-      head_pos[sd.head_off[b] + (j - pend)] = pos;
+      head_src[head0 + (j - pend)] = r;
+      head_pos[head0 + (j - pend)] = pos;
     }
   }
   const uint4* src = reinterpret_cast<const uint4*>(embed + (size_t)tok * d);
@@ -198,17 +209,65 @@ __device__ __forceinline__ bool is_delim(const uint8_t* bm, int id) {
   return bm != nullptr && ((bm[id >> 3] >> (id & 7)) & 1);
 }
 
-__global__ void k_lsp_scan(const float* __restrict__ score, const int32_t* __restrict__ yhat,
-                           const float* __restrict__ margin, const int* __restrict__ seq_off, ScanParams p,
-                           int32_t* __restrict__ o_run, int32_t* __restrict__ o_commit, uint32_t* __restrict__ o_flags,
-                           float* __restrict__ o_tau) {
+// What the scan's launch does besides (one block of 256 threads per sequence; the first warp scans):
+//   * token flips (Fig. 3), when head_pos is given: for every masked position of this step, compares its argmax with the one
+//     the previous step stored for the same absolute position (-1 = not scored before), counts the differences, and stores
+//     the new argmax;
+//   * the results, and the status word, go straight to pinned host memory as well, so that no copy follows the last kernel.
+struct ScanOut {
+  int* dev;                  // 6 arrays of stride ints: run, commit, flags, tau, flips, flip base
+  int* host;                 // the same, pinned host memory (or null)
+  unsigned* host_status;     // 4 words (with host)
+  const unsigned* status;
+  int stride;
+  const int* head_pos;       // null: no flip count
+  int32_t* prev;
+  int prev_stride;
+};
+
+__global__ void __launch_bounds__(256) k_lsp_scan(const float* __restrict__ score, const int32_t* __restrict__ yhat,
+                           const float* __restrict__ margin, const int* __restrict__ seq_off, ScanParams p, ScanOut o) {
+  __shared__ int red[2][8];
   pdl_begin();
   const int b = blockIdx.x;
-  const int lane = threadIdx.x;
+  const int lane = threadIdx.x & 31;
   const int base = seq_off[b];
   const int N = seq_off[b + 1] - base;
+  if (o.head_pos != nullptr) {
+    int flips = 0, scored = 0;
+    for (int i = base + (int)threadIdx.x; i < base + N; i += 256) {
+      int32_t* q = o.prev + (size_t)b * o.prev_stride + o.head_pos[i];
+      const int32_t old = *q, cur = yhat[i];
+      if (old >= 0) { ++scored; flips += (old != cur); }
+      *q = cur;
+    }
+    flips = __reduce_add_sync(0xffffffffu, flips);
+    scored = __reduce_add_sync(0xffffffffu, scored);
+    if (lane == 0) { red[0][threadIdx.x >> 5] = flips; red[1][threadIdx.x >> 5] = scored; }
+    __syncthreads();
+  }
+  if (threadIdx.x >= 32) return;
+  auto put = [&](int which, int v) {
+    o.dev[which * o.stride + b] = v;
+    if (o.host) o.host[which * o.stride + b] = v;
+  };
+  auto emit = [&](int run, int commit, uint32_t flags, float tau) {
+    if (lane != 0) return;
+    put(0, run);
+    put(1, commit);
+    put(2, (int)flags);
+    put(3, __float_as_int(tau));
+    if (o.head_pos != nullptr) {
+      int f = 0, t = 0;
+      for (int i = 0; i < 8; ++i) { f += red[0][i]; t += red[1][i]; }
+      put(4, f);
+      put(5, t);
+    }
+    if (o.host && b == 0)
+      for (int i = 0; i < 4; ++i) o.host_status[i] = o.status[i];
+  };
   if (N <= 0) {
-    if (lane == 0) { o_run[b] = 0; o_commit[b] = 0; o_flags[b] = 0; o_tau[b] = 0.f; }
+    emit(0, 0, 0u, 0.f);
     return;
   }
   const float* sc = score + base;
@@ -218,7 +277,7 @@ __global__ void k_lsp_scan(const float* __restrict__ score, const int32_t* __res
   float tau = p.tau;
   if (p.mode == 2) {
     int L = min(N, max(1, p.fixed_k));
-    if (lane == 0) { o_run[b] = L; o_commit[b] = L; o_flags[b] = 0; o_tau[b] = __int_as_float(0x7fc00000); }
+    emit(L, L, 0u, __int_as_float(0x7fc00000));
     return;
   }
   if (p.mode == 1) {
@@ -291,7 +350,7 @@ __global__ void k_lsp_scan(const float* __restrict__ score, const int32_t* __res
     if (__any_sync(0xffffffffu, near)) flags |= 16u;
     if (__any_sync(0xffffffffu, tie)) flags |= 32u;
   }
-  if (lane == 0) { o_run[b] = Lrun; o_commit[b] = L; o_flags[b] = flags; o_tau[b] = tau; }
+  emit(Lrun, L, flags, tau);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -307,7 +366,7 @@ __global__ void k_commit_append(StepDesc sd, const uint4* __restrict__ stage, ui
                                 size_t cache_seq_v4,     // uint4 per sequence inside a cache plane
                                 int row_v4,              // uint4 per row (n_kv_heads * head_dim * sizeof(T) / 16)
                                 const int32_t* __restrict__ yhat, int32_t* __restrict__ tokens, int tok_stride,
-                                int write_tokens, int copy_rows) {
+                                int write_tokens, int copy_rows, const __grid_constant__ LenInline len) {
   pdl_begin();
   const int b = blockIdx.z;
   const int plane = blockIdx.y;
@@ -318,7 +377,7 @@ __global__ void k_commit_append(StepDesc sd, const uint4* __restrict__ stage, ui
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     dst[i] = src[i];
   if (write_tokens && blockIdx.x == 0 && plane == 0) {
-    const int L = sd.Lc[b];
+    const int L = len.use ? len.v[b] : sd.Lc[b];
     const int ho = sd.head_off[b];
     int32_t* t = tokens + (size_t)b * tok_stride + sd.Fp[b];
     for (int i = threadIdx.x; i < L; i += blockDim.x) t[i] = yhat[ho + i];
@@ -393,38 +452,6 @@ __global__ void __launch_bounds__(256) k_compact_masked(StepDesc sd, const int32
 }
 
 // ---------------------------------------------------------------------------------------------
-// Token flips (Fig. 3): for every masked position of this step, compares its argmax with the one the previous step
-// stored for the same absolute position (-1 = not scored before), counts the differences, and stores the new argmax.
-// One block of 256 threads per sequence.
-// ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_flip_count(const int* __restrict__ head_off, const int* __restrict__ head_pos,
-                                                    const int32_t* __restrict__ yhat, int32_t* __restrict__ prev,
-                                                    int prev_stride, int32_t* __restrict__ o_flips,
-                                                    int32_t* __restrict__ o_base) {
-  __shared__ int red[2][8];
-  pdl_begin();
-  const int b = blockIdx.x;
-  const int a = head_off[b], e = head_off[b + 1];
-  int flips = 0, base = 0;
-  for (int i = a + threadIdx.x; i < e; i += 256) {
-    int32_t* p = prev + (size_t)b * prev_stride + head_pos[i];
-    const int32_t old = *p, cur = yhat[i];
-    if (old >= 0) { ++base; flips += (old != cur); }
-    *p = cur;
-  }
-  flips = (int)warp_sum((float)flips);
-  base = (int)warp_sum((float)base);
-  if ((threadIdx.x & 31) == 0) { red[0][threadIdx.x >> 5] = flips; red[1][threadIdx.x >> 5] = base; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int f = 0, t = 0;
-    for (int i = 0; i < 8; ++i) { f += red[0][i]; t += red[1][i]; }
-    o_flips[b] = f;
-    o_base[b] = t;
-  }
-}
-
-// ---------------------------------------------------------------------------------------------
 // Scattered commit: accepts the Lc_b most confident masked positions of sequence b (rank by counting: position i
 // is accepted iff fewer than Lc_b positions beat it; a tie goes to the lower position) and writes their predictions
 // into the token buffer at their own positions.  One block of 256 threads per sequence; scores staged in shared
@@ -432,11 +459,12 @@ __global__ void __launch_bounds__(256) k_flip_count(const int* __restrict__ head
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_scatter_commit(StepDesc sd, const float* __restrict__ score,
                                                         const int32_t* __restrict__ yhat, const int* __restrict__ head_pos,
-                                                        int32_t* __restrict__ tokens, int tok_stride) {
+                                                        int32_t* __restrict__ tokens, int tok_stride,
+                                                        const __grid_constant__ LenInline len) {
   extern __shared__ float sc_s[];
   pdl_begin();
   const int b = blockIdx.x;
-  const int a = sd.head_off[b], n = sd.head_off[b + 1] - a, L = sd.Lc[b];
+  const int a = sd.head_off[b], n = sd.head_off[b + 1] - a, L = len.use ? len.v[b] : sd.Lc[b];
   for (int i = threadIdx.x; i < n; i += 256) sc_s[i] = score[a + i];
   __syncthreads();
   for (int i = threadIdx.x; i < n; i += 256) {

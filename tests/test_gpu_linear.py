@@ -407,3 +407,20 @@ def test_linear_bf16_one_row_group_on_pairs(M, N, K):
         dec.op_linear(2, A, W, W2, out)
         assert near(out, torch.nn.functional.silu(ref) * up, 2)
         dec.close()
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 512, 64), (64, 1024, 512), (128, 272, 448), (33, 4096, 512), (100, 1024, 576)])
+def test_linear_bf16_short_k_without_a_split(M, N, K):
+    """At most 512 elements of K: whole tiles per CTA instead of K slices on clusters (the last case is beyond the line)."""
+    dec = _dec("bf16")
+    A = S.normal((M, K), 16, 1, 1.0, torch.bfloat16, DEV)
+    W = S.normal((N, K), 16, 2, 0.05, torch.bfloat16, DEV)
+    W2 = S.normal((N, K), 16, 3, 0.05, torch.bfloat16, DEV)
+    out = torch.empty(M, N, dtype=torch.bfloat16, device=DEV)
+    ref, up = A.double() @ W.double().t(), A.double() @ W2.double().t()
+    near = lambda got, want, ulps=1: bool(((got.double() - want).abs() <= ulps / 128 * want.abs() + want.abs().max() / 2560).all())
+    dec.op_linear(0, A, W, None, out)
+    assert near(out, ref)
+    dec.op_linear(2, A, W, W2, out)
+    assert near(out, torch.nn.functional.silu(ref) * up, 2)
+    dec.close()
