@@ -15,7 +15,7 @@
 //   * Persistent: pair p takes tiles p, p + P, ...; the accumulators are double-buffered (2 x BN of 512 columns), so the
 //     epilogue of a tile overlaps the next tile's MMAs.
 //   * BN is a run-time multiple of 32 (64 for the rotary epilogue), chosen so that the last wave of tiles is full (see
-//     pair_width).
+//     pair_shape).
 // Measured (B200, back to back, weights from a ring larger than L2; row-major k_gemm_stream before -> now, us):
 //   rows    12288 x 4096   4096 x 4096   2 x 12288 x 4096 SwiGLU   4096 x 12288
 //    512      58 -> 42      31 -> 17            111 -> 76          56 -> 45
@@ -45,6 +45,8 @@ struct PairArgs {
   int row_groups;   // groups of 256 activation rows
   int band;         // row groups per band: tiles are ordered band by band, within a band column tile by column tile
   int kc;           // chunks of 128 K elements (two atoms; the last one may be half empty: zero-filled)
+  int ks;           // K slices of a tile (plain epilogues, one tile per cluster): pair s of the cluster takes the s-th share of
+                    // the chunks, and the partial tiles are summed through distributed shared memory
   int bn;           // tile width
   int unit;         // rotary epilogue: weight rows per copy when a half tile is not made of whole head halves (else 0)
   int stages;
@@ -68,10 +70,10 @@ __device__ __forceinline__ void tc_mma_f16_pair(uint32_t d_tmem, uint64_t a_desc
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// arrives at the barrier at this offset in both CTAs of the pair once the issued MMAs have completed
-__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
+// arrives at the barrier at this offset in both CTAs of the pair (mask: their cluster ranks) once the issued MMAs have completed
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint16_t mask) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-               "h"((uint16_t)3)
+               "h"(mask)
                : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
@@ -104,11 +106,14 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   auto accf_bar = [&](int b) { return bar_base + 8u * (2 * S + b); };
   auto acce_bar = [&](int b) { return bar_base + 8u * (2 * S + 2 + b); };
 
-  const int rank = (int)cluster_ctarank();
-  const int P = gridDim.x >> 1, pair = blockIdx.x >> 1;
+  const int crank = (int)cluster_ctarank(), rank = crank & 1;           // rank within the pair
+  const unsigned lead = (unsigned)(crank & ~1);                           // the pair's first CTA
+  const int ks = args.ks, slice = crank >> 1;
+  const uint16_t pair_mask = (uint16_t)(3u << lead);
+  const int P = gridDim.x / (unsigned)(2 * ks), pair = blockIdx.x / (unsigned)(2 * ks);
   const int T = args.n_tiles * args.row_groups;
   const int my_tiles = (T - pair + P - 1) / P;            // the host launches at most T pairs
-  const int kc = args.kc;
+  const int kc0 = args.kc * slice / ks, kc = args.kc * (slice + 1) / ks - kc0;      // this pair's chunks
   const int n_units = my_tiles * kc;
   // i-th tile of this pair -> column tile and row group
   auto tile_of = [&](int i, int& tile, int& rg) {
@@ -119,7 +124,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     tile = r / rows;
     rg = b * args.band + r % rows;
   };
-  const uint32_t full0 = cluster_map(bar_base, 0);        // the first CTA's full barriers, in the cluster's window
+  const uint32_t full0 = cluster_map(bar_base, lead);     // the first CTA's full barriers, in the cluster's window
   const CUtensorMap* map_b = rank ? &map_b1 : &map_b0;    // this CTA's half of the weight tile
   auto load_weights = [&](int tile, int c, int s) {
     const uint32_t sb = smem_u32(smem + (size_t)s * STAGE_BYTES) + 2 * A_ATOM;
@@ -134,7 +139,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             tma_load_4d_pair(sb + a * B_ATOM + b * 128, map_b, (j + b) % epi.half, (j + b) / epi.half, 2 * c + a, full0 + 8u * s);
       }
     } else {
-      tma_load_4d_pair(sb, map_b, Epi::kDual ? tile * HALF : tile * BN + rank * HALF, 0, 2 * c, full0 + 8u * s);
+      tma_load_4d_pair(sb, map_b, Epi::kDual ? tile * HALF : tile * BN + rank * HALF, 0, 2 * (kc0 + c), full0 + 8u * s);
     }
   };
 
@@ -197,7 +202,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE_BYTES);
           load_weights(tile, c, s);
         }
-        tma_load_4d_pair(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_a, rg * PR_ROWS + rank * UM_BM, 0, 2 * c, full0 + 8u * s);
+        tma_load_4d_pair(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_a, rg * PR_ROWS + rank * UM_BM, 0, 2 * (kc0 + c), full0 + 8u * s);
       }
       __syncwarp();
       ++issued;
@@ -248,8 +253,8 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
               for (int k = 0; k < 4; ++k)
                 tc_mma_f16_pair(d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (c | a | k) != 0 ? 1u : 0u);
             }
-            tc_commit_pair(empty_bar(s));
-            if (c == kc - 1) tc_commit_pair(accf_bar(buf));
+            tc_commit_pair(empty_bar(s), pair_mask);
+            if (c == kc - 1) tc_commit_pair(accf_bar(buf), pair_mask);
           }
           __syncwarp();
           if (++s == S) { s = 0; ph ^= 1u; }
@@ -265,8 +270,8 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     const int CH = Epi::kDual ? HALF : BN;                        // pair indices (dual) or columns (plain) per tile
     const int nch = CH >> 4, mid = (nch + 1) >> 1;
     const int ch_lo = h ? mid : 0, ch_hi = h ? nch : mid;
-    const uint32_t acce0 = cluster_map(acce_bar(0), 0);
-    for (int i = 0; i < my_tiles; ++i) {
+    const uint32_t acce0 = cluster_map(acce_bar(0), lead);
+    for (int i = 0; i < my_tiles && ks == 1; ++i) {
       const int buf = i & 1, use = i >> 1;
       int tile, rg;
       tile_of(i, tile, rg);
@@ -321,6 +326,26 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           tc_ld16_nowait(t_row + (uint32_t)(ch * 16), a0);
           if (Epi::kDual) tc_ld16_nowait(t_row + (uint32_t)(HALF + ch * 16), a1);
         };
+        if constexpr (kRope) {
+          // (the rotary table's entries one chunk ahead take the registers a second set of accumulator values would)
+          EpiPre<Epi> pre, next;
+          auto fetch = [&](int ch, EpiPre<Epi>& p) {
+            if (live && ch < ch_hi && j0 + ch * 16 < args.n_pairs) p.load(epi, m, j0 + ch * 16);
+          };
+          fetch(ch_lo, pre);
+          float p0[16], p1[16];
+#pragma unroll 1
+          for (int ch = ch_lo; ch < ch_hi; ++ch) {
+            __syncwarp();
+            request(ch, p0, p1);
+            fetch(ch + 1, next);
+            tc_wait_ld();
+            tc_pin16(p0);
+            tc_pin16(p1);
+            if (live && j0 + ch * 16 < args.n_pairs) epi16(epi, m, j0 + ch * 16, p0, p1, pre);
+            pre = next;
+          }
+        } else {
         // the next chunk's tensor-memory loads are in flight while this one is converted and stored
         float p0[16], p1[16], q0[16], q1[16];
         if (ch_lo < ch_hi) request(ch_lo, p0, p1);
@@ -339,6 +364,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             consume(ch + 1, q0, q1);
           }
         }
+        }
         if constexpr (Epi::kReduce) {
           if (live) epi.part[(size_t)m * epi.n_tiles + 2 * tile + h] = red;      // one partial per column half
         }
@@ -346,6 +372,81 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(acce0 + 8u * buf);
+    }
+  }
+  if constexpr (!Epi::kDual && !Epi::kReduce) {
+    if (ks > 1) {
+      // K slices: the pair of slice s finishes the s-th share of the tile's 16-column chunks.  Every CTA publishes the other
+      // shares of its 128 rows in its own shared memory (the pipeline stages are idle once the accumulator is complete), and
+      // after a cluster barrier adds, for its own share, the pieces of the other slices' CTAs with the same rows to its own,
+      // in slice (= K) order.  All threads of all CTAs reach both barriers.
+      const int q = warp & 3, h = (warp - 2) >> 2, r_in = q * 32 + lane, nch = BN >> 4;
+      const int lo = nch * slice / ks, hi = nch * (slice + 1) / ks;                 // this slice's chunks
+      int tile, rg;
+      tile_of(0, tile, rg);
+      const int m = rg * PR_ROWS + rank * UM_BM + r_in, j0 = tile * BN;
+      const bool live = m < args.M;
+      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
+      float4* pub = reinterpret_cast<float4*>(smem);                               // [chunk][quarter][row]
+      bool ok = true;
+      if (warp >= 2) {
+        ok = __all_sync(0xffffffffu, mbar_wait(accf_bar(0), 0u, abort_flag));
+        if (!ok && lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 45u; }
+        tc_fence_after();
+        if (ok) {
+          for (int ch = h; ch < nch; ch += 2) {                                     // the two warps of a quarter alternate
+            if (ch >= lo && ch < hi) continue;
+            float v[16];
+            __syncwarp();
+            tc_ld16(t_row + (uint32_t)(ch * 16), v);
+            if (live) {
+#pragma unroll
+              for (int g = 0; g < 4; ++g) pub[(ch * 4 + g) * UM_BM + r_in] = make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+            }
+          }
+        }
+      }
+      EpiPre<Epi> pre;
+      if (warp >= 2 && live && lo + h < hi && j0 + (lo + h) * 16 < args.n_pairs) pre.load(epi, m, j0 + (lo + h) * 16);
+      cluster_sync();
+      if (warp >= 2 && ok) {
+        for (int ch = lo + h; ch < hi; ch += 2) {
+          float own[16], a[16];
+          __syncwarp();
+          tc_ld16(t_row + (uint32_t)(ch * 16), own);
+          if (live && j0 + ch * 16 < args.n_pairs) {
+            float4 t[2][4];                                                        // (at most three slices)
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+              const int p = x < slice ? x : x + 1;
+              if (p < ks) {
+                const uint32_t peer = cluster_map(smem_u32(smem), (unsigned)(2 * p + rank)) + (uint32_t)((ch * 4 * UM_BM + r_in) * 16);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) t[x][g] = ld_cluster_f4(peer + (uint32_t)(g * UM_BM * 16));
+              }
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) a[i] = 0.f;
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+              if (p >= ks) break;
+              if (p == slice) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) a[i] += own[i];
+              } else {
+                const int x = p < slice ? p : p - 1;
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                  const float4 u = x == 0 ? t[0][g] : t[1][g];
+                  a[4 * g] += u.x; a[4 * g + 1] += u.y; a[4 * g + 2] += u.z; a[4 * g + 3] += u.w;
+                }
+              }
+            }
+            epi16(epi, m, j0 + ch * 16, a, a, pre);
+            if (ch + 2 < hi && j0 + (ch + 2) * 16 < args.n_pairs) pre.load(epi, m, j0 + (ch + 2) * 16);
+          }
+        }
+      }
     }
   }
   tc_fence_before();
@@ -358,18 +459,32 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 }
 
 // ---- host side ------------------------------------------------------------------------------------------------
-// Tile width.  A tile costs about bn + 44 in units of one column's MMA time (the constant: what a tile costs whatever its
-// width; per round of 4096 K elements 11.4 / 13.5 / 16.1 / 18.9 / 21.8 / 24.6 us at 96 / 128 / 160 / 192 / 224 / 256), and the launch takes as many rounds as its fullest pair, so the width that gives the least rounds x (bn + 44)
-// wins.  step: widths are multiples of 32, or 64 for the rotary epilogue (a half tile is then made of whole 32-row boxes
-// inside one head half).
-inline int pair_width(int M, int cols, int n_pairs_of_sms, int step) {
+// Tile width and K slices.  What a chunk of 128 K elements costs a pair is its intake: 32 KB of activations and bn / 8 KB of
+// weights per SM at about 118 GB/s from L2, i.e. 1.06 ns x (bn + 256), which the MMAs of the widest tile just fill.  (Under the
+// power cap, with many rounds, bn + 44 fits better: per 4096 K elements 11.4 / 13.5 / 16.1 / 18.9 / 21.8 / 24.6 us at 96 / 128 /
+// 160 / 192 / 224 / 256 columns.)  A launch takes as many rounds as its fullest pair.  A plain projection whose tiles fit
+// once with two or three K slices each may split: wider tiles re-read the activations less, at 10 to 14 us for the exchange
+// (187 rows, 4096 x 12288: 34.6 us whole, 28.5 in three slices; 3584 x 18944: 48.2, 35.5; but 512 rows, 4096 x 12288: 45.0 whole,
+// 47.9 in two).
+// step: widths are multiples of 32, or 64 for the rotary epilogue (a half tile is then made of whole 32-row boxes inside one
+// head half).
+struct PairShape { int bn, ks; };
+inline PairShape pair_shape(const UmmaState& st, int M, int cols, int K, int step, bool may_split) {
+  const int pairs = st.max_clusters[2];
   const long rg = (M + PR_ROWS - 1) / PR_ROWS;
-  int best = 256;
+  const double chunks = (K + 127) / 128;
+  PairShape best{256, 1};
   double best_cost = 1e30;
   for (int bn = 256; bn >= 96; bn -= step) {
     const long t = (long)((cols + bn - 1) / bn) * rg;
-    const double cost = (double)((t + n_pairs_of_sms - 1) / n_pairs_of_sms) * (bn + 44);
-    if (cost < best_cost - 1e-9) { best_cost = cost; best = bn; }
+    const long rounds = (t + pairs - 1) / pairs;
+    const double cost = chunks * (rounds > 2 ? rounds * (bn + 44) * 1.8 : rounds * (bn + 256)) * 1.06e-3;
+    if (cost < best_cost - 1e-9) { best_cost = cost; best = {bn, 1}; }
+    for (int ks = 2; ks <= 3 && may_split; ++ks) {
+      if (t * ks > pairs || t > st.max_clusters[2 * ks] || chunks < 8 * ks) continue;
+      const double c2 = chunks / ks * (bn + 256) * 1.06e-3 + 14.0;
+      if (c2 < best_cost - 1e-9) { best_cost = c2; best = {bn, ks}; }
+    }
   }
   return best;
 }
@@ -380,8 +495,10 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
   constexpr bool kRope = std::is_same<Epi, EpiQKVRope<bf16>>::value;
   const int cols = Epi::kDual ? 2 * NP : NP;
   const int pairs = st.max_clusters[2];
-  int bn = Epi::kReduce ? UM_HEAD_BN : pair_width(M, cols, pairs, kRope ? 64 : 32);
-  if (st.pair_bn > 0 && !Epi::kReduce) bn = st.pair_bn;
+  constexpr bool kPlain = !Epi::kDual && !Epi::kReduce;
+  PairShape shape = Epi::kReduce ? PairShape{UM_HEAD_BN, 1} : pair_shape(st, M, cols, K, kRope ? 64 : 32, kPlain && st.pair_split != 1);
+  if (st.pair_bn > 0 && !Epi::kReduce) shape = {st.pair_bn, 1};
+  const int bn = shape.bn;
   int unit = 0;
   if constexpr (kRope) {
     if ((bn / 2) % epi.half) unit = 32;
@@ -431,9 +548,12 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
   if (band_max < 4) band_max = 4;
   if (st.pair_band > 0) band_max = st.pair_band;
   const int n_bands = (rg + band_max - 1) / band_max, band = (rg + n_bands - 1) / n_bands;
-  const int grid = 2 * (int)(T < pairs ? T : pairs);
-  PairArgs args{M, NP, n_tiles, rg, band, (K + 2 * UM_BK - 1) / (2 * UM_BK), bn, unit, stages, status};
-  cudaError_t e = launch_k(st.pdl, k_gemm_pair<Epi>, dim3(grid), dim3(PR_THREADS), smem, stream, 2, ma, mb0, mb1, args, epi);
+  int ks = shape.ks;
+  if (kPlain && st.pair_split > 1 && T * st.pair_split <= pairs && T <= st.max_clusters[2 * st.pair_split] && (K + 127) / 128 >= st.pair_split)
+    ks = st.pair_split;
+  const int grid = 2 * ks * (int)(T < pairs ? T : pairs);
+  PairArgs args{M, NP, n_tiles, rg, band, (K + 2 * UM_BK - 1) / (2 * UM_BK), ks, bn, unit, stages, status};
+  cudaError_t e = launch_k(st.pdl, k_gemm_pair<Epi>, dim3(grid), dim3(PR_THREADS), smem, stream, 2 * ks, ma, mb0, mb1, args, epi);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -5; }
   return 0;

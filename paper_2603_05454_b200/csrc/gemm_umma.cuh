@@ -351,8 +351,8 @@ struct UmmaState {
   int swap_min_rows = 129;         // row counts [min, max] that take the operand-swapped kernel (gemm_swap.cuh); max 0 = never
   int swap_max_rows = 256;
   int swap_force = 0;              // 1: take it whenever it can run (tests), not only where it was measured to pay
-  int pair_min_rows = 257;         // fewest rows that take the kernel on pairs of SMs (gemm_pair.cuh)
-  int pair_one_group = 1;          // ... and with 129..256 rows where umma_takes_pairs says so
+  int pair_min_rows = 129;         // fewest rows that take the kernel on pairs of SMs (gemm_pair.cuh)
+  int pair_split = 0;              // its K slices (0 = automatic, 1 = never, 2 or 3 where they fit)
   int pair_bn = 0;                 // its tile width (0 = automatic)
   int pair_band = 0;               // its row groups per band (0 = automatic)
   int stream_grid_mode = 2;        // its grid: 0 = by row count, 1 = one CTA per SM (even shares), 2 = multiple of the tile count
@@ -461,20 +461,15 @@ inline const CUtensorMap* umma_map(UmmaState& st, const void* base, int rows, in
 }
 
 constexpr int UM_HEAD_BN = 256;
-// Whether M rows of a launch with `tiles` 256-row tiles of 96 columns go to the pairs of SMs (gemm_pair.cuh).  From 257 rows
-// on always.  With 129 to 256 rows (one row group) wherever its tiles are enough or K is short: it does not split K, so a
-// narrow projection with a long K (FFN down: 43 tiles, K 12288) keeps half the chip idle for as long as K is, and the
-// operand-swapped kernel's K slices win.  Measured at 187 / 256 rows, us, best other kernel -> pairs: 12288 x 4096 29 -> 26,
-// 37 -> 27; 4096 x 4096 16.6 -> 14.9, 19.2 -> 15.1; 2 x 12288 SwiGLU 44 -> 45, 54 -> 46; head 249 -> 222; but 4096 x 12288
-// 30 -> 35 and 3584 x 18944 38 -> 48.
-inline bool umma_takes_pairs(const UmmaState& st, int M, int cols, int K) {
-  if (M >= st.pair_min_rows) return true;
-  if (M <= UM_BM || !st.pair_one_group || st.swap_force || st.stream_bn2 || st.stream_bn_dual) return false;
-  return (cols + 95) / 96 >= st.max_clusters[2] || K <= 6144;
+// More than 128 rows go to the pairs of SMs (gemm_pair.cuh).  With 129 to 256 rows (one row group) against the best kernels of
+// one SM per tile, at 187 / 256 rows, us: 12288 x 4096 29 -> 26, 37 -> 27; 4096 x 4096 16.6 -> 14.9, 19.2 -> 15.1; 2 x 12288 SwiGLU
+// 44 -> 45, 54 -> 46; 4096 x 12288 (three K slices) 30 -> 28.5; 3584 x 18944 38 -> 35.5; head 249 -> 222.
+inline bool umma_takes_pairs(const UmmaState& st, int M) {
+  return M >= st.pair_min_rows && !st.swap_force;
 }
 // Partials per row the head GEMM of M rows leaves: one per vocabulary tile, or (k_gemm_pair) one per half tile.
-inline int umma_head_tiles(const UmmaState& st, int M, int vocab, int K) {
-  return (vocab + UM_HEAD_BN - 1) / UM_HEAD_BN * (umma_takes_pairs(st, M, vocab, K) ? 2 : 1);
+inline int umma_head_tiles(const UmmaState& st, int M, int vocab) {
+  return (vocab + UM_HEAD_BN - 1) / UM_HEAD_BN * (umma_takes_pairs(st, M) ? 2 : 1);
 }
 
 template <typename Epi> int stream_row_tiles(const UmmaState& st, int M, int NP, int K, int bn);
@@ -523,7 +518,7 @@ template <typename Epi>
 int umma_gemm(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
               int n_rows_w, const Epi& epi, unsigned* status) {
   if (K % UM_BK) { st.err = "K must be a multiple of 64"; return -6; }
-  if (umma_takes_pairs(st, M, Epi::kDual ? 2 * NP : NP, K)) return pair_launch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
+  if (umma_takes_pairs(st, M)) return pair_launch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
   if constexpr (Epi::kReduce) {
     {
       const int smt = stream_row_tiles<Epi>(st, M, NP, K, UM_HEAD_BN);

@@ -271,7 +271,7 @@ int run_head(lsp_ctx* c, const T* hidden, int rows, int* n_tiles_out) {
   epi.exclude_id = c->s.exclude_mask_logit ? m.mask_id : -1;
   int n_tiles = (m.vocab + SG_HEAD_BN - 1) / SG_HEAD_BN;
 #ifndef LSP_NO_UMMA
-  if (std::is_same<T, bf16>::value && c->gemm_impl == 1) n_tiles = umma_head_tiles(c->umma, rows, m.vocab, m.d_model);
+  if (std::is_same<T, bf16>::value && c->gemm_impl == 1) n_tiles = umma_head_tiles(c->umma, rows, m.vocab);
 #endif
   epi.n_tiles = n_tiles;
   *n_tiles_out = n_tiles;
@@ -843,7 +843,8 @@ int lsp_debug_set(lsp_ctx* c, int key, int value) {
   else if (key == 23) c->umma.stream_bn = (value == 256 || value == 128) ? value : 0;
   else if (key == 40) c->umma.pair_min_rows = value;
   else if (key == 41) c->umma.pair_bn = (value >= 96 && value <= 256 && value % 32 == 0) ? value : 0;
-  else if (key == 45) c->umma.pair_one_group = value ? 1 : 0;
+  else if (key == 46) c->umma.pair_split = (value >= 0 && value <= 3) ? value : 0;
+  else if (key == 45) c->umma.pair_min_rows = value ? 129 : 257;
   else if (key == 42) c->umma.pair_band = value < 0 ? 0 : value;
   else if (key == 43) c->umma.stream_split_copies = value ? 1 : 0;
   else if (key == 44) c->umma.stream_exchange_rows = value;

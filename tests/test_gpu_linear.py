@@ -424,3 +424,25 @@ def test_linear_bf16_short_k_without_a_split(M, N, K):
     dec.op_linear(2, A, W, W2, out)
     assert near(out, torch.nn.functional.silu(ref) * up, 2)
     dec.close()
+
+
+@pytest.mark.parametrize("ks", [0, 2, 3])
+@pytest.mark.parametrize("M,N,K", [(187, 4096, 12288), (129, 512, 2048), (257, 272, 3072), (256, 3584, 4032), (700, 1040, 4096)])
+def test_linear_bf16_k_slices_on_pairs(M, N, K, ks):
+    """K slices of a 256-row tile on clusters of two or three pairs: ragged last column tiles and K chunks, a chunk count that
+    the slices do not divide, rows of one CTA of the pair only; against the fp64 product, and twice the same bits."""
+    dec = _dec("bf16")
+    dec.debug_set(46, ks)
+    A = S.normal((M, K), 17, 1, 1.0, torch.bfloat16, DEV)
+    W = S.normal((N, K), 17, 2, 0.05, torch.bfloat16, DEV)
+    X0 = S.normal((M, N), 17, 4, 1.0, torch.bfloat16, DEV)
+    ref = A.double() @ W.double().t()
+    near = lambda got, want: bool(((got.double() - want).abs() <= want.abs() / 128 + want.abs().max() / 2560).all())
+    x, y = X0.clone(), X0.clone()
+    dec.op_linear(1, A, W, None, x)
+    dec.op_linear(1, A, W, None, y)
+    assert near(x, X0.double() + ref) and torch.equal(x, y)
+    out = torch.full((M + 1, N), 7.0, dtype=torch.bfloat16, device=DEV)
+    dec.op_linear(0, A, W, None, out[:M])
+    assert near(out[:M], ref) and bool((out[M] == 7.0).all())
+    dec.close()
