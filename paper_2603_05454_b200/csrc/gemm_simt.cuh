@@ -7,9 +7,10 @@
 // epilogue) and the eight warps of a CTA split K: warp w takes the 16-element steps w, w + 8, ... of the whole tile, loading the next step's operands while it
 // multiplies this one's; the eight partial tiles are summed in warp order through shared memory (the same order every time)
 // and each thread finishes four neighbouring outputs (two pairs).
-// Measured (B200, fp32, us, k_gemm_simt -> k_gemm_simt_split): 65 x 384 (K 256) 15.2 -> 7.7, 128 x 256 (K 1024) 51 -> 18,
-// 300 x 2048 (K 1024; 160 tiles of 64 x 64) 97 -> 78, 1024 x 4096 (K 4096; 1024 tiles) 1007 -> 1668: the line is drawn at two
-// 64 x 64 tiles per SM.
+// Measured (B200, fp32, us, k_gemm_simt -> k_gemm_simt_split): 65 x 384 (K 256) 15.2 -> 5.9, 128 x 256 (K 1024) 51 -> 14.8,
+// 300 x 2048 (K 1024; 160 tiles of 64 x 64) 97 -> 53, 1024 x 4096 (K 4096; 1024 tiles) 1007 -> over 1100: the line is drawn at
+// two 64 x 64 tiles per SM.  Four neighbouring lanes load a row's 64 bytes of a step (a row per lane cost four times the
+// cache lines per instruction: 18 us instead of 14.8), and sixteen warps per CTA gained nothing.
 #pragma once
 #include "epilogues.cuh"
 
@@ -47,20 +48,21 @@ __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* __re
   const int m0 = blockIdx.y * BM, j0 = blockIdx.x * PT;
   float* As = sm + w * WARP_F;
   float* Bs = As + SG_KS * LA;
-  // operand rows of this lane's vectors (null past the edges)
+  // operand rows of this lane's vectors, four neighbouring lanes to a row's 16 elements (null past the edges)
+  static_assert(SG_KS == 16, "four vectors per row");
   const T* ap[NA];
   const T* bp[NB];
 #pragma unroll
   for (int i = 0; i < NA; ++i) {
-    const int v = lane + 32 * i, m = m0 + v % BM;
-    ap[i] = m < M ? A + (size_t)m * K + (v / BM) * 4 : nullptr;
+    const int v = lane + 32 * i, m = m0 + (v >> 2);
+    ap[i] = m < M ? A + (size_t)m * K + (v & 3) * 4 : nullptr;
   }
 #pragma unroll
   for (int i = 0; i < NB; ++i) {
-    const int v = lane + 32 * i, c = v % BN;
+    const int v = lane + 32 * i, c = v >> 2;
     const int j = j0 + (Epi::kDual ? c % PT : c);
     const T* row = (Epi::kDual && c >= PT) ? W1 + (size_t)epi.row1(j) * K : W0 + (size_t)epi.row0(j) * K;
-    bp[i] = j < NP ? row + (v / BN) * 4 : nullptr;
+    bp[i] = j < NP ? row + (v & 3) * 4 : nullptr;
   }
   const int rg = lane / (BN / 8), cg = lane % (BN / 8);         // rows 4 rg .., columns 4 cg .. and BN / 2 + 4 cg ..
   float acc[4][8] = {};
@@ -79,13 +81,13 @@ __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* __re
 #pragma unroll
     for (int i = 0; i < NA; ++i) {
       const int v = lane + 32 * i;
-      float* d = As + (v / BM) * 4 * LA + v % BM;
+      float* d = As + (v & 3) * 4 * LA + (v >> 2);
       d[0] = av[i].x; d[LA] = av[i].y; d[2 * LA] = av[i].z; d[3 * LA] = av[i].w;
     }
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
       const int v = lane + 32 * i;
-      float* d = Bs + (v / BN) * 4 * LB + v % BN;
+      float* d = Bs + (v & 3) * 4 * LB + (v >> 2);
       d[0] = bv[i].x; d[LB] = bv[i].y; d[2 * LB] = bv[i].z; d[3 * LB] = bv[i].w;
     }
     __syncwarp();

@@ -252,13 +252,13 @@ int run_gemm(lsp_ctx* c, const T* A, const T* W0, const T* W1, int M, int NP, in
   }
 #endif
   dim3 grid((NP + SG_BN - 1) / SG_BN, (M + SG_BM - 1) / SG_BM);
-  auto kern = k_gemm_simt<T, Epi>;
   if ((long)grid.x * grid.y < 2l * sm_count(c)) {          // (the line: see gemm_simt.cuh)
     using Tile = SimtTile<Epi>;
     grid = dim3((NP + Tile::PER_TILE - 1) / Tile::PER_TILE, (M + Tile::BM - 1) / Tile::BM);
-    kern = k_gemm_simt_split<T, Epi>;
+    CU(launch_k(c->pdl, k_gemm_simt_split<T, Epi>, grid, dim3(256), 0, c->stream, A, W0, W1, M, NP, K, epi));
+  } else {
+    CU(launch_k(c->pdl, k_gemm_simt<T, Epi>, grid, dim3(256), 0, c->stream, A, W0, W1, M, NP, K, epi));
   }
-  CU(launch_k(c->pdl, kern, grid, dim3(256), 0, c->stream, A, W0, W1, M, NP, K, epi));
   return LSP_OK;
 }
 
@@ -896,9 +896,10 @@ int lsp_denoise_step(lsp_ctx* c, lsp_step_rec* rec) {
 
 namespace {
 
-// Enqueues the commit kernel(s) of a step that read descriptor sd; the block lengths are in len or in sd's Lc array.
+// Enqueues the commit kernel(s) of a step that read descriptor sd; the block lengths are in len or in sd's Lc array.  next_desc:
+// the device descriptor to fill in for the next step (the lagged loop), or null.
 // max_pend: the longest pending block (an upper bound is enough: it only sizes the copy's grid).
-int enqueue_commit(lsp_ctx* c, const StepDesc& sd, const LenInline& len, int B, int max_pend, int max_n) {
+int enqueue_commit(lsp_ctx* c, const StepDesc& sd, const LenInline& len, int B, int max_pend, int max_n, int* next_desc = nullptr) {
   const lsp_model_cfg& m = c->m;
   const size_t kvd = (size_t)m.n_kv_heads * m.head_dim;
   const int row_v4 = (int)(kvd * c->esz / 16);
@@ -917,7 +918,7 @@ int enqueue_commit(lsp_ctx* c, const StepDesc& sd, const LenInline& len, int B, 
   if ((!scattered || max_pend > 0) && (copy || !scattered)) {
     launch_k(c->pdl, k_commit_append, dim3(grid), dim3(256), 0, c->stream, sd, (const uint4*)c->stage, (uint4*)c->kv_cache,
                                                  stage_plane_v4, cache_plane_v4, cache_seq_v4, row_v4, c->yhat,
-                                                 c->tokens, c->tok_stride, scattered ? 0 : 1, copy ? 1 : 0, len);
+                                                 c->tokens, c->tok_stride, scattered ? 0 : 1, copy ? 1 : 0, len, next_desc, c->max_batch + 1, B);
     count_launch(c, CLS_COMMIT);
   }
   if (scattered) {
@@ -933,7 +934,7 @@ int enqueue_commit(lsp_ctx* c, const StepDesc& sd, const LenInline& len, int B, 
 }
 
 // Algorithm 1's loop with the block lengths kept on the device (prefix topology).  Pass j+1 is enqueued before L_j has
-// been read back: the scan's L goes straight into the commit kernel, k_advance derives the next descriptor from it on
+// been read back: the scan's L goes straight into the commit kernel, the commit kernel derives the next descriptor from it on
 // the device, and the host only needs the row counts to size the launches -- and those it knows one step late, because
 // a sequence's rows at step j+1 (pending block + masked suffix) are exactly its masked suffix at step j, N_j, which
 // follows from L_{j-1}.  The LM-head row count is an upper bound (N_j - 1); rows beyond the real ones are inert.
@@ -1012,7 +1013,7 @@ int generate_lagged(lsp_ctx* c, lsp_step_rec* recs, int max_recs, int* n_steps) 
     PassDims pd;
     if (exact) {
       pd = host_descriptor(c);
-      // the device descriptor of this step: the first one is uploaded; later ones were derived on the device (k_advance)
+      // the device descriptor of this step: the first one is uploaded; later ones were derived on the device (advance_descriptor)
       // from the same block lengths and are equal to the host's
       if (launched == 0) { rc = send_descriptor(c, &din); if (rc) return rc; }
     } else {
@@ -1046,12 +1047,8 @@ int generate_lagged(lsp_ctx* c, lsp_step_rec* recs, int max_recs, int* n_steps) 
     int max_pend = 0;
     if (exact) { for (int b = 0; b < B; ++b) if (c->N[b] > 0) max_pend = std::max(max_pend, c->pend[b]); }
     else max_pend = std::min(pd.maxQ, std::max(8, 2 * last_L));
-    rc = enqueue_commit(c, sc, LenInline(), B, max_pend, 0);
+    rc = enqueue_commit(c, sc, LenInline(), B, max_pend, 0, c->d_desc + (size_t)(par ^ 1) * 7 * s);
     if (rc) return rc;
-    launch_k(c->pdl, k_advance, dim3(1), dim3(32), 0, c->stream, sd, c->d_desc + (size_t)(par ^ 1) * 7 * s, s,
-             (const int32_t*)(c->d_scan + mb), B);
-    CU(cudaGetLastError());
-    count_launch(c, CLS_COMMIT);
     c->last_M = pd.M;
     c->score_rows = pd.Mh;
     ++launched;

@@ -354,6 +354,32 @@ __global__ void __launch_bounds__(256) k_lsp_scan(const float* __restrict__ scor
 }
 
 // ---------------------------------------------------------------------------------------------
+// Next step's descriptor, computed on the device from this step's and the scan's block lengths (prefix topology), so
+// that the host can enqueue the next pass without reading L back first:
+//   F += pend;  pend = L;  N -= L;  Fp += L;  rows = pend + N (0 once N = 0);  row_off / head_off = prefix sums.
+// One thread of the commit kernel (whose other threads read the current descriptor; nxt is the other one).
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void advance_descriptor(const StepDesc& cur, int* __restrict__ nxt, int stride, int batch) {
+  int M = 0, Mh = 0;
+  for (int b = 0; b < batch; ++b) {
+    const int N = cur.N[b];
+    const int L = N > 0 ? cur.Lc[b] : 0;
+    const int pend = N > 0 ? cur.pend[b] : 0;
+    const int N2 = N - L;
+    nxt[0 * stride + b] = cur.F[b] + pend;
+    nxt[1 * stride + b] = N2 > 0 ? L : 0;
+    nxt[2 * stride + b] = N2;
+    nxt[3 * stride + b] = M;
+    nxt[4 * stride + b] = Mh;
+    nxt[5 * stride + b] = cur.Fp[b] + L;
+    M += N2 > 0 ? L + N2 : 0;
+    Mh += N2;
+  }
+  nxt[3 * stride + batch] = M;
+  nxt[4 * stride + batch] = Mh;
+}
+
+// ---------------------------------------------------------------------------------------------
 // Commit (Algorithm 1: commit and AppendToCache).  grid = (chunks, n_layers * 2, batch):
 //   * the pending block's K/V rows, staged by the last pass at packed rows [row_off_b, row_off_b + pend_b),
 //     are copied to cache rows [F_b, F_b + pend_b): one contiguous 128-bit-vector copy per (layer, K|V, b);
@@ -366,7 +392,8 @@ __global__ void k_commit_append(StepDesc sd, const uint4* __restrict__ stage, ui
                                 size_t cache_seq_v4,     // uint4 per sequence inside a cache plane
                                 int row_v4,              // uint4 per row (n_kv_heads * head_dim * sizeof(T) / 16)
                                 const int32_t* __restrict__ yhat, int32_t* __restrict__ tokens, int tok_stride,
-                                int write_tokens, int copy_rows, const __grid_constant__ LenInline len) {
+                                int write_tokens, int copy_rows, const __grid_constant__ LenInline len,
+                                int* __restrict__ next_desc, int desc_stride, int batch) {
   pdl_begin();
   const int b = blockIdx.z;
   const int plane = blockIdx.y;
@@ -382,34 +409,8 @@ __global__ void k_commit_append(StepDesc sd, const uint4* __restrict__ stage, ui
     int32_t* t = tokens + (size_t)b * tok_stride + sd.Fp[b];
     for (int i = threadIdx.x; i < L; i += blockDim.x) t[i] = yhat[ho + i];
   }
-}
-
-// ---------------------------------------------------------------------------------------------
-// Next step's descriptor, computed on the device from this step's and the scan's block lengths (prefix topology), so
-// that the host can enqueue the next pass without reading L back first:
-//   F += pend;  pend = L;  N -= L;  Fp += L;  rows = pend + N (0 once N = 0);  row_off / head_off = prefix sums.
-// One thread; runs after the commit kernel of the step (which still reads the current descriptor).
-// ---------------------------------------------------------------------------------------------
-__global__ void k_advance(StepDesc cur, int* __restrict__ nxt, int stride, const int32_t* __restrict__ L_commit, int batch) {
-  pdl_begin();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  int M = 0, Mh = 0;
-  for (int b = 0; b < batch; ++b) {
-    const int N = cur.N[b];
-    const int L = N > 0 ? L_commit[b] : 0;
-    const int pend = N > 0 ? cur.pend[b] : 0;
-    const int N2 = N - L;
-    nxt[0 * stride + b] = cur.F[b] + pend;
-    nxt[1 * stride + b] = N2 > 0 ? L : 0;
-    nxt[2 * stride + b] = N2;
-    nxt[3 * stride + b] = M;
-    nxt[4 * stride + b] = Mh;
-    nxt[5 * stride + b] = cur.Fp[b] + L;
-    M += N2 > 0 ? L + N2 : 0;
-    Mh += N2;
-  }
-  nxt[3 * stride + batch] = M;
-  nxt[4 * stride + batch] = Mh;
+  if (next_desc != nullptr && blockIdx.x == 0 && plane == 0 && b == 0 && threadIdx.x == blockDim.x - 1)
+    advance_descriptor(sd, next_desc, desc_stride, batch);
 }
 
 // ---------------------------------------------------------------------------------------------
