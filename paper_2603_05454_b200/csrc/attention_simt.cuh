@@ -7,7 +7,14 @@
 namespace lsp {
 
 // Queries per block: 4 per warp where that still gives a block per SM, else 1 per warp (the K/V tile is then used by fewer
-// queries, but a small pass is bound by one block's serial walk over the keys: tiny model, 26 -> 19 us a launch).
+// queries, but a small pass is bound by one block's serial walk over the keys: tiny model, 26 -> 19 us a launch; with vector
+// loads a tile ahead and four dot-product chains 12).
+__device__ __forceinline__ float4 as_load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 as_load4(const bf16* p) {
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&u.x), b = *reinterpret_cast<const __nv_bfloat162*>(&u.y);
+  return make_float4(__low2float(a), __high2float(a), __low2float(b), __high2float(b));
+}
 constexpr int AS_BK = 32;   // keys per tile (one per lane)
 
 // grid = (ceil(max_rows_per_seq / (4 QW)), n_heads, batch), block = 128; QW queries per warp.
@@ -22,7 +29,7 @@ __global__ void __launch_bounds__(128) k_attn_simt(const T* __restrict__ q, cons
   constexpr int AS_BQ = 4 * QW;
   __shared__ float Qs[AS_BQ][DH];
   __shared__ float Ks[AS_BK][DH + 1];
-  __shared__ float Vs[AS_BK][DH];
+  __shared__ __align__(16) float Vs[AS_BK][DH];
   pdl_begin();
   const int b = blockIdx.z, h = blockIdx.y;
   const int r0 = sd.row_off[b];
@@ -52,29 +59,45 @@ __global__ void __launch_bounds__(128) k_attn_simt(const T* __restrict__ q, cons
   const T* cv = cache_v + (size_t)b * cache_seq_elems + kvh * DH;
   const T* sk = stage_k + (size_t)r0 * ldkv + kvh * DH;
   const T* sv = stage_v + (size_t)r0 * ldkv + kvh * DH;
-  for (int s0 = 0; s0 < S; s0 += AS_BK) {
-    __syncthreads();
-    {
-      const int key = t >> 2, part = (t & 3) * (DH / 4);
-      const int s = s0 + key;
+  // A tile's keys and values: vector i of thread t is elements 4 (t % (DH / 4)) .. of key t / (DH / 4) + i * KPI.  The next tile's
+  // are fetched while this one's are used.
+  constexpr int VPR = DH / 4, KPI = 128 / VPR, NV = AS_BK / KPI;
+  float4 kreg[NV], vreg[NV];
+  const int vk = t / VPR, ve = (t % VPR) * 4;
+  auto fetch = [&](int s0) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int s = s0 + vk + i * KPI;
       const T* kp = nullptr;
       const T* vp = nullptr;
       if (s < F) { kp = ck + (size_t)s * ldkv; vp = cv + (size_t)s * ldkv; }
       else if (s < S) { kp = sk + (size_t)(s - F) * ldkv; vp = sv + (size_t)(s - F) * ldkv; }
-#pragma unroll 4
-      for (int d = 0; d < DH / 4; ++d) {
-        Ks[key][part + d] = kp ? to_f(kp[part + d]) : 0.f;
-        Vs[key][part + d] = vp ? to_f(vp[part + d]) : 0.f;
-      }
+      kreg[i] = kp ? as_load4(kp + ve) : make_float4(0.f, 0.f, 0.f, 0.f);
+      vreg[i] = vp ? as_load4(vp + ve) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  fetch(0);
+  for (int s0 = 0; s0 < S; s0 += AS_BK) {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int key = vk + i * KPI;
+      Ks[key][ve] = kreg[i].x; Ks[key][ve + 1] = kreg[i].y; Ks[key][ve + 2] = kreg[i].z; Ks[key][ve + 3] = kreg[i].w;
+      *reinterpret_cast<float4*>(&Vs[key][ve]) = vreg[i];
     }
     __syncthreads();
+    if (s0 + AS_BK < S) fetch(s0 + AS_BK);
     const bool kvalid = (s0 + lane) < S;
 #pragma unroll
     for (int i = 0; i < QW; ++i) {
       const int qi = w * QW + i;
-      float dot = 0.f;
-#pragma unroll 8
-      for (int d = 0; d < DH; ++d) dot = fmaf(Qs[qi][d], Ks[lane][d], dot);
+      float d4[4] = {0.f, 0.f, 0.f, 0.f};                     // (four chains: one would be DH dependent steps)
+#pragma unroll 4
+      for (int d = 0; d < DH; d += 4) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) d4[e] = fmaf(Qs[qi][d + e], Ks[lane][d + e], d4[e]);
+      }
+      const float dot = (d4[0] + d4[1]) + (d4[2] + d4[3]);
       const float sc = kvalid ? dot * scale : -INFINITY;
       const float m_new = fmaxf(m_run[i], warp_max(sc));
       const float p = kvalid ? __expf(sc - m_new) : 0.f;
