@@ -49,15 +49,15 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # weight bytes streamed, so the reported figure is the class's mean algorithmic bytes per launch scaled by the
 # captured ratio.  A class whose sources changed since the capture reports null.
 CLASS_SOURCES = {
-    "gemm": ("gemm_stream.cuh", "gemm_swap.cuh", "gemm_umma.cuh", "epilogues.cuh", "common.cuh"),
-    "head": ("gemm_stream.cuh", "gemm_swap.cuh", "gemm_umma.cuh", "epilogues.cuh", "common.cuh"),
+    "gemm": ("gemm_stream.cuh", "gemm_pair.cuh", "gemm_umma.cuh", "epilogues.cuh", "common.cuh"),
+    "head": ("gemm_stream.cuh", "gemm_pair.cuh", "gemm_umma.cuh", "epilogues.cuh", "common.cuh"),
     "attn": ("attention_umma.cuh", "common.cuh"),
     "commit": ("misc_kernels.cuh", "common.cuh"),
 }
 NCU_TRAFFIC = {
-    # k_gemm_stream<128,1,1,EpiStore>, M 64, N 12288, K 4096: profiles/k_gemm_stream_M64_N12288_K4096.md
+    # k_gemm_stream<128,EpiStore>, M 64, N 12288, K 4096: profiles/k_gemm_stream_M64_N12288_K4096.md
     "gemm": {"captured_bytes": 105.06e6, "algorithmic_bytes": 102.8e6, "src": "34127c2c8b24"},
-    # k_gemm_stream<256,1,1,EpiHead>, 64 rows: profiles/k_gemm_stream_head_M64_V126464.md
+    # k_gemm_stream<256,EpiHead>, 64 rows: profiles/k_gemm_stream_head_M64_V126464.md
     "head": {"captured_bytes": 1062.8e6, "algorithmic_bytes": 1037.0e6, "src": "34127c2c8b24"},
     # k_attn_umma, 16 x (128 query rows over 2048 keys): profiles/k_attn_umma_B16_F1920.md
     "attn": {"captured_bytes": 569.2e6, "algorithmic_bytes": 570.4e6, "src": "196044e4044b"},
@@ -620,7 +620,7 @@ def head_line(dev, peaks, peak_kind, steps, warmup, sampler=None):
             "roofline": {"bound": "tensor", "achieved": head.get("tflops"), "peak": peaks["bf16_tflops"],
                          "unit": "TFLOP/s", "frac": (head.get("tflops") or 0) / peaks["bf16_tflops"],
                          "traffic": head.get("traffic"), "peak_kind": "burst, of " + peak_kind,
-                         "kernel": "k_gemm_stream<256,.,.,EpiHead> (LM head with the top-2 / log-sum-exp reduction in its epilogue)"},
+                         "kernel": "k_gemm_pair<EpiHead> (LM head with the top-2 / log-sum-exp reduction in its epilogue)"},
             "e2e": {"value": r["positions"] / (r["e2e_ms"] * 1e-3), "unit": "positions/s",
                     "h2d_bytes_per_step": r["h2d"], "d2h_bytes_per_step": r["d2h"]},
             "gpu_launches": r["launches"], "classes": r["classes"], "clocks": clocks}
@@ -645,7 +645,7 @@ def topology_line(wl, dev, peaks, peak_kind, warmup, sampler=None):
             "roofline": {"bound": "tensor", "achieved": g.get("tflops"), "peak": tc, "unit": "TFLOP/s",
                          "frac": g.get("tensor_frac_sustained"), "traffic": g.get("traffic"),
                          "peak_kind": "sustained, of " + peak_kind,
-                         "kernel": "k_gemm_stream (layer GEMMs; 17 k to 33 k rows per pass: tensor-bound)",
+                         "kernel": "k_gemm_pair (layer GEMMs; 17 k to 33 k rows per pass: tensor-bound)",
                          "timed": f"per-launch CUDA events over the first {n_cls} passes of one more LSP decode"},
             "classes": classes, "topologies": cmp_, "gpu_launches": lsp["gpu_launches"], "clocks": clocks}
 
@@ -716,7 +716,7 @@ def main():
             "tokens_per_pass": r["l_commit_mean"],
             "roofline": {"bound": "hbm", "achieved": gemm.get("gbs"), "peak": peaks["hbm_gbs"], "unit": "GB/s",
                          "frac": gemm.get("hbm_frac"), "traffic": gemm.get("traffic"),
-                         "kernel": "k_gemm_stream (layer projections and FFN; all but the first pass have at most 257 rows: weight-streaming regime)",
+                         "kernel": "k_gemm_stream up to 128 rows, k_gemm_pair above (layer projections and FFN; all but the first pass have at most 257 rows: mostly the weight-streaming regime)",
                          "peak_kind": "of " + peak_kind,
                          "timed": "per-launch CUDA events, second pass over the same K decodes (each event pair adds "
                                   "about 5 us and breaks the overlap between consecutive launches: a lower bound)",

@@ -1,4 +1,4 @@
-// bf16 GEMM on pairs of SMs (tcgen05.mma.cta_group::2), for passes of more than 256 activation rows.
+// bf16 GEMM on pairs of SMs (tcgen05.mma.cta_group::2), for passes of more than 128 activation rows.
 //
 //   acc[m, c] = sum_k A[m, k] * Wt[c, k]        operands and fused epilogues as k_gemm_stream (gemm_umma.cuh)
 //
@@ -16,16 +16,16 @@
 //     epilogue of a tile overlaps the next tile's MMAs.
 //   * BN is a run-time multiple of 32 (64 for the rotary epilogue), chosen so that the last wave of tiles is full (see
 //     pair_shape).
-// Measured (B200, back to back, weights from a ring larger than L2; row-major k_gemm_stream before -> now, us):
+//   * The weight tile's two halves come from the two tensors / row ranges whose columns a fused epilogue pairs (gate and
+//     up, rotate-half partners), so CTA 0 always loads the first and CTA 1 the second of the pair.
+//   * Eight epilogue warps: two per quarter of the accumulator rows, each taking half of the 16-column chunks.  The
+//     residual epilogue fetches its rows of x while it waits for the accumulators.
+// Measured (B200, back to back, weights from a ring larger than L2; one SM per tile before -> now, us):
 //   rows    12288 x 4096   4096 x 4096   2 x 12288 x 4096 SwiGLU   4096 x 12288
 //    512      58 -> 42      31 -> 17            111 -> 76          56 -> 45
 //   1000     104 -> 74      41 -> 28            153 -> 139          86 -> 75
 //   4096     313 -> 271     129 -> 99            559 -> 512         311 -> 297
 //   8240     646 -> 551     260 -> 202           1205 -> 1050        657 -> 596
-//   * The weight tile's two halves come from the two tensors / row ranges whose columns a fused epilogue pairs (gate and
-//     up, rotate-half partners), so CTA 0 always loads the first and CTA 1 the second of the pair.
-//   * Eight epilogue warps: two per quarter of the accumulator rows, each taking half of the 16-column chunks.  The
-//     residual epilogue fetches its rows of x while it waits for the accumulators.
 // Warp roles (320 threads): warp 0 = TMA producer, warp 1 = TMEM allocator and, in the pair's first CTA, MMA issuer,
 // warps 2..9 = epilogue.  Every wait is bounded; on expiry the kernel records (code, site) in the status word, drains and
 // returns.

@@ -4,11 +4,11 @@
 //
 // This header holds the PTX wrappers (mbarrier with bounded waits, TMA tile loads (every CTA fetches its own tiles), tcgen05.mma /
 // .commit / .ld), the shared-memory and instruction descriptors, the vectorised fused epilogues (store / residual /
-// SwiGLU / rotary + K/V staging), the host state (tensor-map cache, tuning fields) and the dispatch that picks tile
-// width and row tiles per CTA.  The kernel itself is the persistent k_gemm_stream of gemm_stream.cuh; the attention
-// kernel (attention_umma.cuh) uses the same wrappers.
+// SwiGLU / rotary + K/V staging), the host state (tensor-map caches, tuning fields) and the dispatch that picks
+// kernel and tile width.  The kernels are k_gemm_stream (gemm_stream.cuh, up to 128 rows) and k_gemm_pair (gemm_pair.cuh, more);
+// the attention kernel (attention_umma.cuh) uses the same wrappers.
 //
-// The B tile is two TMA boxes of BN/2 weight rows each (possibly from two tensors), so accumulator columns
+// The B tile is two blocks of BN/2 weight rows each (possibly from two tensors), so accumulator columns
 // c and c + BN/2 of one thread hold the pair an element-wise fusion needs (gate/up, rotate-half partners).
 // Every wait is bounded by wall-clock time; on expiry a kernel records (code, site) in a status word, lets
 // all roles drain and returns, so a protocol error can never hang the device.
@@ -179,10 +179,6 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr) {
   return d;
 }
 // Instruction descriptor: D = f32, A = B = bf16, both K-major, M = 128, N = BN.
-// (M = 64 puts accumulator row r in tensor-memory lane 32 (r / 16) + r % 16: the lower half of every warp's lane quarter.)
-__host__ __device__ constexpr uint32_t make_idesc_m64(int bn) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(64 >> 4) << 24);
-}
 __host__ __device__ constexpr uint32_t make_idesc(int bn) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(UM_BM >> 4) << 24);
 }
@@ -320,7 +316,6 @@ typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_
 
 struct UmmaState {
   PFN_encodeTiled encode = nullptr;
-  std::map<std::tuple<const void*, int, int, int>, CUtensorMap> cache;
   std::map<std::tuple<const void*, int, int, int, int, int>, CUtensorMap> cache4;
   std::map<std::tuple<const void*, size_t, int, int, int, int>, CUtensorMap> cache5;
   int max_smem = 0;
@@ -331,32 +326,20 @@ struct UmmaState {
   int n_counters = 0;
   int target_ctas = 0;             // 0 = one CTA per SM
   int max_stages = UM_MAX_STAGES;
-  int sm_smem = 233472;            // shared memory per SM
   int pdl = 1;                     // launch with the programmatic-serialisation attribute
   int stream_cluster = 1;          // persistent kernel: K slices of a tile on one thread block cluster, reduced through DSMEM
   int max_clusters[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};   // [c]: clusters of c one-per-SM CTAs that can be resident at once (queried at init)
-  int stream_half_sm = 1;          // persistent kernel: cap shared memory at half an SM when three stages still fit
-  int stream_issuers = 1;          // MMA-issuing warps with one row tile per CTA (two row tiles always use two); measured: no gain from 2
-  int stream_two_tiles = 1;        // 129..256 rows: 1 = two row tiles per CTA, 2 = two row groups
-  int stream_big_mt = 3;           // ... and for more rows: 1 or 2 row tiles per CTA, 3 = whichever fills the SMs better
-  int stream_bn = 0;               // its tile width with one row tile (0 = automatic)
-  int stream_bn2 = 0;              // ... and with two row tiles
+  int stream_even = 0;             // persistent kernel: even shares over all SMs instead of equal K slices per tile
+  int stream_bn = 0;               // its tile width (0 = automatic)
   int stream_bn_dual = 0;          // tile width of dual epilogues: 0 = automatic, 192 or 256
   int stream_exchange = 1;         // clusters of 2 exchange half tiles instead of publishing whole partial tiles
   int stream_exchange_rows = 64;   // ... from this many rows on
   int stream_atoms = 0;            // K atoms per stage: 0 = two when stream_min_stages2 such stages fit, else 1 or 2 as given
   int stream_min_stages2 = 3;
   int stream_split_copies = 0;     // a dual tile's weights by one copy per half and atom even where one copy can bring them all
-  int stream_half_tile1 = 1;       // 129..192 rows on two row tiles, unsplit: 64-row MMAs for the second row tile
-  int swap_min_rows = 129;         // row counts [min, max] that take the operand-swapped kernel (gemm_swap.cuh); max 0 = never
-  int swap_max_rows = 256;
-  int swap_force = 0;              // 1: take it whenever it can run (tests), not only where it was measured to pay
-  int pair_min_rows = 129;         // fewest rows that take the kernel on pairs of SMs (gemm_pair.cuh)
   int pair_split = 0;              // its K slices (0 = automatic, 1 = never, 2 or 3 where they fit)
   int pair_bn = 0;                 // its tile width (0 = automatic)
   int pair_band = 0;               // its row groups per band (0 = automatic)
-  int stream_grid_mode = 2;        // its grid: 0 = by row count, 1 = one CTA per SM (even shares), 2 = multiple of the tile count
-  int stream_even_max_rows = 0;    // mode 0: even shares up to this many activation rows
   std::string err;
 };
 
@@ -373,7 +356,6 @@ inline int umma_init(UmmaState& st) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&st.max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   cudaDeviceGetAttribute(&st.n_sm, cudaDevAttrMultiProcessorCount, dev);
-  cudaDeviceGetAttribute(&st.sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   return 0;
 }
 
@@ -440,146 +422,71 @@ inline const CUtensorMap* umma_map5(UmmaState& st, const WeightView& v, int K, i
   return &st.cache5.emplace(key, m).first->second;
 }
 
-// 2-D bf16 tensor [rows, K] row-major, box = [64 (K), box_rows], 128-byte swizzle, zero fill out of bounds.
-inline const CUtensorMap* umma_map(UmmaState& st, const void* base, int rows, int K, int box_rows) {
-  auto key = std::make_tuple(base, rows, K, box_rows);
-  auto it = st.cache.find(key);
-  if (it != st.cache.end()) return &it->second;
-  CUtensorMap m;
-  cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-  cuuint32_t box[2] = {(cuuint32_t)UM_BK, (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = st.encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) {
-    st.err = "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
-    return nullptr;
-  }
-  return &st.cache.emplace(key, m).first->second;
-}
-
 constexpr int UM_HEAD_BN = 256;
 // More than 128 rows go to the pairs of SMs (gemm_pair.cuh).  With 129 to 256 rows (one row group) against the best kernels of
 // one SM per tile, at 187 / 256 rows, us: 12288 x 4096 29 -> 26, 37 -> 27; 4096 x 4096 16.6 -> 14.9, 19.2 -> 15.1; 2 x 12288 SwiGLU
 // 44 -> 45, 54 -> 46; 4096 x 12288 (three K slices) 30 -> 28.5; 3584 x 18944 38 -> 35.5; head 249 -> 222.
-inline bool umma_takes_pairs(const UmmaState& st, int M) {
-  return M >= st.pair_min_rows && !st.swap_force;
-}
+inline bool umma_takes_pairs(int M) { return M > UM_BM; }
 // Partials per row the head GEMM of M rows leaves: one per vocabulary tile, or (k_gemm_pair) one per half tile.
-inline int umma_head_tiles(const UmmaState& st, int M, int vocab) {
-  return (vocab + UM_HEAD_BN - 1) / UM_HEAD_BN * (umma_takes_pairs(st, M) ? 2 : 1);
+inline int umma_head_tiles(int M, int vocab) {
+  return (vocab + UM_HEAD_BN - 1) / UM_HEAD_BN * (umma_takes_pairs(M) ? 2 : 1);
 }
 
-template <typename Epi> int stream_row_tiles(const UmmaState& st, int M, int NP, int K, int bn);
-template <int NACC, typename Epi>
-int swap_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
-                int n_rows_w, const Epi& epi, unsigned* status);
+template <typename Epi> bool stream_can(const UmmaState& st, int M, int NP, int K, int bn);
 template <typename Epi>
 int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
                 int n_rows_w, const Epi& epi, unsigned* status);
-template <int BN, int MT, int NI, typename Epi>
+template <int BN, typename Epi>
 int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
                   int n_rows_w, const Epi& epi, unsigned* status);
 
-// Instantiation choice for the streaming kernel: tile width 128 or 256, one or two row tiles, one or two MMA issuers
-// (two row tiles always have two).
-template <typename Epi>
-int stream_dispatch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
-                    int n_rows_w, const Epi& epi, unsigned* status, int bn, int mt, int ni) {
-#define LSP_STREAM_CASE(BN_, MT_, NI_) \
-  if (bn == BN_ && mt == MT_ && ni == NI_) \
-    return stream_launch<BN_, MT_, NI_, Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status)
-  if (mt == 2) ni = 2;
-  LSP_STREAM_CASE(256, 1, 1);
-  LSP_STREAM_CASE(256, 1, 2);
-  LSP_STREAM_CASE(256, 2, 2);
-  if constexpr (Epi::kDual && !std::is_same<Epi, EpiQKVRope<bf16>>::value) {    // 96 pairs per tile: whole tiles only (see umma_gemm)
-    if (bn == 192 && mt == 1) ni = 1;
-    LSP_STREAM_CASE(192, 1, 1);
-    LSP_STREAM_CASE(192, 2, 2);
-  }
-  if constexpr (!Epi::kReduce) {
-    LSP_STREAM_CASE(128, 1, 1);
-    LSP_STREAM_CASE(128, 1, 2);
-    LSP_STREAM_CASE(128, 2, 2);
-  }
-#undef LSP_STREAM_CASE
-  st.err = "no streaming-kernel instantiation for this tile shape";
-  return -7;
-}
-
-// Tile-width choice for the persistent kernel (the K split follows from the tile count, see stream_launch).
-//  * The rotary epilogue needs both partners of a pair inside one head: its half tiles are fetched head by head.
-//  * A shape the kernel cannot take (none of a transformer layer's: it would need more than 4096 column tiles in a
-//    launch whose tiles are split between CTAs) is an error, not a fallback.
+// More than 128 rows: pairs of SMs.  Else the streaming kernel (the K split follows from the tile count, see stream_launch)
+// with this tile width, from measurements on the LLaDA and Dream layer shapes at 2 to 128 rows:
+//  * the head 256;
+//  * dual epilogues 256 columns (128 pairs), or 192 (96 pairs) where that makes one fuller wave: with 12288 pairs 128 tiles
+//    instead of 96, i.e. a third more SMs pulling operands, and a quarter less shared-memory fill per CTA.  Only where no tile
+//    would be split between CTAs (the split paths assume a power-of-two chunk count).  (The same idea for the rotary QKV
+//    GEMM, 96-wide tiles that straddle heads, needs 16-row TMA boxes of 2 KB, and those cost far more than the fuller wave
+//    gains: +0.7 ms per LLaDA-shaped pass.  Not kept.)
+//  * plain and rotary ones 128, which needs no K split with 96 tiles, except that a wide GEMM with at most 32 rows takes 256
+//    (its partial tiles are small, and half as many MMA instructions are issued).  A rotary half tile is whole head halves.
+// A shape the kernel cannot take (none of a transformer layer's: it would need more than 4096 column tiles in a launch whose
+// tiles are split between CTAs) is an error, not a fallback.
 template <typename Epi>
 int umma_gemm(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
               int n_rows_w, const Epi& epi, unsigned* status) {
   if (K % UM_BK) { st.err = "K must be a multiple of 64"; return -6; }
-  if (umma_takes_pairs(st, M)) return pair_launch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
-  if constexpr (Epi::kReduce) {
-    {
-      const int smt = stream_row_tiles<Epi>(st, M, NP, K, UM_HEAD_BN);
-      if (smt > 0)
-        return stream_dispatch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status, UM_HEAD_BN, smt,
-                                    st.stream_issuers);
-    }
-    st.err = "the tcgen05 head GEMM cannot take this shape";
-    return -8;
-  } else {
-    const int cols = Epi::kDual ? 2 * NP : NP;
-    if (M >= st.swap_min_rows && M <= st.swap_max_rows) {
-      // 129..256 rows: the tensor pipe bounds the launch, and with the operands swapped its time follows the row count
-      int rc;
-      if constexpr (std::is_same<Epi, EpiQKVRope<bf16>>::value) rc = swap_launch<2, Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
-      else if constexpr (Epi::kDual) rc = st.swap_force ? swap_launch<2, Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status) : 1;   // gate/up: one K slice only, 96 CTAs of 3 MB intake each: the 192-wide row-major tiles win (measured)
-      else if (cols >= 8192) rc = swap_launch<2, Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
-      else rc = swap_launch<1, Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
-      if (rc <= 0) return rc;          // 1 = not a problem that kernel takes
-    }
-    {
-      // Tile width, from measurements on the LLaDA layer shapes at 2..256 rows: dual epilogues take 256 columns (128
-      // pairs); plain ones take 128, which needs no K split with 96 tiles, except that a wide GEMM with at most 32
-      // rows takes 256 (its partial tiles are small, and half as many MMA instructions are issued).  The rotary
-      // epilogue's half tiles are fetched head by head.
-      // With 129..256 rows (two row tiles per CTA) a wide GEMM again takes 256 columns, its K halves on a cluster of 2
-      // that exchanges half tiles: 256 x 256 tiles need a third less shared-memory fill than 256 x 128 ones (QKV-sized
-      // GEMM 38-40 -> 35-37.5 us); a narrow GEMM (36 tiles of 128) is better off with more, smaller tiles.
-      const bool wide_two_tiles = M > UM_BM && M <= 2 * UM_BM && cols >= 8192 && st.stream_exchange && st.stream_cluster;
-      int sbn = Epi::kDual ? 256 : (((M <= 32 || wide_two_tiles) && cols >= 8192) ? 256 : 128), box_rows = 0;
-      if constexpr (std::is_same<Epi, EpiQKVRope<bf16>>::value) {
-        box_rows = epi.half;
-        sbn = (M <= 32 || wide_two_tiles) ? 256 : 128;
-      }
-      if (M > 2 * UM_BM || (M > UM_BM && st.stream_two_tiles == 2)) sbn = 256;   // several row groups: the widest MMA
-      if (M <= UM_BM && st.stream_bn > 0) sbn = st.stream_bn;
-      if (M > UM_BM && M <= 2 * UM_BM && st.stream_bn2 > 0) sbn = st.stream_bn2;
-      if (box_rows > sbn / 2) sbn = 2 * box_rows;
-      if constexpr (Epi::kDual && !std::is_same<Epi, EpiQKVRope<bf16>>::value) {
-        // 192-wide tiles (96 pairs): with 12288 pairs that is 128 tiles instead of 96, i.e. a third more SMs pulling
-        // operands, and a quarter less shared-memory fill per CTA.  Only where no tile would be split between CTAs
-        // (the split paths assume a power-of-two chunk count): one wave of whole tiles, or several row groups.
-        // (The same idea for the rotary QKV GEMM, 96-wide tiles that straddle heads, needs 16-row TMA boxes of 2 KB,
-        // and those cost far more than the fuller wave gains: +0.7 ms per LLaDA-shaped pass.  Not kept.)
-        if (st.stream_bn_dual != 256 && NP % 96 == 0 && st.stream_grid_mode == 2 && st.target_ctas == 0) {
-          const int mt192 = M <= UM_BM ? 1 : 2;
-          const long groups = (M + UM_BM * mt192 - 1) / (UM_BM * mt192);
-          const long t192 = (long)(NP / 96) * groups, t256 = (long)((NP + 127) / 128) * groups;
-          const bool whole192 = (groups == 1 && t192 <= st.n_sm && 2 * t192 > st.n_sm) || (groups > 1 && t192 >= st.n_sm);
-          const bool better = M <= 2 * UM_BM ? (t256 < t192 && t256 < st.n_sm) : false;
-          if (whole192 && (st.stream_bn_dual == 192 || better)) sbn = 192;
-        }
-      }
-      const int smt = stream_row_tiles<Epi>(st, M, NP, K, sbn);
-      if (smt > 0 && (sbn == 128 || sbn == 256 || sbn == 192))
-        return stream_dispatch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status, sbn, smt,
-                                    st.stream_issuers);
-    }
-    st.err = "the tcgen05 GEMM cannot take this shape";
-    return -8;
+  if (umma_takes_pairs(M)) return pair_launch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
+  constexpr bool kRope = std::is_same<Epi, EpiQKVRope<bf16>>::value;
+  const int cols = Epi::kDual ? 2 * NP : NP;
+  int bn = UM_HEAD_BN;
+  if constexpr (kRope) {
+    bn = M <= 32 ? 256 : 128;
+    if (st.stream_bn > 0) bn = st.stream_bn;
+    if (bn / 2 < epi.half) bn = 2 * epi.half;
+  } else if constexpr (Epi::kDual) {
+    const long t192 = NP / 96, t256 = (NP + 127) / 128;
+    const bool whole192 = NP % 96 == 0 && t192 <= st.n_sm && 2 * t192 > st.n_sm;
+    if (whole192 && st.stream_bn_dual != 256 && !st.stream_even && st.target_ctas == 0 &&
+        (st.stream_bn_dual == 192 || (t256 < t192 && t256 < st.n_sm)))
+      bn = 192;
+    else if (st.stream_bn > 0)
+      bn = st.stream_bn;
+  } else if constexpr (!Epi::kReduce) {
+    bn = (M <= 32 && cols >= 8192) ? 256 : 128;
+    if (st.stream_bn > 0) bn = st.stream_bn;
   }
+  if (stream_can<Epi>(st, M, NP, K, bn)) {
+    if (bn == 256) return stream_launch<256, Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
+    if constexpr (!Epi::kReduce) {
+      if (bn == 128) return stream_launch<128, Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
+    }
+    if constexpr (Epi::kDual && !kRope) {
+      if (bn == 192) return stream_launch<192, Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
+    }
+  }
+  st.err = "the tcgen05 GEMM cannot take this shape";
+  return -8;
 }
 
 }  // namespace lsp

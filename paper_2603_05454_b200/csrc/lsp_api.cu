@@ -20,7 +20,6 @@
 #include "misc_kernels.cuh"
 #ifndef LSP_NO_UMMA
 #include "gemm_stream.cuh"
-#include "gemm_swap.cuh"
 #include "gemm_pair.cuh"
 #include "attention_umma.cuh"
 #endif
@@ -181,7 +180,7 @@ struct Layout {
       gemm_scratch, gemm_counters, stage, total;
 };
 
-constexpr size_t kGemmScratchBytes = 80u << 20;   // split-K partial tiles (the streaming GEMM needs 74 MiB at its widest)
+constexpr size_t kGemmScratchBytes = 40u << 20;   // split-K partial tiles (the streaming GEMM needs 37 MiB at its widest)
 constexpr int kGemmCounters = 4096;               // split-K arrival counters
 
 int head_tiles_max(const lsp_model_cfg* m) { return std::max(2, (m->vocab + 63) / 64); }
@@ -271,7 +270,7 @@ int run_head(lsp_ctx* c, const T* hidden, int rows, int* n_tiles_out) {
   epi.exclude_id = c->s.exclude_mask_logit ? m.mask_id : -1;
   int n_tiles = (m.vocab + SG_HEAD_BN - 1) / SG_HEAD_BN;
 #ifndef LSP_NO_UMMA
-  if (std::is_same<T, bf16>::value && c->gemm_impl == 1) n_tiles = umma_head_tiles(c->umma, rows, m.vocab);
+  if (std::is_same<T, bf16>::value && c->gemm_impl == 1) n_tiles = umma_head_tiles(rows, m.vocab);
 #endif
   epi.n_tiles = n_tiles;
   *n_tiles_out = n_tiles;
@@ -818,10 +817,6 @@ int lsp_debug_set(lsp_ctx* c, int key, int value) {
   if (!c) return LSP_ERR_ARG;
   if (key == 28) c->attn_umma_min_rows = value;
   else if (key == 31) c->lag_tail = value < 1 ? 1 : value;
-  else if (key == 36) c->umma.swap_min_rows = value;
-  else if (key == 37) c->umma.swap_max_rows = value;
-  else if (key == 38) c->umma.swap_force = value ? 1 : 0;
-  else if (key == 39) c->umma.stream_half_tile1 = value ? 1 : 0;
   else if (key == 30) c->attn_cluster = value ? 1 : 0;
   else if (key == 3) c->async_ops = value;
   else if (key == 4) c->op_repeat = value < 1 ? 1 : value;
@@ -830,27 +825,21 @@ int lsp_debug_set(lsp_ctx* c, int key, int value) {
   else if (key == 10) c->umma.target_ctas = value;
   else if (key == 11) c->umma.max_stages = value < 1 ? 1 : (value > UM_MAX_STAGES ? UM_MAX_STAGES : value);
   else if (key == 25) { c->pdl = value ? 1 : 0; c->umma.pdl = c->pdl; }
-  else if (key == 17) c->umma.stream_grid_mode = value;
-  else if (key == 18) c->umma.stream_even_max_rows = value;
-  else if (key == 19) c->umma.stream_two_tiles = value == 2 ? 2 : 1;
-  else if (key == 27) c->umma.stream_half_sm = value ? 1 : 0;
+  else if (key == 17) c->umma.stream_even = value == 1 ? 1 : 0;
   else if (key == 29) c->umma.stream_cluster = value ? 1 : 0;
   else if (key == 32) c->umma.stream_bn_dual = (value == 192 || value == 256) ? value : 0;
   else if (key == 33) c->umma.stream_exchange = value ? 1 : 0;
-  else if (key == 26) c->umma.stream_issuers = value == 1 ? 1 : 2;
-  else if (key == 24) c->umma.stream_big_mt = (value == 1 || value == 2) ? value : 3;
-  else if (key == 20) c->umma.stream_bn2 = (value == 256 || value == 128) ? value : 0;
   else if (key == 23) c->umma.stream_bn = (value == 256 || value == 128) ? value : 0;
-  else if (key == 40) c->umma.pair_min_rows = value;
   else if (key == 41) c->umma.pair_bn = (value >= 96 && value <= 256 && value % 32 == 0) ? value : 0;
   else if (key == 46) c->umma.pair_split = (value >= 0 && value <= 3) ? value : 0;
-  else if (key == 45) c->umma.pair_min_rows = value ? 129 : 257;
   else if (key == 42) c->umma.pair_band = value < 0 ? 0 : value;
   else if (key == 43) c->umma.stream_split_copies = value ? 1 : 0;
   else if (key == 44) c->umma.stream_exchange_rows = value;
   else if (key == 21) c->umma.stream_atoms = value;
   else if (key == 22) c->umma.stream_min_stages2 = value < 2 ? 2 : value;
 #endif
+  // knobs of kernel variants that are gone (two row tiles per CTA, swapped operands, two issuers, half an SM): accepted, without effect
+  else if (key == 18 || key == 19 || key == 20 || key == 24 || key == 26 || key == 27 || (key >= 36 && key <= 40) || key == 45) {}
   else return fail(c, LSP_ERR_ARG, "lsp_debug_set: unknown key %d", key);
   return LSP_OK;
 }
@@ -1369,7 +1358,7 @@ int lsp_linear_static(const void* A, const void* W, void* out, int M, int N, int
     if (rc == cudaSuccess) rc = cudaDeviceGetAttribute(&sd.max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (rc == cudaSuccess) rc = cudaDeviceGetAttribute(&sd.n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (rc == cudaSuccess)
-      rc = cudaFuncSetAttribute(k_gemm_stream<kStaticBN, 1, 2, EpiStore<bf16>>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      rc = cudaFuncSetAttribute(k_gemm_stream<kStaticBN, EpiStore<bf16>>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 sd.max_smem);
     sd.setup_rc = rc;
   });
@@ -1380,7 +1369,7 @@ int lsp_linear_static(const void* A, const void* W, void* out, int M, int N, int
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   // stage shape: as many two-atom stages as fit, else one-atom stages
   const int a_rows = (M + 7) / 8 * 8;
-  const int aux = 1024 + UM_BM * 128 + 8 * (2 * ST_MAX_STAGES + 4) + 16;
+  const int aux = 1024 + 8 * (2 * ST_MAX_STAGES + 4) + 16;
   const int atom = a_rows * 128 + kStaticBN * 128;
   const int atoms = (K % 128 == 0 && (sd.max_smem - aux) / (2 * atom) >= 3) ? 2 : 1;
   int stages = (sd.max_smem - aux) / (atoms * atom);
@@ -1407,9 +1396,9 @@ int lsp_linear_static(const void* A, const void* W, void* out, int M, int N, int
     static_msg(err, err_len, "lsp_linear_static: clearing the counters failed (%s)", cudaGetErrorString(e));
     return LSP_ERR_CUDA;
   }
-  StreamArgs args{M, N, n_tiles, 1, 0, 0, 1, kc, a_rows, atoms, 1, 0, stages, 0, partials, counters, status};
+  StreamArgs args{M, N, n_tiles, 0, 0, kc, a_rows, atoms, 1, 0, stages, partials, counters, status};
   EpiStore<bf16> epi{(bf16*)out, N};
-  k_gemm_stream<kStaticBN, 1, 2, EpiStore<bf16>><<<grid, ST_THREADS, smem, stream>>>(ma, mb, mb, args, epi);
+  k_gemm_stream<kStaticBN, EpiStore<bf16>><<<grid, ST_THREADS, smem, stream>>>(ma, mb, mb, args, epi);
   e = cudaGetLastError();
   if (e != cudaSuccess) {
     static_msg(err, err_len, "lsp_linear_static: launch failed (%s)", cudaGetErrorString(e));

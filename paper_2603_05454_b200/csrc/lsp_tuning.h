@@ -19,35 +19,28 @@ extern "C" {
  *   4  lsp_op_linear enqueues the operation this many times
  *   5  repetition r reads its weights at W + (r mod value) * N * K elements, so a buffer of several weight copies keeps
  *      the L2 cold
- * tcgen05 GEMM (the persistent kernel k_gemm_stream):
+ * tcgen05 GEMM, up to 128 rows (the persistent kernel k_gemm_stream):
  *   10 CTAs a launch whose tiles are split is dealt to (0 = by the tile count)          11 maximum pipeline stages
- *   17 grid of the persistent kernel (0 by row count, 1 one CTA per SM with even shares, 2 a multiple of the tile count)
- *   18 row count up to which mode 0 takes even shares
- *   19 129..256 rows: 1 = two row tiles per CTA (default), 2 = two row groups
- *   20 its tile width for those (0 = automatic, 128, 256)
+ *   17 its grid (1: one CTA per SM with even shares; else, the default, a multiple of the tile count)
  *   21 64-element K atoms per pipeline stage (0 = automatic, 1, 2)   22 fewest two-atom stages the automatic choice accepts
- *   23 its tile width for up to 128 rows (0 = automatic, 128, 256)
- *   24 row tiles per CTA above 256 rows (1, 2, 3 = automatic, default)
+ *   23 its tile width (0 = automatic, 128, 256)
  *   25 launch the step's kernels with programmatic dependent launch (1, default) or plainly (0)
- *   26 MMA-issuing warps of the persistent kernel with one row tile per CTA (1, default, or 2)
- *   27 the persistent kernel caps its shared memory at half an SM when three stages still fit (1, default)
  *   29 the K slices of a split tile run as one thread block cluster, reduced through distributed shared memory (1,
  *      default), or through global scratch by the last CTA to arrive (0)
  *   32 tile width of the dual (SwiGLU) GEMM: 0 = automatic (default), 192 or 256
  *   43 a SwiGLU tile's weights come by one copy per half and K atom even where one copy can bring them all (0, default)
  *   33 a cluster of 2 exchanges half tiles (1, default) or publishes whole partial tiles like larger clusters (0)
- * GEMM on pairs of SMs:
- *   40 fewest rows that take it (default 257)   41 its tile width (0 = automatic, 96 ... 256 in steps of 32)
- *   42 most row groups of 256 per band (0 = automatic)   45 with 129..256 rows where it pays (1, default) or not
+ *   44 ... from this many rows on (default 64)
+ * GEMM on pairs of SMs, more than 128 rows (k_gemm_pair):
+ *   41 its tile width (0 = automatic, 96 ... 256 in steps of 32)   42 most row groups of 256 per band (0 = automatic)
+ *   46 its K slices (0 = automatic, 1 = never split, 2 or 3 where they fit)
  * tcgen05 attention:
  *   28 fewest (query row x group head) rows of a (sequence, KV head) for which the tcgen05 kernel is used (default 0)
  *   30 it splits a row tile's keys over a thread block cluster when there are few CTAs (1, default)
- *   39 with 129..192 rows on two row tiles and unsplit tiles, the second row tile's MMAs span 64 rows (1, default)
- *   36, 37 fewest and most activation rows of a GEMM that takes the operand-swapped kernel (defaults 129 and 256;
- *      37 = 0: never)        38 take it whenever it can run (1), not only where it was measured to pay (0, default)
  * decode loop:
  *   31 with device-resident block lengths (lsp_set_option key 4), lsp_generate reads every step before sizing the next
  *      once at most this many masked positions per sequence remain (default 8)
+ * Accepted without effect (they tuned kernel variants that no longer exist): 18, 19, 20, 24, 26, 27, 36 to 40, 45.
  * Unknown key: LSP_ERR_ARG. */
 int lsp_debug_set(lsp_ctx* ctx, int key, int value);
 

@@ -390,23 +390,21 @@ def test_linear_cuda_core_kernels(dtype, M, N, K):
 @pytest.mark.parametrize("M", [129, 187, 256])
 @pytest.mark.parametrize("N,K", [(4096, 4096), (1152, 512), (4608, 3584), (7168, 5120), (4096, 12288), (16, 64)])
 def test_linear_bf16_one_row_group_on_pairs(M, N, K):
-    """129 to 256 rows on both sides of the rule that sends them to the pairs of SMs or to the kernels that split K."""
-    for one_group in (1, 0):
-        dec = _dec("bf16")
-        dec.debug_set(45, one_group)
-        A = S.normal((M, K), 14, 1, 1.0, torch.bfloat16, DEV)
-        W = S.normal((N, K), 14, 2, 0.05, torch.bfloat16, DEV)
-        W2 = S.normal((N, K), 14, 3, 0.05, torch.bfloat16, DEV)
-        X0 = S.normal((M, N), 14, 4, 1.0, torch.bfloat16, DEV)
-        ref, up = A.double() @ W.double().t(), A.double() @ W2.double().t()
-        near = lambda got, want, ulps=1: bool(((got.double() - want).abs() <= ulps / 128 * want.abs() + want.abs().max() / 2560).all())
-        x = X0.clone()
-        dec.op_linear(1, A, W, None, x)
-        assert near(x, X0.double() + ref)
-        out = torch.empty(M, N, dtype=torch.bfloat16, device=DEV)
-        dec.op_linear(2, A, W, W2, out)
-        assert near(out, torch.nn.functional.silu(ref) * up, 2)
-        dec.close()
+    """129 to 256 rows on the pairs of SMs: one row group, tiles narrower than a box, ragged K, K slices or none."""
+    dec = _dec("bf16")
+    A = S.normal((M, K), 14, 1, 1.0, torch.bfloat16, DEV)
+    W = S.normal((N, K), 14, 2, 0.05, torch.bfloat16, DEV)
+    W2 = S.normal((N, K), 14, 3, 0.05, torch.bfloat16, DEV)
+    X0 = S.normal((M, N), 14, 4, 1.0, torch.bfloat16, DEV)
+    ref, up = A.double() @ W.double().t(), A.double() @ W2.double().t()
+    near = lambda got, want, ulps=1: bool(((got.double() - want).abs() <= ulps / 128 * want.abs() + want.abs().max() / 2560).all())
+    x = X0.clone()
+    dec.op_linear(1, A, W, None, x)
+    assert near(x, X0.double() + ref)
+    out = torch.empty(M, N, dtype=torch.bfloat16, device=DEV)
+    dec.op_linear(2, A, W, W2, out)
+    assert near(out, torch.nn.functional.silu(ref) * up, 2)
+    dec.close()
 
 
 @pytest.mark.parametrize("M,N,K", [(1, 512, 64), (64, 1024, 512), (128, 272, 448), (33, 4096, 512), (100, 1024, 576)])
