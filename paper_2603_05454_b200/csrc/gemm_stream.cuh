@@ -84,6 +84,11 @@ __device__ __forceinline__ int st_first_unit(int U, int G, int g) { return (int)
 __device__ __forceinline__ int st_owner(int U, int G, int u) { return (int)(((unsigned)(u + 1) * (unsigned)G + (unsigned)U - 1u) / (unsigned)U) - 1; }
 
 constexpr int ST_THREADS = 192;
+// Every CTA reads the same activations.  Were all to walk K from its start, the whole chip would ask for the same few lines of L2
+// at a time; so column tile t starts t * ST_ROT chunks later (and wraps): a LLaDA-shaped pass of 101 rows 4.25 -> 4.16 ms, of 9
+// rows 3.72 -> 3.68 (1 to 19 chunks: 4.15 to 4.23, 3.68 to 3.70).  The order depends on the tile alone, so the CTAs that share a
+// tile still cover it, and results do not depend on timing.
+constexpr int ST_ROT = 4;
 
 template <int BN, typename Epi>
 __global__ void __launch_bounds__(ST_THREADS, 1)
@@ -127,32 +132,35 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
   int cl_tile = 0;                   // cluster mode: the tile this CTA contributed a K slice to
 
   // Position of the producer in the unit space, advanced without divisions (its loop has to keep ahead of the tensor pipe).
+  // A tile takes its K chunks in rotated order, starting at chunk rot (see ST_ROT).
   struct Pos {
-    int tile, c;
+    int tile, c, rot;
   };
+  auto chunk = [&](const Pos& p) { return p.c + p.rot < args.kc ? p.c + p.rot : p.c + p.rot - args.kc; };
   auto pos_set = [&](Pos& p, int u) {
     p.tile = u / args.kc;
     p.c = u % args.kc;
+    p.rot = p.tile * ST_ROT % args.kc;
   };
   auto pos_next = [&](Pos& p) {
-    if (++p.c == args.kc) { p.c = 0; ++p.tile; }
+    if (++p.c == args.kc) { p.c = 0; ++p.tile; p.rot = p.tile * ST_ROT % args.kc; }
   };
   // the weight tile of one stage: both halves of every K atom (see umma_map5)
   auto load_weights = [&](const Pos& p, int s) {
     const uint32_t sb = smem_u32(smem + (size_t)s * STAGE_BYTES) + AT * A_ATOM;
     const int j = p.tile * (Epi::kDual ? HALF : BN);
-    const int r0 = args.half ? 0 : j, blk = args.half ? j / args.half : 0;
+    const int r0 = args.half ? 0 : j, blk = args.half ? j / args.half : 0, a0 = chunk(p) * AT;
     if (args.one_copy) {
-      tma_load_5d(sb, &map_b0, r0, blk, 0, p.c * AT, full_bar(s));
+      tma_load_5d(sb, &map_b0, r0, blk, 0, a0, full_bar(s));
     } else {
       for (int a = 0; a < AT; ++a) {
-        tma_load_5d(sb + a * B_ATOM, &map_b0, r0, blk, 0, p.c * AT + a, full_bar(s));
-        tma_load_5d(sb + a * B_ATOM + B_HALF_ATOM, &map_b1, r0, blk, 0, p.c * AT + a, full_bar(s));
+        tma_load_5d(sb + a * B_ATOM, &map_b0, r0, blk, 0, a0 + a, full_bar(s));
+        tma_load_5d(sb + a * B_ATOM + B_HALF_ATOM, &map_b1, r0, blk, 0, a0 + a, full_bar(s));
       }
     }
   };
   auto load_acts = [&](const Pos& p, int s) {
-    tma_load_4d(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_a, 0, 0, p.c * AT, full_bar(s));
+    tma_load_4d(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_a, 0, 0, chunk(p) * AT, full_bar(s));
   };
 
   const int n_pre = n_units < S ? n_units : S;      // stages whose weights are requested before the predecessor is done
