@@ -12,8 +12,9 @@
 //     thread issuing (a lane branch around tcgen05.mma costs about 130 cycles per instruction, elect.sync 48 to 88).  With
 //     one atom per stage and a copy per box the same kernel ran 4096 x 4096 outputs (K 4096) in 104 us, so 98, and
 //     512 x 4096 in 25.3, so 17.8.
-//   * Persistent: pair p takes tiles p, p + P, ...; the accumulators are double-buffered (2 x BN of 512 columns), so the
+//   * Persistent: pair p takes every P-th tile (odd rounds in reverse order); the accumulators are double-buffered (2 x BN of 512 columns), so the
 //     epilogue of a tile overlaps the next tile's MMAs.
+//   * A last row group of at most 128 rows runs on 128-row MMAs (see pair_half_last).
 //   * BN is a run-time multiple of 32 (64 for the rotary epilogue), chosen so that the last wave of tiles is full (see
 //     pair_shape).
 //   * The weight tile's two halves come from the two tensors / row ranges whose columns a fused epilogue pairs (gate and
@@ -48,6 +49,7 @@ struct PairArgs {
   int ks;           // K slices of a tile (plain epilogues, one tile per cluster): pair s of the cluster takes the s-th share of
                     // the chunks, and the partial tiles are summed through distributed shared memory
   int bn;           // tile width
+  int half_last;    // the last row group has at most 128 rows and runs with 128-row MMAs (64 rows per CTA)
   int unit;         // rotary epilogue: weight rows per copy when a half tile is not made of whole head halves (else 0)
   int stages;
   unsigned* status;
@@ -83,7 +85,8 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
 template <typename Epi>
 __global__ void __launch_bounds__(PR_THREADS, 1)
 k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b0,
-            const __grid_constant__ CUtensorMap map_b1, PairArgs args, Epi epi) {
+            const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ CUtensorMap map_ah,
+            const __grid_constant__ CUtensorMap map_h0, const __grid_constant__ CUtensorMap map_h1, PairArgs args, Epi epi) {
   extern __shared__ uint8_t smem_raw[];
   pdl_release();
   constexpr int A_ATOM = UM_BM * 128;                     // this CTA's 128 activation rows of one K atom
@@ -112,12 +115,14 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   const uint16_t pair_mask = (uint16_t)(3u << lead);
   const int P = gridDim.x / (unsigned)(2 * ks), pair = blockIdx.x / (unsigned)(2 * ks);
   const int T = args.n_tiles * args.row_groups;
-  const int my_tiles = (T - pair + P - 1) / P;            // the host launches at most T pairs
+  // tiles are dealt in rounds, odd rounds in reverse, so that with an even number of row groups a pair gets some of each
+  const int rest = T % P;
+  const int my_tiles = T / P + ((((T / P) & 1) ? P - 1 - pair : pair) < rest ? 1 : 0);      // the host launches at most T pairs
   const int kc0 = args.kc * slice / ks, kc = args.kc * (slice + 1) / ks - kc0;      // this pair's chunks
   const int n_units = my_tiles * kc;
   // i-th tile of this pair -> column tile and row group
   auto tile_of = [&](int i, int& tile, int& rg) {
-    const int t = pair + i * P;
+    const int t = i * P + ((i & 1) ? P - 1 - pair : pair);
     const int per_band = args.band * args.n_tiles;
     const int b = t / per_band, r = t - b * per_band;
     const int rows = min(args.band, args.row_groups - b * args.band);
@@ -125,8 +130,10 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     rg = b * args.band + r % rows;
   };
   const uint32_t full0 = cluster_map(bar_base, lead);     // the first CTA's full barriers, in the cluster's window
+  constexpr bool kHalf = !kRope && !Epi::kReduce;
+  auto half_rows = [&](int rg) { return kHalf && args.half_last && rg == args.row_groups - 1; };
   const CUtensorMap* map_b = rank ? &map_b1 : &map_b0;    // this CTA's half of the weight tile
-  auto load_weights = [&](int tile, int c, int s) {
+  auto load_weights = [&](int tile, int rg, int c, int s) {
     const uint32_t sb = smem_u32(smem + (size_t)s * STAGE_BYTES) + 2 * A_ATOM;
     if constexpr (kRope) {
       // blocks of the map are head halves; a half tile is HALF consecutive pair indices
@@ -137,6 +144,14 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         for (int b = 0; b < HALF; b += args.unit)
           for (int a = 0; a < 2; ++a)
             tma_load_4d_pair(sb + a * B_ATOM + b * 128, map_b, (j + b) % epi.half, (j + b) / epi.half, 2 * c + a, full0 + 8u * s);
+      }
+    } else if (Epi::kDual && half_rows(rg)) {
+      // the MMA leaves columns [0, HALF) in lanes 0 .. 63 and [HALF, BN) in lanes 64 .. 127: this CTA's half of the weight tile
+      // is then the rank-th half of the tile's gate rows and the same of its up rows, so that a pair stays in one lane
+      const int j = tile * HALF + rank * (HALF / 2);
+      for (int a = 0; a < 2; ++a) {
+        tma_load_4d_pair(sb + a * B_ATOM, &map_h0, j, 0, 2 * c + a, full0 + 8u * s);
+        tma_load_4d_pair(sb + a * B_ATOM + B_ATOM / 2, &map_h1, j, 0, 2 * c + a, full0 + 8u * s);
       }
     } else {
       tma_load_4d_pair(sb, map_b, Epi::kDual ? tile * HALF : tile * BN + rank * HALF, 0, 2 * (kc0 + c), full0 + 8u * s);
@@ -178,8 +193,8 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       int t2 = tile, rg2 = rg, c2 = 0, i2 = 0;
       for (int it = 0; it < n_pre; ++it) {
         if (elect_one()) {
-          if (rank == 0) mbar_expect_tx(full_bar(it), 2 * STAGE_BYTES);
-          load_weights(t2, c2, it);
+          if (rank == 0) mbar_expect_tx(full_bar(it), half_rows(rg2) ? 2 * STAGE_BYTES - 2 * A_ATOM : 2 * STAGE_BYTES);
+          load_weights(t2, rg2, c2, it);
         }
         __syncwarp();
         if (++c2 == kc) { c2 = 0; if (++i2 < my_tiles) tile_of(i2, t2, rg2); }
@@ -199,10 +214,13 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       }
       if (elect_one()) {
         if (it >= n_pre) {
-          if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE_BYTES);
-          load_weights(tile, c, s);
+          if (rank == 0) mbar_expect_tx(full_bar(s), half_rows(rg) ? 2 * STAGE_BYTES - 2 * A_ATOM : 2 * STAGE_BYTES);
+          load_weights(tile, rg, c, s);
         }
-        tma_load_4d_pair(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_a, rg * PR_ROWS + rank * UM_BM, 0, 2 * (kc0 + c), full0 + 8u * s);
+        if (half_rows(rg))
+          tma_load_4d_pair(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_ah, rg * PR_ROWS + rank * 64, 0, 2 * (kc0 + c), full0 + 8u * s);
+        else
+          tma_load_4d_pair(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_a, rg * PR_ROWS + rank * UM_BM, 0, 2 * (kc0 + c), full0 + 8u * s);
       }
       __syncwarp();
       ++issued;
@@ -222,12 +240,16 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   } else if (warp == 1) {
     // ---------------- MMA issuer (first CTA; the whole warp waits, one elected thread issues) ----------------
     if (rank == 0) {
-      const uint32_t idesc = (make_idesc(BN) & ~(31u << 24)) | ((uint32_t)(PR_ROWS >> 4) << 24);
       int s = 0;
       uint32_t ph = 0;
       bool ok = true;
       for (int i = 0; i < my_tiles && ok; ++i) {
         const int buf = i & 1, use = i >> 1;
+        int tile, rg;
+        tile_of(i, tile, rg);
+        const bool half = half_rows(rg);
+        const uint32_t idesc = (make_idesc(BN) & ~(31u << 24)) | ((uint32_t)((half ? PR_ROWS / 2 : PR_ROWS) >> 4) << 24);
+        const uint32_t a_atom = half ? A_ATOM / 2 : A_ATOM;
         if (use >= 1) ok = mbar_wait(acce_bar(buf), (uint32_t)(use - 1) & 1u, abort_flag);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) {
@@ -248,7 +270,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           if (elect_one()) {
 #pragma unroll
             for (int a = 0; a < 2; ++a) {
-              const uint64_t da = make_smem_desc(sa + a * A_ATOM), db = make_smem_desc(sa + 2 * A_ATOM + a * B_ATOM);
+              const uint64_t da = make_smem_desc(sa + a * a_atom), db = make_smem_desc(sa + 2 * A_ATOM + a * B_ATOM);
 #pragma unroll
               for (int k = 0; k < 4; ++k)
                 tc_mma_f16_pair(d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (c | a | k) != 0 ? 1u : 0u);
@@ -268,15 +290,17 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     const int h = (warp - 2) >> 2;                                // column half
     const int r_in = q * 32 + lane;
     const int CH = Epi::kDual ? HALF : BN;                        // pair indices (dual) or columns (plain) per tile
-    const int nch = CH >> 4, mid = (nch + 1) >> 1;
-    const int ch_lo = h ? mid : 0, ch_hi = h ? nch : mid;
     const uint32_t acce0 = cluster_map(acce_bar(0), lead);
     for (int i = 0; i < my_tiles && ks == 1; ++i) {
       const int buf = i & 1, use = i >> 1;
       int tile, rg;
       tile_of(i, tile, rg);
-      const int m = rg * PR_ROWS + rank * UM_BM + r_in;
-      const int j0 = tile * CH;
+      const bool half = half_rows(rg);                            // 64 rows per CTA, lanes 64 .. 127: the second half of the columns
+      const int m = half ? rg * PR_ROWS + rank * 64 + (r_in & 63) : rg * PR_ROWS + rank * UM_BM + r_in;
+      const int j0 = tile * CH + (half && q >= 2 ? CH / 2 : 0);
+      const int nch = half ? CH >> 5 : CH >> 4, mid = (nch + 1) >> 1;
+      const int ch_lo = h ? mid : 0, ch_hi = h ? nch : mid;
+      const uint32_t up = (uint32_t)(half ? HALF / 2 : HALF);     // dual: the second accumulator's first column
       const bool live = m < args.M;
       uint4 xr[16];
       if constexpr (std::is_same<Epi, EpiResidual<bf16>>::value) {
@@ -324,7 +348,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         };
         auto request = [&](int ch, float (&a0)[16], float (&a1)[16]) {
           tc_ld16_nowait(t_row + (uint32_t)(ch * 16), a0);
-          if (Epi::kDual) tc_ld16_nowait(t_row + (uint32_t)(HALF + ch * 16), a1);
+          if (Epi::kDual) tc_ld16_nowait(t_row + up + (uint32_t)(ch * 16), a1);
         };
         if constexpr (kRope) {
           // (the rotary table's entries one chunk ahead take the registers a second set of accumulator values would)
@@ -469,7 +493,17 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 // step: widths are multiples of 32, or 64 for the rotary epilogue (a half tile is then made of whole 32-row boxes inside one
 // head half).
 struct PairShape { int bn, ks; };
-inline PairShape pair_shape(const UmmaState& st, int M, int cols, int K, int step, bool may_split) {
+// A last row group of at most 128 rows runs with 128-row MMAs (64 rows per CTA, which leave the tile's column halves in the two
+// halves of the lanes): 24 KB instead of 32 per SM and K atom at 256 columns and half the tensor work, about 0.75 of a tile's
+// time.
+// 1032 rows, 2 x 18944 x 3584: 222.5 -> 213.3 us; 3584 x 18944: 116.5 -> 114.5; 300 rows, 4096 x 12288: 43.4 -> 41.5, 4096 x 4096: 17.3
+// -> 16.5, 2 x 12288 x 4096 (now 256 columns wide): 74.8 -> 70.0.  The epilogues whose columns cannot be halved that way (rotary
+// pairs inside a head, the head's partials per tile half) and widths that are no multiple of 64 keep 256-row MMAs.
+inline bool pair_half_last(int M, int bn) {
+  const int last = M % PR_ROWS;
+  return M > PR_ROWS && last >= 1 && last <= PR_ROWS / 2 && bn % 64 == 0;
+}
+inline PairShape pair_shape(const UmmaState& st, int M, int cols, int K, int step, bool may_split, bool may_halve) {
   const int pairs = st.max_clusters[2];
   const long rg = (M + PR_ROWS - 1) / PR_ROWS;
   const double chunks = (K + 127) / 128;
@@ -478,7 +512,8 @@ inline PairShape pair_shape(const UmmaState& st, int M, int cols, int K, int ste
   for (int bn = 256; bn >= 96; bn -= step) {
     const long t = (long)((cols + bn - 1) / bn) * rg;
     const long rounds = (t + pairs - 1) / pairs;
-    const double cost = chunks * (rounds > 2 ? rounds * (bn + 44) * 1.8 : rounds * (bn + 256)) * 1.06e-3;
+    const double share = (may_halve && pair_half_last(M, bn)) ? (rg - 0.25) / rg : 1.0;     // of a full tile's time
+    const double cost = share * chunks * (rounds > 2 ? rounds * (bn + 44) * 1.8 : rounds * (bn + 256)) * 1.06e-3;
     if (cost < best_cost - 1e-9) { best_cost = cost; best = {bn, 1}; }
     for (int ks = 2; ks <= 3 && may_split; ++ks) {
       if (t * ks > pairs || t > st.max_clusters[2 * ks] || chunks < 8 * ks) continue;
@@ -496,7 +531,7 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
   const int cols = Epi::kDual ? 2 * NP : NP;
   const int pairs = st.max_clusters[2];
   constexpr bool kPlain = !Epi::kDual && !Epi::kReduce;
-  PairShape shape = Epi::kReduce ? PairShape{UM_HEAD_BN, 1} : pair_shape(st, M, cols, K, kRope ? 64 : 32, kPlain && st.pair_split != 1);
+  PairShape shape = Epi::kReduce ? PairShape{UM_HEAD_BN, 1} : pair_shape(st, M, cols, K, kRope ? 64 : 32, kPlain && st.pair_split != 1, !kRope && !Epi::kReduce);
   if (st.pair_bn > 0 && !Epi::kReduce) shape = {st.pair_bn, 1};
   const int bn = shape.bn;
   int unit = 0;
@@ -516,7 +551,8 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
     if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -3; }
     attr_set = true;
   }
-  CUtensorMap ma, mb0, mb1;
+  CUtensorMap ma, mb0, mb1, mah, mh0, mh1;               // ..h: operands of a half row group
+  const int half_last = (!kRope && !Epi::kReduce && shape.ks == 1 && st.pair_split <= 1 && pair_half_last(M, bn)) ? 1 : 0;
   {
     const CUtensorMap* p = umma_map4(st, A, M, M, 1, K, UM_BM, 1, 2);
     if (!p) return -4;
@@ -535,6 +571,22 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
     }
     if (!p) return -4;
     mb1 = *p;
+    mah = ma;
+    mh0 = mb0;
+    mh1 = mb1;
+    if (half_last) {
+      p = umma_map4(st, A, M, M, 1, K, UM_BM / 2, 1, 2);
+      if (!p) return -4;
+      mah = *p;
+      if (Epi::kDual) {
+        p = umma_map4(st, W0, n_rows_w, n_rows_w, 1, K, bn / 4, 1, 1);
+        if (!p) return -4;
+        mh0 = *p;
+        p = umma_map4(st, W1, n_rows_w, n_rows_w, 1, K, bn / 4, 1, 1);
+        if (!p) return -4;
+        mh1 = *p;
+      }
+    }
   }
   const int per_tile = Epi::kDual ? bn / 2 : bn;
   const int n_tiles = (NP + per_tile - 1) / per_tile;
@@ -552,8 +604,8 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
   if (kPlain && st.pair_split > 1 && T * st.pair_split <= pairs && T <= st.max_clusters[2 * st.pair_split] && (K + 127) / 128 >= st.pair_split)
     ks = st.pair_split;
   const int grid = 2 * ks * (int)(T < pairs ? T : pairs);
-  PairArgs args{M, NP, n_tiles, rg, band, (K + 2 * UM_BK - 1) / (2 * UM_BK), ks, bn, unit, stages, status};
-  cudaError_t e = launch_k(st.pdl, k_gemm_pair<Epi>, dim3(grid), dim3(PR_THREADS), smem, stream, 2 * ks, ma, mb0, mb1, args, epi);
+  PairArgs args{M, NP, n_tiles, rg, band, (K + 2 * UM_BK - 1) / (2 * UM_BK), ks, bn, half_last, unit, stages, status};
+  cudaError_t e = launch_k(st.pdl, k_gemm_pair<Epi>, dim3(grid), dim3(PR_THREADS), smem, stream, 2 * ks, ma, mb0, mb1, mah, mh0, mh1, args, epi);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -5; }
   return 0;

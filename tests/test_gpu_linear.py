@@ -444,3 +444,26 @@ def test_linear_bf16_k_slices_on_pairs(M, N, K, ks):
     dec.op_linear(0, A, W, None, out[:M])
     assert near(out[:M], ref) and bool((out[M] == 7.0).all())
     dec.close()
+
+
+@pytest.mark.parametrize("M", [257, 320, 384, 385, 1032])
+@pytest.mark.parametrize("N,K,bn", [(272, 192, 0), (1040, 4032, 64), (4096, 576, 128), (1536, 512, 192), (3584, 4096, 256), (1024, 512, 224)])
+def test_linear_bf16_half_row_group_on_pairs(M, N, K, bn):
+    """A last row group of at most 128 rows (the fourth row count and the last width are beyond the line) on 128-row MMAs: ragged
+    last column tiles and K chunks, rows of one CTA of the pair only; against the fp64 product."""
+    dec = _dec("bf16")
+    dec.debug_set(46, 1)
+    dec.debug_set(41, bn)
+    A = S.normal((M, K), 19, 1, 1.0, torch.bfloat16, DEV)
+    W = S.normal((N, K), 19, 2, 0.05, torch.bfloat16, DEV)
+    W2 = S.normal((N, K), 19, 3, 0.05, torch.bfloat16, DEV)
+    X0 = S.normal((M, N), 19, 4, 1.0, torch.bfloat16, DEV)
+    ref, up = A.double() @ W.double().t(), A.double() @ W2.double().t()
+    for op, want, ulps in ((0, ref, 1), (1, X0.double() + ref, 1), (2, torch.nn.functional.silu(ref) * up, 2)):
+        out = torch.full((M + 1, N), 7.0, dtype=torch.bfloat16, device=DEV)
+        out[:M] = X0
+        dec.op_linear(op, A, W, W2 if op == 2 else None, out[:M])
+        # one bf16 rounding per stored value (two ulps with the 2-ulp division) and the fp32 sums' absolute error
+        assert bool(((out[:M].double() - want).abs() <= ulps / 128 * want.abs() + want.abs().max() / 2560).all())
+        assert bool((out[M] == 7.0).all())
+    dec.close()
