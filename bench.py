@@ -60,9 +60,9 @@ NCU_TRAFFIC = {
     # k_gemm_stream<256,EpiHead>, 64 rows: profiles/k_gemm_stream_head_M64_V126464.md
     "head": {"captured_bytes": 1062.8e6, "algorithmic_bytes": 1037.0e6, "src": "34127c2c8b24"},
     # k_attn_umma, 16 x (128 query rows over 2048 keys): profiles/k_attn_umma_B16_F1920.md
-    "attn": {"captured_bytes": 569.2e6, "algorithmic_bytes": 570.4e6, "src": "196044e4044b"},
+    "attn": {"captured_bytes": 571.1e6, "algorithmic_bytes": 570.4e6, "src": "37f095fbf04d"},
     # k_commit_append of a 16 x 1920-row prompt block: profiles/k_commit_append_prompt_B16_P1920.md
-    "commit": {"captured_bytes": 1968.9e6, "algorithmic_bytes": 2013.3e6, "src": "10338810cc4a"},
+    "commit": {"captured_bytes": 1967.9e6, "algorithmic_bytes": 2013.3e6, "src": "c5793f4afff8"},
 }
 
 
