@@ -31,6 +31,8 @@
 // warps 2..9 = epilogue.  Every wait is bounded; on expiry the kernel records (code, site) in the status word, drains and
 // returns.
 #pragma once
+#include <algorithm>
+
 #include "gemm_stream.cuh"
 
 namespace lsp {
@@ -49,6 +51,7 @@ struct PairArgs {
   int ks;           // K slices of a tile (plain epilogues, one tile per cluster): pair s of the cluster takes the s-th share of
                     // the chunks, and the partial tiles are summed through distributed shared memory
   int bn;           // tile width
+  int chains;       // head with one tile per pair: accumulators that take K in turn (see umma_head_shape), else 1
   int half_last;    // the last row group has at most 128 rows and runs with 128-row MMAs (64 rows per CTA)
   int unit;         // rotary epilogue: weight rows per copy when a half tile is not made of whole head halves (else 0)
   int stages;
@@ -257,7 +260,8 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           break;
         }
         tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)(buf * 256);
+        uint32_t d = tmem_base + (uint32_t)(buf * 256), acc = 0;              // acc 0: the next MMA overwrites the accumulator
+        int chain = 0, chain_end = 2 * kc / args.chains;                      // (in K atoms)
         for (int c = 0; c < kc; ++c) {
           ok = mbar_wait(full_bar(s), ph, abort_flag);
           ok = __all_sync(0xffffffffu, ok);
@@ -270,10 +274,16 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           if (elect_one()) {
 #pragma unroll
             for (int a = 0; a < 2; ++a) {
+              if (Epi::kReduce && 2 * c + a == chain_end) {
+                chain_end = 2 * kc * (++chain + 1) / args.chains;
+                d += (uint32_t)BN;
+                acc = 0;
+              }
               const uint64_t da = make_smem_desc(sa + a * a_atom), db = make_smem_desc(sa + 2 * A_ATOM + a * B_ATOM);
 #pragma unroll
               for (int k = 0; k < 4; ++k)
-                tc_mma_f16_pair(d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (c | a | k) != 0 ? 1u : 0u);
+                tc_mma_f16_pair(d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, acc | (uint32_t)k ? 1u : 0u);
+              acc = 1;
             }
             tc_commit_pair(empty_bar(s), pair_mask);
             if (c == kc - 1) tc_commit_pair(accf_bar(buf), pair_mask);
@@ -368,6 +378,19 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             tc_pin16(p1);
             if (live && j0 + ch * 16 < args.n_pairs) epi16(epi, m, j0 + ch * 16, p0, p1, pre);
             pre = next;
+          }
+        } else if (Epi::kReduce && args.chains > 1) {
+#pragma unroll 1
+          for (int ch = ch_lo; ch < ch_hi; ++ch) {
+            float sum[16], part[16];
+            tc_ld16(t_row + (uint32_t)(ch * 16), sum);
+#pragma unroll 1
+            for (int x = 1; x < args.chains; ++x) {
+              tc_ld16(t_row + (uint32_t)(x * BN + ch * 16), part);
+#pragma unroll
+              for (int e = 0; e < 16; ++e) sum[e] += part[e];
+            }
+            consume(ch, sum, part);
           }
         } else {
         // the next chunk's tensor-memory loads are in flight while this one is converted and stored
@@ -531,8 +554,16 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
   const int cols = Epi::kDual ? 2 * NP : NP;
   const int pairs = st.max_clusters[2];
   constexpr bool kPlain = !Epi::kDual && !Epi::kReduce;
-  PairShape shape = Epi::kReduce ? PairShape{UM_HEAD_BN, 1} : pair_shape(st, M, cols, K, kRope ? 64 : 32, kPlain && st.pair_split != 1, !kRope && !Epi::kReduce);
-  if (st.pair_bn > 0 && !Epi::kReduce) shape = {st.pair_bn, 1};
+  PairShape shape{UM_HEAD_BN, 1};
+  int chains = 1;
+  if constexpr (Epi::kReduce) {
+    const HeadShape h = umma_head_shape(st, M, NP, K);
+    shape.bn = h.bn;
+    chains = std::min(h.chains, K / UM_BK);
+  } else {
+    shape = pair_shape(st, M, cols, K, kRope ? 64 : 32, kPlain && st.pair_split != 1, !kRope);
+    if (st.pair_bn > 0) shape = {st.pair_bn, 1};
+  }
   const int bn = shape.bn;
   int unit = 0;
   if constexpr (kRope) {
@@ -604,7 +635,7 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
   if (kPlain && st.pair_split > 1 && T * st.pair_split <= pairs && T <= st.max_clusters[2 * st.pair_split] && (K + 127) / 128 >= st.pair_split)
     ks = st.pair_split;
   const int grid = 2 * ks * (int)(T < pairs ? T : pairs);
-  PairArgs args{M, NP, n_tiles, rg, band, (K + 2 * UM_BK - 1) / (2 * UM_BK), ks, bn, half_last, unit, stages, status};
+  PairArgs args{M, NP, n_tiles, rg, band, (K + 2 * UM_BK - 1) / (2 * UM_BK), ks, bn, chains, half_last, unit, stages, status};
   cudaError_t e = launch_k(st.pdl, k_gemm_pair<Epi>, dim3(grid), dim3(PR_THREADS), smem, stream, 2 * ks, ma, mb0, mb1, mah, mh0, mh1, args, epi);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -5; }

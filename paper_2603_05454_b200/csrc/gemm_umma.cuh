@@ -427,9 +427,23 @@ constexpr int UM_HEAD_BN = 256;
 // one SM per tile, at 187 / 256 rows, us: 12288 x 4096 29 -> 26, 37 -> 27; 4096 x 4096 16.6 -> 14.9, 19.2 -> 15.1; 2 x 12288 SwiGLU
 // 44 -> 45, 54 -> 46; 4096 x 12288 (three K slices) 30 -> 28.5; 3584 x 18944 38 -> 35.5; head 249 -> 222.
 inline bool umma_takes_pairs(int M) { return M > UM_BM; }
-// Partials per row the head GEMM of M rows leaves: one per vocabulary tile, or (k_gemm_pair) one per half tile.
-inline int umma_head_tiles(int M, int vocab) {
-  return (vocab + UM_HEAD_BN - 1) / UM_HEAD_BN * (umma_takes_pairs(M) ? 2 : 1);
+// The head's kernel and tile.  Its scores leave in fp32, so the rounding of the sums over K shows: the tensor core truncates at
+// every step, and the error grows with the length of one accumulator's chain (scores of 4096 ids from K = 512, relative to
+// 64 bits: 3.5e-6 in one chain, 1.7e-6 in two, 1.1e-6 in four).  A vocabulary of few tiles leaves tensor memory unused, one tile
+// per pair: K then runs in four accumulators of 128 columns, or two of 256, which the epilogue adds in K order.
+// Rows: more than 128 go to the pairs, as everywhere.  So do 9 to 128 with a short K: the streaming kernel would split the few
+// tiles over its CTAs and sum them from global scratch (4096 ids, K 512: 49 us at 100 rows, 15.7 at 9, 13.0 at 4; pairs 15 to 16).
+struct HeadShape { bool pairs; int bn, chains; };
+inline HeadShape umma_head_shape(const UmmaState& st, int M, int vocab, int K) {
+  const long rg = (M + 255) / 256, t256 = (vocab + 255) / 256 * rg, t128 = (vocab + 127) / 128 * rg, pairs = st.max_clusters[2];
+  if (!(umma_takes_pairs(M) || (M > 8 && K <= 512 && t256 <= pairs))) return {false, UM_HEAD_BN, 1};
+  if (t128 <= pairs) return {true, 128, 4};
+  return {true, UM_HEAD_BN, t256 <= pairs ? 2 : 1};
+}
+// Partials per row the head GEMM leaves: one per vocabulary tile, or (k_gemm_pair) one per half tile.
+inline int umma_head_tiles(const UmmaState& st, int M, int vocab, int K) {
+  const HeadShape s = umma_head_shape(st, M, vocab, K);
+  return (vocab + s.bn - 1) / s.bn * (s.pairs ? 2 : 1);
 }
 
 template <typename Epi> bool stream_can(const UmmaState& st, int M, int NP, int K, int bn);
@@ -456,7 +470,8 @@ template <typename Epi>
 int umma_gemm(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0, const bf16* W1, int M, int NP, int K,
               int n_rows_w, const Epi& epi, unsigned* status) {
   if (K % UM_BK) { st.err = "K must be a multiple of 64"; return -6; }
-  if (umma_takes_pairs(M)) return pair_launch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
+  if (Epi::kReduce ? umma_head_shape(st, M, NP, K).pairs : umma_takes_pairs(M))
+    return pair_launch<Epi>(st, stream, A, W0, W1, M, NP, K, n_rows_w, epi, status);
   constexpr bool kRope = std::is_same<Epi, EpiQKVRope<bf16>>::value;
   const int cols = Epi::kDual ? 2 * NP : NP;
   int bn = UM_HEAD_BN;

@@ -183,7 +183,7 @@ struct Layout {
 constexpr size_t kGemmScratchBytes = 40u << 20;   // split-K partial tiles (the streaming GEMM needs 37 MiB at its widest)
 constexpr int kGemmCounters = 4096;               // split-K arrival counters
 
-int head_tiles_max(const lsp_model_cfg* m) { return std::max(2, (m->vocab + 63) / 64); }
+int head_tiles_max(const lsp_model_cfg* m) { return (m->vocab + 127) / 128 * 2; }      // partials per row: at most one per 64 ids, in pairs
 
 Layout make_layout(const lsp_model_cfg* m, int max_batch, int max_len) {
   const size_t esz = m->dtype == 0 ? 4 : 2;
@@ -270,7 +270,7 @@ int run_head(lsp_ctx* c, const T* hidden, int rows, int* n_tiles_out) {
   epi.exclude_id = c->s.exclude_mask_logit ? m.mask_id : -1;
   int n_tiles = (m.vocab + SG_HEAD_BN - 1) / SG_HEAD_BN;
 #ifndef LSP_NO_UMMA
-  if (std::is_same<T, bf16>::value && c->gemm_impl == 1) n_tiles = umma_head_tiles(rows, m.vocab);
+  if (std::is_same<T, bf16>::value && c->gemm_impl == 1) n_tiles = umma_head_tiles(c->umma, rows, m.vocab, m.d_model);
 #endif
   epi.n_tiles = n_tiles;
   *n_tiles_out = n_tiles;
