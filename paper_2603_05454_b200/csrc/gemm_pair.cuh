@@ -562,13 +562,14 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
     chains = std::min(h.chains, K / UM_BK);
   } else {
     shape = pair_shape(st, M, cols, K, kRope ? 64 : 32, kPlain && st.pair_split != 1, !kRope);
-    if (st.pair_bn > 0) shape = {st.pair_bn, 1};
+    if (st.pair_bn > 0 && (!kRope || st.pair_bn % 64 == 0)) shape = {st.pair_bn, 1};      // (a width that the epilogue can take)
   }
   const int bn = shape.bn;
   int unit = 0;
   if constexpr (kRope) {
     if ((bn / 2) % epi.half) unit = 32;
-    if (epi.half % 32) { st.err = "unsupported head_dim for the paired GEMM"; return -6; }
+    // a half tile is whole boxes, each inside one head half: a box too many would land behind its stage
+    if (epi.half % 32 || bn % 64) { st.err = "unsupported head_dim or tile width for the paired GEMM's rotary epilogue"; return -6; }
   }
   const int stage = 2 * (UM_BM * 128 + bn / 2 * 128);
   const int aux = 1024 + 8 * (2 * PR_MAX_STAGES + 4) + 16;

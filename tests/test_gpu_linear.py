@@ -332,7 +332,8 @@ def test_linear_bf16_on_pairs_of_sms(case):
     dec.close()
 
 
-@pytest.mark.parametrize("dh,hq,hkv,bn", [(128, 4, 2, 128), (128, 4, 2, 192), (128, 5, 5, 256), (64, 6, 2, 192), (64, 6, 2, 128)])
+@pytest.mark.parametrize("dh,hq,hkv,bn", [(128, 4, 2, 128), (128, 4, 2, 192), (128, 5, 5, 256), (64, 6, 2, 192), (64, 6, 2, 128),
+                                              (128, 4, 2, 96), (128, 5, 5, 160), (64, 6, 2, 224)])      # no multiples of 64: automatic
 def test_rotary_projection_on_pairs_of_sms(dh, hq, hkv, bn):
     """The rotary QKV projection of more than 256 rows (half tiles of whole head halves, or of 32-row pieces of them): the
     first layer's cached keys and values against the CUDA-core GEMM's.  Both round the same fp32 value up to the order of its
