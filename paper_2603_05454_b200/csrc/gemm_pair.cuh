@@ -577,12 +577,8 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
   if (stages > PR_MAX_STAGES) stages = PR_MAX_STAGES;
   if (stages < 2) { st.err = "not enough shared memory for the paired GEMM"; return -2; }
   const size_t smem = (size_t)stages * stage + aux;
-  static bool attr_set = false;   // per instantiation
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_pair<Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, st.max_smem);
-    if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -3; }
-    attr_set = true;
-  }
+  const cudaError_t smem_rc = umma_raise_smem(st, k_gemm_pair<Epi>);
+  if (smem_rc != cudaSuccess) { st.err = cudaGetErrorString(smem_rc); return -3; }
   CUtensorMap ma, mb0, mb1, mah, mh0, mh1;               // ..h: operands of a half row group
   const int half_last = (!kRope && !Epi::kReduce && shape.ks == 1 && st.pair_split <= 1 && pair_half_last(M, bn)) ? 1 : 0;
   {

@@ -758,12 +758,8 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
   const StreamShape sh = stream_shape(st, M, BN, K);
   if (sh.stages < 2) { st.err = "not enough shared memory for the streaming GEMM"; return -2; }
   const size_t smem = (size_t)sh.stages * sh.stage_bytes + sh.aux;
-  static bool attr_set = false;   // per instantiation
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_stream<BN, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, st.max_smem);
-    if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -3; }
-    attr_set = true;
-  }
+  const cudaError_t smem_rc = umma_raise_smem(st, k_gemm_stream<BN, Epi>);
+  if (smem_rc != cudaSuccess) { st.err = cudaGetErrorString(smem_rc); return -3; }
   const CUtensorMap* ma = umma_map4(st, A, M, M, 1, K, sh.a_rows, 1, sh.atoms);
   if (!ma) return -4;
   WeightView v{W0, n_rows_w, 1, n_rows_w, 1, 0, BN, 1};

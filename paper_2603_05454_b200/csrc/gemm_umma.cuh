@@ -16,6 +16,7 @@
 #include <cuda.h>
 
 #include <map>
+#include <set>
 #include <string>
 #include <tuple>
 
@@ -340,8 +341,19 @@ struct UmmaState {
   int pair_split = 0;              // its K slices (0 = automatic, 1 = never, 2 or 3 where they fit)
   int pair_bn = 0;                 // its tile width (0 = automatic)
   int pair_band = 0;               // its row groups per band (0 = automatic)
+  std::set<const void*> smem_set;  // kernels whose shared-memory limit has been raised on this context's device
   std::string err;
 };
+
+// Raises a kernel's dynamic shared-memory limit once per library context: the limit belongs to the device (and the CUDA context)
+// current at the call, so a flag per process would leave the kernel's launches on a second one to fail.
+template <typename... KArgs>
+cudaError_t umma_raise_smem(UmmaState& st, void (*kernel)(KArgs...)) {
+  if (st.smem_set.count((const void*)kernel)) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, st.max_smem);
+  if (e == cudaSuccess) st.smem_set.insert((const void*)kernel);
+  return e;
+}
 
 inline int umma_init(UmmaState& st) {
   void* fn = nullptr;
