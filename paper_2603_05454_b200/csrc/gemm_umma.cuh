@@ -234,7 +234,7 @@ struct EpiPre<EpiQKVRope<bf16>> {
   __device__ __forceinline__ void load(const EpiQKVRope<bf16>& e, int m, int j) {
     const int h = j / e.half, i = j % e.half;
     if (h < e.n_heads + e.n_kv_heads) {
-      const float4* c4 = reinterpret_cast<const float4*>(e.cs + (size_t)__ldg(e.row_pos + m) * e.half + i);
+      const float4* c4 = reinterpret_cast<const float4*>(e.cs + (size_t)e.row_pos[m] * e.half + i);
 #pragma unroll
       for (int q = 0; q < 8; ++q) c[q] = __ldg(c4 + q);
     }
