@@ -50,9 +50,9 @@ constexpr int attn_mma_smem_bytes() { return (AM_BM + 4 * AM_BN) * (DH + 8) * 2;
 
 // grid = (ceil(max_rows_per_seq * group / 64), n_kv_heads, batch), block = 128, dynamic smem = attn_mma_smem_bytes.
 template <int DH>
-__global__ void __launch_bounds__(128) k_attn_mma(const bf16* __restrict__ q, const bf16* __restrict__ cache_k,
-                                                  const bf16* __restrict__ cache_v, const bf16* __restrict__ stage_k,
-                                                  const bf16* __restrict__ stage_v, bf16* __restrict__ out, StepDesc sd,
+__global__ void __launch_bounds__(128) k_attn_mma(const bf16* q, const bf16* cache_k,
+                                                  const bf16* cache_v, const bf16* stage_k,
+                                                  const bf16* stage_v, bf16* __restrict__ out, StepDesc sd,
                                                   int n_heads, int n_kv_heads, size_t cache_seq_elems,
                                                   float scale_log2, int inplace) {
   constexpr int LD = DH + 8;            // padded row (elements): 16-byte shift per row, conflict-free ldmatrix

@@ -21,9 +21,9 @@ constexpr int AS_BK = 32;   // keys per tile (one per lane)
 // q: [M, n_heads*DH]; cache_k/v: this layer's planes [batch_max][max_len][n_kv*DH]; stage_k/v: this layer's
 // staged planes [M][n_kv*DH]; out: [M, n_heads*DH].
 template <typename T, int DH, int QW>
-__global__ void __launch_bounds__(128) k_attn_simt(const T* __restrict__ q, const T* __restrict__ cache_k,
-                                                   const T* __restrict__ cache_v, const T* __restrict__ stage_k,
-                                                   const T* __restrict__ stage_v, T* __restrict__ out, StepDesc sd,
+__global__ void __launch_bounds__(128) k_attn_simt(const T* q, const T* cache_k,
+                                                   const T* cache_v, const T* stage_k,
+                                                   const T* stage_v, T* __restrict__ out, StepDesc sd,
                                                    int n_heads, int n_kv_heads, size_t cache_seq_elems,
                                                    float scale, int inplace) {
   constexpr int AS_BQ = 4 * QW;

@@ -87,6 +87,9 @@ __device__ __forceinline__ float warp_min(float v) {
 // waits itself) and then waits until the preceding kernel has completed and its writes are visible.  Kernels with a
 // set-up that touches no global memory call pdl_release() first and pdl_wait() after the set-up.  Both are no-ops in a
 // kernel launched without the attribute.
+// Data that a kernel of the step writes is therefore not read-only for its successors, whose blocks may be resident while it is
+// written: their parameters for it carry no const __restrict__ (which lets the compiler load through the read-only path, without
+// an order against those writes).  Weights and tables do.
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin() { pdl_release(); pdl_wait(); }

@@ -35,7 +35,7 @@ constexpr int SG_HEAD_BN = 64;    // columns per partial of the head, in both ke
 
 // grid = (ceil(NP / PER_TILE), ceil(M / BM)), block = 256.  A: [M, K]; W0/W1: [*, K] row-major.
 template <typename T, typename Epi>
-__global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* __restrict__ A, const T* __restrict__ W0,
+__global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* A, const T* __restrict__ W0,
                                                                    const T* __restrict__ W1, int M, int NP, int K, Epi epi) {
   constexpr int BM = SimtTile<Epi>::BM, BN = SimtTile<Epi>::BN, PT = SimtTile<Epi>::PER_TILE;
   constexpr int LA = BM + 4, LB = BN + 4;                       // padded leading dimensions
@@ -167,7 +167,7 @@ constexpr int SG_BM = 64, SG_BN = SG_HEAD_BN, SG_BK = 16;
 
 // grid = (ceil(NP / 64), ceil(M / 64)), block = 256.  A: [M, K]; W0/W1: [*, K] row-major.
 template <typename T, typename Epi>
-__global__ void __launch_bounds__(256) k_gemm_simt(const T* __restrict__ A, const T* __restrict__ W0,
+__global__ void __launch_bounds__(256) k_gemm_simt(const T* A, const T* __restrict__ W0,
                                                    const T* __restrict__ W1, int M, int NP, int K, Epi epi) {
   __shared__ float As[SG_BK][SG_BM + 4];
   __shared__ float B0s[SG_BK][SG_BN + 4];

@@ -10,7 +10,7 @@ namespace lsp {
 // One block per row.  Also fills row_seq / row_pos and the list of rows that go through the LM head.
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void k_assemble_embed(StepDesc sd, const __grid_constant__ DescInline in, int batch, const int32_t* __restrict__ tokens, int tok_stride,
+__global__ void k_assemble_embed(StepDesc sd, const __grid_constant__ DescInline in, int batch, const int32_t* tokens, int tok_stride,
                                  int mask_id, const T* __restrict__ embed, int d, T* __restrict__ X,
                                  int* __restrict__ row_seq, int* __restrict__ row_pos,
                                  int* __restrict__ head_src, int* __restrict__ head_pos, int scattered) {
@@ -93,8 +93,8 @@ __device__ __forceinline__ uint4 f_to_vec(const float (&v)[8]) {
 // the wait to the last store of a 101-row launch.  With many rows they stay in L2 and the registers they hold (57 a thread
 // instead of 36) cost more: 8240 rows 34 -> 41 us.
 template <typename T, bool kEarly>
-__global__ void __launch_bounds__(RN_THREADS) k_rmsnorm(const T* __restrict__ x, const T* __restrict__ g, T* __restrict__ out,
-                                                       const int* __restrict__ src_rows, int d, float eps) {
+__global__ void __launch_bounds__(RN_THREADS) k_rmsnorm(const T* x, const T* __restrict__ g, T* __restrict__ out,
+                                                       const int* src_rows, int d, float eps) {
   constexpr int E = Vec16<T>::N;                 // elements per 16-byte vector
   __shared__ float red[RN_THREADS / 32];
   pdl_release();
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(RN_THREADS) k_rmsnorm(const T* __restrict__ x,
 // ---------------------------------------------------------------------------------------------
 // Merge of the per-vocab-tile partials of one row into (yhat, p_max, delta).  One warp per row.
 // ---------------------------------------------------------------------------------------------
-__global__ void k_merge_partials(const Top2* __restrict__ part, int n_tiles, int rows, int32_t* __restrict__ yhat,
+__global__ void k_merge_partials(const Top2* part, int n_tiles, int rows, int32_t* __restrict__ yhat,
                                  float* __restrict__ pmax, float* __restrict__ margin) {
   pdl_begin();
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -225,8 +225,8 @@ struct ScanOut {
   int prev_stride;
 };
 
-__global__ void __launch_bounds__(256) k_lsp_scan(const float* __restrict__ score, const int32_t* __restrict__ yhat,
-                           const float* __restrict__ margin, const int* __restrict__ seq_off, ScanParams p, ScanOut o) {
+__global__ void __launch_bounds__(256) k_lsp_scan(const float* score, const int32_t* yhat,
+                           const float* margin, const int* seq_off, ScanParams p, ScanOut o) {
   __shared__ int red[2][8];
   pdl_begin();
   const int b = blockIdx.x;
@@ -386,12 +386,12 @@ __device__ __forceinline__ void advance_descriptor(const StepDesc& cur, int* __r
 //   * block (0, 0, b) also writes yhat_{1:L_b} into the token buffer at [Fp_b, Fp_b + L_b).
 // The host advances F, Fp, pend, N after enqueueing this kernel (stream order makes the commit atomic).
 // ---------------------------------------------------------------------------------------------
-__global__ void k_commit_append(StepDesc sd, const uint4* __restrict__ stage, uint4* __restrict__ cache,
+__global__ void k_commit_append(StepDesc sd, const uint4* stage, uint4* __restrict__ cache,
                                 size_t stage_plane_v4,   // uint4 per (layer, K|V) plane of the staging buffer
                                 size_t cache_plane_v4,   // uint4 per (layer, K|V) plane of the cache
                                 size_t cache_seq_v4,     // uint4 per sequence inside a cache plane
                                 int row_v4,              // uint4 per row (n_kv_heads * head_dim * sizeof(T) / 16)
-                                const int32_t* __restrict__ yhat, int32_t* __restrict__ tokens, int tok_stride,
+                                const int32_t* yhat, int32_t* __restrict__ tokens, int tok_stride,
                                 int write_tokens, int copy_rows, const __grid_constant__ LenInline len,
                                 int* __restrict__ next_desc, int desc_stride, int batch) {
   pdl_begin();
@@ -417,7 +417,7 @@ __global__ void k_commit_append(StepDesc sd, const uint4* __restrict__ stage, ui
 // Scattered topology: lists, in ascending position, the rows of sequence b whose token is still [MASK].
 // One block of 256 threads per sequence; rows [pend_b, pend_b + N_b) of the pass are its generation region.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_compact_masked(StepDesc sd, const int32_t* __restrict__ tokens, int tok_stride,
+__global__ void __launch_bounds__(256) k_compact_masked(StepDesc sd, const int32_t* tokens, int tok_stride,
                                                         int mask_id, int* __restrict__ head_src,
                                                         int* __restrict__ head_pos) {
   __shared__ int warp_cnt[8];
@@ -458,8 +458,8 @@ __global__ void __launch_bounds__(256) k_compact_masked(StepDesc sd, const int32
 // into the token buffer at their own positions.  One block of 256 threads per sequence; scores staged in shared
 // memory (dynamic, 4 bytes per masked position of the longest sequence).
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_scatter_commit(StepDesc sd, const float* __restrict__ score,
-                                                        const int32_t* __restrict__ yhat, const int* __restrict__ head_pos,
+__global__ void __launch_bounds__(256) k_scatter_commit(StepDesc sd, const float* score,
+                                                        const int32_t* yhat, const int* head_pos,
                                                         int32_t* __restrict__ tokens, int tok_stride,
                                                         const __grid_constant__ LenInline len) {
   extern __shared__ float sc_s[];
