@@ -242,6 +242,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (first CTA; the whole warp waits, one elected thread issues) ----------------
+    pdl_wait();            // (its bounded waits must not count the preceding kernel's time)
     if (rank == 0) {
       int s = 0;
       uint32_t ph = 0;

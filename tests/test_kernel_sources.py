@@ -26,3 +26,17 @@ def test_no_kernel_declares_data_of_the_step_read_only(name):
     lengths that the host copies before a plain launch (P, G)."""
     for m in re.finditer(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", _source(name)):
         assert m.group(1) in ("embed", "g", "W0", "W1", "P", "G"), f"{name}: {m.group(1)}"
+
+
+@pytest.mark.parametrize("name", ["gemm_stream.cuh", "gemm_pair.cuh", "attention_umma.cuh"])
+def test_no_role_starts_a_bounded_wait_before_the_preceding_kernel_has_ended(name):
+    """The limit of a wait is for this kernel's own copies and MMAs.  Every role (producer, issuer, epilogue: the branches behind the
+    set-up's barrier) reaches pdl_wait() before its first mbar_wait(), by itself or because all of them do."""
+    body = _source(name)
+    body = body[body.index("tmem_base = *tmem_slot"):]
+    roles = re.split(r"\n  (?:if|\} else if) \(warp == [^\n]*\) \{\n|\n  \} else \{\n", body)
+    assert len(roles) >= 4
+    if "pdl_wait();" in roles[0]:
+        return
+    for r in roles[1:4]:
+        assert "pdl_wait();" in r.split("mbar_wait(")[0]
