@@ -486,6 +486,7 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
 #pragma unroll 1
           for (int c = 0; c < DH; c += 16) {
             float v[16], u[16];
+            __syncwarp();
             if (have) tc_ld16(lane_base + (uint32_t)c, v);
             if (have1) tc_ld16(lane_base + (uint32_t)(DH + c), u);
             if (valid) {

@@ -325,7 +325,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           }
         }
       }
-      if (!mbar_wait(accf_bar(buf), (uint32_t)use & 1u, abort_flag)) {
+      if (!__all_sync(0xffffffffu, mbar_wait(accf_bar(buf), (uint32_t)use & 1u, abort_flag))) {
         if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 44u; }
         break;
       }
@@ -337,6 +337,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         for (int k = 0; k < 8; ++k) {
           if (ch_lo + k < ch_hi) {                                // uniform per warp
             float a[16];
+            __syncwarp();                                         // (rows past the last one part ways above; the load is collective)
             tc_ld16(t_row + (uint32_t)((ch_lo + k) * 16), a);
             if (live && j0 + (ch_lo + k) * 16 < args.n_pairs) {
 #pragma unroll
@@ -356,6 +357,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           const int j = j0 + ch * 16;
           if constexpr (Epi::kReduce) top2_push16(red, a0, j, epi);
           else if (live && j < args.n_pairs) epi16(epi, m, j, a0, a1);
+          __syncwarp();                                           // (rows past the last one part ways above; the next load is collective)
         };
         auto request = [&](int ch, float (&a0)[16], float (&a1)[16]) {
           tc_ld16_nowait(t_row + (uint32_t)(ch * 16), a0);

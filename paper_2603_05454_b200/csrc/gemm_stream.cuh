@@ -307,7 +307,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       if constexpr (!Epi::kReduce) {
         if (whole && r_in < args.M && j0 < args.n_pairs) preA.load(epi, r_in, j0);
       }
-      if (!mbar_wait(accf_bar(buf), (uint32_t)use & 1u, abort_flag)) {
+      if (!__all_sync(0xffffffffu, mbar_wait(accf_bar(buf), (uint32_t)use & 1u, abort_flag))) {
         if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 14u; }
         ok = false;
         break;
@@ -332,6 +332,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             } else {
               if (m < args.M && j0 + c < args.n_pairs) epi16(epi, m, j0 + c, a0, a1, pre);
             }
+            __syncwarp();
           };
           auto request = [&](int c, float (&a0)[16], float (&a1)[16]) {
             tc_ld16_nowait(t_row + c, a0);
@@ -397,6 +398,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
 #pragma unroll
               for (int p = 0; p < P; ++p) {
                 float v[16];
+                __syncwarp();
                 tc_ld16(t_row + p * HALF + ch * 16, v);
                 if (r_in < args.M) {
 #pragma unroll
@@ -417,6 +419,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
 #pragma unroll 1
           for (int c = 0; c < BN; c += 16) {
             float v[16];
+            __syncwarp();
             tc_ld16(t_row + c, v);
             if (r_in < args.M) {
 #pragma unroll
@@ -544,6 +547,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       auto finish = [&](int it, const float4 (&t0)[4], const float4 (&t1)[4], const EpiPre<Epi>& pre) {
         const int ch = o_lo + it;
         float a0[16], a1[16];
+        __syncwarp();
         tc_ld16(t_row + ch * 16, a0);
         if (Epi::kDual) tc_ld16(t_row + HALF + ch * 16, a1);
         if (live(it)) {

@@ -40,3 +40,9 @@ def test_no_role_starts_a_bounded_wait_before_the_preceding_kernel_has_ended(nam
         return
     for r in roles[1:4]:
         assert "pdl_wait();" in r.split("mbar_wait(")[0]
+
+
+@pytest.mark.parametrize("name", ["gemm_stream.cuh", "gemm_pair.cuh", "attention_umma.cuh"])
+def test_warps_leave_on_an_expired_wait_as_one(name):
+    """Tensor-memory loads and full-mask barriers need every lane: whether a wait expired is put to a vote before anyone leaves."""
+    assert not re.search(r"if \(!mbar_wait\(", _source(name))
