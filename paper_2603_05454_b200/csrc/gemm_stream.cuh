@@ -27,6 +27,8 @@
 // Warp roles (192 threads): warp 0 = TMA producer, warp 1 = TMEM allocator + MMA issuer, warps 2..5 = epilogue.
 // Every wait is bounded; on expiry the kernel records (code, site) in the status word, drains and returns.
 #pragma once
+#include <algorithm>
+
 #include "gemm_umma.cuh"
 
 namespace lsp {
@@ -710,8 +712,9 @@ inline int stream_splits(const UmmaState& st, long n_tiles, bool no_split) {
   return splits;
 }
 
-inline int stream_grid(const UmmaState& st, int n_tiles, bool no_split) {
-  if (st.target_ctas > 0) return st.target_ctas;
+inline int stream_grid(const UmmaState& st, int n_tiles, int bn, bool no_split) {
+  // (a forced count: as many as the scratch holds partial tiles for)
+  if (st.target_ctas > 0) return std::min(st.target_ctas, (int)(st.scratch_bytes / stream_scratch_bytes(1, bn)));
   const int splits = stream_splits(st, n_tiles, no_split);
   return (st.stream_even || splits == 0) ? st.n_sm : n_tiles * splits;
 }
@@ -794,7 +797,7 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
   const int n_tiles = (NP + per_tile - 1) / per_tile;
   const int kc = K / (sh.atoms * UM_BK);
   const long T = n_tiles;
-  int grid = stream_grid(st, (int)T, stream_no_split<Epi>(K));
+  int grid = stream_grid(st, (int)T, BN, stream_no_split<Epi>(K));
   if (grid > T * kc) grid = (int)(T * kc);
   if ((double)T * kc * (grid + 1) >= 4.0e9) { st.err = "too many work units for the streaming GEMM"; return -9; }   // 32-bit unit arithmetic
   // K slices of one tile on the CTAs of one cluster: the reduction then stays on chip
@@ -820,7 +823,7 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
 template <typename Epi>
 bool stream_can(const UmmaState& st, int M, int NP, int K, int bn) {
   const long T = (NP + (Epi::kDual ? bn / 2 : bn) - 1) / (Epi::kDual ? bn / 2 : bn);
-  if (st.scratch == nullptr || T > st.n_counters || stream_scratch_bytes(stream_grid(st, (int)T, stream_no_split<Epi>(K)), bn) > st.scratch_bytes)
+  if (st.scratch == nullptr || T > st.n_counters || stream_scratch_bytes(stream_grid(st, (int)T, bn, stream_no_split<Epi>(K)), bn) > st.scratch_bytes)
     return false;
   return stream_shape(st, M, bn, K).stages >= 2;
 }

@@ -425,6 +425,26 @@ def test_linear_bf16_short_k_without_a_split(M, N, K):
     dec.close()
 
 
+@pytest.mark.parametrize("ctas", [1, 100, 161, 320])
+@pytest.mark.parametrize("op,N", [(0, 4096), (2, 1024)])
+def test_linear_bf16_forced_cta_count(ctas, op, N):
+    """A forced number of CTAs (key 10), below and above what the scratch has room for with 256-wide tiles (160): the count is
+    capped, not refused.  One or two bf16 ulps, as above."""
+    dec = _dec("bf16")
+    dec.debug_set(10, ctas)
+    M, K = 64, 4096
+    A = S.normal((M, K), 18, 1, 1.0, torch.bfloat16, DEV)
+    W = S.normal((N, K), 18, 2, 0.05, torch.bfloat16, DEV)
+    W2 = S.normal((N, K), 18, 3, 0.05, torch.bfloat16, DEV)
+    out = torch.empty(M, N, dtype=torch.bfloat16, device=DEV)
+    dec.op_linear(op, A, W, W2 if op == 2 else None, out)
+    want = A.double() @ W.double().t()
+    if op == 2:
+        want = torch.nn.functional.silu(want) * (A.double() @ W2.double().t())
+    assert bool(((out.double() - want).abs() <= (2 if op == 2 else 1) / 128 * want.abs() + want.abs().max() / 2560).all())
+    dec.close()
+
+
 @pytest.mark.parametrize("ks", [0, 2, 3])
 @pytest.mark.parametrize("M,N,K", [(187, 4096, 12288), (129, 512, 2048), (257, 272, 3072), (256, 3584, 4032), (700, 1040, 4096)])
 def test_linear_bf16_k_slices_on_pairs(M, N, K, ks):
