@@ -830,8 +830,14 @@ int lsp_debug_set(lsp_ctx* c, int key, int value) {
   else if (key == 32) c->umma.stream_bn_dual = (value == 192 || value == 256) ? value : 0;
   else if (key == 33) c->umma.stream_exchange = value ? 1 : 0;
   else if (key == 23) c->umma.stream_bn = (value == 256 || value == 128) ? value : 0;
-  else if (key == 41) c->umma.pair_bn = (value >= 96 && value <= 256 && value % 32 == 0) ? value : 0;
-  else if (key == 46) c->umma.pair_split = (value >= 0 && value <= 3) ? value : 0;
+  else if (key == 41) {
+    if (value != 0 && (value < 96 || value > 256 || value % 32)) return fail(c, LSP_ERR_ARG, "lsp_debug_set: key 41 takes 0 or 96 ... 256 in steps of 32, not %d", value);
+    c->umma.pair_bn = value;
+  }
+  else if (key == 46) {
+    if (value < 0 || value > 3) return fail(c, LSP_ERR_ARG, "lsp_debug_set: key 46 takes 0 to 3, not %d", value);
+    c->umma.pair_split = value;
+  }
   else if (key == 42) c->umma.pair_band = value < 0 ? 0 : value;
   else if (key == 43) c->umma.stream_split_copies = value ? 1 : 0;
   else if (key == 44) c->umma.stream_exchange_rows = value;
@@ -839,7 +845,7 @@ int lsp_debug_set(lsp_ctx* c, int key, int value) {
   else if (key == 22) c->umma.stream_min_stages2 = value < 2 ? 2 : value;
 #endif
   // knobs of kernel variants that are gone (two row tiles per CTA, swapped operands, two issuers, half an SM): accepted, without effect
-  else if (key == 18 || key == 19 || key == 20 || key == 24 || key == 26 || key == 27 || (key >= 36 && key <= 40) || key == 45) {}
+  else if (key == 18 || key == 19 || key == 20 || key == 24 || key == 26 || key == 27 || (key >= 36 && key <= 39)) {}
   else return fail(c, LSP_ERR_ARG, "lsp_debug_set: unknown key %d", key);
   return LSP_OK;
 }

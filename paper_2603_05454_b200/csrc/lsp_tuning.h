@@ -41,8 +41,8 @@ extern "C" {
  * decode loop:
  *   31 with device-resident block lengths (lsp_set_option key 4), lsp_generate reads every step before sizing the next
  *      once at most this many masked positions per sequence remain (default 8)
- * Accepted without effect (they tuned kernel variants that no longer exist): 18, 19, 20, 24, 26, 27, 36 to 40, 45.
- * Unknown key: LSP_ERR_ARG. */
+ * Accepted without effect (they tuned kernel variants that no longer exist): 18, 19, 20, 24, 26, 27, 36 to 39.
+ * Unknown key, or a value outside the range of key 41 or 46: LSP_ERR_ARG. */
 int lsp_debug_set(lsp_ctx* ctx, int key, int value);
 
 /* Exercises the bounded-wait recovery path without touching any data: launches one thread that waits, for limit_us

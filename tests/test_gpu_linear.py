@@ -425,6 +425,19 @@ def test_linear_bf16_short_k_without_a_split(M, N, K):
     dec.close()
 
 
+def test_tuning_entry_refuses_what_it_does_not_know():
+    """Keys that never tuned anything, and widths and splits that the paired GEMM does not have, are errors, not silent defaults."""
+    from paper_2603_05454_b200 import LSPError
+    dec = _dec("bf16")
+    for key, value in ((40, 1), (45, 1), (99, 0), (41, 64), (41, 100), (41, 288), (46, 4), (46, -1)):
+        with pytest.raises(LSPError) as e:
+            dec.debug_set(key, value)
+        assert e.value.code == -1
+    for value in (0, 96, 256):
+        dec.debug_set(41, value)
+    dec.close()
+
+
 @pytest.mark.parametrize("ctas", [1, 100, 161, 320])
 @pytest.mark.parametrize("op,N", [(0, 4096), (2, 1024)])
 def test_linear_bf16_forced_cta_count(ctas, op, N):
@@ -468,7 +481,7 @@ def test_linear_bf16_k_slices_on_pairs(M, N, K, ks):
 
 
 @pytest.mark.parametrize("M", [257, 320, 384, 385, 1032])
-@pytest.mark.parametrize("N,K,bn", [(272, 192, 0), (1040, 4032, 64), (4096, 576, 128), (1536, 512, 192), (3584, 4096, 256), (1024, 512, 224)])
+@pytest.mark.parametrize("N,K,bn", [(272, 192, 0), (1040, 4032, 192), (4096, 576, 128), (1536, 512, 192), (3584, 4096, 256), (1024, 512, 224)])
 def test_linear_bf16_half_row_group_on_pairs(M, N, K, bn):
     """A last row group of at most 128 rows (the fourth row count and the last width are beyond the line) on 128-row MMAs: ragged
     last column tiles and K chunks, rows of one CTA of the pair only; against the fp64 product."""
