@@ -38,6 +38,7 @@ struct lsp_ctx {
   char* kv_cache = nullptr;
   int max_batch = 0, max_len = 0, max_rows = 0;
   size_t esz = 0;
+  int n_sm = 0;                     // SMs of the device
   cudaStream_t stream = nullptr;
   int gemm_impl = 1, attn_impl = 2, timing = 0, async_ops = 0, op_repeat = 1, op_rotate = 1, pdl = 1, attn_umma_min_rows = 0, attn_cluster = 1;
   // workspace carve (device)
@@ -106,14 +107,6 @@ enum { CNT_LAUNCHES = 0, CNT_GEMM_BYTES = 1, CNT_GEMM_FLOPS = 2, CNT_ATTN_BYTES 
 void count_launch(lsp_ctx* c, int cls, int n = 1) {
   c->counters[CNT_LAUNCHES] += n;
   c->counters[CNT_CLS_LAUNCHES + cls] += n;
-}
-
-int sm_count(const lsp_ctx* c) {
-#ifndef LSP_NO_UMMA
-  return c->umma.n_sm;
-#else
-  return 148;
-#endif
 }
 
 // Opens a timed segment of kernel class cls (only when per-class timing is on).
@@ -251,7 +244,7 @@ int run_gemm(lsp_ctx* c, const T* A, const T* W0, const T* W1, int M, int NP, in
   }
 #endif
   dim3 grid((NP + SG_BN - 1) / SG_BN, (M + SG_BM - 1) / SG_BM);
-  if ((long)grid.x * grid.y < 2l * sm_count(c)) {          // (the line: see gemm_simt.cuh)
+  if ((long)grid.x * grid.y < 2l * c->n_sm) {          // (the line: see gemm_simt.cuh)
     using Tile = SimtTile<Epi>;
     grid = dim3((NP + Tile::PER_TILE - 1) / Tile::PER_TILE, (M + Tile::BM - 1) / Tile::BM);
     CU(launch_k(c->pdl, k_gemm_simt_split<T, Epi>, grid, dim3(256), 0, c->stream, A, W0, W1, M, NP, K, epi));
@@ -398,7 +391,7 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const Step
     }
   }
   if (!done) {
-    const int qw = (long)((maxQ + 15) / 16) * m.n_heads * B >= sm_count(c) ? 4 : 1;
+    const int qw = (long)((maxQ + 15) / 16) * m.n_heads * B >= c->n_sm ? 4 : 1;
     dim3 grid((maxQ + 4 * qw - 1) / (4 * qw), m.n_heads, B);
     auto kern = dh == 128 ? (qw == 4 ? k_attn_simt<T, 128, 4> : k_attn_simt<T, 128, 1>)
                           : (qw == 4 ? k_attn_simt<T, 64, 4> : k_attn_simt<T, 64, 1>);
@@ -727,6 +720,9 @@ int lsp_init(lsp_ctx** out, const lsp_model_cfg* model, const lsp_sched_cfg* sch
     if (e == cudaSuccess) e = cudaEventCreate(&c->ring_t0[i]);
     if (e == cudaSuccess) e = cudaEventCreate(&c->ring_t1[i]);
   }
+  int dev = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaEventCreate(&c->ev0);
   if (e == cudaSuccess) e = cudaEventCreate(&c->ev1);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, 256, c->stream);

@@ -46,3 +46,8 @@ def test_no_role_starts_a_bounded_wait_before_the_preceding_kernel_has_ended(nam
 def test_warps_leave_on_an_expired_wait_as_one(name):
     """Tensor-memory loads and full-mask barriers need every lane: whether a wait expired is put to a vote before anyone leaves."""
     assert not re.search(r"if \(!mbar_wait\(", _source(name))
+
+
+def test_the_step_driver_assumes_no_sm_count():
+    """The dispatch lines of the CUDA-core kernels (fp32 models among them) are in SMs of the device at hand."""
+    assert not re.search(r"\b148\b", _source("lsp_api.cu")) and "cudaDevAttrMultiProcessorCount" in _source("lsp_api.cu")
