@@ -827,7 +827,7 @@ int lsp_debug_set(lsp_ctx* c, int key, int value) {
   else if (key == 33) c->umma.stream_exchange = value ? 1 : 0;
   else if (key == 23) c->umma.stream_bn = (value == 256 || value == 128) ? value : 0;
   else if (key == 41) {
-    if (value != 0 && (value < 96 || value > 256 || value % 32)) return fail(c, LSP_ERR_ARG, "lsp_debug_set: key 41 takes 0 or 96 ... 256 in steps of 32, not %d", value);
+    if (value != 0 && (value < 64 || value > 256 || value % 32)) return fail(c, LSP_ERR_ARG, "lsp_debug_set: key 41 takes 0 or 64 ... 256 in steps of 32, not %d", value);
     c->umma.pair_bn = value;
   }
   else if (key == 46) {

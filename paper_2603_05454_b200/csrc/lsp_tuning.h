@@ -32,7 +32,7 @@ extern "C" {
  *   33 a cluster of 2 exchanges half tiles (1, default) or publishes whole partial tiles like larger clusters (0)
  *   44 ... from this many rows on (default 64)
  * GEMM on pairs of SMs, more than 128 rows (k_gemm_pair):
- *   41 its tile width (0 = automatic, 96 ... 256 in steps of 32; the rotary projection ignores a width that is no
+ *   41 its tile width (0 = automatic, 64 ... 256 in steps of 32; the rotary projection ignores a width that is no
  *      multiple of 64)   42 most row groups of 256 per band (0 = automatic)
  *   46 its K slices (0 = automatic, 1 = never split, 2 or 3 where they fit)
  * tcgen05 attention:

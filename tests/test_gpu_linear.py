@@ -333,7 +333,8 @@ def test_linear_bf16_on_pairs_of_sms(case):
 
 
 @pytest.mark.parametrize("dh,hq,hkv,bn", [(128, 4, 2, 128), (128, 4, 2, 192), (128, 5, 5, 256), (64, 6, 2, 192), (64, 6, 2, 128),
-                                              (128, 4, 2, 96), (128, 5, 5, 160), (64, 6, 2, 224)])      # no multiples of 64: automatic
+                                              (128, 4, 2, 96), (128, 5, 5, 160), (64, 6, 2, 224),       # no multiples of 64: automatic
+                                              (128, 4, 2, 64), (64, 6, 2, 64)])
 def test_rotary_projection_on_pairs_of_sms(dh, hq, hkv, bn):
     """The rotary QKV projection of more than 256 rows (half tiles of whole head halves, or of 32-row pieces of them): the
     first layer's cached keys and values against the CUDA-core GEMM's.  Both round the same fp32 value up to the order of its
@@ -430,11 +431,11 @@ def test_tuning_entry_refuses_what_it_does_not_know():
     """Keys that never tuned anything, and widths and splits that the paired GEMM does not have, are errors, not silent defaults."""
     from paper_2603_05454_b200 import LSPError
     dec = _dec("bf16")
-    for key, value in ((40, 1), (45, 1), (99, 0), (41, 64), (41, 100), (41, 288), (46, 4), (46, -1)):
+    for key, value in ((40, 1), (45, 1), (99, 0), (41, 32), (41, 100), (41, 288), (46, 4), (46, -1)):
         with pytest.raises(LSPError) as e:
             dec.debug_set(key, value)
         assert e.value.code == -1
-    for value in (0, 96, 256):
+    for value in (0, 64, 96, 256):
         dec.debug_set(41, value)
     dec.close()
 
@@ -482,7 +483,7 @@ def test_linear_bf16_k_slices_on_pairs(M, N, K, ks):
 
 
 @pytest.mark.parametrize("M", [257, 320, 384, 385, 1032])
-@pytest.mark.parametrize("N,K,bn", [(272, 192, 0), (1040, 4032, 192), (4096, 576, 128), (1536, 512, 192), (3584, 4096, 256), (1024, 512, 224)])
+@pytest.mark.parametrize("N,K,bn", [(272, 192, 0), (1040, 4032, 64), (4096, 576, 128), (1536, 512, 192), (3584, 4096, 256), (1024, 512, 224)])
 def test_linear_bf16_half_row_group_on_pairs(M, N, K, bn):
     """A last row group of at most 128 rows (the fourth row count and the last width are beyond the line) on 128-row MMAs: ragged
     last column tiles and K chunks, rows of one CTA of the pair only; against the fp64 product."""
