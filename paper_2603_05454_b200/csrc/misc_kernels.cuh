@@ -190,7 +190,7 @@ __global__ void k_merge_partials(const Top2* part, int n_tiles, int rows, int32_
 }
 
 // ---------------------------------------------------------------------------------------------
-// LSP scan (Sec. 3.2): one warp per sequence.
+// LSP scan (Sec. 3.2): one block per sequence, whose first warp scans (see ScanOut for what the others are for).
 //   fixed mode    : L' = longest left-aligned run with score_i >= tau             (ballot + ffs)
 //   adaptive mode : prefix minimum pm; m is achievable iff pm[m] > pm[m+1]; the largest achievable
 //                   m in [ceil(alpha N), floor(beta N)] is taken, tau = pm[m] (Eq. 2)

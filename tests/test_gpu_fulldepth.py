@@ -8,7 +8,7 @@ host.  Sequences of a batch are independent, so the oracle follows sequence 0 on
 batch run along on the GPU (they shape the launches) and commit their own proposals.
 
 Two policies per workload: the benchmark's fixed threshold (passes of 2 P rows, then about P + G/2) and a fixed block
-size that walks the row count down through the two-row-tile regime into the one-row-tile regime.
+size that walks the row count down through one row group on pairs of SMs into the streaming GEMM.
 
 Every pass is compared element by element: yhat, p_max, delta, and - outside the flagged band - L' and L.
 

@@ -4,7 +4,7 @@
    fp64 logits only for sampled rows and for the left end of every sequence up to one row past the first position that
    fails the threshold, which is all the scan's result depends on.
  * LLaDA-8B- and Dream-7B-shaped layers (full d_model, heads, FFN width; one layer, small vocabulary): teacher-forced
-   decode steps whose row counts cover the tiled GEMM (more than 256 rows) and both shapes of the streaming GEMM.
+   decode steps whose row counts cover the GEMM on pairs of SMs (one and two row groups) and the streaming GEMM.
 """
 import numpy as np
 import pytest
@@ -77,7 +77,7 @@ def test_full_width_layer_teacher_forced_steps(name):
         sh = S.ModelShape(1, 4096, 32, 32, 128, 12288, 8192, dtype="bf16", head_scale=4.0)
     else:
         sh = S.ModelShape(1, 3584, 28, 4, 128, 18944, 8192, dtype="bf16", head_scale=4.0, rope_theta=1e6)
-    # pass 0 has 300 rows (tiled GEMM, three row tiles), pass 1 about 250 (streaming GEMM, two row tiles); the
+    # pass 0 has 300 rows (pairs of SMs, two row groups), pass 1 about 250 (one row group); the
     # fixed-k policy then walks the row count down through the one-row-tile regime
     _teacher_forced(sh, 21, 50, 250, SchedCfg(tau=0.9), (1, 64), max_steps=2)
     _teacher_forced(sh, 22, 8, 150, SchedCfg(mode=2, fixed_k=60), (1, 64), max_steps=3)

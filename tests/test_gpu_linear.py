@@ -60,8 +60,9 @@ def test_linear_bf16(impl, shape):
                                    (17, 4096, 12288), (129, 384, 256), (200, 4096, 4096), (256, 12288, 4096),
                                    (190, 1152, 576)])
 def test_linear_bf16_weight_streaming_kernel(grid_mode, shape):
-    """M <= 256 takes the persistent streaming kernel (one or two row tiles per CTA): tiles split between CTAs
-    (partials in scratch, summed by the last arriver) with both ways of dealing out the work."""
+    """M <= 128 takes the persistent streaming kernel with both ways of dealing out the work: even shares over all SMs (tiles split
+    anywhere, partials in scratch, summed by the last arriver) and equal K slices per tile (on clusters).  The row counts above
+    that go to the pairs of SMs, beside the line."""
     M, N, K = shape
     tdt = torch.bfloat16
     dec = _dec("bf16")
@@ -93,17 +94,20 @@ def test_linear_bf16_weight_streaming_kernel(grid_mode, shape):
 
 
 @pytest.mark.parametrize("case", [
-    # (M, N, K, options): 256 x 256 tiles whose K slices run as one cluster; the fp32 partial tile (256 KB) is larger
-    # than the pipeline's shared memory, so it is reduced one row tile at a time
-    (200, 4096, 4096, {20: 256}), (256, 12288, 4096, {20: 256}), (130, 4096, 12288, {20: 256}),
-    (640, 4096, 12288, {}), (1000, 3584, 3584, {}), (300, 2048, 1024, {}), (257, 512, 2048, {}),
-    (640, 4096, 4096, {29: 0}),
-    (640, 4096, 12288, {33: 0}), (200, 12288, 1024, {20: 256, 33: 0}),      # clusters of 2 without the half-tile exchange
-    # SwiGLU GEMM with 192-wide tiles (96 pairs): one and two row tiles, several row groups, a forced 256 for contrast
-    (100, 12288, 256, {}), (200, 12288, 320, {}), (600, 12288, 256, {32: 192}), (100, 12288, 256, {32: 256}),
-    (300, 9600, 192, {32: 192}),
+    # (M, N, K, options): K slices on clusters of two (64 to 74 tiles of 128 columns), with the half-tile exchange, without it, and
+    # below its row count; of four and eight; through global scratch instead of clusters
+    (100, 8192, 4096, {}), (100, 8192, 4096, {33: 0}), (128, 8192, 1024, {33: 0}), (33, 8192, 1024, {}), (33, 8192, 1024, {44: 0}),
+    (64, 9216, 1088, {33: 0}), (100, 4096, 4096, {}), (128, 1040, 4096, {}), (100, 4096, 4096, {29: 0}), (128, 8192, 1024, {29: 0}),
+    (17, 1040, 2048, {29: 0}),
+    # SwiGLU GEMM with 192-wide tiles (96 pairs) and a forced 256 for contrast
+    (100, 12288, 256, {}), (100, 12288, 256, {32: 256}), (64, 9600, 1024, {32: 192}),
+    # more than 128 rows: pairs of SMs, few tiles and many, with and without K slices
+    (200, 4096, 4096, {}), (256, 12288, 4096, {}), (130, 4096, 12288, {}), (640, 4096, 12288, {}), (1000, 3584, 3584, {}),
+    (300, 2048, 1024, {}), (257, 512, 2048, {}), (640, 4096, 4096, {}), (200, 12288, 1024, {}), (200, 12288, 320, {}),
+    (600, 12288, 256, {}), (300, 9600, 192, {}),
 ])
-def test_linear_bf16_cluster_split_of_two_row_tiles(case):
+def test_linear_bf16_split_tiles(case):
+    """Every way of splitting a tile's K and of summing the slices, against fp64 products; twice the same bits."""
     M, N, K, opts = case
     tdt = torch.bfloat16
     dec = _dec("bf16")
@@ -136,13 +140,12 @@ def test_linear_bf16_cluster_split_of_two_row_tiles(case):
 
 
 def test_linear_bf16_seeded_random_shapes_and_kernel_options():
-    """Sixty seeded random (rows, columns, K, option) combinations across the row regimes (one tile, two tiles, row
-    groups), the split paths (clusters of 2..8, half-tile exchange, rounds, global scratch), the tile widths, and the
-    operand-swapped kernel forced on."""
+    """Sixty seeded random (rows, columns, K, option) combinations across the row regimes (one tile; pairs of SMs with one row group
+    and several), the split paths (clusters of 2..8, half-tile exchange, global scratch, K slices on pairs) and the tile widths."""
     import random
     rng = random.Random(7)
     dec = _dec("bf16")
-    defaults = {29: 1, 33: 1, 20: 0, 23: 0, 32: 0, 17: 2, 24: 3, 36: 129, 38: 0}
+    defaults = {29: 1, 33: 1, 23: 0, 32: 0, 17: 2, 41: 0, 42: 0, 46: 0}
     f64 = lambda t: t.float().cpu().numpy().astype(np.float64)
     rows = [1, 2, 5, 17, 32, 33, 64, 100, 128, 129, 190, 256, 257, 300, 400, 512, 640, 768, 1000, 1100, 1536, 2100]
     done = 0
@@ -152,12 +155,10 @@ def test_linear_bf16_seeded_random_shapes_and_kernel_options():
         if M * N * K > 2e10:
             continue
         opts = {}
-        for key, p, vals in ((29, 0.2, [0]), (33, 0.2, [0]), (20, 0.15, [128, 256]), (23, 0.15, [128, 256]),
-                             (32, 0.15, [192, 256]), (17, 0.1, [1]), (24, 0.1, [1, 2]), (38, 0.3, [1])):
+        for key, p, vals in ((29, 0.2, [0]), (33, 0.2, [0]), (41, 0.15, [96, 128, 224]), (23, 0.15, [128, 256]),
+                             (32, 0.15, [192, 256]), (17, 0.1, [1]), (42, 0.1, [1, 2]), (46, 0.3, [1, 2, 3])):
             if rng.random() < p:
                 opts[key] = rng.choice(vals)
-        if opts.get(38):
-            opts[36] = 1                    # the operand-swapped kernel at every row count up to 256, on any shape it can run
         for k, v in {**defaults, **opts}.items():
             dec.debug_set(k, v)
         A = S.normal((M, K), done, 1, 1.0, torch.bfloat16, DEV)
@@ -231,14 +232,10 @@ def test_linear_bf16_third_model_shape(M):
 
 
 @pytest.mark.parametrize("M", [1, 16, 17, 100, 129, 144, 177, 200, 256])
-def test_linear_bf16_operand_swapped_kernel(M):
-    """The operand-swapped kernel (weights as the 128-row MMA operand, activation rows as N in steps of 16), forced on for
-    every row count up to 256: one and two accumulators, K slices on clusters of 1, 2 and 4, ragged last tiles, all three
-    epilogues, twice (bit-identical: the K slices are summed in rank order)."""
+def test_linear_bf16_layer_shapes_up_to_256_rows(M):
+    """Layer shapes at row counts up to 256, on either side of the line between one SM and pairs of SMs: with and without K slices,
+    ragged last tiles, all three epilogues, twice (bit-identical: the K slices are summed in rank order)."""
     dec = _dec("bf16")
-    dec.debug_set(36, 1)
-    dec.debug_set(37, 256)
-    dec.debug_set(38, 1)
     f64 = lambda t: t.float().cpu().numpy().astype(np.float64)
     rtol = 1.0 / 128
     for (N, K) in ((4096, 4096), (12288, 4096), (1152, 512), (384, 256), (3584, 18944), (4608, 3584), (144, 192)):
@@ -269,12 +266,11 @@ def test_linear_bf16_operand_swapped_kernel(M):
 
 
 @pytest.mark.parametrize("case", [(130, 12288, 256, {}), (150, 12288, 320, {}), (192, 12288, 256, {}), (177, 9600, 192, {}),
-                                  (160, 12288, 256, {32: 256}), (193, 12288, 256, {}), (150, 12288, 256, {39: 0}),
-                                  (140, 12288, 512, {37: 0})])
-def test_linear_bf16_second_row_tile_of_64_rows(case):
-    """129..192 rows on two row tiles with unsplit tiles (the SwiGLU GEMM of a wide FFN): the second row tile runs 64-row
-    MMAs, whose accumulator rows sit in the lower half of every warp's tensor-memory lanes.  Also the neighbouring cases
-    that must not take that path (193 rows; the option off; plain epilogues with the operand-swapped kernel off)."""
+                                  (160, 12288, 256, {41: 256}), (193, 12288, 256, {}), (150, 12288, 256, {41: 128}),
+                                  (140, 12288, 512, {42: 1})])
+def test_linear_bf16_wide_ffn_just_above_one_row_tile(case):
+    """130 to 193 rows of a wide FFN: one row group on pairs of SMs, its second half partly or wholly empty, at the automatic tile
+    width and others, all three epilogues."""
     M, N, K, opts = case
     dec = _dec("bf16")
     for k, v in opts.items():
