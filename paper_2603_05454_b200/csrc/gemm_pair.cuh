@@ -15,8 +15,8 @@
 //   * Persistent: pair p takes every P-th tile (odd rounds in reverse order); the accumulators are double-buffered (2 x BN of 512 columns), so the
 //     epilogue of a tile overlaps the next tile's MMAs.
 //   * A last row group of at most 128 rows runs on 128-row MMAs (see pair_half_last).
-//   * BN is a run-time multiple of 32 (64 for the rotary epilogue), chosen so that the last wave of tiles is full (see
-//     pair_shape).
+//   * BN is a run-time multiple of 32 (64 for the rotary epilogue), the one with the least time by a model of a pair's
+//     intake over all rounds (see pair_shape); whole tiles are dealt, so the last round may still leave pairs idle.
 //   * The weight tile's two halves come from the two tensors / row ranges whose columns a fused epilogue pairs (gate and
 //     up, rotate-half partners), so CTA 0 always loads the first and CTA 1 the second of the pair.
 //   * Eight epilogue warps: two per quarter of the accumulator rows, each taking half of the 16-column chunks.  The
@@ -522,8 +522,8 @@ struct PairShape { int bn, ks; };
 // A last row group of at most 128 rows runs with 128-row MMAs (64 rows per CTA, which leave the tile's column halves in the two
 // halves of the lanes): 24 KB instead of 32 per SM and K atom at 256 columns and half the tensor work, about 0.75 of a tile's
 // time.
-// 1032 rows, 2 x 18944 x 3584: 222.5 -> 213.3 us; 3584 x 18944: 116.5 -> 114.5; 300 rows, 4096 x 12288: 43.4 -> 41.5, 4096 x 4096: 17.3
-// -> 16.5, 2 x 12288 x 4096 (now 256 columns wide): 74.8 -> 70.0.  The epilogues whose columns cannot be halved that way (rotary
+// 1032 rows, 2 x 18944 x 3584: 222.5 -> 209.4 us; 3584 x 18944: 116.5 -> 114.5; 300 rows, 4096 x 12288: 43.4 -> 41.5, 4096 x 4096: 17.3
+// -> 16.5, 2 x 12288 x 4096 (now 256 columns wide): 74.8 -> 68.6.  The epilogues whose columns cannot be halved that way (rotary
 // pairs inside a head, the head's partials per tile half) and widths that are no multiple of 64 keep 256-row MMAs.
 inline bool pair_half_last(int M, int bn) {
   const int last = M % PR_ROWS;

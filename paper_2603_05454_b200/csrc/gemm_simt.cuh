@@ -10,7 +10,9 @@
 // Measured (B200, fp32, us, k_gemm_simt -> k_gemm_simt_split): 65 x 384 (K 256) 15.2 -> 5.9, 128 x 256 (K 1024) 51 -> 14.8,
 // 300 x 2048 (K 1024; 160 tiles of 64 x 64) 97 -> 53, 1024 x 4096 (K 4096; 1024 tiles) 1007 -> over 1100: the line is drawn at
 // two 64 x 64 tiles per SM.  Four neighbouring lanes load a row's 64 bytes of a step (a row per lane cost four times the
-// cache lines per instruction: 18 us instead of 14.8), and sixteen warps per CTA gained nothing.
+// cache lines per instruction: 18 us instead of 14.8), and sixteen warps per CTA gained nothing.  Near the line two launches lose: the
+// head at 250 rows of 2048 ids (K 256) 22.0 -> 25.9 and bf16 1032 x 2 x 1024 (K 256) 49 -> 52; the split sums are the more exact ones
+// (p_max of that head 1.2e-6 from 64 bits, 4.4e-6 before), so the line stays.
 #pragma once
 #include "epilogues.cuh"
 

@@ -437,7 +437,9 @@ inline const CUtensorMap* umma_map5(UmmaState& st, const WeightView& v, int K, i
 constexpr int UM_HEAD_BN = 256;
 // More than 128 rows go to the pairs of SMs (gemm_pair.cuh).  With 129 to 256 rows (one row group) against the best kernels of
 // one SM per tile, at 187 / 256 rows, us: 12288 x 4096 29 -> 26, 37 -> 27; 4096 x 4096 16.6 -> 14.9, 19.2 -> 15.1; 2 x 12288 SwiGLU
-// 44 -> 45, 54 -> 46; 4096 x 12288 (three K slices) 30 -> 28.5; 3584 x 18944 38 -> 35.5; head 249 -> 222.
+// 44.7 -> 46.3, 52.7 -> 48.0; 4096 x 12288 (three K slices) 30 -> 28.5; 3584 x 18944 38 -> 35.5; head 249 -> 199.  (The SwiGLU of
+// 129 to 192 rows is the one launch that lost: 4 %, 43.3 -> 45.0 at 129.  Its MMAs span 256 rows whatever the row count, and its 128 tiles
+// are two rounds of 74 pairs; 64-row MMAs for a second row tile on one SM, which it had, followed the rows more closely.)
 inline bool umma_takes_pairs(int M) { return M > UM_BM; }
 // The head's kernel and tile.  Its scores leave in fp32, so the rounding of the sums over K shows: the tensor core truncates at
 // every step, and the error grows with the length of one accumulator's chain (scores of 4096 ids from K = 512, relative to
