@@ -47,7 +47,9 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # profiles/, keyed by kernel class: the captured launch's traffic and algorithmic bytes, and the hash of the kernel
 # sources the capture was taken on.  The class's launches differ in shape, and traffic grows in proportion to the
 # weight bytes streamed, so the reported figure is the class's mean algorithmic bytes per launch scaled by the
-# captured ratio.  A class whose sources changed since the capture reports null.
+# captured ratio.  A class whose sources changed since the capture reports null, and so do GEMMs and heads of more than 256
+# rows a launch on average (their flops per byte): there the weights are streamed once per band of rows, and no capture
+# stands for that.
 CLASS_SOURCES = {
     "gemm": ("gemm_stream.cuh", "gemm_pair.cuh", "gemm_umma.cuh", "epilogues.cuh", "common.cuh"),
     "head": ("gemm_stream.cuh", "gemm_pair.cuh", "gemm_umma.cuh", "epilogues.cuh", "common.cuh"),
@@ -254,7 +256,8 @@ def class_report(cnt, tms, peaks):
             e["bytes_per_launch"] = round(b / n) if n else None
         t = NCU_TRAFFIC.get(name)
         e["traffic"] = None
-        if t and n and name in work and t.get("src") == source_hash(name):
+        captured_regime = name not in ("gemm", "head") or work[name][1] <= 256 * work[name][0]
+        if t and n and name in work and captured_regime and t.get("src") == source_hash(name):
             e["traffic"] = round(work[name][0] / n * t["captured_bytes"] / t["algorithmic_bytes"])
         out[name] = e
     return out
