@@ -87,11 +87,10 @@ __device__ __forceinline__ int st_owner(int U, int G, int u) { return (int)(((un
 
 constexpr int ST_THREADS = 192;
 // Every CTA reads the same activations.  Were all to walk K from its start, the whole chip would ask for the same few lines of L2
-// at a time; so column tile t starts t * ST_ROT chunks later (and wraps): 12288 x 4096 at 100 rows 25.0 -> 23.2 us, 2 x 12288 x 4096
-// SwiGLU 37.5 -> 35.2, at 8 rows 35.2 -> 33.6.  An odd step, so that the starts of an even number of chunks cover all of them: with 4,
-// 2 x 18944 x 3584 (28 chunks, 7 starts) took 46.1 us at 8 rows, 44.9 without a rotation, 44.6 with 5.  The order depends on the tile
-// alone, so the CTAs that share a tile still cover it, and results do not depend on timing.
-constexpr int ST_ROT = 5;
+// at a time; so column tile t starts t * ST_ROT chunks later (and wraps): a LLaDA-shaped pass of 101 rows 4.25 -> 4.16 ms, of 9
+// rows 3.72 -> 3.68 (1 to 19 chunks: 4.15 to 4.23, 3.68 to 3.70).  The order depends on the tile alone, so the CTAs that share a
+// tile still cover it, and results do not depend on timing.
+constexpr int ST_ROT = 4;
 
 template <int BN, typename Epi>
 __global__ void __launch_bounds__(ST_THREADS, 1)
