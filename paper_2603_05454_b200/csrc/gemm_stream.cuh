@@ -697,17 +697,10 @@ inline size_t stream_scratch_bytes(int n_ctas, int bn) { return (size_t)n_ctas *
 // With a short K (at most 512) a slice would be a stage or two, and the reduction costs more than it saves, except where the
 // epilogue reads its output's old value (see no_split): 64 x 2 x 1024 SwiGLU 9.7 -> 7.2 us, 100 x 1024 6.8 -> 5.2, 64 x 4096
 // 6.2 -> 4.9 unsplit, but a residual update of 100 x 512 7.5 -> 8.0; from K = 1024 on the split wins (64 x 512 6.8, 8.9 without).
-// A dual epilogue of few rows splits all the same, its partial tiles being small and its tiles 256 wide.  SwiGLU up to 16 rows: 1 / 9
-// / 16 / 24 rows of 1024 pairs (K 512) 6.3 / 6.7 / 6.9 / 7.1 us split, 7.4 / 7.4 / 7.3 / 7.3 whole.  The rotary projection as long as its
-// tiles are that wide, 32 rows: eight layers (d 512, 4 heads of 128) at 3 / 16 / 31 rows 355 / 374 / 384 -> 332 / 354 / 371 us; 128-wide
-// ones at 68 rows 378 -> 385.
 // The head, with few tiles and a short K, comes here with at most 8 rows (umma_head_shape) and keeps the split: 4 rows of 4096 ids
 // 15.1 -> 12.9 us, and the shorter sums are more exact.
 template <typename Epi>
-bool stream_no_split(int M, int K) {
-  if (Epi::kDual && M <= (std::is_same<Epi, EpiSwiGLU<bf16>>::value ? 16 : 32)) return false;
-  return K <= 512 && !Epi::kReduce && !std::is_same<Epi, EpiResidual<bf16>>::value;
-}
+bool stream_no_split(int K) { return K <= 512 && !Epi::kReduce && !std::is_same<Epi, EpiResidual<bf16>>::value; }
 inline int stream_splits(const UmmaState& st, long n_tiles, bool no_split) {
   int splits = n_tiles <= st.n_sm ? (int)(st.n_sm / n_tiles) : 0;
   if (no_split && splits > 1) return 1;
@@ -804,7 +797,7 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
   const int n_tiles = (NP + per_tile - 1) / per_tile;
   const int kc = K / (sh.atoms * UM_BK);
   const long T = n_tiles;
-  int grid = stream_grid(st, (int)T, BN, stream_no_split<Epi>(M, K));
+  int grid = stream_grid(st, (int)T, BN, stream_no_split<Epi>(K));
   if (grid > T * kc) grid = (int)(T * kc);
   if ((double)T * kc * (grid + 1) >= 4.0e9) { st.err = "too many work units for the streaming GEMM"; return -9; }   // 32-bit unit arithmetic
   // K slices of one tile on the CTAs of one cluster: the reduction then stays on chip
@@ -830,7 +823,7 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
 template <typename Epi>
 bool stream_can(const UmmaState& st, int M, int NP, int K, int bn) {
   const long T = (NP + (Epi::kDual ? bn / 2 : bn) - 1) / (Epi::kDual ? bn / 2 : bn);
-  if (st.scratch == nullptr || T > st.n_counters || stream_scratch_bytes(stream_grid(st, (int)T, bn, stream_no_split<Epi>(M, K)), bn) > st.scratch_bytes)
+  if (st.scratch == nullptr || T > st.n_counters || stream_scratch_bytes(stream_grid(st, (int)T, bn, stream_no_split<Epi>(K)), bn) > st.scratch_bytes)
     return false;
   return stream_shape(st, M, bn, K).stages >= 2;
 }

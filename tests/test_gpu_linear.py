@@ -405,8 +405,7 @@ def test_linear_bf16_one_row_group_on_pairs(M, N, K):
     dec.close()
 
 
-@pytest.mark.parametrize("M,N,K", [(1, 512, 64), (64, 1024, 512), (128, 272, 448), (33, 4096, 512), (100, 1024, 576),
-                                   (16, 1024, 512), (17, 1024, 512), (9, 208, 192)])
+@pytest.mark.parametrize("M,N,K", [(1, 512, 64), (64, 1024, 512), (128, 272, 448), (33, 4096, 512), (100, 1024, 576)])
 def test_linear_bf16_short_k_without_a_split(M, N, K):
     """At most 512 elements of K: whole tiles per CTA instead of K slices on clusters (the last case is beyond the line)."""
     dec = _dec("bf16")
