@@ -697,6 +697,9 @@ inline size_t stream_scratch_bytes(int n_ctas, int bn) { return (size_t)n_ctas *
 // With a short K (at most 512) a slice would be a stage or two, and the reduction costs more than it saves, except where the
 // epilogue reads its output's old value (see no_split): 64 x 2 x 1024 SwiGLU 9.7 -> 7.2 us, 100 x 1024 6.8 -> 5.2, 64 x 4096
 // 6.2 -> 4.9 unsplit, but a residual update of 100 x 512 7.5 -> 8.0; from K = 1024 on the split wins (64 x 512 6.8, 8.9 without).
+// With few rows a dual epilogue, whose tiles are 256 wide, loses by it: SwiGLU of 1024 pairs (K 512) at 1 / 9 / 16 / 24 rows 6.3 / 6.7 / 6.9 /
+// 7.1 us split, 7.4 / 7.4 / 7.3 / 7.3 whole, eight layers (d 512) at 3 rows 332 and 355.  It stays whole at every row count: a sum whose
+// order changed with the rows moved near-tied predictions of such a model (one token in five of sixty decodes).
 // The head, with few tiles and a short K, comes here with at most 8 rows (umma_head_shape) and keeps the split: 4 rows of 4096 ids
 // 15.1 -> 12.9 us, and the shorter sums are more exact.
 template <typename Epi>
