@@ -58,13 +58,13 @@ CLASS_SOURCES = {
 }
 NCU_TRAFFIC = {
     # k_gemm_stream<128,EpiStore>, M 64, N 12288, K 4096: profiles/k_gemm_stream_M64_N12288_K4096.md
-    "gemm": {"captured_bytes": 104.57e6, "algorithmic_bytes": 102.8e6, "src": "81843e54038f"},
+    "gemm": {"captured_bytes": 104.38e6, "algorithmic_bytes": 102.8e6, "src": "8a89cf02e57d"},
     # k_gemm_stream<256,EpiHead>, 64 rows: profiles/k_gemm_stream_head_M64_V126464.md
-    "head": {"captured_bytes": 1062.4e6, "algorithmic_bytes": 1037.0e6, "src": "81843e54038f"},
+    "head": {"captured_bytes": 1062.3e6, "algorithmic_bytes": 1037.0e6, "src": "8a89cf02e57d"},
     # k_attn_umma, 16 x (128 query rows over 2048 keys): profiles/k_attn_umma_B16_F1920.md
-    "attn": {"captured_bytes": 571.1e6, "algorithmic_bytes": 570.4e6, "src": "37f095fbf04d"},
+    "attn": {"captured_bytes": 569.5e6, "algorithmic_bytes": 570.4e6, "src": "f9ea95f59873"},
     # k_commit_append of a 16 x 1920-row prompt block: profiles/k_commit_append_prompt_B16_P1920.md
-    "commit": {"captured_bytes": 1967.9e6, "algorithmic_bytes": 2013.3e6, "src": "c5793f4afff8"},
+    "commit": {"captured_bytes": 1968.2e6, "algorithmic_bytes": 2013.3e6, "src": "f4033b225a27"},
 }
 
 
