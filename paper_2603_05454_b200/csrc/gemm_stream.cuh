@@ -24,7 +24,13 @@
 // tensor maps, gemm_umma.cuh): against a lane branch and a copy per half tile and K atom 2 x 12288 x 4096 SwiGLU at 101 rows
 // 38.7 -> 35.5 us, 12288 x 4096 25.7 -> 24.7, 3584 x 18944 at 9 rows 28.8 -> 26.4; a LLaDA-shaped pass of 9 rows
 // 4.20 -> 3.95 ms, of 101 rows 4.82 -> 4.51.
-// Warp roles (192 threads): warp 0 = TMA producer, warp 1 = TMEM allocator + MMA issuer, warps 2..5 = epilogue.
+// The activations have a producer of their own: where the preceding kernel has just ended (the O and down projections start when
+// its CTAs leave the SMs) their first request would queue behind the 200 KB of weights that fill the ring, and the first MMA came 5 us
+// after the launch's start instead of 3 (a LLaDA-shaped pass of 9 rows 3.74 -> 3.63 ms, of 101 rows 4.28 -> 4.19).  And the issuer looks at
+// the next stage between this one's MMAs: waiting for it behind the commit leaves the tensor pipe empty meanwhile (8 MMAs of 128 columns
+// 749 -> 659 cycles a stage; the passes another 2 to 4 %).
+// Warp roles (224 threads): warp 0 = TMA producer of the weights, warp 6 = of the activations, warp 1 = TMEM allocator + MMA issuer,
+// warps 2..5 = epilogue.
 // Every wait is bounded; on expiry the kernel records (code, site) in the status word, drains and returns.
 #pragma once
 #include <algorithm>
@@ -85,7 +91,7 @@ __device__ __forceinline__ int st_first_unit(int U, int G, int g) { return (int)
 // CTA that owns unit u
 __device__ __forceinline__ int st_owner(int U, int G, int u) { return (int)(((unsigned)(u + 1) * (unsigned)G + (unsigned)U - 1u) / (unsigned)U) - 1; }
 
-constexpr int ST_THREADS = 192;
+constexpr int ST_THREADS = 224;
 // Every CTA reads the same activations.  Were all to walk K from its start, the whole chip would ask for the same few lines of L2
 // at a time; so column tile t starts t * ST_ROT chunks later (and wraps): a LLaDA-shaped pass of 101 rows 4.25 -> 4.16 ms, of 9
 // rows 3.72 -> 3.68 (1 to 19 chunks: 4.15 to 4.23, 3.68 to 3.70).  The order depends on the tile alone, so the CTAs that share a
@@ -160,6 +166,19 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         tma_load_5d(sb + a * B_ATOM + B_HALF_ATOM, &map_b1, r0, blk, 0, a0 + a, full_bar(s));
       }
     }
+  // The weights are never written by any kernel, so the first stages' weight tiles can be requested at once, while a preceding
+  // kernel (launched with programmatic serialisation) is still running: the first one here, the others after the set-up's
+  // barrier, which nobody is to wait for them at (a full ring's requests take the copy engine 2 us).
+  Pos pw;
+  pos_set(pw, u0);
+  auto request_weights = [&](int s) {
+    if (elect_one()) {
+      mbar_expect_tx(full_bar(s), STAGE_BYTES);
+      load_weights(pw, s);
+    }
+    __syncwarp();
+    pos_next(pw);
+  };
   };
   auto load_acts = [&](const Pos& p, int s) {
     tma_load_4d(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_a, 0, 0, chunk(p) * AT, full_bar(s));
@@ -181,20 +200,8 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 0) {
-    // The weights are never written by any kernel, so the first stages' weight tiles can be requested at once, while a
-    // preceding kernel (launched with programmatic serialisation) is still running; the activations follow after
-    // pdl_wait().  This warp is also the producer below.
     __syncwarp();
-    Pos p;
-    pos_set(p, u0);
-    for (int it = 0; it < n_pre; ++it) {
-      if (elect_one()) {
-        mbar_expect_tx(full_bar(it), STAGE_BYTES);
-        load_weights(p, it);
-      }
-      __syncwarp();
-      pos_next(p);
-    }
+    if (n_pre > 0) request_weights(0);
   }
   if (threadIdx.x == 64) tma_prefetch_map(&map_a);      // its first use comes right after pdl_wait()
   if (warp == 1) {
@@ -207,33 +214,43 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_wait();          // barriers and tensor memory are set up; from here on the kernel reads what its predecessor wrote
-
+  // barriers and tensor memory are set up; every role waits for the preceding kernel before it reads what that wrote, and before
+  // its first bounded wait
   if (warp == 0) {
-    // ---------------- TMA producer: one uninterrupted stream over this CTA's units ----------------
-    int issued = 0;
+  } else if (warp == 6) {
+    // ---------------- TMA producer of the activations ----------------
+    // (the same stages in the same order; they may arrive ahead of the stage's arming: its phase ends with both.  A warp of its
+    // own: behind the weights that fill the ring its first request would wait 2 us.)
+    pdl_wait();
+    if (kRope) pdl_release();        // the attention that follows reads older keys and values ahead of its own wait
     Pos p;
     pos_set(p, u0);
     int s = 0;
     uint32_t ph = 0;
     for (int it = 0; it < n_units; ++it) {
-      if (it >= n_pre) {
-        if (!__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, abort_flag))) {
-          if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 11u; }
-          break;
-        }
+      if (it >= n_pre && !__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, abort_flag))) {
+        if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 15u; }
+        break;
       }
-      if (elect_one()) {
-        if (it >= n_pre) {                   // else the stage is armed and its weights are on their way
-          mbar_expect_tx(full_bar(s), STAGE_BYTES);
-          load_weights(p, s);
-        }
-        load_acts(p, s);
-      }
+      if (elect_one()) load_acts(p, s);
       __syncwarp();
-      ++issued;
       if (++s == S) { s = 0; ph ^= 1u; }
       pos_next(p);
+    }
+    // ---------------- TMA producer of the weights: one uninterrupted stream over this CTA's units ----------------
+    for (int it = 1; it < n_pre; ++it) request_weights(it);
+    pdl_wait();
+      pdl_wait();
+    int issued = n_pre, s = 0;
+    uint32_t ph = 1;
+    for (int it = n_pre; it < n_units; ++it) {
+      if (!__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, abort_flag))) {
+        if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 11u; }
+        break;
+      }
+      request_weights(s);
+      ++issued;
+      if (++s == S) { s = 0; ph ^= 1u; }
     }
     // do not leave while copies may still be landing in this CTA's shared memory
     const int first = issued > S ? issued - S : 0;
@@ -246,7 +263,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     {
       constexpr uint32_t idesc = make_idesc(BN);
       int seg = 0;
-      bool ok = true;
+      bool ok = true, ready = false;           // ready: stage s has been seen full
       int s = 0;
       uint32_t ph = 0;
       for (int u = u0; u < u1 && ok;) {
@@ -260,10 +277,19 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
           break;
         }
         tc_fence_after();
+            __syncwarp();
+            acc = 1;
+          }
+          // the next stage is looked at between this one's MMAs, while the tensor pipe still has work
+          ready = __all_sync(0xffffffffu, mbar_test(full_bar(s2), ph2));
+          if (elect_one()) {
+            const uint64_t da = make_smem_desc(sa + (AT - 1) * A_ATOM), db = make_smem_desc(sb + (AT - 1) * B_ATOM);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tc_mma_f16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, acc | (uint32_t)k);
         const uint32_t d_tmem = tmem_base + (uint32_t)(buf * SET_COLS);
         uint32_t acc = 0;                               // 0: the segment's first MMA overwrites the accumulator
         for (; u < seg_end; ++u) {
-          ok = __all_sync(0xffffffffu, mbar_wait(full_bar(s), ph, abort_flag));
+          if (!ready) ok = __all_sync(0xffffffffu, mbar_wait(full_bar(s), ph, abort_flag));
           if (!ok) {
             if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 13u; }
             break;
@@ -271,20 +297,23 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
           tc_fence_after();
           const uint32_t sa = smem_u32(smem + (size_t)s * STAGE_BYTES);
           const uint32_t sb = sa + AT * A_ATOM;
-          if (elect_one()) {
-            for (int j = 0; j < AT; ++j) {
-              const uint64_t da = make_smem_desc(sa + j * A_ATOM);
-              const uint64_t db = make_smem_desc(sb + j * B_ATOM);
+          int s2 = s + 1;
+          uint32_t ph2 = ph;
+    pdl_wait();
+          if (s2 == S) { s2 = 0; ph2 ^= 1u; }
+          if (AT == 2) {
+            if (elect_one()) {
+              const uint64_t da = make_smem_desc(sa), db = make_smem_desc(sb);
 #pragma unroll
-              for (int k = 0; k < 4; ++k)
-                tc_mma_f16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, acc | (uint32_t)(j | k));
+              for (int k = 0; k < 4; ++k) tc_mma_f16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, acc | (uint32_t)k);
             }
             tc_commit(empty_bar(s));
             if (u == seg_end - 1) tc_commit(accf_bar(buf));
           }
           __syncwarp();
           acc = 1;
-          if (++s == S) { s = 0; ph ^= 1u; }
+          s = s2;
+          ph = ph2;
         }
         ++seg;
       }
