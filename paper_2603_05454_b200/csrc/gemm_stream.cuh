@@ -166,19 +166,6 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         tma_load_5d(sb + a * B_ATOM + B_HALF_ATOM, &map_b1, r0, blk, 0, a0 + a, full_bar(s));
       }
     }
-  // The weights are never written by any kernel, so the first stages' weight tiles can be requested at once, while a preceding
-  // kernel (launched with programmatic serialisation) is still running: the first one here, the others after the set-up's
-  // barrier, which nobody is to wait for them at (a full ring's requests take the copy engine 2 us).
-  Pos pw;
-  pos_set(pw, u0);
-  auto request_weights = [&](int s) {
-    if (elect_one()) {
-      mbar_expect_tx(full_bar(s), STAGE_BYTES);
-      load_weights(pw, s);
-    }
-    __syncwarp();
-    pos_next(pw);
-  };
   };
   auto load_acts = [&](const Pos& p, int s) {
     tma_load_4d(smem_u32(smem + (size_t)s * STAGE_BYTES), &map_a, 0, 0, chunk(p) * AT, full_bar(s));
@@ -199,6 +186,19 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  // The weights are never written by any kernel, so the first stages' weight tiles can be requested at once, while a preceding
+  // kernel (launched with programmatic serialisation) is still running: the first one here, the others after the set-up's
+  // barrier, which nobody is to wait for them at (a full ring's requests take the copy engine 2 us).
+  Pos pw;
+  pos_set(pw, u0);
+  auto request_weights = [&](int s) {
+    if (elect_one()) {
+      mbar_expect_tx(full_bar(s), STAGE_BYTES);
+      load_weights(pw, s);
+    }
+    __syncwarp();
+    pos_next(pw);
+  };
   if (warp == 0) {
     __syncwarp();
     if (n_pre > 0) request_weights(0);
@@ -217,30 +217,9 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
   // barriers and tensor memory are set up; every role waits for the preceding kernel before it reads what that wrote, and before
   // its first bounded wait
   if (warp == 0) {
-  } else if (warp == 6) {
-    // ---------------- TMA producer of the activations ----------------
-    // (the same stages in the same order; they may arrive ahead of the stage's arming: its phase ends with both.  A warp of its
-    // own: behind the weights that fill the ring its first request would wait 2 us.)
-    pdl_wait();
-    if (kRope) pdl_release();        // the attention that follows reads older keys and values ahead of its own wait
-    Pos p;
-    pos_set(p, u0);
-    int s = 0;
-    uint32_t ph = 0;
-    for (int it = 0; it < n_units; ++it) {
-      if (it >= n_pre && !__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, abort_flag))) {
-        if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 15u; }
-        break;
-      }
-      if (elect_one()) load_acts(p, s);
-      __syncwarp();
-      if (++s == S) { s = 0; ph ^= 1u; }
-      pos_next(p);
-    }
     // ---------------- TMA producer of the weights: one uninterrupted stream over this CTA's units ----------------
     for (int it = 1; it < n_pre; ++it) request_weights(it);
     pdl_wait();
-      pdl_wait();
     int issued = n_pre, s = 0;
     uint32_t ph = 1;
     for (int it = n_pre; it < n_units; ++it) {
@@ -258,9 +237,29 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       volatile uint32_t no_abort = 0;
       mbar_wait(full_bar((int)(it % S)), (uint32_t)(it / S) & 1u, &no_abort);
     }
+  } else if (warp == 6) {
+    // ---------------- TMA producer of the activations ----------------
+    // (the same stages in the same order; they may arrive ahead of the stage's arming: its phase ends with both.  A warp of its
+    // own: behind the weights that fill the ring its first request would wait 2 us.)
+    pdl_wait();
+    Pos p;
+    pos_set(p, u0);
+    int s = 0;
+    uint32_t ph = 0;
+    for (int it = 0; it < n_units; ++it) {
+      if (it >= n_pre && !__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, abort_flag))) {
+        if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 15u; }
+        break;
+      }
+      if (elect_one()) load_acts(p, s);
+      __syncwarp();
+      if (++s == S) { s = 0; ph ^= 1u; }
+      pos_next(p);
+    }
   } else if (warp == 1) {
     // ---------------- MMA issuer (the whole warp waits, one elected thread issues) ----------------
     {
+      pdl_wait();
       constexpr uint32_t idesc = make_idesc(BN);
       int seg = 0;
       bool ok = true, ready = false;           // ready: stage s has been seen full
@@ -277,15 +276,6 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
           break;
         }
         tc_fence_after();
-            __syncwarp();
-            acc = 1;
-          }
-          // the next stage is looked at between this one's MMAs, while the tensor pipe still has work
-          ready = __all_sync(0xffffffffu, mbar_test(full_bar(s2), ph2));
-          if (elect_one()) {
-            const uint64_t da = make_smem_desc(sa + (AT - 1) * A_ATOM), db = make_smem_desc(sb + (AT - 1) * B_ATOM);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) tc_mma_f16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, acc | (uint32_t)k);
         const uint32_t d_tmem = tmem_base + (uint32_t)(buf * SET_COLS);
         uint32_t acc = 0;                               // 0: the segment's first MMA overwrites the accumulator
         for (; u < seg_end; ++u) {
@@ -299,7 +289,6 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
           const uint32_t sb = sa + AT * A_ATOM;
           int s2 = s + 1;
           uint32_t ph2 = ph;
-    pdl_wait();
           if (s2 == S) { s2 = 0; ph2 ^= 1u; }
           if (AT == 2) {
             if (elect_one()) {
@@ -307,6 +296,15 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
 #pragma unroll
               for (int k = 0; k < 4; ++k) tc_mma_f16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, acc | (uint32_t)k);
             }
+            __syncwarp();
+            acc = 1;
+          }
+          // the next stage is looked at between this one's MMAs, while the tensor pipe still has work
+          ready = __all_sync(0xffffffffu, mbar_test(full_bar(s2), ph2));
+          if (elect_one()) {
+            const uint64_t da = make_smem_desc(sa + (AT - 1) * A_ATOM), db = make_smem_desc(sb + (AT - 1) * B_ATOM);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tc_mma_f16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, acc | (uint32_t)k);
             tc_commit(empty_bar(s));
             if (u == seg_end - 1) tc_commit(accf_bar(buf));
           }
@@ -320,6 +318,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     }
   } else {
     // ---------------- epilogue (warps 2..5) ----------------
+    pdl_wait();
     const int q = warp & 3;
     const int r_in = q * 32 + lane;                       // accumulator lane this thread reads
     constexpr int CH = Epi::kDual ? HALF : BN;            // pair indices (dual) or columns (plain) per tile
