@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(AU_THREADS, 1)
 k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_ck,
             const __grid_constant__ CUtensorMap map_cv, const __grid_constant__ CUtensorMap map_sk,
             const __grid_constant__ CUtensorMap map_sv, bf16* __restrict__ out, StepDesc sd, int n_heads, int n_kv_heads, int max_len,
-            float scale_log2, int cluster, int inplace, unsigned* status) {
+            float scale_log2, int cluster, int inplace, int early, unsigned* status) {
   constexpr int DH = 128;
   extern __shared__ uint8_t smem_raw[];
   pdl_release();
@@ -173,7 +173,11 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   // tensor memory columns: O of group 0 at 0, O of group 1 at 128, S buffer s at 256 + 128 s
-  pdl_wait();
+  // early: the kernel before this one is the QKV projection, which releases this launch only after its own wait.  Everything
+  // older than it is complete then: the descriptor and the cached keys and values are read while it still runs.  In a small pass
+  // the queries were there 2.4 us after the wait and the first keys 3.5 (of 11.5 in all); LLaDA-shaped passes of 9 / 101 / 187 rows
+  // 3.63 -> 3.57, 4.17 -> 4.13, 5.21 -> 5.15 ms.
+  if (!early) pdl_wait();
 
   const int r0 = sd.row_off[b];
   const int Qn = sd.row_off[b + 1] - r0;
@@ -195,22 +199,9 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     // ---------------- TMA producers: one warp streams the K tiles, another the V tiles (one elected thread issues) ----------------
     const bool is_v = warp == AU_W_TMAV;
     const int full = is_v ? B_VF : B_KF, empty = is_v ? B_VE : B_KE;
-    int issued = 0;
-    if (!is_v && n_tiles > 0 && elect_one()) {
-      // the Q tile (positions past the sequence's end bring other rows or zeros; rows are independent and those are never
-      // stored)
-      mbar_expect_tx(bar(B_Q), (uint32_t)(pos_tile * G * 256));
-      tma_load_5d_q(smem_u32(Qs), &map_q, kvh, r0 + pos0, 0, bar(B_Q));
-      tma_load_5d_q(smem_u32(Qs) + AU_ATOM, &map_q, kvh, r0 + pos0, 1, bar(B_Q));
-    }
-    __syncwarp();
-    for (int t = 0; t < n_tiles; ++t) {
-      const int s = t & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(bar(empty + s), ((uint32_t)(t >> 1) & 1u) ^ 1u, abort_flag))) {
-        if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 21u; }
-        break;
-      }
+    auto load_tile = [&](int t) {
       if (elect_one()) {
+        const int s = t & 1;
         mbar_expect_tx(bar(full + s), AU_TILE);
         const uint32_t dst = smem_u32(KVs + (size_t)s * 2 * AU_TILE) + (is_v ? AU_TILE : 0);
         const int gt = rank + t * C;                    // tile index in the sequence's key range
@@ -221,6 +212,26 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         tma_load_2d(dst + AU_ATOM, mp, kvh * DH + 64, row, bar(full + s));
       }
       __syncwarp();
+    };
+    // the first tiles, as far as no row of theirs is written by the QKV projection
+    int issued = 0;
+    if (early)
+      while (issued < min(2, n_tiles) && (inplace ? (rank + issued * C + 1) * AU_BN <= F - Qn : rank + issued * C < n_c)) load_tile(issued++);
+    pdl_wait();
+    if (!is_v && n_tiles > 0 && elect_one()) {
+      // the Q tile (positions past the sequence's end bring other rows or zeros; rows are independent and those are never
+      // stored)
+      mbar_expect_tx(bar(B_Q), (uint32_t)(pos_tile * G * 256));
+      tma_load_5d_q(smem_u32(Qs), &map_q, kvh, r0 + pos0, 0, bar(B_Q));
+      tma_load_5d_q(smem_u32(Qs) + AU_ATOM, &map_q, kvh, r0 + pos0, 1, bar(B_Q));
+    }
+    __syncwarp();
+    for (int t = issued; t < n_tiles; ++t) {
+      if (!__all_sync(0xffffffffu, mbar_wait(bar(empty + (t & 1)), ((uint32_t)(t >> 1) & 1u) ^ 1u, abort_flag))) {
+        if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 21u; }
+        break;
+      }
+      load_tile(t);
       ++issued;
     }
     // do not leave while copies may still be landing in this CTA's shared memory
@@ -230,6 +241,7 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   } else if (warp == AU_W_QK) {
     // ---------------- MMA issuer 1: S = Q K^T of every tile (the whole warp waits, one elected thread issues: a lane branch
     // around the MMAs would cost more than they take, see elect_one) ----------------
+    pdl_wait();
     constexpr uint32_t idesc_qk = make_idesc(AU_BN);
     bool ok = n_tiles == 0 || __all_sync(0xffffffffu, mbar_wait(bar(B_Q), 0u, abort_flag));
     if (!ok && lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(status, 1u); status[1] = 26u; }
@@ -258,6 +270,7 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     }
   } else if (warp == AU_W_PV) {
     // ---------------- MMA issuer 2: O_w += P_w V of every tile (w = tile parity) ----------------
+    pdl_wait();
     constexpr uint32_t idesc_pv = make_idesc(DH) | (1u << 16);          // B operand (V) is MN-major
     for (int t = 0; t < n_tiles; ++t) {
       const int s = t & 1;                  // K/V stage, S buffer and softmax group of this tile
@@ -284,6 +297,7 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   } else {
     // ---------------- softmax (two groups of four warps, one row per thread; group w takes the tiles of parity w, with
     // its own running maximum, row sum and accumulator O_w) and, for group 0, the epilogue ----------------
+    pdl_wait();
     const int w = warp >> 2;                           // softmax group
     const int r = threadIdx.x & 127;
     const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);

@@ -91,10 +91,10 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ CUtensorMap map_ah,
             const __grid_constant__ CUtensorMap map_h0, const __grid_constant__ CUtensorMap map_h1, PairArgs args, Epi epi) {
   extern __shared__ uint8_t smem_raw[];
-  pdl_release();
   constexpr int A_ATOM = UM_BM * 128;                     // this CTA's 128 activation rows of one K atom
   constexpr uint32_t TMEM_COLS = 512;
   constexpr bool kRope = std::is_same<Epi, EpiQKVRope<bf16>>::value;
+  if (!kRope) pdl_release();
   const int BN = args.bn, HALF = BN / 2;
   const int B_ATOM = HALF * 128;
   const int STAGE_BYTES = 2 * (A_ATOM + B_ATOM);          // two K atoms
@@ -204,6 +204,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       }
     }
     pdl_wait();
+    if (kRope) pdl_release();        // the attention that follows reads older keys and values ahead of its own wait
     int s = 0, issued = 0;
     uint32_t ph = 0;
     bool ok = true;

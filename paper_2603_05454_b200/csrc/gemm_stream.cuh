@@ -103,8 +103,8 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
 k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b0,
               const __grid_constant__ CUtensorMap map_b1, StreamArgs args, Epi epi) {
   extern __shared__ uint8_t smem_raw[];
-  pdl_release();
   constexpr bool kRope = std::is_same<Epi, EpiQKVRope<bf16>>::value;
+  if (!kRope) pdl_release();
   constexpr int HALF = BN / 2;
   constexpr int B_HALF_ATOM = HALF * 128;               // bytes of one half-tile atom (64 K elements)
   constexpr int B_ATOM = BN * 128;
@@ -242,6 +242,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     // (the same stages in the same order; they may arrive ahead of the stage's arming: its phase ends with both.  A warp of its
     // own: behind the weights that fill the ring its first request would wait 2 us.)
     pdl_wait();
+    if (kRope) pdl_release();        // the attention that follows reads older keys and values ahead of its own wait
     Pos p;
     pos_set(p, u0);
     int s = 0;

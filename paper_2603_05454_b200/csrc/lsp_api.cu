@@ -330,9 +330,10 @@ int check_status(lsp_ctx* c) {
 
 // Suffix-over-prefix attention of layer l (Sec. 3.2: every query row of the pass sees the cached prefix [0, F_b) and all
 // of the pass's own rows).  Reads the uploaded descriptor (F, row_off), Q from q, K/V from the cache and the staging
-// planes of layer l; writes out.  q_rows: rows of Qb.  max_q: most query rows of one sequence; max_keys: most keys of one sequence.
+// planes of layer l; writes out.  early: the launch before it is the tcgen05 QKV projection of the same layer (see k_attn_umma).
+// q_rows: rows of Qb.  max_q: most query rows of one sequence; max_keys: most keys of one sequence.
 template <typename T>
-int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const StepDesc& sd, int B, int maxQ, int max_keys, int inplace) {
+int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const StepDesc& sd, int B, int maxQ, int max_keys, int inplace, int early) {
   const lsp_model_cfg& m = c->m;
   const int dh = m.head_dim, kvd = m.n_kv_heads * dh;
   const size_t plane = (size_t)c->max_rows * kvd;
@@ -370,7 +371,7 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const Step
       // at most two key tiles per CTA: the kernel with rolled softmax loops
       auto kern = (max_keys + AU_BN - 1) / AU_BN <= 2 * cl ? k_attn_umma<true> : k_attn_umma<false>;
       launch_k(c->pdl, kern, g3, dim3(AU_THREADS), (size_t)AU_SMEM, c->stream, cl, map_q, mp[0], mp[1], mp[2], mp[3],
-               Att, sd, m.n_heads, m.n_kv_heads, c->max_len, sl2, cl, inplace, c->d_status);
+               Att, sd, m.n_heads, m.n_kv_heads, c->max_len, sl2, cl, inplace, early, c->d_status);
       c->last_attn_kernel = 2;
       c->last_attn_cluster = cl;
       done = true;
@@ -462,7 +463,8 @@ int enqueue_pass(lsp_ctx* c, const StepDesc& sd, const DescInline& din, int B, c
     {
       c->counters[CNT_ATTN_BYTES] += pd.attn_bytes;
       c->counters[CNT_ATTN_FLOPS] += pd.attn_flops;
-      const int rc = run_attention<T>(c, l, Qb, M, Att, sd, B, pd.maxQ, pd.max_keys, c->kv_inplace);
+      const int rc = run_attention<T>(c, l, Qb, M, Att, sd, B, pd.maxQ, pd.max_keys, c->kv_inplace,
+                                      c->gemm_impl == 1 ? 1 : 0);
       if (rc) return rc;
     }
     {
@@ -1244,8 +1246,8 @@ int lsp_op_attention(lsp_ctx* c, int layer, const void* q, const void* k_new, co
   char* stK = c->stage + (size_t)(2 * layer) * plane;
   CU(cudaMemcpyAsync(stK, k_new, (size_t)M * kvd * c->esz, cudaMemcpyDeviceToDevice, c->stream));
   CU(cudaMemcpyAsync(stK + plane, v_new, (size_t)M * kvd * c->esz, cudaMemcpyDeviceToDevice, c->stream));
-  const int rc = c->m.dtype == 0 ? run_attention<float>(c, layer, (const float*)q, M, (float*)out, desc_of(c), batch, maxQ, max_keys, 0)
-                                 : run_attention<bf16>(c, layer, (const bf16*)q, M, (bf16*)out, desc_of(c), batch, maxQ, max_keys, 0);
+  const int rc = c->m.dtype == 0 ? run_attention<float>(c, layer, (const float*)q, M, (float*)out, desc_of(c), batch, maxQ, max_keys, 0, 0)
+                                 : run_attention<bf16>(c, layer, (const bf16*)q, M, (bf16*)out, desc_of(c), batch, maxQ, max_keys, 0, 0);
   if (rc) return rc;
   CU(cudaMemcpyAsync(c->h_status, c->d_status, 16, cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
