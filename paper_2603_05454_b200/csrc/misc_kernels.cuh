@@ -114,50 +114,62 @@ __global__ void __launch_bounds__(RN_THREADS) k_rmsnorm(const T* x, const T* __r
       }
     }
   }
-  pdl_wait();
-  const uint4* xr = reinterpret_cast<const uint4*>(x + (size_t)(src_rows ? src_rows[r] : r) * d);
-  if (in_regs) {
+  // With early gains the row's code runs once ahead of the wait, on the gains in place of the row and storing nothing: its
+  // instructions then wait in the SM instead of being fetched, behind a stream of weights, once the row is there (LLaDA-shaped passes
+  // of 9 / 40 / 101 rows 3.60 -> 3.56, 3.86 -> 3.82, 4.19 -> 4.16 ms).
+  float inv = 0.f;
+#pragma unroll 1
+  for (int turn = kEarly && in_regs ? 0 : 1; turn < 2; ++turn) {
+    if (turn == 1) pdl_wait();
+    const uint4* xr = turn == 1 ? reinterpret_cast<const uint4*>(x + (size_t)(src_rows ? src_rows[r] : r) * d) : gr;
+    ss = 0.f;
+    if (in_regs) {
 #pragma unroll
-    for (int j = 0; j < RN_VPT; ++j) {
-      const int i = threadIdx.x + j * RN_THREADS;
-      keep[j] = (i < nv) ? xr[i] : make_uint4(0u, 0u, 0u, 0u);
-    }
+      for (int j = 0; j < RN_VPT; ++j) {
+        const int i = threadIdx.x + j * RN_THREADS;
+        keep[j] = (i < nv) ? xr[i] : make_uint4(0u, 0u, 0u, 0u);
+      }
 #pragma unroll
-    for (int j = 0; j < RN_VPT; ++j) {
-      float v[E];
-      vec_to_f(keep[j], v);
-#pragma unroll
-      for (int e = 0; e < E; ++e) ss += v[e] * v[e];
-    }
-  } else {
-    for (int i = threadIdx.x; i < nv; i += RN_THREADS) {
-      float v[E];
-      vec_to_f(xr[i], v);
-#pragma unroll
-      for (int e = 0; e < E; ++e) ss += v[e] * v[e];
-    }
-  }
-  ss = warp_sum(ss);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  float tot = 0.f;
-#pragma unroll
-  for (int w = 0; w < RN_THREADS / 32; ++w) tot += red[w];      // same order in every thread
-  const float inv = rsqrtf(__fdividef(tot, (float)d) + eps);      // fast division: no IEEE slow-path subroutine in the kernel
-  if (in_regs) {
-#pragma unroll
-    for (int j = 0; j < RN_VPT; ++j) {
-      const int i = threadIdx.x + j * RN_THREADS;
-      if (i < nv) {
-        float v[E], gv[E];
+      for (int j = 0; j < RN_VPT; ++j) {
+        float v[E];
         vec_to_f(keep[j], v);
-        vec_to_f(kEarly ? gain[kEarly ? j : 0] : __ldg(gr + i), gv);
 #pragma unroll
-        for (int e = 0; e < E; ++e) v[e] = v[e] * inv * gv[e];
-        o[i] = f_to_vec(v);
+        for (int e = 0; e < E; ++e) ss += v[e] * v[e];
+      }
+    } else {
+      for (int i = threadIdx.x; i < nv; i += RN_THREADS) {
+        float v[E];
+        vec_to_f(xr[i], v);
+#pragma unroll
+        for (int e = 0; e < E; ++e) ss += v[e] * v[e];
       }
     }
-  } else {
+    ss = warp_sum(ss);
+    if (kEarly) __syncthreads();                 // the previous turn's sums have been read
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    float tot = 0.f;
+#pragma unroll
+    for (int w = 0; w < RN_THREADS / 32; ++w) tot += red[w];      // same order in every thread
+    inv = rsqrtf(__fdividef(tot, (float)d) + eps);      // fast division: no IEEE slow-path subroutine in the kernel
+    if (in_regs) {
+#pragma unroll
+      for (int j = 0; j < RN_VPT; ++j) {
+        const int i = threadIdx.x + j * RN_THREADS;
+        if (i < nv) {
+          float v[E], gv[E];
+          vec_to_f(keep[j], v);
+          vec_to_f(kEarly ? gain[kEarly ? j : 0] : __ldg(gr + i), gv);
+#pragma unroll
+          for (int e = 0; e < E; ++e) v[e] = v[e] * inv * gv[e];
+          const uint4 y = f_to_vec(v);
+          if (!kEarly || turn == 1) o[i] = y;
+        }
+      }
+    }
+  }
+  if (!in_regs) {
+    const uint4* xr = reinterpret_cast<const uint4*>(x + (size_t)(src_rows ? src_rows[r] : r) * d);
     for (int i = threadIdx.x; i < nv; i += RN_THREADS) {
       float v[E], gv[E];
       vec_to_f(xr[i], v);
