@@ -488,8 +488,10 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
 //    would be split between CTAs (the split paths assume a power-of-two chunk count).  (The same idea for the rotary QKV
 //    GEMM, 96-wide tiles that straddle heads, needs 16-row TMA boxes of 2 KB, and those cost far more than the fuller wave
 //    gains: +0.7 ms per LLaDA-shaped pass.  Not kept.)
-//  * plain and rotary ones 128, which needs no K split with 96 tiles, except that a wide GEMM with at most 32 rows takes 256
-//    (its partial tiles are small, and half as many MMA instructions are issued).  A rotary half tile is whole head halves.
+//  * plain and rotary ones 128, which needs no K split with 96 tiles.  With at most 32 rows a wide plain GEMM takes 256 (its partial
+//    tiles are small, and half as many MMA instructions are issued), and so does a rotary one whose 128-wide tiles would be split
+//    anyway; 96 whole tiles of 128 save the K slices' sum instead (12288 x 4096 in a pass of 9 rows: 3.57 -> 3.53 ms per pass).  A
+//    rotary half tile is whole head halves.
 // A shape the kernel cannot take (none of a transformer layer's: it would need more than 4096 column tiles in a launch whose
 // tiles are split between CTAs) is an error, not a fallback.
 template <typename Epi>
@@ -502,7 +504,8 @@ int umma_gemm(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W0,
   const int cols = Epi::kDual ? 2 * NP : NP;
   int bn = UM_HEAD_BN;
   if constexpr (kRope) {
-    bn = M <= 32 ? 256 : 128;
+    const long t128 = (cols + 127) / 128;
+    bn = M <= 32 && (2 * t128 <= st.n_sm || t128 > st.n_sm) ? 256 : 128;
     if (st.stream_bn > 0) bn = st.stream_bn;
     if (bn / 2 < epi.half) bn = 2 * epi.half;
   } else if constexpr (Epi::kDual) {
