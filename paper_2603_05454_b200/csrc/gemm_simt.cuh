@@ -14,6 +14,7 @@
 // head at 250 rows of 2048 ids (K 256) 22.0 -> 25.9 and bf16 1032 x 2 x 1024 (K 256) 49 -> 52; the split sums are the more exact ones
 // (p_max of that head 1.2e-6 from 64 bits, 4.4e-6 before), so the line stays.
 #pragma once
+#include "cluster.cuh"
 #include "epilogues.cuh"
 
 namespace lsp {
@@ -28,6 +29,14 @@ __device__ __forceinline__ float4 load4(const bf16* p) {
 
 constexpr int SG_KS = 16;         // K elements per step
 constexpr int SG_WARPS = 8;
+constexpr int SG_MAX_SLICES = 4;
+// K slices of a tile (the CTAs of a cluster): where the tiles leave SMs idle, as long as every warp keeps two steps (a slice of one
+// step per warp would cost the sum across the cluster, over a microsecond, for less than it saves).
+inline int simt_slices(long tiles, int K, int n_sm, bool reduce) {
+  int s = 1;
+  while (!reduce && 2 * s <= SG_MAX_SLICES && 2 * s * tiles <= n_sm && K / SG_KS >= 2 * s * SG_WARPS * 2) s *= 2;
+  return s;
+}
 // tile: rows x weight rows (a paired epilogue's tile holds half as many pairs); the head reduces 64 columns per partial
 template <typename Epi> struct SimtTile {
   static constexpr int BM = Epi::kReduce ? 16 : 32, BN = Epi::kReduce ? 64 : 32;
@@ -35,10 +44,11 @@ template <typename Epi> struct SimtTile {
 };
 constexpr int SG_HEAD_BN = 64;    // columns per partial of the head, in both kernels
 
-// grid = (ceil(NP / PER_TILE), ceil(M / BM)), block = 256.  A: [M, K]; W0/W1: [*, K] row-major.
+// grid = (ceil(NP / PER_TILE) * slices, ceil(M / BM)), block = 256, clusters of slices CTAs along x: the K slices of a tile.  A: [M, K];
+// W0/W1: [*, K] row-major.
 template <typename T, typename Epi>
 __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* A, const T* __restrict__ W0,
-                                                                   const T* __restrict__ W1, int M, int NP, int K, Epi epi) {
+                                                                   const T* __restrict__ W1, int M, int NP, int K, int slices, Epi epi) {
   constexpr int BM = SimtTile<Epi>::BM, BN = SimtTile<Epi>::BN, PT = SimtTile<Epi>::PER_TILE;
   constexpr int LA = BM + 4, LB = BN + 4;                       // padded leading dimensions
   constexpr int NA = BM * SG_KS / 4 / 32, NB = BN * SG_KS / 4 / 32;      // 4-element vectors per lane and step
@@ -47,7 +57,8 @@ __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* A, c
   __shared__ __align__(16) float sm[SG_WARPS * (WARP_F > RED_F ? WARP_F : RED_F)];
   pdl_begin();
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-  const int m0 = blockIdx.y * BM, j0 = blockIdx.x * PT;
+  const int tile = blockIdx.x / (unsigned)slices, slice = blockIdx.x % (unsigned)slices;
+  const int m0 = blockIdx.y * BM, j0 = tile * PT;
   float* As = sm + w * WARP_F;
   float* Bs = As + SG_KS * LA;
   // operand rows of this lane's vectors, four neighbouring lanes to a row's 16 elements (null past the edges)
@@ -76,9 +87,9 @@ __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* A, c
 #pragma unroll
     for (int i = 0; i < NB; ++i) bv[i] = bp[i] ? load4(bp[i] + k0) : zero;
   };
-  const int steps = K / SG_KS;
-  if (w < steps) load(w * SG_KS);
-  for (int s = w; s < steps; s += SG_WARPS) {
+  const int lo = K / SG_KS * slice / slices, steps = K / SG_KS * (slice + 1) / slices;
+  if (lo + w < steps) load((lo + w) * SG_KS);
+  for (int s = lo + w; s < steps; s += SG_WARPS) {
     __syncwarp();
 #pragma unroll
     for (int i = 0; i < NA; ++i) {
@@ -116,6 +127,27 @@ __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* A, c
   __syncthreads();
   constexpr int TPR = BN / 4;            // threads per output row
   const int row = t / TPR, m = m0 + row;
+  // K slices: every CTA leaves its sums in its shared memory, and the first one adds them in slice (= K) order (true: this CTA
+  // finishes the tile)
+  auto sum_slices = [&](float (&v)[4]) -> bool {
+    if (Epi::kReduce || slices == 1) return true;
+    float4* out = reinterpret_cast<float4*>(sm);
+    __syncthreads();                     // the warps' partial tiles have been read
+    if (slice > 0) out[t] = make_float4(v[0], v[1], v[2], v[3]);
+    cluster_sync();
+    if (slice == 0) {
+      const uint32_t a = smem_u32(out + t);
+      float4 p[SG_MAX_SLICES - 1];
+#pragma unroll
+      for (int x = 1; x < SG_MAX_SLICES; ++x)
+        if (x < slices) p[x - 1] = ld_cluster_f4(cluster_map(a, (unsigned)x));
+#pragma unroll
+      for (int x = 1; x < SG_MAX_SLICES; ++x)
+        if (x < slices) { v[0] += p[x - 1].x; v[1] += p[x - 1].y; v[2] += p[x - 1].z; v[3] += p[x - 1].w; }
+    }
+    cluster_sync();                      // nobody leaves while its sums may still be read
+    return slice == 0;
+  };
   if constexpr (Epi::kDual) {
     const int p = (t % TPR) * 2;         // two pairs: columns p, p + 1 and PT + p, PT + p + 1
     float a0[2] = {}, a1[2] = {};
@@ -125,7 +157,10 @@ __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* A, c
       const float2 u = *reinterpret_cast<const float2*>(r), v = *reinterpret_cast<const float2*>(r + PT);
       a0[0] += u.x; a0[1] += u.y; a1[0] += v.x; a1[1] += v.y;
     }
-    if (m < M) {
+    float a[4] = {a0[0], a0[1], a1[0], a1[1]};
+    const bool mine = sum_slices(a);
+    a0[0] = a[0]; a0[1] = a[1]; a1[0] = a[2]; a1[1] = a[3];
+    if (mine && m < M) {
 #pragma unroll
       for (int e = 0; e < 2; ++e)
         if (j0 + p + e < NP) epi.elem(m, j0 + p + e, a0[e], a1[e]);
@@ -138,6 +173,7 @@ __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* A, c
       const float4 u = *reinterpret_cast<const float4*>(sm + x * RED_F + row * BN + c);
       a[0] += u.x; a[1] += u.y; a[2] += u.z; a[3] += u.w;
     }
+    const bool mine = sum_slices(a);
     if constexpr (Epi::kReduce) {
       Top2 r = top2_empty();
 #pragma unroll
@@ -145,8 +181,8 @@ __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* A, c
         if (epi.valid(j0 + c + e)) top2_push(r, a[e], j0 + c + e);
 #pragma unroll
       for (int o = 1; o < TPR; o <<= 1) r = top2_merge(r, top2_shfl_xor(r, o));
-      if (t % TPR == 0 && m < M) epi.part[(size_t)m * epi.n_tiles + blockIdx.x] = r;
-    } else if (m < M) {
+      if (t % TPR == 0 && m < M) epi.part[(size_t)m * epi.n_tiles + tile] = r;
+    } else if (mine && m < M) {
 #pragma unroll
       for (int e = 0; e < 4; ++e)
         if (j0 + c + e < NP) epi.elem(m, j0 + c + e, a[e], 0.f);

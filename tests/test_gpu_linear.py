@@ -385,6 +385,13 @@ def test_linear_cuda_core_kernels(dtype, M, N, K):
     _check(dtype, 0, M, N, K, seed=13)
 
 
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("M,N,K", [(1, 16, 512), (40, 256, 512), (33, 272, 832), (128, 256, 1024), (64, 64, 4096)])
+def test_linear_cuda_core_k_slices_on_a_cluster(dtype, M, N, K):
+    """Few tiles and a long K: two or four K slices, of unequal length where K is no multiple, summed by the cluster's first CTA."""
+    _check(dtype, 0, M, N, K, seed=12)
+
+
 @pytest.mark.parametrize("M", [129, 187, 256])
 @pytest.mark.parametrize("N,K", [(4096, 4096), (1152, 512), (4608, 3584), (7168, 5120), (4096, 12288), (16, 64)])
 def test_linear_bf16_one_row_group_on_pairs(M, N, K):
