@@ -126,4 +126,96 @@ __global__ void __launch_bounds__(128) k_attn_simt(const T* q, const T* cache_k,
   }
 }
 
+// Small passes: one query per CTA, its keys split over the four warps in tiles of 32 (one key per lane).  A lane reads its key's row and
+// the warp the tile's value rows straight from memory, all requested before the first is used, and the warps' partial results are merged
+// at the end: with 128 keys every warp has one tile, where the kernel above walks four in series.  Every query reads all keys and
+// values itself, so this is for as many CTAs as are resident at once (the dispatch: at most three per SM).
+template <typename T, int DH>
+__global__ void __launch_bounds__(128) k_attn_simt_split(const T* q, const T* cache_k, const T* cache_v, const T* stage_k, const T* stage_v,
+                                                         T* __restrict__ out, StepDesc sd, int n_heads, int n_kv_heads,
+                                                         size_t cache_seq_elems, float scale, int inplace) {
+  constexpr int NV = DH / 4, NC = DH / 32;             // 4-element vectors of a row; elements of the output per lane
+  __shared__ __align__(16) float qs[4][DH];            // a copy per warp: no barrier before the merge
+  __shared__ float part[4][DH], pm[4], pl[4];
+  pdl_begin();
+  const int b = blockIdx.z, h = blockIdx.y, qi = blockIdx.x;
+  const int r0 = sd.row_off[b], Qn = sd.row_off[b + 1] - r0;
+  if (qi >= Qn) return;
+  const int S = sd.F[b] + Qn;
+  const int F = inplace ? S : sd.F[b];      // in-place layout: this pass's K/V rows already sit behind the prefix in the cache
+  const int kvh = h / (n_heads / n_kv_heads), ldq = n_heads * DH, ldkv = n_kv_heads * DH;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const T* ck = cache_k + (size_t)b * cache_seq_elems + kvh * DH;
+  const T* cv = cache_v + (size_t)b * cache_seq_elems + kvh * DH;
+  const T* sk = stage_k + (size_t)r0 * ldkv + kvh * DH;
+  const T* sv = stage_v + (size_t)r0 * ldkv + kvh * DH;
+  float qr[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) qr[c] = to_f(q[(size_t)(r0 + qi) * ldq + h * DH + lane + 32 * c]);
+  float m = -INFINITY, l = 0.f, acc[NC] = {};
+  for (int s0 = 32 * w; s0 < S; s0 += 128) {
+    const int key = s0 + lane;
+    const T* kp = key < F ? ck + (size_t)key * ldkv : sk + (size_t)(key < S ? key - F : 0) * ldkv;
+    if (key >= S) kp = sk;                  // (a row of this pass, there is one)
+    float4 kr[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) kr[i] = as_load4(kp + 4 * i);
+    float v[32][NC];
+    auto load_v = [&]() {
+#pragma unroll
+      for (int k = 0; k < 32; ++k) {
+        const int kk = s0 + k;
+        const T* vp = kk < F ? cv + (size_t)kk * ldkv : sv + (size_t)(kk - F) * ldkv;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) v[k][c] = kk < S ? to_f(vp[lane + 32 * c]) : 0.f;
+      }
+    };
+    if (DH == 64) load_v();                 // (with 128 elements a row the key's registers are needed first)
+    if (s0 == 32 * w) {
+#pragma unroll
+      for (int c = 0; c < NC; ++c) qs[w][lane + 32 * c] = qr[c];
+      __syncwarp();
+    }
+    float d4[4] = {};
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const float4 qv = *reinterpret_cast<const float4*>(qs[w] + 4 * i);
+      d4[0] = fmaf(qv.x, kr[i].x, d4[0]);
+      d4[1] = fmaf(qv.y, kr[i].y, d4[1]);
+      d4[2] = fmaf(qv.z, kr[i].z, d4[2]);
+      d4[3] = fmaf(qv.w, kr[i].w, d4[3]);
+    }
+    const float sc = key < S ? ((d4[0] + d4[1]) + (d4[2] + d4[3])) * scale : -INFINITY;
+    const float m_new = fmaxf(m, warp_max(sc));
+    const float p = key < S ? __expf(sc - m_new) : 0.f;
+    const float corr = __expf(m - m_new);
+    l = l * corr + warp_sum(p);
+    m = m_new;
+    if (DH != 64) load_v();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[c] *= corr;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+      const float pk = __shfl_sync(0xffffffffu, p, k);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[c] = fmaf(pk, v[k][c], acc[c]);
+    }
+  }
+  if (lane == 0) { pm[w] = m; pl[w] = l; }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) part[w][lane + 32 * c] = acc[c];
+  __syncthreads();
+  if (t < DH) {
+    const float mx = fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3]));
+    float sum = 0.f, ls = 0.f;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const float f = pm[x] == -INFINITY ? 0.f : __expf(pm[x] - mx);
+      ls += f * pl[x];
+      sum += f * part[x][t];
+    }
+    out[(size_t)(r0 + qi) * ldq + h * DH + t] = from_f<T>(sum / ls);
+  }
+}
+
 }  // namespace lsp

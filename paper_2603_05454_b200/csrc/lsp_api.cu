@@ -393,6 +393,12 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const Step
       done = true;
     }
   }
+  if (!done && (long)maxQ * m.n_heads * B <= 3l * c->n_sm) {
+    auto kern = dh == 128 ? k_attn_simt_split<T, 128> : k_attn_simt_split<T, 64>;
+    launch_k(c->pdl, kern, dim3(maxQ, m.n_heads, B), dim3(128), 0, c->stream, Qb, cK, cV, stK, stV, Att, sd, m.n_heads, m.n_kv_heads,
+             (size_t)c->max_len * kvd, scale, inplace);
+    done = true;
+  }
   if (!done) {
     const int qw = (long)((maxQ + 15) / 16) * m.n_heads * B >= c->n_sm ? 4 : 1;
     dim3 grid((maxQ + 4 * qw - 1) / (4 * qw), m.n_heads, B);

@@ -97,6 +97,13 @@ def test_attention_other_kernels_against_the_oracle(attn_impl):
     _run_case(8, 2, [129, 5], [33, 70], 256, attn_impl=attn_impl)
 
 
+@pytest.mark.parametrize("F,rows", [([0], [1]), ([30], [2]), ([31], [1]), ([127, 128], [1, 3]), ([300, 0, 17], [5, 12, 1])])
+def test_attention_few_queries_on_cuda_cores(F, rows):
+    """One query per CTA with the keys split over its warps: fewer keys than warps' tiles, tiles that end inside the prefix, at its
+    end and inside the staged rows; memory that was never written holds NaN."""
+    _run_case(8, 2, F, rows, 512, attn_impl=0, seed=6, poison=True)
+
+
 def test_attention_ignores_memory_it_never_wrote():
     """Cache rows past the prefix and staging rows past the pass hold NaN bit patterns (memory the caller handed over
     uninitialised): a ragged last key tile brings such rows into shared memory, and they must not reach the output."""
