@@ -439,8 +439,9 @@ int enqueue_pass(lsp_ctx* c, const StepDesc& sd, const DescInline& din, int B, c
   T* Att = (T*)c->Att;
   T* Hf = (T*)c->Hf;
   seg_begin(c, CLS_MISC);
-  launch_k(c->pdl, k_assemble_embed<T>, dim3(M), dim3(128), 0, c->stream, sd, din, B, c->tokens, c->tok_stride, m.mask_id, (const T*)c->embed, d, X,
-                                               c->row_seq, c->row_pos, c->head_src, c->head_pos, scattered ? 1 : 0);
+  const bool norm0 = d / Vec16<T>::N <= RN_VPT * RN_THREADS;       // a row fits the block's registers: the first norm goes with the embedding
+  launch_k(c->pdl, k_assemble_embed<T>, dim3(M), dim3(RN_THREADS), 0, c->stream, sd, din, B, c->tokens, c->tok_stride, m.mask_id, (const T*)c->embed,
+           d, X, c->row_seq, c->row_pos, c->head_src, c->head_pos, scattered ? 1 : 0, (const T*)c->attn_norm[0], norm0 ? Nrm : (T*)nullptr, m.rms_eps);
   CU(cudaGetLastError());
   if (scattered) {
     launch_k(c->pdl, k_compact_masked, dim3(B), dim3(256), 0, c->stream, sd, (const int32_t*)c->tokens, c->tok_stride, m.mask_id,
@@ -456,11 +457,13 @@ int enqueue_pass(lsp_ctx* c, const StepDesc& sd, const DescInline& din, int B, c
     // this pass's K/V: the staging planes, or (in-place layout) each row's own slot in the cache planes
     T* stK = c->kv_inplace ? (T*)c->kv_cache + (size_t)(2 * l) * cplane : (T*)c->stage + (size_t)(2 * l) * plane;
     T* stV = stK + (c->kv_inplace ? cplane : plane);
-    seg_begin(c, CLS_MISC);
-    run_rmsnorm<T>(c, X, c->attn_norm[l], Nrm, nullptr, M);
-    seg_end(c);
-    count_launch(c, CLS_MISC);
-    CU(cudaGetLastError());
+    if (l > 0 || !norm0) {
+      seg_begin(c, CLS_MISC);
+      run_rmsnorm<T>(c, X, c->attn_norm[l], Nrm, nullptr, M);
+      seg_end(c);
+      count_launch(c, CLS_MISC);
+      CU(cudaGetLastError());
+    }
     {
       EpiQKVRope<T> e{Qb, stK, stV, c->rope_cs, c->row_pos, m.n_heads, m.n_kv_heads, dh / 2, c->row_seq,
                       c->kv_inplace ? c->max_len : 0};

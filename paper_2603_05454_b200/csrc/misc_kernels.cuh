@@ -4,65 +4,6 @@
 
 namespace lsp {
 
-// ---------------------------------------------------------------------------------------------
-// Row assembly + embedding (input of Algorithm 1's forward pass): packed row r of sequence b is position
-// F_b + j; the first pend_b rows carry the tokens committed by the previous step, the rest [MASK].
-// One block per row.  Also fills row_seq / row_pos and the list of rows that go through the LM head.
-// ---------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void k_assemble_embed(StepDesc sd, const __grid_constant__ DescInline in, int batch, const int32_t* tokens, int tok_stride,
-                                 int mask_id, const T* __restrict__ embed, int d, T* __restrict__ X,
-                                 int* __restrict__ row_seq, int* __restrict__ row_pos,
-                                 int* __restrict__ head_src, int* __restrict__ head_pos, int scattered) {
-  pdl_begin();
-  const int r = blockIdx.x;
-  if (in.use && r == 0) {              // leave the descriptor for the step's other kernels
-    for (int i = threadIdx.x; i <= batch; i += blockDim.x) {
-      const_cast<int*>(sd.F)[i] = in.v[0][i];
-      const_cast<int*>(sd.pend)[i] = in.v[1][i];
-      const_cast<int*>(sd.N)[i] = in.v[2][i];
-      const_cast<int*>(sd.row_off)[i] = in.v[3][i];
-      const_cast<int*>(sd.head_off)[i] = in.v[4][i];
-      const_cast<int*>(sd.Fp)[i] = in.v[5][i];
-    }
-  }
-  auto at = [&](int a, const int* p, int i) { return in.use ? in.v[a][i] : p[i]; };
-  // The grid may be larger than the pass (a host that sizes launches from an upper bound of the row counts): rows past
-  // the last real one are zero vectors that belong to no sequence, and the spare head slots point at row 0.
-  if (r >= at(4, sd.head_off, batch) && threadIdx.x == 0) head_src[r] = 0;
-  if (r >= at(3, sd.row_off, batch)) {
-    if (threadIdx.x == 0) { row_seq[r] = -1; row_pos[r] = 0; }
-    uint4* z = reinterpret_cast<uint4*>(X + (size_t)r * d);
-    for (int i = threadIdx.x; i < d * (int)sizeof(T) / 16; i += blockDim.x) z[i] = make_uint4(0u, 0u, 0u, 0u);
-    return;
-  }
-  int b = 0;
-  while (b + 1 < batch && r >= at(3, sd.row_off, b + 1)) ++b;
-  const int j = r - at(3, sd.row_off, b);
-  const int F = at(0, sd.F, b), pend = at(1, sd.pend, b), head0 = at(4, sd.head_off, b);
-  const int pos = F + j;
-  // prefix topology: rows past the pending block are the masked suffix; scattered topology: every row reads the token
-  // buffer (committed positions hold their token, the others the mask id) and k_compact_masked lists the masked rows
-  const int tok = (scattered || j < pend) ? tokens[(size_t)b * tok_stride + pos] : mask_id;
-  if (threadIdx.x == 0) {
-    row_seq[r] = b;
-    row_pos[r] = pos;
-    if (!scattered && j >= pend) {
-      head_src[head0 + (j - pend)] = r;
-      head_pos[head0 + (j - pend)] = pos;
-    }
-  }
-  const uint4* src = reinterpret_cast<const uint4*>(embed + (size_t)tok * d);
-  uint4* dst = reinterpret_cast<uint4*>(X + (size_t)r * d);
-  const int nv = d * (int)sizeof(T) / 16;
-  for (int i = threadIdx.x; i < nv; i += blockDim.x) dst[i] = __ldg(src + i);
-}
-
-// ---------------------------------------------------------------------------------------------
-// RMSNorm: out[r] = x[src[r]] / sqrt(mean(x^2) + eps) * g, fp32 arithmetic, one block per output row.
-// The row is read once with 128-bit loads and kept in registers between the reduction and the scaling
-// (up to RN_VPT vectors per thread; longer rows fall back to a second read).
-// ---------------------------------------------------------------------------------------------
 constexpr int RN_THREADS = 256;
 constexpr int RN_VPT = 4;      // 16-byte vectors per thread held in registers
 
@@ -88,6 +29,120 @@ __device__ __forceinline__ uint4 f_to_vec(const float (&v)[8]) {
   return r;
 }
 
+// ---------------------------------------------------------------------------------------------
+// Row assembly + embedding (input of Algorithm 1's forward pass): packed row r of sequence b is position
+// F_b + j; the first pend_b rows carry the tokens committed by the previous step, the rest [MASK].
+// One block per row.  Also fills row_seq / row_pos and the list of rows that go through the LM head, and, with norm_out, applies the
+// first layer's RMSNorm to the row while it is in registers (as k_rmsnorm does, to the bit; a launch less per pass, about 3.5 us).
+// ---------------------------------------------------------------------------------------------
+template <typename T>
+__global__ void __launch_bounds__(RN_THREADS) k_assemble_embed(StepDesc sd, const __grid_constant__ DescInline in, int batch, const int32_t* tokens, int tok_stride,
+                                 int mask_id, const T* __restrict__ embed, int d, T* __restrict__ X,
+                                 int* __restrict__ row_seq, int* __restrict__ row_pos,
+                                 int* __restrict__ head_src, int* __restrict__ head_pos, int scattered, const T* __restrict__ g,
+                                 T* __restrict__ norm_out, float eps) {
+  constexpr int E = Vec16<T>::N;
+  __shared__ float red[RN_THREADS / 32];
+  pdl_release();
+  const int r = blockIdx.x;
+  const int nv = d / E;
+  uint4 keep[RN_VPT], gain[RN_VPT];
+  const uint4* gr = reinterpret_cast<const uint4*>(g);
+  if (norm_out != nullptr) {
+#pragma unroll
+    for (int j = 0; j < RN_VPT; ++j) {
+      const int i = threadIdx.x + j * RN_THREADS;
+      gain[j] = (i < nv) ? __ldg(gr + i) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+  pdl_wait();
+  if (in.use && r == 0) {              // leave the descriptor for the step's other kernels
+    for (int i = threadIdx.x; i <= batch; i += blockDim.x) {
+      const_cast<int*>(sd.F)[i] = in.v[0][i];
+      const_cast<int*>(sd.pend)[i] = in.v[1][i];
+      const_cast<int*>(sd.N)[i] = in.v[2][i];
+      const_cast<int*>(sd.row_off)[i] = in.v[3][i];
+      const_cast<int*>(sd.head_off)[i] = in.v[4][i];
+      const_cast<int*>(sd.Fp)[i] = in.v[5][i];
+    }
+  }
+  auto at = [&](int a, const int* p, int i) { return in.use ? in.v[a][i] : p[i]; };
+  // The grid may be larger than the pass (a host that sizes launches from an upper bound of the row counts): rows past
+  // the last real one are zero vectors that belong to no sequence, and the spare head slots point at row 0.
+  if (r >= at(4, sd.head_off, batch) && threadIdx.x == 0) head_src[r] = 0;
+  if (r >= at(3, sd.row_off, batch)) {
+    if (threadIdx.x == 0) { row_seq[r] = -1; row_pos[r] = 0; }
+    uint4* z = reinterpret_cast<uint4*>(X + (size_t)r * d);
+    uint4* zn = reinterpret_cast<uint4*>(norm_out + (size_t)r * d);
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+      z[i] = make_uint4(0u, 0u, 0u, 0u);
+      if (norm_out != nullptr) zn[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    return;
+  }
+  int b = 0;
+  while (b + 1 < batch && r >= at(3, sd.row_off, b + 1)) ++b;
+  const int j = r - at(3, sd.row_off, b);
+  const int F = at(0, sd.F, b), pend = at(1, sd.pend, b), head0 = at(4, sd.head_off, b);
+  const int pos = F + j;
+  // prefix topology: rows past the pending block are the masked suffix; scattered topology: every row reads the token
+  // buffer (committed positions hold their token, the others the mask id) and k_compact_masked lists the masked rows
+  const int tok = (scattered || j < pend) ? tokens[(size_t)b * tok_stride + pos] : mask_id;
+  if (threadIdx.x == 0) {
+    row_seq[r] = b;
+    row_pos[r] = pos;
+    if (!scattered && j >= pend) {
+      head_src[head0 + (j - pend)] = r;
+      head_pos[head0 + (j - pend)] = pos;
+    }
+  }
+  const uint4* src = reinterpret_cast<const uint4*>(embed + (size_t)tok * d);
+  uint4* dst = reinterpret_cast<uint4*>(X + (size_t)r * d);
+  if (norm_out == nullptr) {
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) dst[i] = __ldg(src + i);
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < RN_VPT; ++j) {
+    const int i = threadIdx.x + j * RN_THREADS;
+    keep[j] = (i < nv) ? __ldg(src + i) : make_uint4(0u, 0u, 0u, 0u);
+  }
+  float ss = 0.f;
+#pragma unroll
+  for (int j = 0; j < RN_VPT; ++j) {
+    float v[E];
+    vec_to_f(keep[j], v);
+#pragma unroll
+    for (int e = 0; e < E; ++e) ss += v[e] * v[e];
+  }
+  ss = warp_sum(ss);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float tot = 0.f;
+#pragma unroll
+  for (int w = 0; w < RN_THREADS / 32; ++w) tot += red[w];
+  const float inv = rsqrtf(__fdividef(tot, (float)d) + eps);
+  uint4* o = reinterpret_cast<uint4*>(norm_out + (size_t)r * d);
+#pragma unroll
+  for (int j = 0; j < RN_VPT; ++j) {
+    const int i = threadIdx.x + j * RN_THREADS;
+    if (i < nv) {
+      float v[E], gv[E];
+      vec_to_f(keep[j], v);
+      vec_to_f(gain[j], gv);
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = v[e] * inv * gv[e];
+      dst[i] = keep[j];
+      o[i] = f_to_vec(v);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// RMSNorm: out[r] = x[src[r]] / sqrt(mean(x^2) + eps) * g, fp32 arithmetic, one block per output row.
+// The row is read once with 128-bit loads and kept in registers between the reduction and the scaling
+// (up to RN_VPT vectors per thread; longer rows fall back to a second read).
+// ---------------------------------------------------------------------------------------------
 // kEarly: the gains are fetched before the wait for the preceding kernel (they are weights, written by no kernel).  In a small
 // pass they come from HBM, behind its weight stream, and would be a second round trip after the reduction: 3.6 -> 2.4 us from
 // the wait to the last store of a 101-row launch.  With many rows they stay in L2 and the registers they hold (57 a thread

@@ -256,6 +256,14 @@ def test_bf16_model_with_learned_norm_gains():
     _teacher_forced(sh, 42, 200, 140, SchedCfg(mode=2, fixed_k=50), (1, 400), gains_seed=6, max_steps=3)
 
 
+@pytest.mark.parametrize("dtype,d", [("fp32", 4096), ("fp32", 4160), ("bf16", 8192), ("bf16", 8256)])
+def test_first_norm_of_rows_that_do_and_do_not_fit_the_embedding_kernel(dtype, d):
+    """The first layer's norm runs in the embedding kernel while a row fits its registers (4096 fp32 or 8192 bf16 elements)."""
+    from paper_2603_05454_b200 import SchedCfg
+    sh = S.ModelShape(1, d, 2, 2, 64, 64, 256, dtype=dtype, head_scale=1.0, w_std=0.02)
+    _teacher_forced(sh, 43, 5, 7, SchedCfg(mode=2, fixed_k=3), (1, 16), gains_seed=7)
+
+
 @pytest.mark.parametrize("dtype,dh", [("bf16", 128), ("bf16", 64), ("fp32", 64)])
 def test_decode_does_not_read_memory_it_never_wrote(dtype, dh):
     """The cache and the workspace arrive uninitialised (here: NaN bit patterns), the context is larger than the decode
