@@ -22,6 +22,7 @@
 #include "gemm_stream.cuh"
 #include "gemm_pair.cuh"
 #include "attention_umma.cuh"
+#include "attention_rows.cuh"
 #endif
 
 using namespace lsp;
@@ -40,7 +41,7 @@ struct lsp_ctx {
   size_t esz = 0;
   int n_sm = 0;                     // SMs of the device
   cudaStream_t stream = nullptr;
-  int gemm_impl = 1, attn_impl = 2, timing = 0, async_ops = 0, op_repeat = 1, op_rotate = 1, pdl = 1, attn_umma_min_rows = 0, attn_cluster = 1;
+  int gemm_impl = 1, attn_impl = 2, timing = 0, async_ops = 0, op_repeat = 1, op_rotate = 1, pdl = 1, attn_umma_min_rows = 0, attn_cluster = 1, attn_rows = 0;
   // workspace carve (device)
   char *X = nullptr, *Nrm = nullptr, *Qb = nullptr, *Att = nullptr, *Hf = nullptr, *stage = nullptr;
   Top2* part = nullptr;
@@ -370,10 +371,19 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const Step
       dim3 g3(row_tiles * cl, m.n_kv_heads, B);
       const float sl2 = scale * 1.4426950408889634f;
       const CUtensorMap* mp = &c->attn_maps[4 * l];
-      // at most two key tiles per CTA: the kernel with rolled softmax loops
-      auto kern = (max_keys + AU_BN - 1) / AU_BN <= 2 * cl ? k_attn_umma<true> : k_attn_umma<false>;
-      launch_k(c->pdl, kern, g3, dim3(AU_THREADS), (size_t)AU_SMEM, c->stream, cl, map_q, mp[0], mp[1], mp[2], mp[3],
-               Att, sd, m.n_heads, m.n_kv_heads, c->max_len, sl2, cl, inplace, early, c->d_status);
+      // two row tiles per CTA where that still gives every SM a CTA (see attention_rows.cuh)
+      const int pairs = (row_tiles + 1) / 2;
+      const bool by_rows = c->attn_rows == 2 || (c->attn_rows == 0 && row_tiles > 1 && pairs * m.n_kv_heads * B >= c->n_sm);
+      if (by_rows) {
+        launch_k(c->pdl, k_attn_rows, dim3(pairs, m.n_kv_heads, B), dim3(AU_THREADS), (size_t)AR_SMEM, c->stream, map_q, mp[0], mp[1], mp[2], mp[3],
+                 Att, sd, m.n_heads, m.n_kv_heads, c->max_len, sl2, inplace, early, c->d_status);
+        cl = 1;
+      } else {
+        // at most two key tiles per CTA: the kernel with rolled softmax loops
+        auto kern = (max_keys + AU_BN - 1) / AU_BN <= 2 * cl ? k_attn_umma<true> : k_attn_umma<false>;
+        launch_k(c->pdl, kern, g3, dim3(AU_THREADS), (size_t)AU_SMEM, c->stream, cl, map_q, mp[0], mp[1], mp[2], mp[3],
+                 Att, sd, m.n_heads, m.n_kv_heads, c->max_len, sl2, cl, inplace, early, c->d_status);
+      }
       c->last_attn_kernel = 2;
       c->last_attn_cluster = cl;
       done = true;
@@ -772,7 +782,8 @@ int lsp_init(lsp_ctx** out, const lsp_model_cfg* model, const lsp_sched_cfg* sch
       const size_t plane = (size_t)max_batch * max_len * kvd * 2;      // bytes of one (layer, K|V) plane, cache and staging alike
       c->attn_maps.resize((size_t)4 * model->n_layers);
       bool ok = cudaFuncSetAttribute(k_attn_umma<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AU_SMEM) == cudaSuccess &&
-                cudaFuncSetAttribute(k_attn_umma<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AU_SMEM) == cudaSuccess;
+                cudaFuncSetAttribute(k_attn_umma<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AU_SMEM) == cudaSuccess &&
+                cudaFuncSetAttribute(k_attn_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, AR_SMEM) == cudaSuccess;
       for (int l = 0; l < model->n_layers && ok; ++l) {
         const char* ck = c->kv_cache + (size_t)(2 * l) * plane;
         const char* sk = c->stage + (size_t)(2 * l) * plane;
@@ -827,6 +838,10 @@ int lsp_debug_set(lsp_ctx* c, int key, int value) {
   if (key == 28) c->attn_umma_min_rows = value;
   else if (key == 31) c->lag_tail = value < 1 ? 1 : value;
   else if (key == 30) c->attn_cluster = value ? 1 : 0;
+  else if (key == 47) {
+    if (value < 0 || value > 2) return fail(c, LSP_ERR_ARG, "lsp_debug_set: key 47 takes 0 to 2, not %d", value);
+    c->attn_rows = value;
+  }
   else if (key == 3) c->async_ops = value;
   else if (key == 4) c->op_repeat = value < 1 ? 1 : value;
   else if (key == 5) c->op_rotate = value < 1 ? 1 : value;

@@ -38,11 +38,12 @@ extern "C" {
  * tcgen05 attention:
  *   28 fewest (query row x group head) rows of a (sequence, KV head) for which the tcgen05 kernel is used (default 0)
  *   30 it splits a row tile's keys over a thread block cluster when there are few CTAs (1, default)
+ *   47 two row tiles per CTA (k_attn_rows): 0 = where that gives every SM a CTA (default), 1 = never, 2 = always
  * decode loop:
  *   31 with device-resident block lengths (lsp_set_option key 4), lsp_generate reads every step before sizing the next
  *      once at most this many masked positions per sequence remain (default 8)
  * Accepted without effect (they tuned kernel variants that no longer exist): 18, 19, 20, 24, 26, 27, 36 to 39.
- * Unknown key, or a value outside the range of key 41 or 46: LSP_ERR_ARG. */
+ * Unknown key, or a value outside the range of key 41, 46 or 47: LSP_ERR_ARG. */
 int lsp_debug_set(lsp_ctx* ctx, int key, int value);
 
 /* Exercises the bounded-wait recovery path without touching any data: launches one thread that waits, for limit_us

@@ -20,7 +20,7 @@ ATOL = 2e-2
 MEASURED_CEILING = 1.6e-2
 
 
-def _run_case(hq, hkv, cache_len, rows, max_len, attn_impl=None, expect_cluster=None, seed=0, poison=False):
+def _run_case(hq, hkv, cache_len, rows, max_len, attn_impl=None, expect_cluster=None, seed=0, poison=False, opts=()):
     from paper_2603_05454_b200 import LSPDecoder, SchedCfg
     dh, B = 128, len(rows)
     sh = S.ModelShape(1, 128 * hq, hq, hkv, dh, 64, 256, dtype="bf16")
@@ -32,6 +32,8 @@ def _run_case(hq, hkv, cache_len, rows, max_len, attn_impl=None, expect_cluster=
     dec = LSPDecoder(sh, w, SchedCfg(), B, max_len, device=DEV)
     if attn_impl is not None:
         dec.set_option(1, attn_impl)
+    for key, value in opts:
+        dec.debug_set(key, value)
     M = int(sum(rows))
     bf = torch.bfloat16
     q = S.normal((M, hq * dh), seed, 1, 1.0, bf, DEV)
@@ -153,3 +155,17 @@ def test_attention_row_tiles_that_a_group_does_not_fill(case):
     hq, hkv, F, rows, max_len = case
     _run_case(hq, hkv, F, rows, max_len)
     _run_case(hq, hkv, F, rows, max_len, seed=1, poison=True)
+
+
+@pytest.mark.parametrize("hq,hkv,F,rows", [
+    (4, 4, [0], [1]),                            # one row, one ragged tile
+    (4, 4, [128], [128]),                        # whole tiles, one row tile: the second softmax group has no rows
+    (4, 4, [127, 129, 300], [129, 256, 257]),    # ragged key tiles on either side; the second row tile of one row, whole; a third
+    (8, 2, [640, 5, 0], [3, 0, 300]),            # a finished sequence
+    (28, 4, [535, 130], [258, 19]),              # groups that do not divide 128
+    (32, 8, [1500], [515]),                      # many key tiles: the accumulators are rescaled and the stages wrap
+])
+def test_attention_with_two_row_tiles_per_cta(hq, hkv, F, rows):
+    """The kernel of the large passes at every row count, also over memory that was never written."""
+    _run_case(hq, hkv, F, rows, 2048, seed=8, opts=[(47, 2)])
+    _run_case(hq, hkv, F, rows, 2048, seed=9, opts=[(47, 2)], poison=True)
