@@ -53,7 +53,11 @@ struct PairArgs {
   int bn;           // tile width
   int chains;       // head with one tile per pair: accumulators that take K in turn (see umma_head_shape), else 1
   int half_last;    // the last row group has at most 128 rows and runs with 128-row MMAs (64 rows per CTA)
-  int unit;         // rotary epilogue: weight rows per copy when a half tile is not made of whole head halves (else 0)
+  int unit;         // rotary epilogue: 0 where a half tile is made of whole head halves; else 32, and tiles 2 g and 2 g + 1 are the first and
+                    // the second 32 frequencies of bn / 64 heads: one copy brings such rows of several heads, where a tile of
+                    // consecutive pairs would take one per 32 rows and K atom (six a stage at 192 columns: 12288 x 4096 with 512 rows
+                    // took 57 us where the same tiles of a plain epilogue take 42; LLaDA-shaped passes of 187 / 512 rows 4.87 ->
+                    // 4.80, 7.93 -> 7.77 ms)
   int stages;
   unsigned* status;
 };
@@ -139,15 +143,9 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   auto load_weights = [&](int tile, int rg, int c, int s) {
     const uint32_t sb = smem_u32(smem + (size_t)s * STAGE_BYTES) + 2 * A_ATOM;
     if constexpr (kRope) {
-      // blocks of the map are head halves; a half tile is HALF consecutive pair indices
-      const int j = tile * HALF;
-      if (args.unit == 0) {
-        tma_load_4d_pair(sb, map_b, 0, j / epi.half, 2 * c, full0 + 8u * s);
-      } else {
-        for (int b = 0; b < HALF; b += args.unit)
-          for (int a = 0; a < 2; ++a)
-            tma_load_4d_pair(sb + a * B_ATOM + b * 128, map_b, (j + b) % epi.half, (j + b) / epi.half, 2 * c + a, full0 + 8u * s);
-      }
+      // blocks of the map are head halves
+      if (args.unit == 0) tma_load_4d_pair(sb, map_b, 0, tile * HALF / epi.half, 2 * c, full0 + 8u * s);
+      else tma_load_4d_pair(sb, map_b, (tile & 1) * 32, (tile >> 1) * (HALF / 32), 2 * c, full0 + 8u * s);
     } else if (Epi::kDual && half_rows(rg)) {
       // the MMA leaves columns [0, HALF) in lanes 0 .. 63 and [HALF, BN) in lanes 64 .. 127: this CTA's half of the weight tile
       // is then the rank-th half of the tile's gate rows and the same of its up rows, so that a pair stays in one lane
@@ -326,6 +324,20 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           }
         }
       }
+      // rotary table entries of the first two chunks, fetched while the MMAs run, then two chunks ahead (fetched behind the last MMA,
+      // one ahead: LLaDA-shaped passes of 187 / 512 rows 5.14 -> 5.04, 8.12 -> 8.04 ms)
+      EpiPre<Epi> pre, next;
+      auto pair_at = [&](int ch) {                                // pair index of a chunk
+        if (kRope && args.unit) return ((tile >> 1) * (HALF / 32) + (ch >> 1)) * 64 + (tile & 1) * 32 + (ch & 1) * 16;
+        return j0 + ch * 16;
+      };
+      auto fetch = [&](int ch, EpiPre<Epi>& p) {
+        if (live && ch < ch_hi && pair_at(ch) < args.n_pairs) p.load(epi, m, pair_at(ch));
+      };
+      if constexpr (kRope) {
+        fetch(ch_lo, pre);
+        fetch(ch_lo + 1, next);
+      }
       if (!__all_sync(0xffffffffu, mbar_wait(accf_bar(buf), (uint32_t)use & 1u, abort_flag))) {
         if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 44u; }
         break;
@@ -365,23 +377,18 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           if (Epi::kDual) tc_ld16_nowait(t_row + up + (uint32_t)(ch * 16), a1);
         };
         if constexpr (kRope) {
-          // (the rotary table's entries one chunk ahead take the registers a second set of accumulator values would)
-          EpiPre<Epi> pre, next;
-          auto fetch = [&](int ch, EpiPre<Epi>& p) {
-            if (live && ch < ch_hi && j0 + ch * 16 < args.n_pairs) p.load(epi, m, j0 + ch * 16);
-          };
-          fetch(ch_lo, pre);
+          // (the rotary table's entries ahead take the registers a second set of accumulator values would)
           float p0[16], p1[16];
 #pragma unroll 1
           for (int ch = ch_lo; ch < ch_hi; ++ch) {
             __syncwarp();
             request(ch, p0, p1);
-            fetch(ch + 1, next);
             tc_wait_ld();
             tc_pin16(p0);
             tc_pin16(p1);
-            if (live && j0 + ch * 16 < args.n_pairs) epi16(epi, m, j0 + ch * 16, p0, p1, pre);
+            if (live && pair_at(ch) < args.n_pairs) epi16(epi, m, pair_at(ch), p0, p1, pre);
             pre = next;
+            fetch(ch + 2, next);
           }
         } else if (Epi::kReduce && args.chains > 1) {
 #pragma unroll 1
@@ -590,11 +597,11 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
     if (!p) return -4;
     ma = *p;
     if constexpr (kRope) {
-      const int blocks = n_rows_w / (2 * epi.half), br = unit ? unit : epi.half, bb = unit ? 1 : bn / 2 / epi.half;
-      p = umma_map4(st, W0, epi.half, 2 * epi.half, blocks, K, br, bb, unit ? 1 : 2);
+      const int blocks = n_rows_w / (2 * epi.half), br = unit ? unit : epi.half, bb = bn / 2 / br;
+      p = umma_map4(st, W0, epi.half, 2 * epi.half, blocks, K, br, bb, 2);
       if (!p) return -4;
       mb0 = *p;
-      p = umma_map4(st, W1 + (size_t)epi.half * K, epi.half, 2 * epi.half, blocks, K, br, bb, unit ? 1 : 2);
+      p = umma_map4(st, W1 + (size_t)epi.half * K, epi.half, 2 * epi.half, blocks, K, br, bb, 2);
     } else {
       p = umma_map4(st, W0, n_rows_w, n_rows_w, 1, K, bn / 2, 1, 2);
       if (!p) return -4;
@@ -621,7 +628,11 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
     }
   }
   const int per_tile = Epi::kDual ? bn / 2 : bn;
-  const int n_tiles = (NP + per_tile - 1) / per_tile;
+  int n_tiles = (NP + per_tile - 1) / per_tile;
+  if constexpr (kRope) {
+    const int heads = NP / epi.half, nb = bn / 64;
+    if (unit) n_tiles = (heads + nb - 1) / nb * 2;
+  }
   const int rg = (M + PR_ROWS - 1) / PR_ROWS;
   const long T = (long)n_tiles * rg;
   if (T > (1l << 24)) { st.err = "too many tiles for the paired GEMM"; return -9; }
