@@ -424,7 +424,8 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const Step
 
 template <typename T>
 void run_rmsnorm(lsp_ctx* c, const T* x, const void* gains, T* out, const int* src_rows, int rows) {
-  auto kern = rows <= 1024 ? k_rmsnorm<T, true> : k_rmsnorm<T, false>;
+  const bool early = rows <= 1024 && c->m.d_model / Vec16<T>::N <= RN_VPT * RN_THREADS;
+  auto kern = early ? k_rmsnorm_early<T> : k_rmsnorm<T>;
   launch_k(c->pdl, kern, dim3(rows), dim3(RN_THREADS), 0, c->stream, x, (const T*)gains, out, src_rows, c->m.d_model, c->m.rms_eps);
 }
 
@@ -449,7 +450,8 @@ int enqueue_pass(lsp_ctx* c, const StepDesc& sd, const DescInline& din, int B, c
   T* Att = (T*)c->Att;
   T* Hf = (T*)c->Hf;
   seg_begin(c, CLS_MISC);
-  const bool norm0 = d / Vec16<T>::N <= RN_VPT * RN_THREADS;       // a row fits the block's registers: the first norm goes with the embedding
+  // where a row fits the block's registers the first norm goes with the embedding (not with many rows: the registers cost more, as in run_rmsnorm)
+  const bool norm0 = M <= 1024 && d / Vec16<T>::N <= RN_VPT * RN_THREADS;
   launch_k(c->pdl, k_assemble_embed<T>, dim3(M), dim3(RN_THREADS), 0, c->stream, sd, din, B, c->tokens, c->tok_stride, m.mask_id, (const T*)c->embed,
            d, X, c->row_seq, c->row_pos, c->head_src, c->head_pos, scattered ? 1 : 0, (const T*)c->attn_norm[0], norm0 ? Nrm : (T*)nullptr, m.rms_eps);
   CU(cudaGetLastError());

@@ -143,11 +143,7 @@ __global__ void __launch_bounds__(RN_THREADS) k_assemble_embed(StepDesc sd, cons
 // The row is read once with 128-bit loads and kept in registers between the reduction and the scaling
 // (up to RN_VPT vectors per thread; longer rows fall back to a second read).
 // ---------------------------------------------------------------------------------------------
-// kEarly: the gains are fetched before the wait for the preceding kernel (they are weights, written by no kernel).  In a small
-// pass they come from HBM, behind its weight stream, and would be a second round trip after the reduction: 3.6 -> 2.4 us from
-// the wait to the last store of a 101-row launch.  With many rows they stay in L2 and the registers they hold (57 a thread
-// instead of 36) cost more: 8240 rows 34 -> 41 us.
-template <typename T, bool kEarly>
+template <typename T>
 __global__ void __launch_bounds__(RN_THREADS) k_rmsnorm(const T* x, const T* __restrict__ g, T* __restrict__ out,
                                                        const int* src_rows, int d, float eps) {
   constexpr int E = Vec16<T>::N;                 // elements per 16-byte vector
@@ -158,73 +154,52 @@ __global__ void __launch_bounds__(RN_THREADS) k_rmsnorm(const T* x, const T* __r
   uint4* o = reinterpret_cast<uint4*>(out + (size_t)r * d);
   const int nv = d / E;                          // d is a multiple of 64
   const bool in_regs = nv <= RN_VPT * RN_THREADS;
-  uint4 keep[RN_VPT], gain[kEarly ? RN_VPT : 1];
+  uint4 keep[RN_VPT];
   float ss = 0.f;
-  if constexpr (kEarly) {
-    if (in_regs) {
+  pdl_wait();
+  const uint4* xr = reinterpret_cast<const uint4*>(x + (size_t)(src_rows ? src_rows[r] : r) * d);
+  if (in_regs) {
 #pragma unroll
-      for (int j = 0; j < RN_VPT; ++j) {
-        const int i = threadIdx.x + j * RN_THREADS;
-        gain[j] = (i < nv) ? __ldg(gr + i) : make_uint4(0u, 0u, 0u, 0u);
-      }
+    for (int j = 0; j < RN_VPT; ++j) {
+      const int i = threadIdx.x + j * RN_THREADS;
+      keep[j] = (i < nv) ? xr[i] : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int j = 0; j < RN_VPT; ++j) {
+      float v[E];
+      vec_to_f(keep[j], v);
+#pragma unroll
+      for (int e = 0; e < E; ++e) ss += v[e] * v[e];
+    }
+  } else {
+    for (int i = threadIdx.x; i < nv; i += RN_THREADS) {
+      float v[E];
+      vec_to_f(xr[i], v);
+#pragma unroll
+      for (int e = 0; e < E; ++e) ss += v[e] * v[e];
     }
   }
-  // With early gains the row's code runs once ahead of the wait, on the gains in place of the row and storing nothing: its
-  // instructions then wait in the SM instead of being fetched, behind a stream of weights, once the row is there (LLaDA-shaped passes
-  // of 9 / 40 / 101 rows 3.60 -> 3.56, 3.86 -> 3.82, 4.19 -> 4.16 ms).
-  float inv = 0.f;
-#pragma unroll 1
-  for (int turn = kEarly && in_regs ? 0 : 1; turn < 2; ++turn) {
-    if (turn == 1) pdl_wait();
-    const uint4* xr = turn == 1 ? reinterpret_cast<const uint4*>(x + (size_t)(src_rows ? src_rows[r] : r) * d) : gr;
-    ss = 0.f;
-    if (in_regs) {
+  ss = warp_sum(ss);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float tot = 0.f;
 #pragma unroll
-      for (int j = 0; j < RN_VPT; ++j) {
-        const int i = threadIdx.x + j * RN_THREADS;
-        keep[j] = (i < nv) ? xr[i] : make_uint4(0u, 0u, 0u, 0u);
-      }
+  for (int w = 0; w < RN_THREADS / 32; ++w) tot += red[w];      // same order in every thread
+  const float inv = rsqrtf(__fdividef(tot, (float)d) + eps);      // fast division: no IEEE slow-path subroutine in the kernel
+  if (in_regs) {
 #pragma unroll
-      for (int j = 0; j < RN_VPT; ++j) {
-        float v[E];
+    for (int j = 0; j < RN_VPT; ++j) {
+      const int i = threadIdx.x + j * RN_THREADS;
+      if (i < nv) {
+        float v[E], gv[E];
         vec_to_f(keep[j], v);
+        vec_to_f(__ldg(gr + i), gv);
 #pragma unroll
-        for (int e = 0; e < E; ++e) ss += v[e] * v[e];
-      }
-    } else {
-      for (int i = threadIdx.x; i < nv; i += RN_THREADS) {
-        float v[E];
-        vec_to_f(xr[i], v);
-#pragma unroll
-        for (int e = 0; e < E; ++e) ss += v[e] * v[e];
+        for (int e = 0; e < E; ++e) v[e] = v[e] * inv * gv[e];
+        o[i] = f_to_vec(v);
       }
     }
-    ss = warp_sum(ss);
-    if (kEarly) __syncthreads();                 // the previous turn's sums have been read
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-    __syncthreads();
-    float tot = 0.f;
-#pragma unroll
-    for (int w = 0; w < RN_THREADS / 32; ++w) tot += red[w];      // same order in every thread
-    inv = rsqrtf(__fdividef(tot, (float)d) + eps);      // fast division: no IEEE slow-path subroutine in the kernel
-    if (in_regs) {
-#pragma unroll
-      for (int j = 0; j < RN_VPT; ++j) {
-        const int i = threadIdx.x + j * RN_THREADS;
-        if (i < nv) {
-          float v[E], gv[E];
-          vec_to_f(keep[j], v);
-          vec_to_f(kEarly ? gain[kEarly ? j : 0] : __ldg(gr + i), gv);
-#pragma unroll
-          for (int e = 0; e < E; ++e) v[e] = v[e] * inv * gv[e];
-          const uint4 y = f_to_vec(v);
-          if (!kEarly || turn == 1) o[i] = y;
-        }
-      }
-    }
-  }
-  if (!in_regs) {
-    const uint4* xr = reinterpret_cast<const uint4*>(x + (size_t)(src_rows ? src_rows[r] : r) * d);
+  } else {
     for (int i = threadIdx.x; i < nv; i += RN_THREADS) {
       float v[E], gv[E];
       vec_to_f(xr[i], v);
@@ -232,6 +207,70 @@ __global__ void __launch_bounds__(RN_THREADS) k_rmsnorm(const T* x, const T* __r
 #pragma unroll
       for (int e = 0; e < E; ++e) v[e] = v[e] * inv * gv[e];
       o[i] = f_to_vec(v);
+    }
+  }
+}
+
+// The same for at most 1024 rows of at most RN_VPT vectors per thread: the gains are fetched before the wait for the preceding kernel
+// (they are weights, written by no kernel).  In a small pass they come from HBM, behind its weight stream, and would be a second
+// round trip after the reduction: 3.6 -> 2.4 us from the wait to the last store of a 101-row launch.  With many rows they stay in L2 and
+// the registers they hold (80 a thread instead of 37; held to 64 they spill: 101 rows 4.09 -> 4.20 ms a pass) cost more: 8240 rows 34 -> 41 us.
+// And the row's code runs once ahead of the wait, on the gains in place of the row and storing nothing: its instructions then wait in
+// the SM instead of being fetched, behind a stream of weights, once the row is there (LLaDA-shaped passes of 9 / 40 / 101 rows
+// 3.60 -> 3.56, 3.86 -> 3.82, 4.19 -> 4.16 ms).
+template <typename T>
+__global__ void __launch_bounds__(RN_THREADS) k_rmsnorm_early(const T* x, const T* __restrict__ g, T* __restrict__ out,
+                                                             const int* src_rows, int d, float eps) {
+  constexpr int E = Vec16<T>::N;                 // elements per 16-byte vector
+  __shared__ float red[RN_THREADS / 32];
+  pdl_release();
+  const int r = blockIdx.x;
+  const uint4* gr = reinterpret_cast<const uint4*>(g);
+  uint4* o = reinterpret_cast<uint4*>(out + (size_t)r * d);
+  const int nv = d / E;                          // d is a multiple of 64
+  uint4 keep[RN_VPT], gain[RN_VPT];
+#pragma unroll
+  for (int j = 0; j < RN_VPT; ++j) {
+    const int i = threadIdx.x + j * RN_THREADS;
+    gain[j] = (i < nv) ? __ldg(gr + i) : make_uint4(0u, 0u, 0u, 0u);
+  }
+#pragma unroll 1
+  for (int turn = 0; turn < 2; ++turn) {
+    if (turn == 1) pdl_wait();
+    const uint4* xr = turn == 1 ? reinterpret_cast<const uint4*>(x + (size_t)(src_rows ? src_rows[r] : r) * d) : gr;
+    float ss = 0.f;
+#pragma unroll
+    for (int j = 0; j < RN_VPT; ++j) {
+      const int i = threadIdx.x + j * RN_THREADS;
+      keep[j] = (i < nv) ? xr[i] : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int j = 0; j < RN_VPT; ++j) {
+      float v[E];
+      vec_to_f(keep[j], v);
+#pragma unroll
+      for (int e = 0; e < E; ++e) ss += v[e] * v[e];
+    }
+    ss = warp_sum(ss);
+    __syncthreads();                             // the dry turn's sums have been read
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    float tot = 0.f;
+#pragma unroll
+    for (int w = 0; w < RN_THREADS / 32; ++w) tot += red[w];      // same order in every thread
+    const float inv = rsqrtf(__fdividef(tot, (float)d) + eps);
+#pragma unroll
+    for (int j = 0; j < RN_VPT; ++j) {
+      const int i = threadIdx.x + j * RN_THREADS;
+      if (i < nv) {
+        float v[E], gv[E];
+        vec_to_f(keep[j], v);
+        vec_to_f(gain[j], gv);
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = v[e] * inv * gv[e];
+        const uint4 y = f_to_vec(v);
+        if (turn == 1) o[i] = y;
+      }
     }
   }
 }
