@@ -51,20 +51,20 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # rows a launch on average (their flops per byte): there the weights are streamed once per band of rows, and no capture
 # stands for that.
 CLASS_SOURCES = {
-    "gemm": ("gemm_stream.cuh", "gemm_pair.cuh", "gemm_umma.cuh", "epilogues.cuh", "common.cuh"),
-    "head": ("gemm_stream.cuh", "gemm_pair.cuh", "gemm_umma.cuh", "epilogues.cuh", "common.cuh"),
-    "attn": ("attention_umma.cuh", "common.cuh"),
+    "gemm": ("gemm_stream.cuh", "gemm_pair.cuh", "gemm_umma.cuh", "epilogues.cuh", "cluster.cuh", "common.cuh"),
+    "head": ("gemm_stream.cuh", "gemm_pair.cuh", "gemm_umma.cuh", "epilogues.cuh", "cluster.cuh", "common.cuh"),
+    "attn": ("attention_umma.cuh", "attention_rows.cuh", "common.cuh"),
     "commit": ("misc_kernels.cuh", "common.cuh"),
 }
 NCU_TRAFFIC = {
     # k_gemm_stream<128,EpiStore>, M 64, N 12288, K 4096: profiles/k_gemm_stream_M64_N12288_K4096.md
-    "gemm": {"captured_bytes": 104.38e6, "algorithmic_bytes": 102.8e6, "src": "8a89cf02e57d"},
+    "gemm": {"captured_bytes": 104.38e6, "algorithmic_bytes": 102.8e6, "src": "9afdf6ac6d78"},
     # k_gemm_stream<256,EpiHead>, 64 rows: profiles/k_gemm_stream_head_M64_V126464.md
-    "head": {"captured_bytes": 1062.3e6, "algorithmic_bytes": 1037.0e6, "src": "8a89cf02e57d"},
+    "head": {"captured_bytes": 1062.3e6, "algorithmic_bytes": 1037.0e6, "src": "9afdf6ac6d78"},
     # k_attn_umma, 16 x (128 query rows over 2048 keys): profiles/k_attn_umma_B16_F1920.md
-    "attn": {"captured_bytes": 569.5e6, "algorithmic_bytes": 570.4e6, "src": "f9ea95f59873"},
+    "attn": {"captured_bytes": 570.2e6, "algorithmic_bytes": 570.4e6, "src": "acda8c1a1de6"},
     # k_commit_append of a 16 x 1920-row prompt block: profiles/k_commit_append_prompt_B16_P1920.md
-    "commit": {"captured_bytes": 1968.2e6, "algorithmic_bytes": 2013.3e6, "src": "f4033b225a27"},
+    "commit": {"captured_bytes": 1969.9e6, "algorithmic_bytes": 2013.3e6, "src": "7475a23aa56d"},
 }
 
 
