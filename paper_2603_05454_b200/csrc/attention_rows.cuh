@@ -1,8 +1,8 @@
 // Suffix-over-prefix attention of large passes on the 5th-generation tensor cores (tcgen05 + TMEM), head_dim 128, bf16: the contract of
 // attention_umma.cuh, whose kernel takes the passes with few CTAs.
 //
-// Measured against that kernel, passes in ms: 16 x 515 rows over 2100 keys (32 heads) 103.6 -> 101.0; 4 x 1024 over 1024 (28 heads, 4 KV) 46.1
-// -> 45.4; 8 x 154 over 560 18.8 -> 18.3; with fewer CTAs than SMs it loses (4 x 258 rows, 4 KV heads: 13.07 and 13.23).
+// Measured against that kernel, passes in ms: 16 x 515 rows over 2100 keys (32 heads) 105.1 -> 103.0; 8 x 154 over 560 18.8 -> 18.5;
+// 8 x 205 over 900 (28 heads, 4 KV) 27.7 -> 27.5; 4 x 1024 over 1024 no difference (46.7, 46.6).
 // What bounds that kernel with many key tiles is shared memory: per 128 x 128 score tile it writes 64 KB of keys and values and 32 KB of
 // softmax weights, and its MMAs read 128 KB: about 1800 of the 2470 cycles a tile takes.  Here
 //   * a CTA owns TWO row tiles of 128 (position, head of the group) rows of one (sequence, KV head), which share every K / V tile: half
@@ -13,7 +13,13 @@
 //     their store nor the MMAs' reads of them touch shared memory.
 // One warp issues all MMAs.  They execute in order, so P V of a tile and Q K^T of the next one follow each other without a wait, and
 // scores that have arrived tell the softmax group that its previous P V is complete.
-// The running maximum is raised lazily, as in attention_umma.cuh.
+// The running maximum is raised lazily, as in attention_umma.cuh, from the fifth tile on; in the first four it follows the scores (to a
+// quarter), and the row sum adds the weights as they were rounded.  Here a row has one maximum where that kernel has two: only the
+// weight of a key that was the maximum is 1 and without rounding error, and the sum of the rounded weights takes out what their errors
+// share.  Error against 64 bits relative to that kernel's, 500 to 4300 keys, scores of standard deviation 0.3 / 1 / 4: fp32 sum and all
+// tiles lazy 1.003 / 1.022 / 1.07 at worst; now 1.001 / 0.993 / 0.92.  With two key tiles that kernel's two maxima are all there are
+// (1.015), so it takes those passes.  The launch of 16 x 515 rows over 2100 keys alone 458 -> 494 us (that kernel 464); in passes, which run at
+// the power limit, it stays the faster one: see above.
 // Warps 0..3 and 4..7 = softmax groups 0 and 1; warps 8 and 11 = TMA producers of the K and the V tiles, warp 9 = TMEM allocator and MMA
 // issuer.  Every wait is bounded; on expiry the kernel records (code, site), drains and returns.
 #pragma once
@@ -229,7 +235,7 @@ k_attn_rows(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
       const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * scale_log2;
       float corr = 1.f;
       bool raise = false;
-      if (mx > m_used + 8.f) {                          // also the first tile (m_used = -inf)
+      if (mx > m_used + (t < 4 ? 0.25f : 8.f)) {        // also the first tile (m_used = -inf)
         corr = ex2_approx(m_used - mx);
         m_used = mx;
         raise = t > 0;
@@ -270,9 +276,9 @@ k_attn_rows(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
           f2_unpack(x2, p0, p1);
           p0 = ex2_approx(p0);
           p1 = ex2_approx(p1);
-          sum2[j & 1] = f2_add(sum2[j & 1], f2_pack(p0, p1));
           const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
           pk[j] = *reinterpret_cast<const uint32_t*>(&pb);
+          sum2[j & 1] = f2_add(sum2[j & 1], f2_pack(__uint_as_float(pk[j] << 16), __uint_as_float(pk[j] & 0xffff0000u)));
         }
         tc_st16u(s_col + (uint32_t)(16 * c), pk);
       }

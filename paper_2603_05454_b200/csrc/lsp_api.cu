@@ -371,9 +371,9 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const Step
       dim3 g3(row_tiles * cl, m.n_kv_heads, B);
       const float sl2 = scale * 1.4426950408889634f;
       const CUtensorMap* mp = &c->attn_maps[4 * l];
-      // two row tiles per CTA where that still gives every SM a CTA (see attention_rows.cuh)
+      // two row tiles per CTA where that still gives every SM a CTA and the keys are more than two tiles (see attention_rows.cuh)
       const int pairs = (row_tiles + 1) / 2;
-      const bool by_rows = c->attn_rows == 2 || (c->attn_rows == 0 && row_tiles > 1 && pairs * m.n_kv_heads * B >= c->n_sm);
+      const bool by_rows = c->attn_rows == 2 || (c->attn_rows == 0 && row_tiles > 1 && max_keys > 2 * AU_BN && pairs * m.n_kv_heads * B >= c->n_sm);
       if (by_rows) {
         launch_k(c->pdl, k_attn_rows, dim3(pairs, m.n_kv_heads, B), dim3(AU_THREADS), (size_t)AR_SMEM, c->stream, map_q, mp[0], mp[1], mp[2], mp[3],
                  Att, sd, m.n_heads, m.n_kv_heads, c->max_len, sl2, inplace, early, c->d_status);
