@@ -50,6 +50,7 @@ struct StreamArgs {
                     // r-th K slice; the partial tiles are then reduced through distributed shared memory (see the kernel)
   int exchange;     // clusters of 2: each CTA publishes only the half its peer finishes and keeps its own half in tensor memory
   int kc;           // K chunks (one per stage) per tile
+  int chains;       // rotary epilogue, one whole tile per CTA: accumulators that take K in turn, added in K order (else 1)
   int a_rows;       // activation box rows (M rounded up to a multiple of 8)
   int atoms;        // 64-element K atoms per stage (1 or 2)
   int one_copy;     // 1: one copy brings both halves and all atoms of a stage's weight tile (map_b0); 0: one per half and atom
@@ -92,7 +93,8 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
   constexpr int SET_COLS = BN;                            // columns of one accumulator set
   constexpr int NBUF = 2;                                 // accumulator sets in tensor memory
   // tensor memory is allocated in powers of two (192-wide tiles use 384 of 512 columns)
-  constexpr uint32_t TMEM_COLS = (NBUF * SET_COLS <= 128) ? 128 : (NBUF * SET_COLS <= 256 ? 256 : 512);
+  constexpr bool kChains = kRope && BN == 128;            // (see args.chains: up to four accumulators of one tile)
+  constexpr uint32_t TMEM_COLS = kChains ? 512 : (NBUF * SET_COLS <= 128) ? 128 : (NBUF * SET_COLS <= 256 ? 256 : 512);
   const int A_ATOM = args.a_rows * 128;
   const int AT = args.atoms;
   const int STAGE_BYTES = AT * (A_ATOM + B_ATOM);
@@ -125,13 +127,19 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     int tile, c, rot;
   };
   auto chunk = [&](const Pos& p) { return p.c + p.rot < args.kc ? p.c + p.rot : p.c + p.rot - args.kc; };
+  // With several accumulators (chain i takes chunks [kc i / chains, kc (i + 1) / chains) of that order) two neighbouring tiles have the
+  // order of the 256-wide tile they make up, and the odd one starts with its second accumulator.
+  auto chain_lo = [&](int i) { return args.kc * i / args.chains; };
+  auto rot_of = [&](int tile) {
+    return (kChains && args.chains > 1 ? (tile >> 1) * ST_ROT + chain_lo(tile & 1) : tile * ST_ROT) % args.kc;
+  };
   auto pos_set = [&](Pos& p, int u) {
     p.tile = u / args.kc;
     p.c = u % args.kc;
-    p.rot = p.tile * ST_ROT % args.kc;
+    p.rot = rot_of(p.tile);
   };
   auto pos_next = [&](Pos& p) {
-    if (++p.c == args.kc) { p.c = 0; ++p.tile; p.rot = p.tile * ST_ROT % args.kc; }
+    if (++p.c == args.kc) { p.c = 0; ++p.tile; p.rot = rot_of(p.tile); }
   };
   // the weight tile of one stage: both halves of every K atom (see umma_map5)
   auto load_weights = [&](const Pos& p, int s) {
@@ -257,9 +265,21 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
           break;
         }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(buf * SET_COLS);
-        uint32_t acc = 0;                               // 0: the segment's first MMA overwrites the accumulator
+        uint32_t d_tmem = tmem_base + (uint32_t)(buf * SET_COLS);
+        uint32_t acc = 0;                               // 0: the next MMA overwrites the accumulator
+        int chain = 0, next_acc = seg_end;              // the first unit of the next accumulator
+        if (kChains && args.chains > 1) {
+          chain = vt & 1;
+          d_tmem += (uint32_t)(chain * BN);
+          next_acc = u + chain_lo(chain + 1) - chain_lo(chain);
+        }
         for (; u < seg_end; ++u) {
+          if (kChains && u == next_acc) {
+            if (++chain == args.chains) chain = 0;
+            d_tmem = tmem_base + (uint32_t)(chain * BN);
+            acc = 0;
+            next_acc = u + chain_lo(chain + 1) - chain_lo(chain);
+          }
           if (!ready) ok = __all_sync(0xffffffffu, mbar_wait(full_bar(s), ph, abort_flag));
           if (!ok) {
             if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 13u; }
@@ -359,6 +379,18 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
               tc_wait_ld();
               tc_pin16(p0);
               tc_pin16(p1);
+              if constexpr (kChains) {
+#pragma unroll 1
+                for (int x = 1; x < args.chains; ++x) {            // in K order
+                  float v[16];
+                  tc_ld16(t_row + (uint32_t)(x * BN + c), v);
+#pragma unroll
+                  for (int i = 0; i < 16; ++i) p0[i] += v[i];
+                  tc_ld16(t_row + (uint32_t)(x * BN + HALF + c), v);
+#pragma unroll
+                  for (int i = 0; i < 16; ++i) p1[i] += v[i];
+                }
+              }
               consume(c, p0, p1, preA);
               preA = preB;
             }
@@ -822,7 +854,13 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
       exchange = (splits == 2 && st.stream_exchange && M >= st.stream_exchange_rows) ? 1 : 0;
     }
   }
-  StreamArgs args{M, NP, n_tiles, cluster, exchange, kc, sh.a_rows, sh.atoms, one_copy, rot_half, sh.stages, st.scratch, st.counters, status};
+  // a rotary tile of few rows that 256-wide tiles would split over K (see umma_gemm): as many accumulators as that had slices
+  int chains = 1;
+  if constexpr (std::is_same<Epi, EpiQKVRope<bf16>>::value && BN == 128) {
+    if (M <= 32 && grid == T && st.stream_bn == 0)
+      chains = std::max(1, std::min(stream_splits(st, (T + 1) / 2, stream_no_split<Epi>(K)), std::min(4, kc)));
+  }
+  StreamArgs args{M, NP, n_tiles, cluster, exchange, kc, chains, sh.a_rows, sh.atoms, one_copy, rot_half, sh.stages, st.scratch, st.counters, status};
   cudaError_t e = launch_k(st.pdl, k_gemm_stream<BN, Epi>, dim3(grid), dim3(ST_THREADS), smem, stream, cluster, *ma, mb0v,
                            mb1v, args, e2);
   if (e == cudaSuccess) e = cudaGetLastError();

@@ -1428,7 +1428,7 @@ int lsp_linear_static(const void* A, const void* W, void* out, int M, int N, int
     static_msg(err, err_len, "lsp_linear_static: clearing the counters failed (%s)", cudaGetErrorString(e));
     return LSP_ERR_CUDA;
   }
-  StreamArgs args{M, N, n_tiles, 0, 0, kc, a_rows, atoms, 1, 0, stages, partials, counters, status};
+  StreamArgs args{M, N, n_tiles, 0, 0, kc, 1, a_rows, atoms, 1, 0, stages, partials, counters, status};
   EpiStore<bf16> epi{(bf16*)out, N};
   k_gemm_stream<kStaticBN, EpiStore<bf16>><<<grid, ST_THREADS, smem, stream>>>(ma, mb, mb, args, epi);
   e = cudaGetLastError();

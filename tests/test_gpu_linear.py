@@ -357,6 +357,31 @@ def test_rotary_projection_on_pairs_of_sms(dh, hq, hkv, bn):
     assert bool(((kv[0] - kv[1]).abs() <= (kv[1].abs() + typical) / 128).all())
 
 
+@pytest.mark.parametrize("P", [5, 28])
+@pytest.mark.parametrize("dh,hq,hkv,d", [(128, 32, 32, 4096), (128, 72, 2, 1088), (128, 120, 12, 1152), (64, 64, 64, 1024), (128, 73, 1, 576),
+                                         (128, 32, 32, 512)])
+def test_rotary_projection_of_few_rows_keeps_its_sums(dh, hq, hkv, d, P):
+    """75 to 148 whole tiles of 128 columns add K in the slices, and in the order, of the 256-wide tiles (23 = 256) that are split over two
+    or three CTAs: the cache rows of the two are equal to the bit."""
+    from paper_2603_05454_b200 import LSPDecoder, SchedCfg
+    G = 4
+    sh = S.ModelShape(1, d, hq, hkv, dh, 64, 256, dtype="bf16")
+    w = S.make_weights(sh, 3, device=DEV)
+    rows = []
+    for width in (0, 256):
+        dec = LSPDecoder(sh, w, SchedCfg(), 1, P + G, device=DEV)
+        dec.debug_set(23, width)
+        tokens = torch.zeros(1, P + G, dtype=torch.int32, device=DEV)
+        tokens[:, :P] = S.make_prompt(1, P, sh, 7).to(DEV)
+        dec.begin(tokens, [P], [G])
+        dec.denoise_step()
+        dec.commit([1])
+        rows.append(dec.kv_view()[:, :, 0, :P].clone())
+        dec.close()
+    assert rows[0].float().abs().max() > 0.1
+    assert torch.equal(*rows), float((rows[0].float() - rows[1].float()).abs().max())
+
+
 @pytest.mark.parametrize("M,N,K,opts", [(5, 12288, 256, {}), (100, 384, 192, {}), (200, 12288, 320, {}), (128, 1152, 576, {43: 1}),
                                         (200, 12288, 320, {43: 1}), (64, 9600, 1024, {29: 0})])
 @pytest.mark.parametrize("up_first", [False, True])
