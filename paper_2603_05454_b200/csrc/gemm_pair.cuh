@@ -235,10 +235,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     if (rank == 0) {
       for (int it = issued > S ? issued - S : 0; it < issued; ++it) mbar_wait(full_bar(it % S), (uint32_t)(it / S) & 1u, &no_abort);
     }
-    if (!ok) {                             // after a failure the peer may not have counted these copies: let them land
-      const uint64_t t0 = globaltimer_ns();
-      while (globaltimer_ns() - t0 < 1000000ull) {}
-    }
+    if (!ok) um_let_land();                // (the peer may not have counted these copies)
   } else if (warp == 1) {
     // ---------------- MMA issuer (first CTA; the whole warp waits, one elected thread issues) ----------------
     pdl_wait();            // (its bounded waits must not count the preceding kernel's time)

@@ -219,12 +219,9 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       ++issued;
       if (++s == S) { s = 0; ph ^= 1u; }
     }
-    // do not leave while copies may still be landing in this CTA's shared memory
-    const int first = issued > S ? issued - S : 0;
-    for (int it = first; it < issued; ++it) {
-      volatile uint32_t no_abort = 0;
-      mbar_wait(full_bar((int)(it % S)), (uint32_t)(it / S) & 1u, &no_abort);
-    }
+    // do not leave while copies, these or the activations', may still be landing in this CTA's shared memory
+    // (after a failure: see the end)
+    for (int it = issued > S ? issued - S : 0; it < issued; ++it) mbar_wait(full_bar(it % S), (uint32_t)(it / S) & 1u, abort_flag);
   } else if (warp == 6) {
     // ---------------- TMA producer of the activations ----------------
     // (the same stages in the same order; they may arrive ahead of the stage's arming: its phase ends with both.  A warp of its
@@ -714,6 +711,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       cluster_sync();      // nobody leaves while a peer may still read its shared memory
     }
   }
+  if ((warp == 0 || warp == 6) && *abort_flag) um_let_land();
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {

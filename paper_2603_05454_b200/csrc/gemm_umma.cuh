@@ -79,6 +79,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// After a failure a stage may hold copies of one producer and none of the other, and its barrier then never completes.  Each producer
+// stays this long (1 ms; a copy takes microseconds) behind its last copy instead, so that none lands in the memory of a CTA that is gone.
+__device__ __forceinline__ void um_let_land() {
+  const uint64_t t0 = globaltimer_ns();
+  while (globaltimer_ns() - t0 < 1000000ull) {}
+}
+
 // Self-test of the bounded-wait protocol: one thread waits on a barrier that nobody ever arrives at, gives up after
 // limit_ns and reports it exactly as the kernels' roles do: (code 1, site 99) in the status word.  Nothing else runs,
 // nothing is in flight, the context stays usable.

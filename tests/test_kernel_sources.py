@@ -48,6 +48,21 @@ def test_warps_leave_on_an_expired_wait_as_one(name):
     assert not re.search(r"if \(!mbar_wait\(", _source(name))
 
 
+@pytest.mark.parametrize("name,warps", [("gemm_stream.cuh", [0, 6]), ("gemm_pair.cuh", [0])])
+def test_producers_that_share_a_stage_outstay_their_copies_after_a_failure(name, warps):
+    """A stage's barrier counts the copies of two producers (the weights' and the activations' warp, the two CTAs of a pair).  One that gives
+    up leaves the other's copies on a barrier that never completes, so after a failure every warp that issues copies stays for a time."""
+    body = _source(name)
+    body = body[body.index("tmem_base = *tmem_slot"):]
+    roles = re.split(r"\n  (?:if|\} else if) \(warp == ([^\n]*)\) \{\n|\n  \} else \{\n", body)
+    issuing = [int(w) for w, r in zip(roles[1::2], roles[2::2]) if re.search(r"request_weights\(|load_weights\(|load_acts\(", r)]
+    assert issuing == warps
+    if len(warps) == 1:
+        assert "if (!ok) um_let_land();" in roles[2]
+    else:
+        assert "if ((" + " || ".join(f"warp == {w}" for w in warps) + ") && *abort_flag) um_let_land();\n  tc_fence_before();\n  __syncthreads();" in body
+
+
 def test_the_step_driver_assumes_no_sm_count():
     """The dispatch lines of the CUDA-core kernels (fp32 models among them) are in SMs of the device at hand."""
     assert not re.search(r"\b148\b", _source("lsp_api.cu")) and "cudaDevAttrMultiProcessorCount" in _source("lsp_api.cu")
