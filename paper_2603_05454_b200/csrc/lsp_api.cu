@@ -71,6 +71,7 @@ struct lsp_ctx {
   int* h_ring = nullptr;            // kRing x (6 max_batch + 4) ints
   cudaEvent_t ring_done[kRing] = {}, ring_t0[kRing] = {}, ring_t1[kRing] = {};
   int kv_inplace = 0;               // K/V layout: 0 = staging planes + append copy, 1 = written in place (see lsp_set_option key 3)
+  int rotary_late = 0;              // the last GEMM launched was a rotary one that releases its successor behind its own wait
   int last_attn_kernel = 0, last_attn_cluster = 1;   // what the last attention launch was (see lsp_get_counters)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   float timing_ms[8] = {0};
@@ -223,6 +224,7 @@ int check_model(const lsp_model_cfg* m) {
 // ---- GEMM dispatch ------------------------------------------------------------------------------------
 template <typename T, typename Epi>
 int run_gemm(lsp_ctx* c, const T* A, const T* W0, const T* W1, int M, int NP, int K, int n_rows_w, const Epi& epi) {
+  c->rotary_late = 0;
   if (M <= 0) return LSP_OK;
   {
     // algorithmic work of this launch: every operand and result once
@@ -240,6 +242,7 @@ int run_gemm(lsp_ctx* c, const T* A, const T* W0, const T* W1, int M, int NP, in
     if (c->gemm_impl == 1) {
       const int rc = umma_gemm<Epi>(c->umma, c->stream, A, W0, W1, M, NP, K, n_rows_w, epi, c->d_status);
       if (rc != 0) return fail(c, LSP_ERR_CUDA, "tcgen05 GEMM launch failed (%d): %s", rc, c->umma.err.c_str());
+      c->rotary_late = std::is_same<Epi, EpiQKVRope<bf16>>::value ? 1 : 0;
       return LSP_OK;
     }
   }
@@ -333,7 +336,8 @@ int check_status(lsp_ctx* c) {
 
 // Suffix-over-prefix attention of layer l (Sec. 3.2: every query row of the pass sees the cached prefix [0, F_b) and all
 // of the pass's own rows).  Reads the uploaded descriptor (F, row_off), Q from q, K/V from the cache and the staging
-// planes of layer l; writes out.  early: the launch before it is the tcgen05 QKV projection of the same layer (see k_attn_umma).
+// planes of layer l; writes out.  early: the launch before it is a tcgen05 rotary projection, whose kernels release this launch
+// behind their own wait (see k_attn_umma).
 // q_rows: rows of Qb.  max_q: most query rows of one sequence; max_keys: most keys of one sequence.
 template <typename T>
 int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const StepDesc& sd, int B, int maxQ, int max_keys, int inplace, int early) {
@@ -486,8 +490,7 @@ int enqueue_pass(lsp_ctx* c, const StepDesc& sd, const DescInline& din, int B, c
     {
       c->counters[CNT_ATTN_BYTES] += pd.attn_bytes;
       c->counters[CNT_ATTN_FLOPS] += pd.attn_flops;
-      const int rc = run_attention<T>(c, l, Qb, M, Att, sd, B, pd.maxQ, pd.max_keys, c->kv_inplace,
-                                      c->gemm_impl == 1 ? 1 : 0);
+      const int rc = run_attention<T>(c, l, Qb, M, Att, sd, B, pd.maxQ, pd.max_keys, c->kv_inplace, c->rotary_late);
       if (rc) return rc;
     }
     {

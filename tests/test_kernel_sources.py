@@ -63,6 +63,14 @@ def test_producers_that_share_a_stage_outstay_their_copies_after_a_failure(name,
         assert "if ((" + " || ".join(f"warp == {w}" for w in warps) + ") && *abort_flag) um_let_land();\n  tc_fence_before();\n  __syncthreads();" in body
 
 
+def test_attention_starts_early_only_behind_a_rotary_projection_that_was_launched():
+    """Which kernel ran decides, not which one was asked for."""
+    src = _source("lsp_api.cu")
+    assert re.findall(r"rotary_late = ([^;]+);", src) == ["0", "0", "std::is_same<Epi, EpiQKVRope<bf16>>::value ? 1 : 0"]
+    last = re.findall(r"run_attention<\w+>\(.*, ([^,\n]+)\)[;\n]", src)
+    assert last == ["c->rotary_late", "0", "0"]
+
+
 def test_the_step_driver_assumes_no_sm_count():
     """The dispatch lines of the CUDA-core kernels (fp32 models among them) are in SMs of the device at hand."""
     assert not re.search(r"\b148\b", _source("lsp_api.cu")) and "cudaDevAttrMultiProcessorCount" in _source("lsp_api.cu")
