@@ -28,21 +28,61 @@ def test_no_kernel_declares_data_of_the_step_read_only(name):
         assert m.group(1) in ("embed", "g", "W0", "W1", "P", "G"), f"{name}: {m.group(1)}"
 
 
-@pytest.mark.parametrize("name", ["gemm_stream.cuh", "gemm_pair.cuh", "attention_umma.cuh"])
-def test_no_role_starts_a_bounded_wait_before_the_preceding_kernel_has_ended(name):
-    """The limit of a wait is for this kernel's own copies and MMAs.  Every role (producer, issuer, epilogue: the branches behind the
-    set-up's barrier) reaches pdl_wait() before its first mbar_wait(), by itself or because all of them do."""
+TCGEN05 = ["gemm_stream.cuh", "gemm_pair.cuh", "attention_umma.cuh", "attention_rows.cuh"]
+
+
+def _roles(name):
+    """Set-up, roles (the branches on the warp behind the set-up's barrier; the last one with what follows them) of a tcgen05 kernel."""
     body = _source(name)
-    body = body[body.index("tmem_base = *tmem_slot"):]
-    roles = re.split(r"\n  (?:if|\} else if) \(warp == [^\n]*\) \{\n|\n  \} else \{\n", body)
-    assert len(roles) >= 4
-    if "pdl_wait();" in roles[0]:
-        return
-    for r in roles[1:4]:
-        assert "pdl_wait();" in r.split("mbar_wait(")[0]
+    at = body.index("tmem_base = *tmem_slot")
+    return body[:at], re.split(r"\n  (?:if|\} else if) \(warp [^\n]*\) \{\n|\n  \} else \{\n", body[at:])
 
 
-@pytest.mark.parametrize("name", ["gemm_stream.cuh", "gemm_pair.cuh", "attention_umma.cuh"])
+@pytest.mark.parametrize("name,n_roles", list(zip(TCGEN05, [4, 3, 4, 3])))
+def test_no_role_starts_a_bounded_wait_before_the_preceding_kernel_has_ended(name, n_roles):
+    """The limit of a wait is for this kernel's own copies and MMAs.  Every role (producers, issuers, epilogue or softmax) reaches
+    pdl_wait(), whatever early says, before its first mbar_wait()."""
+    setup, (ahead, *roles) = _roles(name)
+    roles = [r for r in roles if "mbar_wait(" in r]
+    assert len(roles) == n_roles
+    assert "mbar_wait(" not in ahead and "mbar_wait(" not in setup[setup.index("__global__"):]
+    for r in roles:
+        assert re.search(r"^ +pdl_wait\(\);", r.split("mbar_wait(")[0], re.M)
+
+
+@pytest.mark.parametrize("name", ["gemm_stream.cuh", "gemm_pair.cuh"])
+def test_a_rotary_projection_releases_the_attention_behind_its_own_wait(name):
+    """The attention reads the descriptor and older cache rows ahead of its wait: the projection before it must not let it start until
+    everything older has ended."""
+    body = _source(name)
+    assert [m.group(0) for m in re.finditer(r"[^\n]*pdl_release\(\);", body)] == ["  if (!kRope) pdl_release();", "    if (kRope) pdl_release();"]
+    assert re.search(r"\n    pdl_wait\(\);\s*\n    if \(kRope\) pdl_release\(\);", body)
+
+
+@pytest.mark.parametrize("name", ["attention_umma.cuh", "attention_rows.cuh"])
+def test_attention_reads_only_older_rows_ahead_of_its_wait(name):
+    """Ahead of the wait: nothing but the descriptor, and K / V tiles of cache rows that this pass's projection does not write (in place:
+    those that end ahead of the pass's first row)."""
+    _, (ahead, *roles) = _roles(name)
+    assert "if (!early) pdl_wait();" in ahead
+    copies = [r for r in roles if re.search(r"tma_load|load_tile\(", r)]
+    assert len(copies) == 1
+    early = copies[0].split("pdl_wait();")[0]
+    loads = early[early.index("int issued = 0;"):]
+    assert re.search(r"if \(early\)\s+while \(issued < min\(2, n_tiles\) && \(inplace \? [^?]*\* AU_BN <= F - Qn : [^?]* < n_c\)\) "
+                     r"load_tile\(issued\+\+\);\s*$", loads)
+    assert "load_tile(" not in early[:early.index("auto load_tile")]
+
+
+def test_attention_starts_early_only_behind_a_rotary_projection_that_was_launched():
+    """Which kernel ran decides, not which one was asked for."""
+    src = _source("lsp_api.cu")
+    assert re.findall(r"rotary_late = ([^;]+);", src) == ["0", "0", "std::is_same<Epi, EpiQKVRope<bf16>>::value ? 1 : 0"]
+    last = re.findall(r"run_attention<\w+>\(.*, ([^,\n]+)\)[;\n]", src)
+    assert last == ["c->rotary_late", "0", "0"]
+
+
+@pytest.mark.parametrize("name", TCGEN05)
 def test_warps_leave_on_an_expired_wait_as_one(name):
     """Tensor-memory loads and full-mask barriers need every lane: whether a wait expired is put to a vote before anyone leaves."""
     assert not re.search(r"if \(!mbar_wait\(", _source(name))
@@ -61,14 +101,6 @@ def test_producers_that_share_a_stage_outstay_their_copies_after_a_failure(name,
         assert "if (!ok) um_let_land();" in roles[2]
     else:
         assert "if ((" + " || ".join(f"warp == {w}" for w in warps) + ") && *abort_flag) um_let_land();\n  tc_fence_before();\n  __syncthreads();" in body
-
-
-def test_attention_starts_early_only_behind_a_rotary_projection_that_was_launched():
-    """Which kernel ran decides, not which one was asked for."""
-    src = _source("lsp_api.cu")
-    assert re.findall(r"rotary_late = ([^;]+);", src) == ["0", "0", "std::is_same<Epi, EpiQKVRope<bf16>>::value ? 1 : 0"]
-    last = re.findall(r"run_attention<\w+>\(.*, ([^,\n]+)\)[;\n]", src)
-    assert last == ["c->rotary_late", "0", "0"]
 
 
 def test_the_step_driver_assumes_no_sm_count():
