@@ -236,7 +236,7 @@ int lsp_last_timing(lsp_ctx* ctx, float* ms);
  * plus Q and O), 4 KV-append bytes (read + write), 5 LM-head bytes, 6 LM-head flops, 7 denoiser passes,
  * 8..13 kernel launches by class (same classes as lsp_last_timing 0..5), 14 attention flops
  * (4 * queries * keys * n_heads * head_dim per layer), 15 committed tokens; not counters but the last attention
- * launch: 16 its kernel (0 CUDA cores, 1 mma.sync, 2 tcgen05), 17 the thread block cluster size its key tiles were
+ * launch: 16 its kernel (0 CUDA cores, 1 mma.sync, 2 tcgen05, 3 tcgen05 with two row tiles per CTA), 17 the thread block cluster size its key tiles were
  * split over (1 = no split). */
 int lsp_get_counters(lsp_ctx* ctx, double* out);
 int lsp_reset_counters(lsp_ctx* ctx);

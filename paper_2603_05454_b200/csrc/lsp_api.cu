@@ -334,14 +334,34 @@ int check_status(lsp_ctx* c) {
   return LSP_OK;
 }
 
+// Launch shape of one denoiser pass.  The row counts may be upper bounds of what the device-side descriptor says (the
+// lagged loop sizes a pass before it has read the previous block lengths): rows past the real ones are inert.
+struct PassDims {
+  int M = 0, Mh = 0;            // packed rows of the pass; rows that go through the LM head
+  int maxQ = 0, max_keys = 0;   // most rows / most keys of one sequence
+  long row_tiles = 0, row_pairs = 0;          // per KV head: tiles of 128 (position, head of the group) rows with rows in them; pairs of such
+  double attn_bytes = 0, attn_flops = 0;      // algorithmic attention work per layer (accounting only)
+  // a sequence of the pass: its rows and keys, query heads per KV head
+  void add(int rows, int keys, int group) {
+    M += rows;
+    maxQ = std::max(maxQ, rows);
+    if (rows <= 0) return;
+    max_keys = std::max(max_keys, keys);
+    const int per_tile = std::max(1, 128 / group), t = (rows + per_tile - 1) / per_tile;
+    row_tiles += t;
+    row_pairs += (t + 1) / 2;
+  }
+};
+
 // Suffix-over-prefix attention of layer l (Sec. 3.2: every query row of the pass sees the cached prefix [0, F_b) and all
 // of the pass's own rows).  Reads the uploaded descriptor (F, row_off), Q from q, K/V from the cache and the staging
 // planes of layer l; writes out.  early: the launch before it is a tcgen05 rotary projection, whose kernels release this launch
 // behind their own wait (see k_attn_umma).
-// q_rows: rows of Qb.  max_q: most query rows of one sequence; max_keys: most keys of one sequence.
+// q_rows: rows of Qb.
 template <typename T>
-int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const StepDesc& sd, int B, int maxQ, int max_keys, int inplace, int early) {
+int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const StepDesc& sd, int B, const PassDims& pd, int inplace, int early) {
   const lsp_model_cfg& m = c->m;
+  const int maxQ = pd.maxQ, max_keys = pd.max_keys;
   const int dh = m.head_dim, kvd = m.n_kv_heads * dh;
   const size_t plane = (size_t)c->max_rows * kvd;
   const size_t cplane = (size_t)c->max_batch * c->max_len * kvd;
@@ -375,9 +395,14 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const Step
       dim3 g3(row_tiles * cl, m.n_kv_heads, B);
       const float sl2 = scale * 1.4426950408889634f;
       const CUtensorMap* mp = &c->attn_maps[4 * l];
-      // two row tiles per CTA where that still gives every SM a CTA and the keys are more than two tiles (see attention_rows.cuh)
+      // Two row tiles per CTA (attention_rows.cuh) where that still gives every SM a CTA with rows, the keys are more than two tiles, and it
+      // saves rounds: a CTA takes about 1.6 times as long as one of a single row tile.  Rounds of one and two row tiles per CTA, passes
+      // in ms (8 to 14 key tiles): 2 and 2 17.8 and 18.2, 15.9 and 16.1; 3 and 2 20.4 20.3, 21.0 21.1, 24.6 25.1; 4 and 2 27.5 27.4, 25.7 24.4; 5 and 3
+      // 33.5 33.3; 6 and 3 40.1 39.3; 7 and 4 44.4 43.7; 7 and 5 47.7 47.6; 6 and 4 41.0 41.3.  (The launch alone at 2 and 2: 45.5 and 59.5 us.)
       const int pairs = (row_tiles + 1) / 2;
-      const bool by_rows = c->attn_rows == 2 || (c->attn_rows == 0 && row_tiles > 1 && max_keys > 2 * AU_BN && pairs * m.n_kv_heads * B >= c->n_sm);
+      const long rounds1 = (pd.row_tiles * m.n_kv_heads + c->n_sm - 1) / c->n_sm, rounds2 = (pd.row_pairs * m.n_kv_heads + c->n_sm - 1) / c->n_sm;
+      const bool by_rows = c->attn_rows == 2 || (c->attn_rows == 0 && max_keys > 2 * AU_BN && pd.row_pairs * m.n_kv_heads >= c->n_sm &&
+                                                 5 * rounds1 > 8 * rounds2);
       if (by_rows) {
         launch_k(c->pdl, k_attn_rows, dim3(pairs, m.n_kv_heads, B), dim3(AU_THREADS), (size_t)AR_SMEM, c->stream, map_q, mp[0], mp[1], mp[2], mp[3],
                  Att, sd, m.n_heads, m.n_kv_heads, c->max_len, sl2, inplace, early, c->d_status);
@@ -388,7 +413,7 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const Step
         launch_k(c->pdl, kern, g3, dim3(AU_THREADS), (size_t)AU_SMEM, c->stream, cl, map_q, mp[0], mp[1], mp[2], mp[3],
                  Att, sd, m.n_heads, m.n_kv_heads, c->max_len, sl2, cl, inplace, early, c->d_status);
       }
-      c->last_attn_kernel = 2;
+      c->last_attn_kernel = by_rows ? 3 : 2;
       c->last_attn_cluster = cl;
       done = true;
     }
@@ -432,14 +457,6 @@ void run_rmsnorm(lsp_ctx* c, const T* x, const void* gains, T* out, const int* s
   auto kern = early ? k_rmsnorm_early<T> : k_rmsnorm<T>;
   launch_k(c->pdl, kern, dim3(rows), dim3(RN_THREADS), 0, c->stream, x, (const T*)gains, out, src_rows, c->m.d_model, c->m.rms_eps);
 }
-
-// Launch shape of one denoiser pass.  The row counts may be upper bounds of what the device-side descriptor says (the
-// lagged loop sizes a pass before it has read the previous block lengths): rows past the real ones are inert.
-struct PassDims {
-  int M = 0, Mh = 0;            // packed rows of the pass; rows that go through the LM head
-  int maxQ = 0, max_keys = 0;   // most rows / most keys of one sequence
-  double attn_bytes = 0, attn_flops = 0;      // algorithmic attention work per layer (accounting only)
-};
 
 // Enqueues one pass (Algorithm 1: forward pass, scores, scan) that reads descriptor sd on the device.
 template <typename T>
@@ -490,7 +507,7 @@ int enqueue_pass(lsp_ctx* c, const StepDesc& sd, const DescInline& din, int B, c
     {
       c->counters[CNT_ATTN_BYTES] += pd.attn_bytes;
       c->counters[CNT_ATTN_FLOPS] += pd.attn_flops;
-      const int rc = run_attention<T>(c, l, Qb, M, Att, sd, B, pd.maxQ, pd.max_keys, c->kv_inplace, c->rotary_late);
+      const int rc = run_attention<T>(c, l, Qb, M, Att, sd, B, pd, c->kv_inplace, c->rotary_late);
       if (rc) return rc;
     }
     {
@@ -550,11 +567,9 @@ PassDims host_descriptor(lsp_ctx* c) {
     h[3 * s + b] = pd.M;
     h[4 * s + b] = pd.Mh;
     h[5 * s + b] = c->Fp[b];
-    pd.M += rows;
+    pd.add(rows, c->F[b] + rows, m.n_heads / m.n_kv_heads);
     pd.Mh += c->N[b];
-    pd.maxQ = std::max(pd.maxQ, rows);
     if (rows > 0) {
-      pd.max_keys = std::max(pd.max_keys, c->F[b] + rows);
       // algorithmic attention traffic: every key/value row of the sequence once per layer, plus Q and O
       pd.attn_bytes += (2.0 * (c->F[b] + rows) * kvd + 2.0 * rows * qd) * c->esz;
       pd.attn_flops += 4.0 * rows * (c->F[b] + rows) * qd;
@@ -1044,11 +1059,9 @@ int generate_lagged(lsp_ctx* c, lsp_step_rec* recs, int max_recs, int* n_steps) 
       // host state is that before step launched - 1: this step's rows of sequence b are N there (if it goes on at all)
       for (int b = 0; b < B; ++b) {
         const int rows = c->N[b] >= 2 ? c->N[b] : 0;
-        pd.M += rows;
+        pd.add(rows, total[b], c->m.n_heads / c->m.n_kv_heads);
         pd.Mh += rows > 0 ? rows - 1 : 0;
-        pd.maxQ = std::max(pd.maxQ, rows);
         if (rows > 0) {
-          pd.max_keys = std::max(pd.max_keys, total[b]);
           pd.attn_bytes += (2.0 * total[b] * kvd + 2.0 * rows * qd) * c->esz;
           pd.attn_flops += 4.0 * rows * (double)total[b] * qd;
         }
@@ -1256,17 +1269,16 @@ int lsp_op_attention(lsp_ctx* c, int layer, const void* q, const void* k_new, co
     return fail(c, LSP_ERR_ARG, "lsp_op_attention: layer %d or batch %d out of range", layer, batch);
   const int s = c->max_batch + 1;
   int* h = c->h_desc;
-  int M = 0, maxQ = 0, max_keys = 0;
+  PassDims pd;
   for (int b = 0; b < batch; ++b) {
     if (cache_len[b] < 0 || rows[b] < 0 || cache_len[b] + rows[b] > c->max_len)
       return fail(c, LSP_ERR_ARG, "lsp_op_attention: sequence %d has %d cached + %d new positions, more than max_len %d", b,
                   cache_len[b], rows[b], c->max_len);
     h[0 * s + b] = cache_len[b];
-    h[3 * s + b] = M;
-    M += rows[b];
-    maxQ = std::max(maxQ, rows[b]);
-    if (rows[b] > 0) max_keys = std::max(max_keys, cache_len[b] + rows[b]);
+    h[3 * s + b] = pd.M;
+    pd.add(rows[b], cache_len[b] + rows[b], c->m.n_heads / c->m.n_kv_heads);
   }
+  const int M = pd.M;
   h[3 * s + batch] = M;
   c->proposed = false;                 // the descriptor of a pending lsp_denoise_step is overwritten
   if (M == 0) return LSP_OK;
@@ -1277,8 +1289,8 @@ int lsp_op_attention(lsp_ctx* c, int layer, const void* q, const void* k_new, co
   char* stK = c->stage + (size_t)(2 * layer) * plane;
   CU(cudaMemcpyAsync(stK, k_new, (size_t)M * kvd * c->esz, cudaMemcpyDeviceToDevice, c->stream));
   CU(cudaMemcpyAsync(stK + plane, v_new, (size_t)M * kvd * c->esz, cudaMemcpyDeviceToDevice, c->stream));
-  const int rc = c->m.dtype == 0 ? run_attention<float>(c, layer, (const float*)q, M, (float*)out, desc_of(c), batch, maxQ, max_keys, 0, 0)
-                                 : run_attention<bf16>(c, layer, (const bf16*)q, M, (bf16*)out, desc_of(c), batch, maxQ, max_keys, 0, 0);
+  const int rc = c->m.dtype == 0 ? run_attention<float>(c, layer, (const float*)q, M, (float*)out, desc_of(c), batch, pd, 0, 0)
+                                 : run_attention<bf16>(c, layer, (const bf16*)q, M, (bf16*)out, desc_of(c), batch, pd, 0, 0);
   if (rc) return rc;
   CU(cudaMemcpyAsync(c->h_status, c->d_status, 16, cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));

@@ -38,7 +38,8 @@ extern "C" {
  * tcgen05 attention:
  *   28 fewest (query row x group head) rows of a (sequence, KV head) for which the tcgen05 kernel is used (default 0)
  *   30 it splits a row tile's keys over a thread block cluster when there are few CTAs (1, default)
- *   47 two row tiles per CTA (k_attn_rows): 0 = where that gives every SM a CTA (default), 1 = never, 2 = always
+ *   47 two row tiles per CTA (k_attn_rows): 0 = where that gives every SM a CTA and saves rounds
+ *      (default), 1 = never, 2 = always
  * decode loop:
  *   31 with device-resident block lengths (lsp_set_option key 4), lsp_generate reads every step before sizing the next
  *      once at most this many masked positions per sequence remain (default 8)

@@ -167,8 +167,34 @@ def test_attention_row_tiles_that_a_group_does_not_fill(case):
 ])
 def test_attention_with_two_row_tiles_per_cta(hq, hkv, F, rows):
     """The kernel of the large passes at every row count, also over memory that was never written."""
-    _run_case(hq, hkv, F, rows, 2048, seed=8, opts=[(47, 2)])
-    _run_case(hq, hkv, F, rows, 2048, seed=9, opts=[(47, 2)], poison=True)
+    for seed, poison in ((8, False), (9, True)):
+        _, cnt = _run_case(hq, hkv, F, rows, 2048, seed=seed, opts=[(47, 2)], poison=poison)
+        assert int(cnt["attn_kernel"]) == 3
+
+
+@pytest.mark.parametrize("hq,hkv,F,rows,kernel", [
+    (32, 32, [300] * 4, [500] * 4, 3),                 # four row tiles each: 512 CTAs in four rounds of 148, or 256 in two
+    (32, 32, [700] * 3, [296] * 3, 2),                 # three: two rounds either way, of longer CTAs
+    (32, 32, [300] * 4, [380] * 4, 2),                 # three rounds or two: no gain
+    (32, 32, [300] + [900] * 7, [600] + [0] * 7, 2),   # 160 CTAs with rows and none for the finished sequences
+    (32, 32, [300] * 8, [600] + [20] * 7, 2),          # the same with a few rows each
+    (32, 32, [0] * 8, [256] * 8, 2),                   # two key tiles
+    (32, 32, [1] * 8, [256] * 8, 3),
+    (28, 4, [300] * 12, [234] * 12, 3),                # 13 tiles of 18 positions: 624 CTAs or 336
+])
+def test_attention_takes_two_row_tiles_per_cta_where_that_saves_rounds(hq, hkv, F, rows, kernel):
+    """The rule counts CTAs that have rows; launch counts are for 148 SMs."""
+    from paper_2603_05454_b200 import LSPDecoder, SchedCfg
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the row counts are for 148 SMs")
+    sh = S.ModelShape(1, 64, hq, hkv, 128, 64, 256, dtype="bf16")
+    dec = LSPDecoder(sh, S.make_weights(sh, 0, device=DEV), SchedCfg(), len(rows), max(map(sum, zip(F, rows))), device=DEV)
+    q, k, v = (torch.zeros(sum(rows), h * 128, dtype=torch.bfloat16, device=DEV) for h in (hq, hkv, hkv))
+    dec.kv_view().zero_()
+    dec.op_attention(0, q, k, v, torch.empty_like(q), F, rows)
+    got = int(dec.counters()["attn_kernel"])
+    dec.close()
+    assert got == kernel
 
 
 @pytest.mark.parametrize("hq,hkv,F,rows", [(32, 32, 300, 200), (32, 8, 700, 257), (28, 4, 0, 600)])
