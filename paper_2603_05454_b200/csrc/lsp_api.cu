@@ -471,10 +471,11 @@ int enqueue_pass(lsp_ctx* c, const StepDesc& sd, const DescInline& din, int B, c
   T* Att = (T*)c->Att;
   T* Hf = (T*)c->Hf;
   seg_begin(c, CLS_MISC);
-  // where a row fits the block's registers the first norm goes with the embedding (not with many rows: the registers cost more, as in run_rmsnorm)
+  // where a row fits the block's registers the first norm goes with the embedding (not with many rows: see k_assemble_embed)
   const bool norm0 = M <= 1024 && d / Vec16<T>::N <= RN_VPT * RN_THREADS;
-  launch_k(c->pdl, k_assemble_embed<T>, dim3(M), dim3(RN_THREADS), 0, c->stream, sd, din, B, c->tokens, c->tok_stride, m.mask_id, (const T*)c->embed,
-           d, X, c->row_seq, c->row_pos, c->head_src, c->head_pos, scattered ? 1 : 0, (const T*)c->attn_norm[0], norm0 ? Nrm : (T*)nullptr, m.rms_eps);
+  launch_k(c->pdl, norm0 ? k_assemble_embed<T, true> : k_assemble_embed<T, false>, dim3(M), dim3(norm0 ? RN_THREADS : EMBED_THREADS), 0, c->stream,
+           sd, din, B, c->tokens, c->tok_stride, m.mask_id, (const T*)c->embed, d, X, c->row_seq, c->row_pos, c->head_src, c->head_pos,
+           scattered ? 1 : 0, (const T*)c->attn_norm[0], Nrm, m.rms_eps);
   CU(cudaGetLastError());
   if (scattered) {
     launch_k(c->pdl, k_compact_masked, dim3(B), dim3(256), 0, c->stream, sd, (const int32_t*)c->tokens, c->tok_stride, m.mask_id,

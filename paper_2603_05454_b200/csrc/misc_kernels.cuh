@@ -32,15 +32,18 @@ __device__ __forceinline__ uint4 f_to_vec(const float (&v)[8]) {
 // ---------------------------------------------------------------------------------------------
 // Row assembly + embedding (input of Algorithm 1's forward pass): packed row r of sequence b is position
 // F_b + j; the first pend_b rows carry the tokens committed by the previous step, the rest [MASK].
-// One block per row.  Also fills row_seq / row_pos and the list of rows that go through the LM head, and, with norm_out, applies the
+// One block per row.  Also fills row_seq / row_pos and the list of rows that go through the LM head, and, kNorm, applies the
 // first layer's RMSNorm to the row while it is in registers (as k_rmsnorm does, to the bit; a launch less per pass, about 3.5 us).
+// kNorm is for at most 1024 rows of at most RN_VPT vectors per thread: its 64 registers and 256 threads leave 4 rows on an SM, the copy
+// alone (32 registers, 128 threads) 16 (8240 rows of 4096 copied by the kernel with the norm in it +17 us, 4096 of 3584 +6).
 // ---------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(RN_THREADS) k_assemble_embed(StepDesc sd, const __grid_constant__ DescInline in, int batch, const int32_t* tokens, int tok_stride,
-                                 int mask_id, const T* __restrict__ embed, int d, T* __restrict__ X,
-                                 int* __restrict__ row_seq, int* __restrict__ row_pos,
-                                 int* __restrict__ head_src, int* __restrict__ head_pos, int scattered, const T* __restrict__ g,
-                                 T* __restrict__ norm_out, float eps) {
+constexpr int EMBED_THREADS = 128;      // without the norm
+template <typename T, bool kNorm>
+__global__ void __launch_bounds__(kNorm ? RN_THREADS : EMBED_THREADS)
+k_assemble_embed(StepDesc sd, const __grid_constant__ DescInline in, int batch, const int32_t* tokens, int tok_stride, int mask_id,
+                 const T* __restrict__ embed, int d, T* __restrict__ X, int* __restrict__ row_seq, int* __restrict__ row_pos,
+                 int* __restrict__ head_src, int* __restrict__ head_pos, int scattered, const T* __restrict__ g, T* __restrict__ norm_out,
+                 float eps) {
   constexpr int E = Vec16<T>::N;
   __shared__ float red[RN_THREADS / 32];
   pdl_release();
@@ -48,7 +51,7 @@ __global__ void __launch_bounds__(RN_THREADS) k_assemble_embed(StepDesc sd, cons
   const int nv = d / E;
   uint4 keep[RN_VPT], gain[RN_VPT];
   const uint4* gr = reinterpret_cast<const uint4*>(g);
-  if (norm_out != nullptr) {
+  if constexpr (kNorm) {
 #pragma unroll
     for (int j = 0; j < RN_VPT; ++j) {
       const int i = threadIdx.x + j * RN_THREADS;
@@ -76,7 +79,7 @@ __global__ void __launch_bounds__(RN_THREADS) k_assemble_embed(StepDesc sd, cons
     uint4* zn = reinterpret_cast<uint4*>(norm_out + (size_t)r * d);
     for (int i = threadIdx.x; i < nv; i += blockDim.x) {
       z[i] = make_uint4(0u, 0u, 0u, 0u);
-      if (norm_out != nullptr) zn[i] = make_uint4(0u, 0u, 0u, 0u);
+      if (kNorm) zn[i] = make_uint4(0u, 0u, 0u, 0u);
     }
     return;
   }
@@ -98,7 +101,7 @@ __global__ void __launch_bounds__(RN_THREADS) k_assemble_embed(StepDesc sd, cons
   }
   const uint4* src = reinterpret_cast<const uint4*>(embed + (size_t)tok * d);
   uint4* dst = reinterpret_cast<uint4*>(X + (size_t)r * d);
-  if (norm_out == nullptr) {
+  if constexpr (!kNorm) {
     for (int i = threadIdx.x; i < nv; i += blockDim.x) dst[i] = __ldg(src + i);
     return;
   }
