@@ -103,40 +103,40 @@ k_assemble_embed(StepDesc sd, const __grid_constant__ DescInline in, int batch, 
   uint4* dst = reinterpret_cast<uint4*>(X + (size_t)r * d);
   if constexpr (!kNorm) {
     for (int i = threadIdx.x; i < nv; i += blockDim.x) dst[i] = __ldg(src + i);
-    return;
-  }
+  } else {
 #pragma unroll
-  for (int j = 0; j < RN_VPT; ++j) {
-    const int i = threadIdx.x + j * RN_THREADS;
-    keep[j] = (i < nv) ? __ldg(src + i) : make_uint4(0u, 0u, 0u, 0u);
-  }
-  float ss = 0.f;
+    for (int j = 0; j < RN_VPT; ++j) {
+      const int i = threadIdx.x + j * RN_THREADS;
+      keep[j] = (i < nv) ? __ldg(src + i) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    float ss = 0.f;
 #pragma unroll
-  for (int j = 0; j < RN_VPT; ++j) {
-    float v[E];
-    vec_to_f(keep[j], v);
-#pragma unroll
-    for (int e = 0; e < E; ++e) ss += v[e] * v[e];
-  }
-  ss = warp_sum(ss);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  float tot = 0.f;
-#pragma unroll
-  for (int w = 0; w < RN_THREADS / 32; ++w) tot += red[w];
-  const float inv = rsqrtf(__fdividef(tot, (float)d) + eps);
-  uint4* o = reinterpret_cast<uint4*>(norm_out + (size_t)r * d);
-#pragma unroll
-  for (int j = 0; j < RN_VPT; ++j) {
-    const int i = threadIdx.x + j * RN_THREADS;
-    if (i < nv) {
-      float v[E], gv[E];
+    for (int j = 0; j < RN_VPT; ++j) {
+      float v[E];
       vec_to_f(keep[j], v);
-      vec_to_f(gain[j], gv);
 #pragma unroll
-      for (int e = 0; e < E; ++e) v[e] = v[e] * inv * gv[e];
-      dst[i] = keep[j];
-      o[i] = f_to_vec(v);
+      for (int e = 0; e < E; ++e) ss += v[e] * v[e];
+    }
+    ss = warp_sum(ss);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    float tot = 0.f;
+#pragma unroll
+    for (int w = 0; w < RN_THREADS / 32; ++w) tot += red[w];
+    const float inv = rsqrtf(__fdividef(tot, (float)d) + eps);
+    uint4* o = reinterpret_cast<uint4*>(norm_out + (size_t)r * d);
+#pragma unroll
+    for (int j = 0; j < RN_VPT; ++j) {
+      const int i = threadIdx.x + j * RN_THREADS;
+      if (i < nv) {
+        float v[E], gv[E];
+        vec_to_f(keep[j], v);
+        vec_to_f(gain[j], gv);
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = v[e] * inv * gv[e];
+        dst[i] = keep[j];
+        o[i] = f_to_vec(v);
+      }
     }
   }
 }
