@@ -45,8 +45,9 @@ template <typename Epi> struct SimtTile {
 constexpr int SG_HEAD_BN = 64;    // columns per partial of the head, in both kernels
 
 // grid = (ceil(NP / PER_TILE) * slices, ceil(M / BM)), block = 256, clusters of slices CTAs along x: the K slices of a tile.  A: [M, K];
-// W0/W1: [*, K] row-major.
-template <typename T, typename Epi>
+// W0/W1: [*, K] row-major.  kSliced: slices > 1 (a kernel of its own: with the slices' arithmetic and sums as run-time branches a launch
+// without them took 0.2 to 0.3 us more: fp32, K 256, 33 x 1024 7.2 -> 7.5, 64 x 2 x 1024 8.3 -> 8.6).
+template <typename T, typename Epi, bool kSliced>
 __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* A, const T* __restrict__ W0,
                                                                    const T* __restrict__ W1, int M, int NP, int K, int slices, Epi epi) {
   constexpr int BM = SimtTile<Epi>::BM, BN = SimtTile<Epi>::BN, PT = SimtTile<Epi>::PER_TILE;
@@ -57,7 +58,7 @@ __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* A, c
   __shared__ __align__(16) float sm[SG_WARPS * (WARP_F > RED_F ? WARP_F : RED_F)];
   pdl_begin();
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-  const int tile = blockIdx.x / (unsigned)slices, slice = blockIdx.x % (unsigned)slices;
+  const int tile = kSliced ? blockIdx.x / (unsigned)slices : blockIdx.x, slice = kSliced ? blockIdx.x % (unsigned)slices : 0;
   const int m0 = blockIdx.y * BM, j0 = tile * PT;
   float* As = sm + w * WARP_F;
   float* Bs = As + SG_KS * LA;
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* A, c
 #pragma unroll
     for (int i = 0; i < NB; ++i) bv[i] = bp[i] ? load4(bp[i] + k0) : zero;
   };
-  const int lo = K / SG_KS * slice / slices, steps = K / SG_KS * (slice + 1) / slices;
+  const int lo = kSliced ? K / SG_KS * slice / slices : 0, steps = kSliced ? K / SG_KS * (slice + 1) / slices : K / SG_KS;
   if (lo + w < steps) load((lo + w) * SG_KS);
   for (int s = lo + w; s < steps; s += SG_WARPS) {
     __syncwarp();
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(32 * SG_WARPS) k_gemm_simt_split(const T* A, c
   // K slices: every CTA leaves its sums in its shared memory, and the first one adds them in slice (= K) order (true: this CTA
   // finishes the tile)
   auto sum_slices = [&](float (&v)[4]) -> bool {
-    if (Epi::kReduce || slices == 1) return true;
+    if constexpr (!kSliced) return true;
     float4* out = reinterpret_cast<float4*>(sm);
     __syncthreads();                     // the warps' partial tiles have been read
     if (slice > 0) out[t] = make_float4(v[0], v[1], v[2], v[3]);

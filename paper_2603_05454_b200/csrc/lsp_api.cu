@@ -253,7 +253,11 @@ int run_gemm(lsp_ctx* c, const T* A, const T* W0, const T* W1, int M, int NP, in
     grid = dim3((NP + Tile::PER_TILE - 1) / Tile::PER_TILE, (M + Tile::BM - 1) / Tile::BM);
     const int slices = simt_slices((long)grid.x * grid.y, K, c->n_sm, Epi::kReduce);
     grid.x *= slices;
-    CU(launch_k(c->pdl, k_gemm_simt_split<T, Epi>, grid, dim3(256), 0, c->stream, slices, A, W0, W1, M, NP, K, slices, epi));
+    auto kern = k_gemm_simt_split<T, Epi, false>;
+    if constexpr (!Epi::kReduce) {
+      if (slices > 1) kern = k_gemm_simt_split<T, Epi, true>;
+    }
+    CU(launch_k(c->pdl, kern, grid, dim3(256), 0, c->stream, slices, A, W0, W1, M, NP, K, slices, epi));
   } else {
     CU(launch_k(c->pdl, k_gemm_simt<T, Epi>, grid, dim3(256), 0, c->stream, A, W0, W1, M, NP, K, epi));
   }
