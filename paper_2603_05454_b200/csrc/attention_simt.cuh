@@ -186,9 +186,11 @@ __global__ void __launch_bounds__(128) k_attn_simt_split(const T* q, const T* ca
       d4[3] = fmaf(qv.w, kr[i].w, d4[3]);
     }
     const float sc = key < S ? ((d4[0] + d4[1]) + (d4[2] + d4[3])) * scale : -INFINITY;
+    // (a score that overflowed to -inf has no weight, also where a warp has met no other yet: the kernel above has by then unless it
+    // is the first tile's)
     const float m_new = fmaxf(m, warp_max(sc));
-    const float p = key < S ? __expf(sc - m_new) : 0.f;
-    const float corr = __expf(m - m_new);
+    const float p = sc == -INFINITY ? 0.f : __expf(sc - m_new);
+    const float corr = m_new == -INFINITY ? 1.f : __expf(m - m_new);
     l = l * corr + warp_sum(p);
     m = m_new;
     if (DH != 64) load_v();

@@ -172,6 +172,34 @@ def test_attention_with_two_row_tiles_per_cta(hq, hkv, F, rows):
         assert int(cnt["attn_kernel"]) == 3
 
 
+@pytest.mark.parametrize("dh", [64, 128])
+@pytest.mark.parametrize("lo,hi", [(32, 64), (96, 160), (40, 190)])
+def test_attention_on_cuda_cores_with_scores_that_overflow(dh, lo, hi):
+    """fp32 scores of keys [lo, hi) below the type's range: they get no weight and the other keys give the result, also where they
+    fill a warp's first tile of 32 keys.  (Keys 0 .. 31 are finite.)"""
+    from paper_2603_05454_b200 import LSPDecoder, SchedCfg
+    F, Q, H = 180, 12, 2
+    sh = S.ModelShape(1, 64, H, H, dh, 64, 256, dtype="fp32")
+    dec = LSPDecoder(sh, S.make_weights(sh, 0, device=DEV), SchedCfg(), 1, 256, device=DEV)
+    q, k, v = (S.normal((Q, H * dh), 4, i, 1.0, torch.float32, DEV) for i in (1, 2, 3))
+    q[:, ::dh] = 1e20                                     # the first element of every head: finite keys have none of it
+    k[:, ::dh] = 0.0
+    kv = dec.kv_view()
+    kv[0, :, 0, :F] = S.normal((2, F, H, dh), 4, 5, 1.0, torch.float32, DEV)
+    kv[0, 0, 0, :F, :, 0] = 0.0
+    keys, vals = (torch.cat([kv[0, i, 0, :F], x.view(Q, H, dh)]).double() for i, x in ((0, k), (1, v)))
+    kv[0, 0, 0, lo:min(hi, F), :, 0] = -1e20
+    k.view(Q, H, dh)[:max(0, hi - F), :, 0] = -1e20
+    out = torch.empty_like(q)
+    dec.op_attention(0, q, k, v, out, [F], [Q])
+    dec.close()
+    z = torch.einsum("qhd,khd->hqk", q.view(Q, H, dh).double(), keys) / dh ** 0.5
+    z[:, :, lo:hi] = -float("inf")
+    ref = torch.einsum("hqk,khd->qhd", torch.softmax(z, -1), vals).reshape(Q, H * dh)
+    assert bool(torch.isfinite(out).all())
+    assert float((out.double() - ref).abs().max()) <= 2e-5        # fp32 sums of 192 terms, as the fp32 decodes
+
+
 @pytest.mark.parametrize("hq,hkv,F,rows,kernel", [
     (32, 32, [300] * 4, [500] * 4, 3),                 # four row tiles each: 512 CTAs in four rounds of 148, or 256 in two
     (32, 32, [700] * 3, [296] * 3, 2),                 # three: two rounds either way, of longer CTAs
