@@ -189,8 +189,9 @@ __global__ void __launch_bounds__(128) k_attn_simt_split(const T* q, const T* ca
     // (a score that overflowed to -inf has no weight, also where a warp has met no other yet: the kernel above has by then unless it
     // is the first tile's)
     const float m_new = fmaxf(m, warp_max(sc));
-    const float p = sc == -INFINITY ? 0.f : __expf(sc - m_new);
-    const float corr = m_new == -INFINITY ? 1.f : __expf(m - m_new);
+    const float m_ref = m_new == -INFINITY ? 0.f : m_new;
+    const float p = key < S ? __expf(sc - m_ref) : 0.f;
+    const float corr = __expf(m - m_ref);
     l = l * corr + warp_sum(p);
     m = m_new;
     if (DH != 64) load_v();
