@@ -436,7 +436,10 @@ int run_attention(lsp_ctx* c, int l, const T* Qb, int q_rows, T* Att, const Step
       done = true;
     }
   }
-  if (!done && (long)maxQ * m.n_heads * B <= 3l * c->n_sm) {
+  // (bf16 rows of 64 elements over at most 40 keys, one tile and a bit: a warp has nearly all of them, and the other kernel shares their
+  // loads: 12 queries of 16 heads over 12 / 32 keys 9.0 and 10.5, 9.9 and 11.9 us; over 52 equal; over 112 17.7 and 13.9)
+  const bool few_keys = sizeof(T) == 2 && dh == 64 && max_keys <= 40;
+  if (!done && !few_keys && (long)maxQ * m.n_heads * B <= 3l * c->n_sm) {
     auto kern = dh == 128 ? k_attn_simt_split<T, 128> : k_attn_simt_split<T, 64>;
     launch_k(c->pdl, kern, dim3(maxQ, m.n_heads, B), dim3(128), 0, c->stream, Qb, cK, cV, stK, stV, Att, sd, m.n_heads, m.n_kv_heads,
              (size_t)c->max_len * kvd, scale, inplace);
