@@ -534,14 +534,21 @@ inline bool pair_half_last(int M, int bn) {
   const int last = M % PR_ROWS;
   return M > PR_ROWS && last >= 1 && last <= PR_ROWS / 2 && bn % 64 == 0;
 }
-inline PairShape pair_shape(const UmmaState& st, int M, int cols, int K, int step, bool may_split, bool may_halve) {
+// Column tiles of width bn.  rot_half: pair indices per head of a rotary epilogue (else 0); where a half tile is no whole head halves, two
+// tiles are the halves of bn / 64 heads (see PairArgs::unit), and the last two may stand for fewer.
+inline int pair_tiles(int cols, int bn, int rot_half) {
+  if (rot_half == 0 || bn / 2 % rot_half == 0) return (cols + bn - 1) / bn;
+  const int heads = cols / (2 * rot_half), nb = bn / 64;
+  return (heads + nb - 1) / nb * 2;
+}
+inline PairShape pair_shape(const UmmaState& st, int M, int cols, int K, int step, bool may_split, bool may_halve, int rot_half) {
   const int pairs = st.max_clusters[2];
   const long rg = (M + PR_ROWS - 1) / PR_ROWS;
   const double chunks = (K + 127) / 128;
   PairShape best{256, 1};
   double best_cost = 1e30;
   for (int bn = 256; bn >= 96; bn -= step) {
-    const long t = (long)((cols + bn - 1) / bn) * rg;
+    const long t = (long)pair_tiles(cols, bn, rot_half) * rg;
     const long rounds = (t + pairs - 1) / pairs;
     const double share = (may_halve && pair_half_last(M, bn)) ? (rg - 0.25) / rg : 1.0;     // of a full tile's time
     const double cost = share * chunks * (rounds > 2 ? rounds * (bn + 44) * 1.8 : rounds * (bn + 256)) * 1.06e-3;
@@ -563,13 +570,14 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
   const int pairs = st.max_clusters[2];
   constexpr bool kPlain = !Epi::kDual && !Epi::kReduce;
   PairShape shape{UM_HEAD_BN, 1};
-  int chains = 1;
+  int chains = 1, rot_half = 0;
+  if constexpr (kRope) rot_half = epi.half;
   if constexpr (Epi::kReduce) {
     const HeadShape h = umma_head_shape(st, M, NP, K);
     shape.bn = h.bn;
     chains = std::min(h.chains, K / UM_BK);
   } else {
-    shape = pair_shape(st, M, cols, K, kRope ? 64 : 32, kPlain && st.pair_split != 1, !kRope);
+    shape = pair_shape(st, M, cols, K, kRope ? 64 : 32, kPlain && st.pair_split != 1, !kRope, rot_half);
     if (st.pair_bn > 0 && (!kRope || st.pair_bn % 64 == 0)) shape = {st.pair_bn, 1};      // (a width that the epilogue can take)
   }
   const int bn = shape.bn;
@@ -624,12 +632,7 @@ int pair_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16* W
       }
     }
   }
-  const int per_tile = Epi::kDual ? bn / 2 : bn;
-  int n_tiles = (NP + per_tile - 1) / per_tile;
-  if constexpr (kRope) {
-    const int heads = NP / epi.half, nb = bn / 64;
-    if (unit) n_tiles = (heads + nb - 1) / nb * 2;
-  }
+  const int n_tiles = pair_tiles(cols, bn, rot_half);
   const int rg = (M + PR_ROWS - 1) / PR_ROWS;
   const long T = (long)n_tiles * rg;
   if (T > (1l << 24)) { st.err = "too many tiles for the paired GEMM"; return -9; }

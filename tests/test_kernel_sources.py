@@ -103,6 +103,15 @@ def test_producers_that_share_a_stage_outstay_their_copies_after_a_failure(name,
         assert "if ((" + " || ".join(f"warp == {w}" for w in warps) + ") && *abort_flag) um_let_land();\n  tc_fence_before();\n  __syncthreads();" in body
 
 
+def test_the_paired_gemm_models_the_tiles_that_it_launches():
+    """The choice of a tile width and the launch count column tiles by one function (rotary tiles of several heads come in twos)."""
+    src = _source("gemm_pair.cuh")
+    assert re.findall(r"[^\n]*pair_tiles\([^\n]*", src) == [
+        "inline int pair_tiles(int cols, int bn, int rot_half) {",
+        "    const long t = (long)pair_tiles(cols, bn, rot_half) * rg;",
+        "  const int n_tiles = pair_tiles(cols, bn, rot_half);"]
+
+
 def test_the_step_driver_assumes_no_sm_count():
     """The dispatch lines of the CUDA-core kernels (fp32 models among them) are in SMs of the device at hand."""
     assert not re.search(r"\b148\b", _source("lsp_api.cu")) and "cudaDevAttrMultiProcessorCount" in _source("lsp_api.cu")
