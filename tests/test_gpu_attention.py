@@ -114,11 +114,13 @@ def test_attention_ignores_memory_it_never_wrote():
     _run_case(8, 2, [129, 5, 250], [3, 0, 60], 320, attn_impl=1, seed=5, poison=True)
 
 
-@pytest.mark.parametrize("hq,hkv,F,rows", [
-    (32, 32, [525 + 3 * b for b in range(7)], [50] * 7),      # five and more key tiles per CTA, the last cached one ragged
-    (32, 32, [490, 493], [43, 38]),                            # the same on clusters of 2
+@pytest.mark.parametrize("hq,hkv,F,rows,key47", [
+    (32, 32, [525 + 3 * b for b in range(7)], [50] * 7, 0),      # five and more key tiles per CTA, the last cached one ragged
+    (32, 32, [490, 493], [43, 38], 0),                            # the same on clusters of 2
+    (32, 32, [525 + 3 * b for b in range(4)], [200, 190, 131, 257], 2),      # two row tiles per CTA, both of whose groups clear rows
+    (28, 4, [390, 130, 7], [300, 40, 129], 2),
 ])
-def test_attention_repeats_bit_for_bit_with_ragged_tiles(hq, hkv, F, rows):
+def test_attention_repeats_bit_for_bit_with_ragged_tiles(hq, hkv, F, rows, key47):
     """The rows of a ragged V tile past the last key are cleared in shared memory; done while the stage still waited for an
     earlier tile, the clear took rows of that tile's V (one launch in four on the first case).  Repeated launches over several
     layers (more K/V than the L2 cache holds) must give the first launch's bits."""
@@ -131,6 +133,7 @@ def test_attention_repeats_bit_for_bit_with_ragged_tiles(hq, hkv, F, rows):
                  w_down=z(d, 64))
     dec = LSPDecoder(sh, dict(embed=z(256, d), w_head=z(256, d), final_norm=z(d), layers=[layer] * L), SchedCfg(), B, max(F) + max(rows),
                      device=DEV)
+    dec.debug_set(47, key47)
     M, bf = int(sum(rows)), torch.bfloat16
     q, kn, vn = (S.normal((M, h * dh), 0, i, 1.0, bf, DEV) for i, h in ((1, hq), (2, hkv), (3, hkv)))
     dec.kv_view().normal_(generator=torch.Generator(device=DEV).manual_seed(0))

@@ -14,7 +14,7 @@ NEAR = oscan.FLAG_NEAR_THRESHOLD | oscan.FLAG_NEAR_TIE
 
 
 def _teacher_forced(shape, seed, P, G, sched, delim, impl=None, attn_impl=None, max_steps=None, gains_seed=None,
-                    max_batch=1, extra_len=0, poison=False, inplace=False):
+                    max_batch=1, extra_len=0, poison=False, inplace=False, opts=()):
     """Runs the GPU path step by step, committing the ORACLE's lengths, and compares every step's outputs."""
     from paper_2603_05454_b200 import LSPDecoder
     tol = tol_for(shape.dtype)
@@ -56,6 +56,8 @@ def _teacher_forced(shape, seed, P, G, sched, delim, impl=None, attn_impl=None, 
         dec.set_option(1, attn_impl)
         if attn_impl == 2:
             dec.debug_set(28, 0)          # the tcgen05 kernel at every row count, not only from its default threshold
+    for key, value in opts:
+        dec.debug_set(key, value)
     tokens = torch.zeros(1, P + G, dtype=torch.int32, device=DEV)
     tokens[0, :P] = prompt[0].to(DEV)
     dec.begin(tokens, [P], [G])
@@ -66,6 +68,8 @@ def _teacher_forced(shape, seed, P, G, sched, delim, impl=None, attn_impl=None, 
         rec = dec.denoise_step()[0]
         y, p, m = dec.scores()
         assert rec["n_before"] == o["n_before"] and rec["rows"] == o["rows"]
+        if (47, 2) in opts:
+            assert int(dec.counters()["attn_kernel"]) == 3
         used_p, used_z = max(used_p, float(np.abs(p - o["pmax"]).max())), max(used_z, float(np.abs(m - o["delta"]).max()))
         assert np.abs(p - o["pmax"]).max() <= tol_p, (o["step"], np.abs(p - o["pmax"]).max(), tol_p)
         assert np.abs(m - o["delta"]).max() <= tol_z, (o["step"], np.abs(m - o["delta"]).max(), tol_z)
@@ -316,6 +320,18 @@ def test_in_place_kv_layout_matches_the_oracle(dtype, dh, hq, hkv):
     sh = S.ModelShape(2, hq * dh, hq, hkv, dh, 512, 2048, dtype=dtype, head_scale=1.5, w_std=0.5 / (hq * dh) ** 0.5)
     _teacher_forced(sh, 61, 150, 170, SchedCfg(mode=2, fixed_k=45), (1, 200), max_steps=4, inplace=True)
     _teacher_forced(sh, 62, 40, 90, SchedCfg(tau=0.04), (1, 400), inplace=True, poison=True, extra_len=50, max_batch=2)
+
+
+@pytest.mark.parametrize("inplace", [False, True])
+@pytest.mark.parametrize("hq,hkv,P", [(4, 2, 127), (7, 1, 255), (4, 4, 383)])
+def test_two_row_tiles_per_cta_in_passes_whose_prefix_crosses_a_key_tile(hq, hkv, P, inplace):
+    """k_attn_rows reads key tiles of the prefix ahead of its wait for the projection, in place only those that end ahead of the pass's
+    first row.  One position is committed at a time, so the passes have prefixes of 0, then one below, at and one above a multiple of 128;
+    the cache and the staging planes held NaN."""
+    from paper_2603_05454_b200 import SchedCfg
+    sh = S.ModelShape(2, hq * 128, hq, hkv, 128, 512, 2048, dtype="bf16", head_scale=1.5, w_std=0.5 / (hq * 128) ** 0.5)
+    steps, _ = _teacher_forced(sh, 63, P, 150, SchedCfg(mode=2, fixed_k=1), (1, 2), max_steps=4, inplace=inplace, poison=True, opts=[(47, 2)])
+    assert steps == 4
 
 
 def test_in_place_kv_layout_free_running_batch_equals_the_staged_layout_where_unflagged():
