@@ -213,6 +213,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     for (int it = n_pre; it < n_units; ++it) {
       if (!__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, abort_flag))) {
         if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 11u; }
+        um_let_land();
         break;
       }
       request_weights(s);
@@ -220,8 +221,12 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       if (++s == S) { s = 0; ph ^= 1u; }
     }
     // do not leave while copies, these or the activations', may still be landing in this CTA's shared memory
-    // (after a failure: see the end)
-    for (int it = issued > S ? issued - S : 0; it < issued; ++it) mbar_wait(full_bar(it % S), (uint32_t)(it / S) & 1u, abort_flag);
+    for (int it = issued > S ? issued - S : 0; it < issued; ++it) {
+      if (!__all_sync(0xffffffffu, mbar_wait(full_bar(it % S), (uint32_t)(it / S) & 1u, abort_flag))) {
+        um_let_land();
+        break;
+      }
+    }
   } else if (warp == 6) {
     // ---------------- TMA producer of the activations ----------------
     // (the same stages in the same order; they may arrive ahead of the stage's arming: its phase ends with both.  A warp of its
@@ -235,6 +240,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     for (int it = 0; it < n_units; ++it) {
       if (it >= n_pre && !__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, abort_flag))) {
         if (lane == 0 && !*abort_flag) { *abort_flag = 1; atomicExch(args.status, 1u); args.status[1] = 15u; }
+        um_let_land();
         break;
       }
       if (elect_one()) load_acts(p, s);
@@ -711,7 +717,6 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       cluster_sync();      // nobody leaves while a peer may still read its shared memory
     }
   }
-  if ((warp == 0 || warp == 6) && *abort_flag) um_let_land();
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {

@@ -99,8 +99,12 @@ def test_producers_that_share_a_stage_outstay_their_copies_after_a_failure(name,
     assert issuing == warps
     if len(warps) == 1:
         assert "if (!ok) um_let_land();" in roles[2]
-    else:
-        assert "if ((" + " || ".join(f"warp == {w}" for w in warps) + ") && *abort_flag) um_let_land();\n  tc_fence_before();\n  __syncthreads();" in body
+        return
+    for w, r in zip(roles[1::2], roles[2::2]):
+        if w in map(str, warps):          # every wait of such a warp that expires
+            waits = re.split(r"if \(!__all_sync\(0xffffffffu, mbar_wait\(|&& !__all_sync\(0xffffffffu, mbar_wait\(", r)[1:]
+            assert len(waits) == (2 if w == "0" else 1) == r.count("mbar_wait(")
+            assert all(re.search(r"um_let_land\(\);\s*break;", x) for x in waits)
 
 
 def test_the_paired_gemm_models_the_tiles_that_it_launches():
