@@ -79,7 +79,9 @@ constexpr int ST_THREADS = 224;
 // tile still cover it, and results do not depend on timing.
 constexpr int ST_ROT = 4;
 
-template <int BN, typename Epi>
+// kChains: the rotary epilogue's several accumulators (args.chains), one whole tile per CTA: a kernel of its own, because the one without
+// them runs with up to 128 rows and was 0.5 to 0.8 % of a pass slower for them.
+template <int BN, typename Epi, bool kChains = false>
 __global__ void __launch_bounds__(ST_THREADS, 1)
 k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b0,
               const __grid_constant__ CUtensorMap map_b1, StreamArgs args, Epi epi) {
@@ -93,7 +95,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
   constexpr int SET_COLS = BN;                            // columns of one accumulator set
   constexpr int NBUF = 2;                                 // accumulator sets in tensor memory
   // tensor memory is allocated in powers of two (192-wide tiles use 384 of 512 columns)
-  constexpr bool kChains = kRope && BN == 128;            // (see args.chains: up to four accumulators of one tile)
+  static_assert(!kChains || (kRope && BN == 128), "up to four accumulators of a tile");
   constexpr uint32_t TMEM_COLS = kChains ? 512 : (NBUF * SET_COLS <= 128) ? 128 : (NBUF * SET_COLS <= 256 ? 256 : 512);
   const int A_ATOM = args.a_rows * 128;
   const int AT = args.atoms;
@@ -131,7 +133,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
   // order of the 256-wide tile they make up, and the odd one starts with its second accumulator.
   auto chain_lo = [&](int i) { return args.kc * i / args.chains; };
   auto rot_of = [&](int tile) {
-    return (kChains && args.chains > 1 ? (tile >> 1) * ST_ROT + chain_lo(tile & 1) : tile * ST_ROT) % args.kc;
+    return (kChains ? (tile >> 1) * ST_ROT + chain_lo(tile & 1) : tile * ST_ROT) % args.kc;
   };
   auto pos_set = [&](Pos& p, int u) {
     p.tile = u / args.kc;
@@ -271,7 +273,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         uint32_t d_tmem = tmem_base + (uint32_t)(buf * SET_COLS);
         uint32_t acc = 0;                               // 0: the next MMA overwrites the accumulator
         int chain = 0, next_acc = seg_end;              // the first unit of the next accumulator
-        if (kChains && args.chains > 1) {
+        if (kChains) {
           chain = vt & 1;
           d_tmem += (uint32_t)(chain * BN);
           next_acc = u + chain_lo(chain + 1) - chain_lo(chain);
@@ -333,7 +335,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       const int tile = vt;
       const int tile_u0 = vt * args.kc;
       const int seg_end = min(u1, tile_u0 + args.kc);
-      const bool whole = (u == tile_u0) && (seg_end == tile_u0 + args.kc);
+      const bool whole = kChains || ((u == tile_u0) && (seg_end == tile_u0 + args.kc));
       const int buf = seg % NBUF, use = seg / NBUF;
       const int j0 = tile * CH;
       // what the first chunk's epilogue reads is fetched while the MMAs run (see EpiPre)
@@ -562,7 +564,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       u = seg_end;
     }
   }
-  if (args.exchange) {
+  if (!kChains && args.exchange) {
     // Pair exchange: after the barrier each CTA adds, for its own half of the chunks, its accumulator (still in tensor
     // memory) and the peer's published piece, and runs the fused epilogue.  One row per thread, as in the plain epilogue;
     // the next chunk's piece and what its epilogue reads are requested before the current one is finished.
@@ -641,7 +643,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       cluster_sync();
     }
     cluster_sync();      // nobody leaves while its peer may still read its shared memory
-  } else if (args.cluster > 1) {
+  } else if (!kChains && args.cluster > 1) {
     // Split-K reduction inside the cluster: every CTA's partial tile sits in its shared memory; after the barrier CTA
     // rank r sums, for its share of the 16-column chunks, the partials of all ranks in rank order (= K order, so the
     // result does not depend on timing) straight from their shared memory, and runs the fused epilogue on them.
@@ -812,8 +814,6 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
   const StreamShape sh = stream_shape(st, M, BN, K);
   if (sh.stages < 2) { st.err = "not enough shared memory for the streaming GEMM"; return -2; }
   const size_t smem = (size_t)sh.stages * sh.stage_bytes + sh.aux;
-  const cudaError_t smem_rc = umma_raise_smem(st, k_gemm_stream<BN, Epi>);
-  if (smem_rc != cudaSuccess) { st.err = cudaGetErrorString(smem_rc); return -3; }
   const CUtensorMap* ma = umma_map4(st, A, M, M, 1, K, sh.a_rows, 1, sh.atoms);
   if (!ma) return -4;
   WeightView v{W0, n_rows_w, 1, n_rows_w, 1, 0, BN, 1};
@@ -864,7 +864,13 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
       chains = std::max(1, std::min(stream_splits(st, (T + 1) / 2, stream_no_split<Epi>(K)), std::min(4, kc)));
   }
   StreamArgs args{M, NP, n_tiles, cluster, exchange, kc, chains, sh.a_rows, sh.atoms, one_copy, rot_half, sh.stages, st.scratch, st.counters, status};
-  cudaError_t e = launch_k(st.pdl, k_gemm_stream<BN, Epi>, dim3(grid), dim3(ST_THREADS), smem, stream, cluster, *ma, mb0v,
+  auto kern = k_gemm_stream<BN, Epi>;
+  if constexpr (std::is_same<Epi, EpiQKVRope<bf16>>::value && BN == 128) {
+    if (chains > 1) kern = k_gemm_stream<BN, Epi, true>;
+  }
+  const cudaError_t smem_rc = umma_raise_smem(st, kern);
+  if (smem_rc != cudaSuccess) { st.err = cudaGetErrorString(smem_rc); return -3; }
+  cudaError_t e = launch_k(st.pdl, kern, dim3(grid), dim3(ST_THREADS), smem, stream, cluster, *ma, mb0v,
                            mb1v, args, e2);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) { st.err = cudaGetErrorString(e); return -5; }

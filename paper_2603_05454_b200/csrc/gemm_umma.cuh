@@ -497,10 +497,10 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
 //    gains: +0.7 ms per LLaDA-shaped pass.  Not kept.)
 //  * plain and rotary ones 128, which needs no K split with 96 tiles.  With at most 32 rows a wide plain GEMM takes 256 (its partial
 //    tiles are small, and half as many MMA instructions are issued), and so does a rotary one whose 128-wide tiles would be split
-//    anyway; 96 whole tiles of 128 save the K slices' sum instead (12288 x 4096 in passes of 9 / 32 rows: 3.70 -> 3.57, 3.86 -> 3.69 ms).  K
+//    anyway; 96 whole tiles of 128 save the K slices' sum instead (12288 x 4096 in passes of 9 / 32 rows: 3.70 -> 3.58, 3.86 -> 3.68 ms).  K
 //    then runs in as many accumulators as the 256-wide tiles would have slices, chunk by chunk in their order: one chain would be
-//    longer than theirs, and the tensor core's error grows with the chain (see umma_head_shape); it would save another 0.8 %.  The
-//    results are those of the 256-wide tiles to the bit.
+//    longer than theirs, and the tensor core's error grows with the chain (see umma_head_shape); it was no faster (9 rows 3.58 and 3.58
+//    ms).  The results are those of the 256-wide tiles to the bit.
 //    A rotary half tile is whole head halves.
 // A shape the kernel cannot take (none of a transformer layer's: it would need more than 4096 column tiles in a launch whose
 // tiles are split between CTAs) is an error, not a fallback.
