@@ -11,15 +11,19 @@
 //     end; while one group computes, the tensor pipe works for the other;
 //   * the weights P go to tensor memory, over the scores they were computed from, and are the A operand of P V from there: neither
 //     their store nor the MMAs' reads of them touch shared memory.
-// One warp issues all MMAs.  They execute in order, so P V of a tile and Q K^T of the next one follow each other without a wait, and
-// scores that have arrived tell the softmax group that its previous P V is complete.
+// One warp issues all MMAs.  They execute in the order of issue, so P V of a tile and Q K^T of the next one, which writes over P, follow
+// each other without a wait.  (PTX states that order for MMAs into one accumulator; between two the kernel rests on the one tensor pipe of
+// an SM, as the published attention kernels for this chip that keep P over S do.  A wait in between would put another 530 cycles into the
+// chain of about 4000 that a tile takes.)  A commit covers all that was issued before it, so scores that have arrived tell the softmax
+// group that its previous P V is complete.
 // The running maximum is raised lazily, as in attention_umma.cuh, from the fifth tile on; in the first four it follows the scores (to a
 // quarter), and the row sum adds the weights as they were rounded.  Here a row has one maximum where that kernel has two: only the
 // weight of a key that was the maximum is 1 and without rounding error, and the sum of the rounded weights takes out what their errors
 // share.  Error against 64 bits relative to that kernel's, 500 to 4300 keys, scores of standard deviation 0.3 / 1 / 4: fp32 sum and all
-// tiles lazy 1.003 / 1.022 / 1.07 at worst; now 1.001 / 0.993 / 0.92.  With two key tiles that kernel's two maxima are all there are
-// (1.015), so it takes those passes.  The launch of 16 x 515 rows over 2100 keys alone 458 -> 494 us (that kernel 464); in passes, which run at
-// the power limit, it stays the faster one: see above.
+// tiles lazy 1.003 / 1.022 / 1.07 at worst; now 1.001 / 0.998 / 0.92.  With two key tiles that kernel's two maxima are all there are
+// (1.015), so it takes those passes.  The launch of 16 x 515 rows over 2100 keys alone 458 -> 494 us (that kernel 464); in passes, which
+// run at the power limit, it stays the faster one: see above.  (O gathers all key tiles in one accumulator where that kernel has two: the
+// bias of the tensor core's truncation is 1.6e-5 of an output at 4300 keys of one sign, 0.9e-5 there, under a rounding to bf16 of 1.4e-3.)
 // Warps 0..3 and 4..7 = softmax groups 0 and 1; warps 8 and 11 = TMA producers of the K and the V tiles, warp 9 = TMEM allocator and MMA
 // issuer.  Every wait is bounded; on expiry the kernel records (code, site), drains and returns.
 #pragma once
