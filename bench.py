@@ -58,13 +58,15 @@ CLASS_SOURCES = {
 }
 NCU_TRAFFIC = {
     # k_gemm_stream<128,EpiStore>, M 64, N 12288, K 4096: profiles/k_gemm_stream_M64_N12288_K4096.md
-    "gemm": {"captured_bytes": 104.38e6, "algorithmic_bytes": 102.8e6, "src": "9afdf6ac6d78"},
+    "gemm": {"captured_bytes": 104.71e6, "algorithmic_bytes": 102.8e6, "src": "c77653dd2af2"},
     # k_gemm_stream<256,EpiHead>, 64 rows: profiles/k_gemm_stream_head_M64_V126464.md
-    "head": {"captured_bytes": 1062.3e6, "algorithmic_bytes": 1037.0e6, "src": "9afdf6ac6d78"},
+    "head": {"captured_bytes": 1062.2e6, "algorithmic_bytes": 1037.0e6, "src": "c77653dd2af2"},
     # k_attn_umma, 16 x (128 query rows over 2048 keys): profiles/k_attn_umma_B16_F1920.md
-    "attn": {"captured_bytes": 570.2e6, "algorithmic_bytes": 570.4e6, "src": "acda8c1a1de6"},
+    "attn": {"captured_bytes": 569.7e6, "algorithmic_bytes": 570.4e6, "src": "3b011640f8e1"},
+    # k_attn_rows, 16 x (2048 query rows over 2048 keys): profiles/k_attn_rows.md
+    "attn_rows": {"captured_bytes": 1053.3e6, "algorithmic_bytes": 1073.7e6, "src": "3b011640f8e1"},
     # k_commit_append of a 16 x 1920-row prompt block: profiles/k_commit_append_prompt_B16_P1920.md
-    "commit": {"captured_bytes": 1969.9e6, "algorithmic_bytes": 2013.3e6, "src": "7475a23aa56d"},
+    "commit": {"captured_bytes": 1968.0e6, "algorithmic_bytes": 2013.3e6, "src": "342142007f56"},
 }
 
 
@@ -254,7 +256,8 @@ def class_report(cnt, tms, peaks):
                 e["tflops"] = round(f / (ms * 1e-3) / 1e12, 1)
                 e["tensor_frac_sustained"] = round(e["tflops"] / tc, 4)
             e["bytes_per_launch"] = round(b / n) if n else None
-        t = NCU_TRAFFIC.get(name)
+        # attention of 256 and more rows a sequence (about 200 flops per byte and up) runs two row tiles per CTA
+        t = NCU_TRAFFIC.get("attn_rows" if name == "attn" and work[name][1] > 200 * work[name][0] else name)
         e["traffic"] = None
         captured_regime = name not in ("gemm", "head") or work[name][1] <= 256 * work[name][0]
         if t and n and name in work and captured_regime and t.get("src") == source_hash(name):
