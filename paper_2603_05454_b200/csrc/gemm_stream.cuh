@@ -79,7 +79,7 @@ constexpr int ST_THREADS = 224;
 // tile still cover it, and results do not depend on timing.
 constexpr int ST_ROT = 4;
 
-// kChains: the rotary epilogue's several accumulators (args.chains), one whole tile per CTA: a kernel of its own, because the one without
+// kChains: the rotary epilogue of few rows, whose tiles take K as args.chains slices, one whole tile per CTA: a kernel of its own, as the one without
 // them runs with up to 128 rows and was 0.5 to 0.8 % of a pass slower for them.
 template <int BN, typename Epi, bool kChains = false>
 __global__ void __launch_bounds__(ST_THREADS, 1)
@@ -274,7 +274,7 @@ k_gemm_stream(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         uint32_t acc = 0;                               // 0: the next MMA overwrites the accumulator
         int chain = 0, next_acc = seg_end;              // the first unit of the next accumulator
         if (kChains) {
-          chain = vt & 1;
+          chain = (vt & 1) % args.chains;
           d_tmem += (uint32_t)(chain * BN);
           next_acc = u + chain_lo(chain + 1) - chain_lo(chain);
         }
@@ -857,8 +857,8 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
       exchange = (splits == 2 && st.stream_exchange && M >= st.stream_exchange_rows) ? 1 : 0;
     }
   }
-  // a rotary tile of few rows that 256-wide tiles would split over K (see umma_gemm): as many accumulators as that had slices
-  int chains = 1;
+  // rotary tiles of few rows in place of 256-wide ones (see umma_gemm): as many accumulators as those would have K slices
+  int chains = 0;
   if constexpr (std::is_same<Epi, EpiQKVRope<bf16>>::value && BN == 128) {
     if (M <= 32 && grid == T && st.stream_bn == 0)
       chains = std::max(1, std::min(stream_splits(st, (T + 1) / 2, stream_no_split<Epi>(K)), std::min(4, kc)));
@@ -866,7 +866,7 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
   StreamArgs args{M, NP, n_tiles, cluster, exchange, kc, chains, sh.a_rows, sh.atoms, one_copy, rot_half, sh.stages, st.scratch, st.counters, status};
   auto kern = k_gemm_stream<BN, Epi>;
   if constexpr (std::is_same<Epi, EpiQKVRope<bf16>>::value && BN == 128) {
-    if (chains > 1) kern = k_gemm_stream<BN, Epi, true>;
+    if (chains > 0) kern = k_gemm_stream<BN, Epi, true>;
   }
   const cudaError_t smem_rc = umma_raise_smem(st, kern);
   if (smem_rc != cudaSuccess) { st.err = cudaGetErrorString(smem_rc); return -3; }

@@ -359,10 +359,10 @@ def test_rotary_projection_on_pairs_of_sms(dh, hq, hkv, bn):
 
 @pytest.mark.parametrize("P", [5, 28])
 @pytest.mark.parametrize("dh,hq,hkv,d", [(128, 32, 32, 4096), (128, 72, 2, 1088), (128, 120, 12, 1152), (64, 64, 64, 1024), (128, 73, 1, 576),
-                                         (128, 32, 32, 512)])
+                                         (128, 32, 32, 512), (128, 112, 16, 320), (64, 70, 70, 192)])
 def test_rotary_projection_of_few_rows_keeps_its_sums(dh, hq, hkv, d, P):
-    """75 to 148 whole tiles of 128 columns add K in the slices, and in the order, of the 256-wide tiles (23 = 256) that are split over two
-    or three CTAs: the cache rows of the two are equal to the bit."""
+    """75 to 148 whole tiles of 128 columns add K in the slices, and in the order, of the 256-wide tiles (23 = 256) that would be split over two
+    or three CTAs, or not (K <= 512): the cache rows of the two are equal to the bit."""
     from paper_2603_05454_b200 import LSPDecoder, SchedCfg
     G = 4
     sh = S.ModelShape(1, d, hq, hkv, dh, 64, 256, dtype="bf16")
