@@ -785,6 +785,11 @@ inline StreamShape stream_shape(const UmmaState& st, int M, int bn, int K) {
   return sh;
 }
 
+// Most bytes between the two halves (gate and up) of a weight tile that one copy brings.  A tensor map takes strides up to 2^40, but a box
+// that spans more than a gigabyte read elsewhere: with the tensors 1.18 GB apart (64 pairs, K 512) a launch ended in an illegal memory
+// access, at 0.83 GB and below it does not.  Halves further apart come by a copy each: with those 30 cases up to 4.4 GB apart are right.
+constexpr size_t ST_MAX_SPAN = (size_t)1 << 29;
+
 // Asks the runtime how many clusters of 2 ... 8 CTAs of the streaming kernel (one CTA per SM) can be resident at once.
 inline void stream_query_clusters(UmmaState& st) {
   auto kern = k_gemm_stream<128, EpiStore<bf16>>;
@@ -827,7 +832,7 @@ int stream_launch(UmmaState& st, cudaStream_t stream, const bf16* A, const bf16*
     const bool flip = (uintptr_t)W1 < (uintptr_t)W0;
     const size_t dist = flip ? (const char*)W0 - (const char*)W1 : (const char*)W1 - (const char*)W0;
     v = WeightView{flip ? W1 : W0, n_rows_w, 1, n_rows_w, 2, dist, BN / 2, 1};
-    if (dist == 0 || dist >= ((size_t)1 << 40) || (dist & 15) || st.stream_split_copies) { one_copy = 0; v.base = W0; v.halves = 1; }
+    if (dist == 0 || dist >= ST_MAX_SPAN || (dist & 15) || st.stream_split_copies) { one_copy = 0; v.base = W0; v.halves = 1; }
     else if (flip) e2.flip = 1;
   }
   const CUtensorMap* mb0 = umma_map5(st, v, K, one_copy ? sh.atoms : 1);

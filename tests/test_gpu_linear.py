@@ -401,6 +401,23 @@ def test_swiglu_weights_by_one_copy_in_either_order(M, N, K, opts, up_first):
     dec.close()
 
 
+@pytest.mark.parametrize("up_first", [False, True])
+@pytest.mark.parametrize("gap", [0x20000000, 0x46402C00])
+def test_swiglu_weights_far_apart(gap, up_first):
+    """Gate and up projection half a gigabyte and more apart: no copy spans the two (see ST_MAX_SPAN)."""
+    dec = _dec("bf16")
+    M, N, K, bf = 26, 192, 512, torch.bfloat16
+    A, W, W2 = S.normal((M, K), 3, 1, 1.0, bf, DEV), S.normal((N, K), 3, 2, 0.05, bf, DEV), S.normal((N, K), 3, 3, 0.05, bf, DEV)
+    both = torch.empty(gap + N * K * 2, dtype=torch.uint8, device=DEV)
+    at = lambda o, t: both[o:o + N * K * 2].view(bf).view(N, K).copy_(t)  # noqa: E731
+    w, w2 = at(gap if up_first else 0, W), at(0 if up_first else gap, W2)
+    out = torch.empty(M, N, dtype=bf, device=DEV)
+    dec.op_linear(2, A, w, w2, out)
+    dec.close()
+    ref = torch.nn.functional.silu(A.double() @ W.double().t()) * (A.double() @ W2.double().t())
+    assert bool(((out.double() - ref).abs() <= ref.abs() / 128 + 1e-3 * ref.abs().max()).all())      # one bf16 ulp, sums that cancel
+
+
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
 @pytest.mark.parametrize("M,N,K", [(1, 16, 64), (31, 48, 64), (33, 1040, 192), (128, 256, 1024), (129, 384, 256),
                                    (1200, 1024, 128), (1217, 1040, 64)])
