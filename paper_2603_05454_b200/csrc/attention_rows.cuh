@@ -104,12 +104,12 @@ k_attn_rows(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   // tensor memory columns: O of row tile w at 128 w; its scores at 256 + 128 w, over whose first 64 columns the weights go
   if (!early) pdl_wait();        // (see k_attn_umma)
 
-  const int r0 = sd.row_off[b];
-  const int Qn = sd.row_off[b + 1] - r0;
+  const int r0 = __ldcg(sd.row_off + b);
+  const int Qn = __ldcg(sd.row_off + b + 1) - r0;
   const int pos_tile = AU_BM / G;                       // whole query positions of G heads each per row tile
   const int pos0 = (int)blockIdx.x * 2 * pos_tile;
   const int n_w = pos0 >= Qn ? 0 : pos0 + pos_tile >= Qn ? 1 : 2;        // row tiles with rows
-  const int F = sd.F[b] + (inplace ? Qn : 0);
+  const int F = __ldcg(sd.F + b) + (inplace ? Qn : 0);
   const int n_c = (F + AU_BN - 1) / AU_BN, n_s = inplace ? 0 : (Qn + AU_BN - 1) / AU_BN;
   const int n_tiles = n_w > 0 ? n_c + n_s : 0;
   const int ldq = n_heads * DH;

@@ -176,11 +176,12 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   // early: the kernel before this one is the QKV projection, which releases this launch only after its own wait.  Everything
   // older than it is complete then: the descriptor and the cached keys and values are read while it still runs.  In a small pass
   // the queries were there 2.4 us after the wait and the first keys 3.5 (of 11.5 in all); LLaDA-shaped passes of 9 / 101 / 187 rows
-  // 3.63 -> 3.57, 4.17 -> 4.13, 5.21 -> 5.15 ms.
+  // 3.63 -> 3.57, 4.17 -> 4.13, 5.21 -> 5.15 ms.  (The descriptor by loads past L1: only the wait is stated to make a line that an
+  // earlier kernel left there invalid.)
   if (!early) pdl_wait();
 
-  const int r0 = sd.row_off[b];
-  const int Qn = sd.row_off[b + 1] - r0;
+  const int r0 = __ldcg(sd.row_off + b);
+  const int Qn = __ldcg(sd.row_off + b + 1) - r0;
   // With clusters (size C along x) the C CTAs of a cluster share one row tile and deal its key tiles round-robin:
   // rank r takes tiles r, r + C, ...; their partial (m, l, O) are merged through distributed shared memory at the end.
   const int C = cluster > 1 ? cluster : 1;
@@ -189,7 +190,7 @@ k_attn_umma(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   const int pos_tile = AU_BM / G;
   const int pos0 = (int)(blockIdx.x / C) * pos_tile;
   // in-place layout: this pass's K/V rows already sit behind the prefix in the cache, so every key tile is a cache tile
-  const int F = sd.F[b] + (inplace ? Qn : 0);
+  const int F = __ldcg(sd.F + b) + (inplace ? Qn : 0);
   const int n_c = (F + AU_BN - 1) / AU_BN, n_s = inplace ? 0 : (Qn + AU_BN - 1) / AU_BN;
   const int n_all = (pos0 < Qn) ? n_c + n_s : 0;       // a CTA past the last row does nothing
   const int n_tiles = n_all > rank ? (n_all - rank + C - 1) / C : 0;   // this CTA's tiles; t below counts them

@@ -65,6 +65,7 @@ def test_attention_reads_only_older_rows_ahead_of_its_wait(name):
     those that end ahead of the pass's first row)."""
     _, (ahead, *roles) = _roles(name)
     assert "if (!early) pdl_wait();" in ahead
+    assert len(re.findall(r"__ldcg\(sd\.\w+ \+ b(?: \+ 1)?\)", ahead)) == len(re.findall(r"\bsd\.", ahead)) == 3      # past L1
     copies = [r for r in roles if re.search(r"tma_load|load_tile\(", r)]
     assert len(copies) == 1
     early = copies[0].split("pdl_wait();")[0]
