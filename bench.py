@@ -62,9 +62,9 @@ NCU_TRAFFIC = {
     # k_gemm_stream<256,EpiHead>, 64 rows: profiles/k_gemm_stream_head_M64_V126464.md
     "head": {"captured_bytes": 1063.1e6, "algorithmic_bytes": 1037.0e6, "src": "8993dfc1061c"},
     # k_attn_umma, 16 x (128 query rows over 2048 keys): profiles/k_attn_umma_B16_F1920.md
-    "attn": {"captured_bytes": 569.7e6, "algorithmic_bytes": 570.4e6, "src": "3b011640f8e1"},
+    "attn": {"captured_bytes": 569.9e6, "algorithmic_bytes": 570.4e6, "src": "d3cb1b41f6dd"},
     # k_attn_rows, 16 x (2048 query rows over 2048 keys): profiles/k_attn_rows.md
-    "attn_rows": {"captured_bytes": 1053.3e6, "algorithmic_bytes": 1073.7e6, "src": "3b011640f8e1"},
+    "attn_rows": {"captured_bytes": 1053.0e6, "algorithmic_bytes": 1073.7e6, "src": "d3cb1b41f6dd"},
     # k_commit_append of a 16 x 1920-row prompt block: profiles/k_commit_append_prompt_B16_P1920.md
     "commit": {"captured_bytes": 1968.0e6, "algorithmic_bytes": 2013.3e6, "src": "342142007f56"},
 }
